@@ -3,16 +3,18 @@
 // 6-point degree-4 triangle rule (Strang & Fix / Dunavant) on both triangles.
 //
 // Structure of one apply y = B_far x:
-//   1. far_prep_kernel   (per source triangle)  densities at the 6 source
+//   1. far_prep_kernel   (per source rule point)  densities at the 6 source
 //      points and the surface-curl vector of the phi density, FP32;
-//   2. far_kernel        (per test point)       N-body sum over all source
+//   2. far_kernel        (per test triangle)       N-body sum over all source
 //      points staged through shared memory in tiles of triangles; both
 //      wavenumbers are evaluated from one distance; the source range is split
 //      over gridDim.y so that the grid fills every SM; partial sums per test
-//      point go to d_part (no atomics);
-//   3. gather_kernel     (per vertex)           sums the partials of the test
-//      points of the incident triangles with the test weights (FP64) and adds
-//      the near-field CSR product (touching pairs, Sauter-Schwab values).
+//      point (u1, u2) and per test triangle (curl term) go to d_part, d_partA
+//      (no atomics);
+//   3. gather_kernel     (a group of lanes per vertex)  sums the partials of
+//      the test points of the incident triangles with the test weights (FP64)
+//      and adds the near-field CSR product (touching pairs, Sauter-Schwab
+//      values).
 //
 // Kernel identities (G = e^{ikr}/(4 pi r), d = x - y, r = |d|):
 //   dG/dn_y = H (y - x).n_y,  dG/dn_x = H (x - y).n_x,
@@ -46,11 +48,32 @@ constexpr int FAR_THREADS = 128;
 // resident blocks per SM the one-right-hand-side kernel is compiled for
 // (registers per thread = 65536 / (FAR_THREADS x FAR_MIN_BLOCKS))
 #ifndef OSRC_FAR_MIN_BLOCKS
-#define OSRC_FAR_MIN_BLOCKS 4
+#define OSRC_FAR_MIN_BLOCKS 2
 #endif
 // largest k_max x (bounding-box diagonal) for the plain (FP32 k r) variant
 constexpr double FAR_PLAIN_MAX_PHASE = 32.0 * 3.14159265358979323846;
 constexpr int FAR_TS = 64;  // source triangles per shared-memory tile
+#ifndef OSRC_FAR_QUNROLL
+#define OSRC_FAR_QUNROLL 3
+#endif
+#ifndef OSRC_FAR_HUNROLL
+#define OSRC_FAR_HUNROLL 2
+#endif
+constexpr int FAR_QUNROLL = OSRC_FAR_QUNROLL, FAR_HUNROLL = OSRC_FAR_HUNROLL;  // unrolls of the rule-point loops
+constexpr int FAR_MIN_TPS = 16;  // fewest source triangles per split
+// test triangles per block: 32 below FAR_TRIS32_NT triangles, 64 below
+// FAR_TRIS64_NT, else FAR_THREADS (128).  Measured: 5136 triangles on four
+// objects 2.136 ms with 128, 2.145 with 64, 2.256 with 32; 296 triangles
+// 38 us with 32 sharing the sources between four warps, 46 us without
+constexpr int FAR_TRIS32_NT = 2048;
+constexpr int FAR_TRIS64_NT = 4096;
+constexpr int FAR_MAX_NS = 64;   // most source splits
+// lanes of the gather per vertex: a block up to GATHER_BLOCK_NV vertices, a
+// warp up to GATHER_WARP_NV, then 8 (150 vertices: block 38 us an apply, warp
+// 41; 642: warp 10.28 ms a solve, block 10.38, 8 lanes 10.60; 2568: 8 lanes
+// 2.140 ms an apply, warp 2.145)
+constexpr int GATHER_BLOCK_NV = 400;
+constexpr int GATHER_WARP_NV = 1500;
 
 __global__ void far_geom_kernel(const double *__restrict__ verts, const int *__restrict__ tris,
                                 int nt, float4 *__restrict__ pt, float4 *__restrict__ poff,
@@ -96,7 +119,17 @@ __global__ void far_geom_kernel(const double *__restrict__ verts, const int *__r
     cen[2 * t + 1] = make_float4(lo[0], lo[1], lo[2], 0.f);
     const double h = n[0] * P[0][0] + n[1] * P[0][1] + n[2] * P[0][2];
     tn[t] = make_float4((float)n[0], (float)n[1], (float)n[2], (float)h);
-    tv[t] = make_int4(v[0], v[1], v[2], 0);
+    // w: bits of n.(P0 - x_0) with the FP32 normal and the FP32 first rule
+    // point x_0, the distance of x_0 from the plane that its rounding made
+    {
+        const double x0 = (1.0 - 2.0 * kQa1) * P[0][0] + kQa1 * (P[1][0] + P[2][0]);
+        const double x1 = (1.0 - 2.0 * kQa1) * P[0][1] + kQa1 * (P[1][1] + P[2][1]);
+        const double x2 = (1.0 - 2.0 * kQa1) * P[0][2] + kQa1 * (P[1][2] + P[2][2]);
+        const double off = (double)(float)n[0] * (P[0][0] - (double)(float)x0) +
+                           (double)(float)n[1] * (P[0][1] - (double)(float)x1) +
+                           (double)(float)n[2] * (P[0][2] - (double)(float)x2);
+        tv[t] = make_int4(v[0], v[1], v[2], __float_as_int((float)off));
+    }
     double *g = tgeo + 16 * (size_t)t;
     g[0] = area;
     g[1] = n[0];
@@ -109,25 +142,27 @@ __global__ void far_geom_kernel(const double *__restrict__ verts, const int *__r
     g[13] = g[14] = g[15] = 0.0;
 }
 
-// Source data of one apply, duplicated into (value, value) pairs and stored
-// with both signs, so that the far kernel's packed FP32 instructions (two
-// test points per thread) take every operand of a complex multiply-add
-// straight from shared memory, without moves or negations:
-//   sP[5k]   = (-y.x, -y.x, -y.y, -y.y)     sP[5k+1] = (-y.z, -y.z, psi.re, psi.re)
-//   sP[5k+2] = (psi.im, psi.im, -psi.re, -psi.re)
-//   sP[5k+3] = (-psi.im, -psi.im, phi.re, phi.re)
-//   sP[5k+4] = (phi.im, phi.im, -phi.re, -phi.re)   sP5[k] = (-phi.im, -phi.im)
+// Source data of one apply, duplicated into (value, value) pairs, the values
+// that enter with both signs stored with both, so that the far kernel's
+// packed FP32 instructions (two test points per pair of lanes) take every
+// operand of a complex multiply-add straight from shared memory, without
+// moves or negations:
+//   sP[4k]   = (-y.x, -y.x, -y.y, -y.y)     sP[4k+1] = (-y.z, -y.z, psi.re, psi.re)
+//   sP[4k+2] = (psi.im, psi.im, -psi.im, -psi.im)
+//   sP[4k+3] = (phi.re, phi.re, phi.im, phi.im)    sP5[k] = (-phi.im, -phi.im)
 // with psi_q = w_q |s| sum_b lambda_b(q) psi_b (the same for phi); per
 // triangle c_s = |s| sum_b phi_b curl phi_b as
-//   sC[5t] = (cx.re, cx.re, cx.im, cx.im)   sC[5t+1] = (-cx.im, -cx.im, cy.re, cy.re)
-//   sC[5t+2] = (cy.im, cy.im, -cy.im, -cy.im)   sC[5t+3] = (cz.re, cz.re, cz.im, cz.im)
-//   sC[5t+4] = (-cz.im, -cz.im, 0, 0)
+//   sC[2t] = (cx.re, cx.im, cy.re, cy.im)   sC[2t+1] = (cz.re, cz.im, 0, 0)
+// One thread per rule point (FP64 is slow here and its chains are short this
+// way: the 150-vertex hull's densities took 11 us with a thread per
+// triangle); threads q < 3 also form component q of c_s.
 __global__ void far_prep_kernel(const double2 *__restrict__ x, int nv, int nt,
                                 const int *__restrict__ tris, const float4 *__restrict__ pt,
                                 const double *__restrict__ tgeo, float4 *__restrict__ sP,
                                 float2 *__restrict__ sP5, float4 *__restrict__ sC) {
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= nt) return;
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= 6 * nt) return;
+    const int t = k / 6, q = k - 6 * (k / 6);
     double2 ps[3], ph[3];
     for (int a = 0; a < 3; ++a) {
         const int v = tris[3 * t + a];
@@ -136,40 +171,30 @@ __global__ void far_prep_kernel(const double2 *__restrict__ x, int nv, int nt,
     }
     const double *g = tgeo + 16 * (size_t)t;
     const double area = g[0];
-    for (int q = 0; q < 6; ++q) {
-        double b[3], w;
-        rule_point(q, b, w);
-        const double W = w * area;
-        double2 s = cd(0, 0), f = cd(0, 0);
-        for (int a = 0; a < 3; ++a) {
-            s = cadd(s, cscale(ps[a], b[a]));
-            f = cadd(f, cscale(ph[a], b[a]));
-        }
-        const float4 p = pt[6 * t + q];
-        const float psr = (float)(W * s.x), psi = (float)(W * s.y);
-        const float phr = (float)(W * f.x), phi = (float)(W * f.y);
-        const size_t k = 6 * (size_t)t + q;
-        float4 *d = sP + 5 * k;
-        d[0] = make_float4(-p.x, -p.x, -p.y, -p.y);
-        d[1] = make_float4(-p.z, -p.z, psr, psr);
-        d[2] = make_float4(psi, psi, -psr, -psr);
-        d[3] = make_float4(-psi, -psi, phr, phr);
-        d[4] = make_float4(phi, phi, -phr, -phr);
-        sP5[k] = make_float2(-phi, -phi);
+    double b[3], w;
+    rule_point(q, b, w);
+    const double W = w * area;
+    double2 s = cd(0, 0), f = cd(0, 0);
+    for (int a = 0; a < 3; ++a) {
+        s = cadd(s, cscale(ps[a], b[a]));
+        f = cadd(f, cscale(ph[a], b[a]));
     }
-    float cr[3], ci[3];
-    for (int j = 0; j < 3; ++j) {
+    const float4 p = pt[k];
+    const float psr = (float)(W * s.x), psi = (float)(W * s.y);
+    const float phr = (float)(W * f.x), phi = (float)(W * f.y);
+    float4 *d = sP + 4 * (size_t)k;
+    d[0] = make_float4(-p.x, -p.x, -p.y, -p.y);
+    d[1] = make_float4(-p.z, -p.z, psr, psr);
+    d[2] = make_float4(psi, psi, -psi, -psi);
+    d[3] = make_float4(phr, phr, phi, phi);
+    sP5[k] = make_float2(-phi, -phi);
+    if (q < 3) {
         double2 cv = cd(0, 0);
-        for (int a = 0; a < 3; ++a) cv = cadd(cv, cscale(ph[a], g[4 + 3 * a + j]));
-        cr[j] = (float)(cv.x * area);
-        ci[j] = (float)(cv.y * area);
+        for (int a = 0; a < 3; ++a) cv = cadd(cv, cscale(ph[a], g[4 + 3 * a + q]));
+        float2 *c = reinterpret_cast<float2 *>(sC + 2 * (size_t)t);
+        c[q] = make_float2((float)(cv.x * area), (float)(cv.y * area));
+        if (q == 0) c[3] = make_float2(0.f, 0.f);
     }
-    float4 *c = sC + 5 * (size_t)t;
-    c[0] = make_float4(cr[0], cr[0], ci[0], ci[0]);
-    c[1] = make_float4(-ci[0], -ci[0], cr[1], cr[1]);
-    c[2] = make_float4(ci[1], ci[1], -ci[1], -ci[1]);
-    c[3] = make_float4(cr[2], cr[2], ci[2], ci[2]);
-    c[4] = make_float4(-ci[2], -ci[2], 0.f, 0.f);
 }
 
 typedef float2 f2;
@@ -188,13 +213,18 @@ struct FarConst2 {
     f2 k0, k1, nk0, nk1, rho, irho, dk0, dk1;
 };
 
-// Accumulators of the two test points of a thread, packed (point a, point b):
-// tile sums of u1, u2 (complex) and of the curl vector A (3 complex), and
-// the per-source-triangle sums T1n = -sum_q Hs phi_q, U = sum_q Gk phi_q,
-// T3 = sum_q w_q Gd.
+// Accumulators of two test points, packed (point a, point b): tile sums of
+// u1, u2 (complex) and the per-source-triangle sums T1n = -sum_q Hs phi_q,
+// U = sum_q Gk phi_q.
 struct PairAcc {
-    f2 u1r, u1i, u2r, u2i, axr, axi, ayr, ayi, azr, azi;
-    f2 t1r, t1i, ur, ui, t3r, t3i;
+    f2 u1r, u1i, u2r, u2i;
+    f2 t1r, t1i, ur, ui;
+};
+
+// Unweighted sums of G0 and G1 over the pairs of a thread and the source
+// points of one weight class (lane x: test points 0..2, lane y: 3..5).
+struct CurlAcc {
+    f2 g0r, g0i, g1r, g1i;
 };
 
 // Per (test triangle, source triangle) data of the centred (large k r)
@@ -203,12 +233,29 @@ struct PairAcc {
 // revolution in [-1/2, 1/2], from float-float arithmetic (about 48 bits).
 struct CenterPair {
     f2 Dx, Dy, Dz, rc, b0, b1;
+    float lx, ly, lz;  // low parts of D
 };
 
 __device__ __forceinline__ void two_sum(float a, float b, float &s, float &e) {
     s = a + b;
     const float v = s - a;
     e = (a - (s - v)) + (b - v);
+}
+
+// s + e += v exactly up to the rounding of e
+__device__ __forceinline__ void comp_add(float &s, float &e, float v) {
+    float t, d;
+    two_sum(s, v, t, d);
+    s = t;
+    e += d;
+}
+
+// the same with Dekker's FastTwoSum (exact for |s| >= |v|, else the error
+// term misses at most a rounding of v: sums whose terms rarely exceed them)
+__device__ __forceinline__ void comp_add_fast(float &s, float &e, float v) {
+    const float t = s + v;
+    e += v - (t - s);
+    s = t;
 }
 
 // a - b for float-float a = (ah, al), b = (bh, bl); result (h, l)
@@ -264,6 +311,9 @@ __device__ __forceinline__ CenterPair center_pair(const float4 &cth, const float
     c.Dx = dup2(dh[0]);
     c.Dy = dup2(dh[1]);
     c.Dz = dup2(dh[2]);
+    c.lx = dl[0];
+    c.ly = dl[1];
+    c.lz = dl[2];
     c.rc = dup2(rh);
     // reduced centroid phases in radians (in [-pi, pi])
     c.b0 = dup2(6.28318530717958647692f * ff_phase_rev(rh, rl, k0h, k0l));
@@ -271,10 +321,15 @@ __device__ __forceinline__ CenterPair center_pair(const float4 &cth, const float
     return c;
 }
 
-// One source point against the two test points of the thread, both
-// wavenumbers, packed FP32 arithmetic.  P[0..4], P5 hold the signed
-// duplicated source data; (mnx, mny, mnz) is the negated test-triangle
-// normal; wq2 the rule weight.  Plain variant: (X, Y, Z) are the test points
+// One source point against the six test points of a triangle (three pairs),
+// both wavenumbers, packed FP32 arithmetic.  P0..P3, P5 hold the signed
+// duplicated source data; (y - x).n_x is the same for every test point (they
+// lie in the triangle's plane) and is formed once: from the first test point,
+// corrected by pdn = n.(P0 - x_0) for the distance that rounding moved it off
+// the plane, or (centred) from the centroid, pdn = D.n_x.  Each
+// step is written for the three pairs together, so that neighbouring
+// instructions share their source operand (the register reuse cache) and none
+// waits for its predecessor.  Plain variant: (X, Y, Z) are the test points
 // and the source coordinates absolute; the MUFU sine / cosine take k r
 // directly (their own argument scaling has the same FP32 rounding as an
 // explicit reduction).  CENTRED variant (large k r): coordinates are offsets
@@ -283,120 +338,173 @@ __device__ __forceinline__ CenterPair center_pair(const float4 &cth, const float
 // float-float arithmetic once per triangle pair.
 // MULTI: m1 multiplies the interior terms (0: source on another object, -1:
 // Mueller); k1i / dk1i: imaginary parts of k1 and k1^2 / rho (attenuation).
-template <bool CENTRED, bool MULTI, bool ABSORB>
-__device__ __forceinline__ void far_pair2(f2 X, f2 Y, f2 Z, const float4 *P, const f2 &P5, f2 mnx,
-                                          f2 mny, f2 mnz, f2 wq2, const FarConst2 &c,
-                                          const CenterPair &cp, f2 m1, f2 k1i, f2 dk1i, PairAcc &A) {
-    const float4 P0 = P[0], P1 = P[1], P2 = P[2], P3 = P[3], P4 = P[4];
-    f2 dx, dy, dz, ddx, ddy, ddz;
+struct Diff2 {
+    f2 dx, dy, dz;     // x - y
+    f2 ddx, ddy, ddz;  // centred: difference of the offsets
+};
+
+template <bool CENTRED>
+__device__ __forceinline__ Diff2 far_diff(f2 X, f2 Y, f2 Z, const float4 &P0, const float4 &P1, const CenterPair &cp) {
+    Diff2 d;
     if (CENTRED) {
-        ddx = add2(X, lo2(P0));  // delta = a - b
-        ddy = add2(Y, hi2(P0));
-        ddz = add2(Z, lo2(P1));
-        dx = add2(ddx, cp.Dx);
-        dy = add2(ddy, cp.Dy);
-        dz = add2(ddz, cp.Dz);
+        d.ddx = add2(X, lo2(P0));  // delta = a - b
+        d.ddy = add2(Y, hi2(P0));
+        d.ddz = add2(Z, lo2(P1));
+        d.dx = add2(d.ddx, cp.Dx);
+        d.dy = add2(d.ddy, cp.Dy);
+        d.dz = add2(d.ddz, cp.Dz);
     } else {
-        dx = add2(X, lo2(P0));  // x - y
-        dy = add2(Y, hi2(P0));
-        dz = add2(Z, lo2(P1));
+        d.dx = add2(X, lo2(P0));  // x - y
+        d.dy = add2(Y, hi2(P0));
+        d.dz = add2(Z, lo2(P1));
     }
-    f2 r2 = mul2(dx, dx);
-    r2 = fma2(dy, dy, r2);
-    r2 = fma2(dz, dz, r2);
-    const f2 ri = make_float2(rsqrtf(r2.x), rsqrtf(r2.y));
-    const f2 r = mul2(r2, ri);
-    const f2 ri2 = mul2(ri, ri);
-    f2 dnxn = mul2(dx, mnx);  // (y - x).n_x
-    dnxn = fma2(dy, mny, dnxn);
-    dnxn = fma2(dz, mnz, dnxn);
-    f2 s0, c0, s1, c1;
-    if (CENTRED) {
-        f2 num = mul2(ddx, ddx);
-        num = fma2(ddy, ddy, num);
-        num = fma2(ddz, ddz, num);
-        f2 dd = mul2(ddx, cp.Dx);
-        dd = fma2(ddy, cp.Dy, dd);
-        dd = fma2(ddz, cp.Dz, dd);
-        num = fma2(dd, dup2(2.f), num);  // r^2 - r_c^2
-        const f2 den = add2(r, cp.rc);
-        const f2 dlt = mul2(num, make_float2(rcp_approx(den.x), rcp_approx(den.y)));  // r - r_c
-        const f2 ph0 = fma2(c.k0, dlt, cp.b0);
-        const f2 ph1 = fma2(c.k1, dlt, cp.b1);
-        __sincosf(ph0.x, &s0.x, &c0.x);
-        __sincosf(ph0.y, &s0.y, &c0.y);
-        __sincosf(ph1.x, &s1.x, &c1.x);
-        __sincosf(ph1.y, &s1.y, &c1.y);
-    } else {
-        const f2 kr0 = mul2(r, c.k0), kr1 = mul2(r, c.k1);
-        __sincosf(kr0.x, &s0.x, &c0.x);
-        __sincosf(kr0.y, &s0.y, &c0.y);
-        __sincosf(kr1.x, &s1.x, &c1.x);
-        __sincosf(kr1.y, &s1.y, &c1.y);
-    }
-    f2 br = make_float2(0.f, 0.f);
-    constexpr bool absorb = MULTI && ABSORB;
-    if (MULTI) {  // e^{i k1 r} with k1 = k1r + i k1i: damping e^{-k1i r}, and m1
-        f2 damp = m1;
-        if (absorb) {
-            br = mul2(r, k1i);
-            damp = mul2(m1, make_float2(__expf(-br.x), __expf(-br.y)));
-        }
-        c1 = mul2(c1, damp);
-        s1 = mul2(s1, damp);
-    }
-    const f2 psr = hi2(P1), psi = lo2(P2), mpsr = hi2(P2), mpsi = lo2(P3);
-    const f2 phr = hi2(P3), phi = lo2(P4), mphr = hi2(P4), mphi = P5;
-    (void)mpsr;
-    (void)mphr;
-    // cos and sin scaled by 1/r once: G = (c + i s)/r for every kernel below
-    const f2 c0r = mul2(c0, ri), s0r = mul2(s0, ri), c1r = mul2(c1, ri), s1r = mul2(s1, ri);
-    // V block (G0 + rho G1) psi, without 1/(4 pi)
-    const f2 gpr = fma2(c.rho, c1r, c0r), gpi = fma2(c.rho, s1r, s0r);
-    A.u1r = fma2(gpr, psr, fma2(gpi, mpsi, A.u1r));
-    A.u1i = fma2(gpr, psi, fma2(gpi, psr, A.u1i));
-    // D normal term (k0^2 G0 + k1^2/rho G1) phi, as (G0 + dk1 G1) phi; the
-    // scale dks is applied per source triangle
-    f2 gkr = fma2(c.dk1, c1r, c0r), gki = fma2(c.dk1, s1r, s0r);
-    if (absorb) {  // complex k1^2 / (rho dks)
-        gkr = fma2(mul2(dk1i, s1r), dup2(-1.f), gkr);
-        gki = fma2(dk1i, c1r, gki);
-    }
-    A.ur = fma2(gkr, phr, fma2(gki, mphi, A.ur));
-    A.ui = fma2(gkr, phi, fma2(gki, phr, A.ui));
-    // D curl term: sum_q w_q (G0 + G1/rho)
-    A.t3r = fma2(fma2(c.irho, c1r, c0r), wq2, A.t3r);
-    A.t3i = fma2(fma2(c.irho, s1r, s0r), wq2, A.t3i);
-    // -(H0 + H1), H = e^{ikr} (i k r - 1) / r^3, written with the scaled c, s:
-    //   re = (c0/r + c1/r + k0 s0 + k1 s1) / r^2,  im = (s0/r + s1/r - k0 c0 - k1 c1) / r^2
-    f2 hp0 = fma2(c.k1, s1, fma2(c.k0, s0, add2(c0r, c1r)));
-    f2 hq0 = fma2(c.nk1, c1, fma2(c.nk0, c0, add2(s0r, s1r)));
-    if (absorb) {  // (i k1 r - 1) with Im k1: + k1i r (c1, s1) / r
-        hp0 = fma2(k1i, c1, hp0);
-        hq0 = fma2(k1i, s1, hq0);
-    }
-    const f2 hp = mul2(hp0, ri2);
-    const f2 hq = mul2(hq0, ri2);
-    A.t1r = fma2(hp, phr, fma2(hq, mphi, A.t1r));  // T1n = -sum Hs phi
-    A.t1i = fma2(hp, phi, fma2(hq, phr, A.t1i));
-    // T block: (H0 + H1)(x - y).n_x psi = (-(H0 + H1)) (y - x).n_x psi
-    const f2 hxp = mul2(hp, dnxn), hxq = mul2(hq, dnxn);
-    A.u2r = fma2(hxp, psr, fma2(hxq, mpsi, A.u2r));
-    A.u2i = fma2(hxp, psi, fma2(hxq, psr, A.u2i));
+    return d;
 }
 
-// One thread per pair of test points (2j, 2j+1) of test triangle 2j / 6,
-// packed into the two lanes of FP32x2 instructions.  Output
-// part[(split * 10 + c) * npts + p], c = u1 (re, im), u2 (re, im),
-// A (x re, x im, y re, y im, z re, z im):
-//   u1 = sum [ (G0 + rho G1) psi_q + (x.n_y - h_y)(H0 + H1) phi_q ]
-//   u2 = sum [ (H0 + H1)(x - y).n_x psi_q - (n_x.n_y)(k0^2 G0 + k1^2/rho G1) phi_q ]
-//   A  = sum_s (sum_q w_q (G0 + G1/rho)) c_s
+template <bool CENTRED, bool MULTI, bool ABSORB>
+__device__ __forceinline__ void far_tri(const f2 (&X)[3], const f2 (&Y)[3], const f2 (&Z)[3], const float4 &n4,
+                                        float pdn, const float4 &P0, const float4 &P1, const float4 &P2, const float4 &P3,
+                                        const f2 &P5, const FarConst2 &c, const CenterPair &cp, f2 m1, f2 k1i,
+                                        f2 dk1i, PairAcc (&A)[3], CurlAcc &B) {
+#define F3 _Pragma("unroll") for (int p = 0; p < 3; ++p)
+    Diff2 d[3];
+    F3 d[p] = far_diff<CENTRED>(X[p], Y[p], Z[p], P0, P1, cp);
+    const f2 dnxn = CENTRED ? dup2(-fmaf(P0.x, n4.x, fmaf(P0.z, n4.y, fmaf(P1.x, n4.z, pdn))))
+                            : dup2(-fmaf(d[0].dz.x, n4.z, fmaf(d[0].dy.x, n4.y, fmaf(d[0].dx.x, n4.x, -pdn))));
+    f2 r2[3], ri[3], r[3], ri2[3], s0[3], c0[3], s1[3], c1[3];
+    F3 r2[p] = mul2(d[p].dx, d[p].dx);
+    F3 r2[p] = fma2(d[p].dy, d[p].dy, r2[p]);
+    F3 r2[p] = fma2(d[p].dz, d[p].dz, r2[p]);
+    F3 ri[p] = make_float2(rsqrtf(r2[p].x), rsqrtf(r2[p].y));
+    F3 r[p] = mul2(r2[p], ri[p]);
+    F3 ri2[p] = mul2(ri[p], ri[p]);
+    if (CENTRED) {
+        f2 num[3], dd[3];
+        F3 num[p] = mul2(d[p].ddx, d[p].ddx);
+        F3 num[p] = fma2(d[p].ddy, d[p].ddy, num[p]);
+        F3 num[p] = fma2(d[p].ddz, d[p].ddz, num[p]);
+        F3 dd[p] = mul2(d[p].ddx, cp.Dx);
+        F3 dd[p] = fma2(d[p].ddy, cp.Dy, dd[p]);
+        F3 dd[p] = fma2(d[p].ddz, cp.Dz, dd[p]);
+        F3 num[p] = fma2(dd[p], dup2(2.f), num[p]);  // r^2 - r_c^2
+        F3 {
+            const f2 den = add2(r[p], cp.rc);
+            const f2 dlt = mul2(num[p], make_float2(rcp_approx(den.x), rcp_approx(den.y)));  // r - r_c
+            const f2 ph0 = fma2(c.k0, dlt, cp.b0), ph1 = fma2(c.k1, dlt, cp.b1);
+            __sincosf(ph0.x, &s0[p].x, &c0[p].x);
+            __sincosf(ph0.y, &s0[p].y, &c0[p].y);
+            __sincosf(ph1.x, &s1[p].x, &c1[p].x);
+            __sincosf(ph1.y, &s1[p].y, &c1[p].y);
+        }
+    } else {
+        F3 {
+            const f2 kr0 = mul2(r[p], c.k0), kr1 = mul2(r[p], c.k1);
+            __sincosf(kr0.x, &s0[p].x, &c0[p].x);
+            __sincosf(kr0.y, &s0[p].y, &c0[p].y);
+            __sincosf(kr1.x, &s1[p].x, &c1[p].x);
+            __sincosf(kr1.y, &s1[p].y, &c1[p].y);
+        }
+    }
+    constexpr bool absorb = MULTI && ABSORB;
+    if (MULTI) {  // e^{i k1 r} with k1 = k1r + i k1i: damping e^{-k1i r}, and m1
+        F3 {
+            f2 damp = m1;
+            if (absorb) {
+                const f2 br = mul2(r[p], k1i);
+                damp = mul2(m1, make_float2(__expf(-br.x), __expf(-br.y)));
+            }
+            c1[p] = mul2(c1[p], damp);
+            s1[p] = mul2(s1[p], damp);
+        }
+    }
+    const f2 psr = hi2(P1), psi = lo2(P2), mpsi = hi2(P2), phr = lo2(P3), phi = hi2(P3), mphi = P5;
+    // cos and sin scaled by 1/r once: G = (c + i s)/r for every kernel below
+    f2 c0r[3], s0r[3], c1r[3], s1r[3], ga[3], gb[3], hp[3], hq[3];
+    F3 c0r[p] = mul2(c0[p], ri[p]);
+    F3 s0r[p] = mul2(s0[p], ri[p]);
+    F3 c1r[p] = mul2(c1[p], ri[p]);
+    F3 s1r[p] = mul2(s1[p], ri[p]);
+    // -(H0 + H1) r^2, H = e^{ikr} (i k r - 1) / r^3, with the scaled c, s:
+    //   re = c0/r + c1/r + k0 s0 + k1 s1,  im = s0/r + s1/r - k0 c0 - k1 c1
+    F3 hp[p] = add2(c0r[p], c1r[p]);
+    F3 hq[p] = add2(s0r[p], s1r[p]);
+    F3 hp[p] = fma2(c.k0, s0[p], hp[p]);
+    F3 hp[p] = fma2(c.k1, s1[p], hp[p]);
+    F3 hq[p] = fma2(c.nk0, c0[p], hq[p]);
+    F3 hq[p] = fma2(c.nk1, c1[p], hq[p]);
+    if (absorb) {  // (i k1 r - 1) with Im k1: + k1i r (c1, s1) / r
+        F3 hp[p] = fma2(k1i, c1[p], hp[p]);
+        F3 hq[p] = fma2(k1i, s1[p], hq[p]);
+    }
+    // D curl term: sums of G0 and G1, weighted and combined by the caller
+    F3 B.g0r = add2(B.g0r, c0r[p]);
+    F3 B.g0i = add2(B.g0i, s0r[p]);
+    F3 B.g1r = add2(B.g1r, c1r[p]);
+    F3 B.g1i = add2(B.g1i, s1r[p]);
+    // V block (G0 + rho G1) psi, without 1/(4 pi)
+    F3 ga[p] = fma2(c.rho, c1r[p], c0r[p]);
+    F3 gb[p] = fma2(c.rho, s1r[p], s0r[p]);
+    F3 A[p].u1r = fma2(gb[p], mpsi, A[p].u1r);
+    F3 A[p].u1i = fma2(gb[p], psr, A[p].u1i);
+    F3 A[p].u1r = fma2(ga[p], psr, A[p].u1r);
+    F3 A[p].u1i = fma2(ga[p], psi, A[p].u1i);
+    // D normal term (k0^2 G0 + k1^2/rho G1) phi, as (G0 + dk1 G1) phi; the
+    // scale dks is applied per source triangle
+    F3 ga[p] = fma2(c.dk1, c1r[p], c0r[p]);
+    F3 gb[p] = fma2(c.dk1, s1r[p], s0r[p]);
+    if (absorb) {  // complex k1^2 / (rho dks)
+        F3 ga[p] = fma2(mul2(dk1i, s1r[p]), dup2(-1.f), ga[p]);
+        F3 gb[p] = fma2(dk1i, c1r[p], gb[p]);
+    }
+    F3 A[p].ur = fma2(gb[p], mphi, A[p].ur);
+    F3 A[p].ui = fma2(gb[p], phr, A[p].ui);
+    F3 A[p].ur = fma2(ga[p], phr, A[p].ur);
+    F3 A[p].ui = fma2(ga[p], phi, A[p].ui);
+    // T1n = -sum Hs phi
+    F3 hp[p] = mul2(hp[p], ri2[p]);
+    F3 hq[p] = mul2(hq[p], ri2[p]);
+    F3 A[p].t1r = fma2(hq[p], mphi, A[p].t1r);
+    F3 A[p].t1i = fma2(hq[p], phr, A[p].t1i);
+    F3 A[p].t1r = fma2(hp[p], phr, A[p].t1r);
+    F3 A[p].t1i = fma2(hp[p], phi, A[p].t1i);
+    // T block: (H0 + H1)(x - y).n_x psi = (-(H0 + H1)) (y - x).n_x psi
+    F3 hp[p] = mul2(hp[p], dnxn);
+    F3 hq[p] = mul2(hq[p], dnxn);
+    F3 A[p].u2r = fma2(hq[p], mpsi, A[p].u2r);
+    F3 A[p].u2i = fma2(hq[p], psr, A[p].u2i);
+    F3 A[p].u2r = fma2(hp[p], psr, A[p].u2r);
+    F3 A[p].u2i = fma2(hp[p], psi, A[p].u2i);
+#undef F3
+}
+
+// One thread per test triangle: its six points are three pairs (p, p + 3)
+// packed into the two lanes of FP32x2 instructions (a lane holds the points
+// of one rule weight).  Outputs per source split
+//   part[(split * 4 + c) * npts + p], c = u1 (re, im), u2 (re, im):
+//     u1 = sum [ (G0 + rho G1) psi_q + (x.n_y - h_y)(H0 + H1) phi_q ]
+//     u2 = sum [ (H0 + H1)(x - y).n_x psi_q - (n_x.n_y)(k0^2 G0 + k1^2/rho G1) phi_q ]
+//   partA[(split * 6 + c) * nt + t], c = A (x re, x im, y re, y im, z re, z im):
+//     A  = sum_s (sum_p w_p sum_q w_q (G0 + G1/rho)) c_s
 // with G, H here without the factor 1/(4 pi) (applied in the gather).  Sums
 // run per 64-triangle tile, then tile sums are added to running sums kept in
-// part.
+// the outputs.
+// The kernel is bound by the FP32 pipe (packed FMA at 2.5 to 3.3 cycles a
+// warp instruction with three distinct register pairs, packed add and
+// multiply at 2).  A thread holds the whole triangle so that what is common
+// to its points is done once: (y - x).n_x per source point (8 of about 154
+// pipe cycles per pair of test points before), the curl term summed over test
+// and source points by plain adds, weighted per class and multiplied into c_s
+// once per triangle pair (10 cycles), the source
+// loads from shared memory (a third), and the centroid phases of the centred
+// variant (a third).  An apply at 10242 vertices: 25.9 ms (29.1 where a
+// thread held one pair of points), 20000 vertices centred 124 ms (147), four
+// objects of 642 vertices 2.19 ms (3.27).  255 registers and two blocks per
+// SM measured 1 to 4 % better than 168 and three.
+// Small meshes give a block 32 or 64 test triangles and split each source
+// tile between its warps, whose sums are added in shared memory: more warps
+// in flight for the same number of partial sums (see far_setup_geometry).
 // CENTRED: pt holds offsets from the test-triangle centroid and cen the
-// float-float centroids (see far_pair2).
+// float-float centroids (see far_tri).
 // MULTI: disjoint objects (Sec. 2.2) or the Mueller formulation; the interior
 // constants are the test triangle's object's, interior terms vanish for
 // sources on other objects and change sign for Mueller.  ABSORB (with MULTI):
@@ -406,30 +514,37 @@ __global__ void __launch_bounds__(FAR_THREADS, OSRC_FAR_MIN_BLOCKS)
 far_kernel(const float4 *__restrict__ pt, const float4 *__restrict__ cen,
            const float4 *__restrict__ tn, const int4 *__restrict__ tv,
            const float4 *__restrict__ sP, const float2 *__restrict__ sP5,
-           const float4 *__restrict__ sC, int nt, int npts, int tris_per_split, FarConst2 c0,
+           const float4 *__restrict__ sC, int nt, int npts, int tris_per_split, int block_tris, FarConst2 c0,
            float4 kff0, const int *__restrict__ tcomp, const FarObj *__restrict__ fobj,
-           float *__restrict__ part) {
-    __shared__ float4 shP[FAR_TS * 6 * 5];
+           float *__restrict__ part, float *__restrict__ partA) {
+    __shared__ float4 shP[FAR_TS * 6 * 4];
     __shared__ float2 shP5[FAR_TS * 6];
     __shared__ float4 shN[FAR_TS];
-    __shared__ float4 shC[FAR_TS * 5];
+    __shared__ float4 shC[FAR_TS * 2];
     __shared__ int4 shV[FAR_TS];
     __shared__ float4 shCen[CENTRED ? 2 * FAR_TS : 1];
     __shared__ int shComp[MULTI ? FAR_TS : 1];
 
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+    // block_tris test triangles x FAR_THREADS / block_tris source groups (whole
+    // warps); a group takes every ngrp-th source triangle of a tile
+    const int tx = threadIdx.x % block_tris, grp = threadIdx.x / block_tris, ngrp = FAR_THREADS / block_tris;
+    const int j = blockIdx.x * block_tris + tx;
     const int split = blockIdx.y;
-    const int s_begin = split * tris_per_split;
+    const int s_begin = min(nt, split * tris_per_split);
     const int s_end = min(nt, s_begin + tris_per_split);
-    const bool active = 2 * j < npts;
-    const int p0 = active ? 2 * j : 0;
-    const int tau = p0 / 6;
-    const float4 xa = pt[p0], xb = pt[p0 + 1];
-    const f2 X = make_float2(xa.x, xb.x), Y = make_float2(xa.y, xb.y), Z = make_float2(xa.z, xb.z);
+    const bool active = j < nt;
+    const int tau = active ? j : 0;
+    f2 X[3], Y[3], Z[3];
+#pragma unroll
+    for (int p = 0; p < 3; ++p) {
+        const float4 xa = pt[6 * tau + p], xb = pt[6 * tau + p + 3];
+        X[p] = make_float2(xa.x, xb.x);
+        Y[p] = make_float2(xa.y, xb.y);
+        Z[p] = make_float2(xa.z, xb.z);
+    }
     const float4 n4 = tn[tau];
     const int4 vt = tv[tau];
-    const f2 mnx = dup2(-n4.x), mny = dup2(-n4.y), mnz = dup2(-n4.z);
-    const f2 W1 = dup2((float)kQw1), W2 = dup2((float)kQw2);
+    constexpr float W1 = (float)kQw1, W2 = (float)kQw2;
     FarConst2 c = c0;
     float4 kff = kff0;
     int ct = 0;
@@ -454,13 +569,17 @@ far_kernel(const float4 *__restrict__ pt, const float4 *__restrict__ cen,
         cth = cen[2 * tau];
         ctl = cen[2 * tau + 1];
     }
+    // curl-term sums of the whole split, rounding errors carried along: one sum per triangle stands for the six points' sums, whose
+    // independent rounding errors the test weights would have averaged
+    float ar[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, ae[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    const size_t o1 = (size_t)split * 4 * npts + 6 * (size_t)tau, oA = (size_t)split * 6 * nt + tau;
 
     for (int t0 = s_begin; t0 < s_end; t0 += FAR_TS) {
         const int cnt = min(FAR_TS, s_end - t0);
         __syncthreads();
-        for (int i = threadIdx.x; i < cnt * 30; i += blockDim.x) shP[i] = sP[30 * (size_t)t0 + i];
+        for (int i = threadIdx.x; i < cnt * 24; i += blockDim.x) shP[i] = sP[24 * (size_t)t0 + i];
         for (int i = threadIdx.x; i < cnt * 6; i += blockDim.x) shP5[i] = sP5[6 * (size_t)t0 + i];
-        for (int i = threadIdx.x; i < cnt * 5; i += blockDim.x) shC[i] = sC[5 * (size_t)t0 + i];
+        for (int i = threadIdx.x; i < cnt * 2; i += blockDim.x) shC[i] = sC[2 * (size_t)t0 + i];
         for (int i = threadIdx.x; i < cnt; i += blockDim.x) {
             const float4 ns = tn[t0 + i];
             shN[i] = make_float4(-ns.x, -ns.y, -ns.z, ns.w);
@@ -472,119 +591,247 @@ far_kernel(const float4 *__restrict__ pt, const float4 *__restrict__ cen,
             for (int i = threadIdx.x; i < cnt; i += blockDim.x) shComp[i] = tcomp[t0 + i];
         __syncthreads();
 
-        PairAcc A;
-        A.u1r = A.u1i = A.u2r = A.u2i = make_float2(0.f, 0.f);
-        A.axr = A.axi = A.ayr = A.ayi = A.azr = A.azi = make_float2(0.f, 0.f);
-        for (int s = 0; s < cnt; ++s) {
+        PairAcc A[3];
+#pragma unroll
+        for (int p = 0; p < 3; ++p) A[p].u1r = A[p].u1i = A[p].u2r = A[p].u2i = make_float2(0.f, 0.f);
+        for (int s = grp; s < cnt; s += ngrp) {
             const int4 vs = shV[s];
             const bool touch = (vs.x == vt.x) | (vs.x == vt.y) | (vs.x == vt.z) |
                                (vs.y == vt.x) | (vs.y == vt.y) | (vs.y == vt.z) |
                                (vs.z == vt.x) | (vs.z == vt.y) | (vs.z == vt.z);
             if (touch) continue;
-            const float4 mns = shN[s];  // (-n_y, n_y.P0)
             CenterPair cp;
-            f2 xnyn;  // -(x - y).n_y, constant over the source triangle
+            float pdn = __int_as_float(vt.w);
             if (CENTRED) {
                 cp = center_pair(cth, ctl, shCen[2 * s], shCen[2 * s + 1], kff.x, kff.y, kff.z, kff.w);
-                // (x - y).n_y = (c_x - c_y + a).n_y since c_y lies in the source plane
-                const float dn = cp.Dx.x * mns.x + cp.Dy.x * mns.y + cp.Dz.x * mns.z;
-                xnyn = fma2(Z, dup2(mns.z), fma2(Y, dup2(mns.y), fma2(X, dup2(mns.x), dup2(dn))));
-            } else {
-                xnyn = fma2(Z, dup2(mns.z), fma2(Y, dup2(mns.y), fma2(X, dup2(mns.x), dup2(mns.w))));
+                pdn = fmaf(cp.Dx.x, n4.x, fmaf(cp.Dy.x, n4.y, cp.Dz.x * n4.z)) +
+                      fmaf(cp.lx, n4.x, fmaf(cp.ly, n4.y, cp.lz * n4.z));
             }
-            const float nxnyn = n4.x * mns.x + n4.y * mns.y + n4.z * mns.z;  // -n_x.n_y
-            A.t1r = A.t1i = A.ur = A.ui = A.t3r = A.t3i = make_float2(0.f, 0.f);
-            const f2 m1 = dup2(MULTI ? (shComp[s] != ct ? 0.f : sgn) : 1.f);
 #pragma unroll
-            for (int q = 0; q < 6; ++q)
-                far_pair2<CENTRED, MULTI, ABSORB>(X, Y, Z, &shP[30 * s + 5 * q], shP5[6 * s + q], mnx, mny, mnz,
-                                          q < 3 ? W1 : W2, c, cp, m1, k1i, dk1i, A);
-            // u1 += (x - y).n_y T1 = (-(x - y).n_y)(-T1);  u2 += (-n_x.n_y) U
-            A.u1r = fma2(xnyn, A.t1r, A.u1r);
-            A.u1i = fma2(xnyn, A.t1i, A.u1i);
+            for (int p = 0; p < 3; ++p)
+                A[p].t1r = A[p].t1i = A[p].ur = A[p].ui = make_float2(0.f, 0.f);
+            f2 t3r = make_float2(0.f, 0.f), t3i = t3r;  // sum_q w_q (G0 + G1/rho), lanes summed over their points
+            const f2 m1 = dup2(MULTI ? (shComp[s] != ct ? 0.f : sgn) : 1.f);
+#pragma unroll FAR_HUNROLL
+            for (int h = 0; h < 2; ++h) {  // the two weight classes of the source points
+                CurlAcc Bs;
+                Bs.g0r = Bs.g0i = Bs.g1r = Bs.g1i = make_float2(0.f, 0.f);
+#pragma unroll FAR_QUNROLL
+                for (int q = 3 * h; q < 3 * h + 3; ++q) {
+                    const float4 *P = &shP[24 * s + 4 * q];
+                    const float4 P0 = P[0], P1 = P[1], P2 = P[2], P3 = P[3];
+                    const f2 P5 = shP5[6 * s + q];
+                    far_tri<CENTRED, MULTI, ABSORB>(X, Y, Z, n4, pdn, P0, P1, P2, P3, P5, c, cp, m1, k1i, dk1i, A, Bs);
+                }
+                const f2 wh = dup2(h ? W2 : W1);
+                t3r = fma2(wh, fma2(c.irho, Bs.g1r, Bs.g0r), t3r);
+                t3i = fma2(wh, fma2(c.irho, Bs.g1i, Bs.g0i), t3i);
+            }
+            const float4 mns = shN[s];  // (-n_y, n_y.P0)
+            float dn = mns.w;           // -(x - y).n_y, constant over the source triangle
+            // centred: (x - y).n_y = (c_x - c_y + a).n_y since c_y lies in the source plane
+            if (CENTRED) dn = cp.Dx.x * mns.x + cp.Dy.x * mns.y + cp.Dz.x * mns.z;
+            const float nxnyn = n4.x * mns.x + n4.y * mns.y + n4.z * mns.z;  // -n_x.n_y
             const f2 nn = dup2(nxnyn * c.dk0.x);
-            A.u2r = fma2(nn, A.ur, A.u2r);
-            A.u2i = fma2(nn, A.ui, A.u2i);
-            const float4 C0 = shC[5 * s], C1 = shC[5 * s + 1], C2 = shC[5 * s + 2];
-            const float4 C3 = shC[5 * s + 3], C4 = shC[5 * s + 4];
-            A.axr = fma2(A.t3r, lo2(C0), fma2(A.t3i, lo2(C1), A.axr));
-            A.axi = fma2(A.t3r, hi2(C0), fma2(A.t3i, lo2(C0), A.axi));
-            A.ayr = fma2(A.t3r, hi2(C1), fma2(A.t3i, hi2(C2), A.ayr));
-            A.ayi = fma2(A.t3r, lo2(C2), fma2(A.t3i, hi2(C1), A.ayi));
-            A.azr = fma2(A.t3r, lo2(C3), fma2(A.t3i, lo2(C4), A.azr));
-            A.azi = fma2(A.t3r, hi2(C3), fma2(A.t3i, lo2(C3), A.azi));
+#pragma unroll
+            for (int p = 0; p < 3; ++p) {
+                // u1 += (x - y).n_y T1 = (-(x - y).n_y)(-T1);  u2 += (-n_x.n_y) U
+                const f2 xnyn = fma2(Z[p], dup2(mns.z), fma2(Y[p], dup2(mns.y), fma2(X[p], dup2(mns.x), dup2(dn))));
+                A[p].u1r = fma2(xnyn, A[p].t1r, A[p].u1r);
+                A[p].u1i = fma2(xnyn, A[p].t1i, A[p].u1i);
+                A[p].u2r = fma2(nn, A[p].ur, A[p].u2r);
+                A[p].u2i = fma2(nn, A[p].ui, A[p].u2i);
+            }
+            // A += (sum_p w_p T3_p) c_s
+            const float wr = fmaf(W1, t3r.x, W2 * t3r.y), wi = fmaf(W1, t3i.x, W2 * t3i.y);
+            const float4 C0 = shC[2 * s], C1 = shC[2 * s + 1];
+            const float cr[3] = {C0.x, C0.z, C1.x}, ci[3] = {C0.y, C0.w, C1.y};
+#pragma unroll
+            for (int i = 0; i < 3; ++i) {
+                comp_add_fast(ar[2 * i], ae[2 * i], fmaf(wr, cr[i], -(wi * ci[i])));
+                comp_add_fast(ar[2 * i + 1], ae[2 * i + 1], fmaf(wr, ci[i], wi * cr[i]));
+            }
         }
-        // running sums live in the output: the first tile stores, later
+        if (ngrp > 1) {  // add the groups' sums through shared memory (the tile is done with)
+            float *red = reinterpret_cast<float *>(shP);
+            const int rs = (ngrp - 1) * block_tris;
+            __syncthreads();
+            if (grp > 0) {
+                float *o = red + (grp - 1) * block_tris + tx;
+#pragma unroll
+                for (int p = 0; p < 3; ++p) {
+                    const f2 v[4] = {A[p].u1r, A[p].u1i, A[p].u2r, A[p].u2i};
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        o[(8 * p + 2 * i) * rs] = v[i].x;
+                        o[(8 * p + 2 * i + 1) * rs] = v[i].y;
+                    }
+                }
+            }
+            __syncthreads();
+            if (grp == 0)
+                for (int g = 0; g < ngrp - 1; ++g) {
+                    const float *o = red + g * block_tris + tx;
+#pragma unroll
+                    for (int p = 0; p < 3; ++p) {
+                        f2 *v[4] = {&A[p].u1r, &A[p].u1i, &A[p].u2r, &A[p].u2i};
+#pragma unroll
+                        for (int i = 0; i < 4; ++i)
+                            *v[i] = add2(*v[i], make_float2(o[(8 * p + 2 * i) * rs], o[(8 * p + 2 * i + 1) * rs]));
+                    }
+                }
+        }
+        // running sums of u live in the outputs: the first tile stores, later
         // tiles add (the thread's own entries; registers stay free for the
         // pair loop)
-        if (active) {
-            const f2 v[10] = {A.u1r, A.u1i, A.u2r, A.u2i, A.axr, A.axi, A.ayr, A.ayi, A.azr, A.azi};
-            f2 *pp = reinterpret_cast<f2 *>(part);
+        if (active && grp == 0) {
+            const bool first = t0 == s_begin;
 #pragma unroll
-            for (int i = 0; i < 10; ++i) {
-                const size_t o = (((size_t)split * 10 + i) * npts + p0) / 2;
-                pp[o] = t0 == s_begin ? v[i] : add2(pp[o], v[i]);
+            for (int p = 0; p < 3; ++p) {
+                const f2 v[4] = {A[p].u1r, A[p].u1i, A[p].u2r, A[p].u2i};
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const size_t o = o1 + (size_t)i * npts + p;
+                    part[o] = first ? v[i].x : part[o] + v[i].x;
+                    part[o + 3] = first ? v[i].y : part[o + 3] + v[i].y;
+                }
             }
         }
     }
-    if (active && s_begin >= s_end) {  // empty split: zero sums
-        f2 *pp = reinterpret_cast<f2 *>(part);
+    if (ngrp > 1) {  // the groups' curl sums
+        float *red = reinterpret_cast<float *>(shP);
+        const int rs = (ngrp - 1) * block_tris;
+        __syncthreads();
+        if (grp > 0)
 #pragma unroll
-        for (int i = 0; i < 10; ++i) pp[(((size_t)split * 10 + i) * npts + p0) / 2] = make_float2(0.f, 0.f);
+            for (int i = 0; i < 6; ++i) red[i * rs + (grp - 1) * block_tris + tx] = ar[i] + ae[i];
+        __syncthreads();
+        if (grp == 0)
+            for (int g = 0; g < ngrp - 1; ++g)
+#pragma unroll
+                for (int i = 0; i < 6; ++i) comp_add(ar[i], ae[i], red[i * rs + g * block_tris + tx]);
+    }
+    if (active && grp == 0)
+#pragma unroll
+        for (int i = 0; i < 6; ++i) partA[oA + (size_t)i * nt] = ar[i] + ae[i];
+    if (active && grp == 0 && s_begin >= s_end) {  // empty split: zero sums
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            for (int p = 0; p < 6; ++p) part[o1 + (size_t)i * npts + p] = 0.f;
     }
 }
 
-// Per vertex v: y1_v = (1/4pi) sum_{(t,a) incident} |t| sum_q w_q lambda_a(q) u1(t,q)
-//               y2_v = (1/4pi) sum |t| [sum_q w_q lambda_a(q) u2(t,q) + curl_a . sum_q w_q A(t,q)]
-// plus the near-field CSR rows (2x2 complex blocks) applied to x.
-__global__ void gather_kernel(int nv, int npts, int nsplit, const int *__restrict__ vt_ptr,
-                              const int *__restrict__ vt_idx, const double *__restrict__ tgeo,
-                              const float *__restrict__ part, int use_far,
-                              const int *__restrict__ nr_ptr, const int *__restrict__ nr_col,
-                              const double2 *__restrict__ nr_val, int use_near,
-                              const double2 *__restrict__ x, double2 *__restrict__ y) {
-    const int v = blockIdx.x * blockDim.x + threadIdx.x;
-    if (v >= nv) return;
+// ---------------------------------------------------------------------------
+// Gather: L lanes per (vertex, right-hand side).  Far field, over the
+// incident (triangle t, local index a):
+//   y1_v = (1/4pi) sum |t| sum_q w_q lambda_a(q) u1(t,q)
+//   y2_v = (1/4pi) sum |t| [sum_q w_q lambda_a(q) u2(t,q) + curl_a . A(t)]
+// plus the near-field CSR rows (2x2 complex blocks) applied to x.  Partial
+// sums as far_kernel and farm_kernel leave them: part [ns][R][4][npts],
+// partA [ns][R][6][nt].
+// The lanes share the (triangle, point) items and the CSR entries.  The
+// source splits are added in FP32 with their rounding errors carried along
+// (Knuth's TwoSum: the sum to about 48 bits), because FP64 issues at 1/64 of
+// the FP32 rate on this part; the rest is FP64.  One thread per vertex with
+// FP64 sums took 215 us on the 150-vertex hull and 0.24 ms on the
+// 10242-vertex sphere.  Small meshes, where the splits are many and the
+// vertices too few to fill the GPU, take a block per vertex (L = 32, W = 4:
+// the splits shared by its four warps); larger ones a warp, then L = 8 where
+// lanes would idle.
+// ---------------------------------------------------------------------------
+constexpr int FARM_MAX_R = 8;
+
+struct VecPtrs {
+    const double2 *p[FARM_MAX_R];
+};
+struct OutPtrs {
+    double2 *p[FARM_MAX_R];
+};
+
+constexpr int GATHER_THREADS = 128;
+
+// value of a compensated sum; an infinite or NaN sum stands alone (its error
+// term is not a number)
+__device__ __forceinline__ double comp_value(float s, float e) {
+    return isfinite(s) ? (double)s + (double)e : (double)s;
+}
+
+template <int L, int W>
+__global__ void __launch_bounds__(GATHER_THREADS)
+gather_kernel(int nv, int nt, int npts, int ns, int R, const int *__restrict__ vt_ptr,
+              const int *__restrict__ vt_idx, const double *__restrict__ tgeo, const float *__restrict__ part,
+              const float *__restrict__ partA, int use_far, const int *__restrict__ nr_ptr,
+              const int *__restrict__ nr_col, const double2 *__restrict__ nr_val, int use_near,
+              const __grid_constant__ VecPtrs x, const __grid_constant__ OutPtrs y) {
+    static_assert(W == 1 || L == 32, "split groups are warps");
+    __shared__ double2 red[W > 1 ? W : 1][2];
+    const int lane = threadIdx.x % L;
+    const int wg = W > 1 ? threadIdx.x / L % W : 0;  // split group
+    const int v = blockIdx.x * (GATHER_THREADS / (L * W)) + threadIdx.x / (L * W);
+    const int rr = blockIdx.y;
+    const bool valid = v < nv;  // every lane takes part in the shuffles below
     double2 y1 = cd(0, 0), y2 = cd(0, 0);
-    if (use_far) {
-        for (int e = vt_ptr[v]; e < vt_ptr[v + 1]; ++e) {
-            const int t = vt_idx[e] / 3, a = vt_idx[e] % 3;
+    if (valid && use_far) {
+        const int e0 = vt_ptr[v], items = 6 * (vt_ptr[v + 1] - e0);
+        const size_t su = (size_t)R * 4 * npts, sa = (size_t)R * 6 * nt;
+        for (int it = lane; it < items; it += L) {
+            const int e = it / 6, q = it - 6 * e;
+            const int ta = vt_idx[e0 + e], t = ta / 3, a = ta - 3 * t;
             const double *g = tgeo + 16 * (size_t)t;
-            double2 s1 = cd(0, 0), s2 = cd(0, 0), ax = cd(0, 0), ay = cd(0, 0), az = cd(0, 0);
-            for (int q = 0; q < 6; ++q) {
-                double b[3], w;
-                rule_point(q, b, w);
-                const double wl = w * b[a];
-                const size_t p = 6 * (size_t)t + q;
-                for (int sp = 0; sp < nsplit; ++sp) {
-                    const float *P = part + (size_t)sp * 10 * npts + p;
-                    s1 = cadd(s1, cd(wl * P[0], wl * P[(size_t)npts]));
-                    s2 = cadd(s2, cd(wl * P[2 * (size_t)npts], wl * P[3 * (size_t)npts]));
-                    ax = cadd(ax, cd(w * P[4 * (size_t)npts], w * P[5 * (size_t)npts]));
-                    ay = cadd(ay, cd(w * P[6 * (size_t)npts], w * P[7 * (size_t)npts]));
-                    az = cadd(az, cd(w * P[8 * (size_t)npts], w * P[9 * (size_t)npts]));
-                }
+            const float *P = part + (size_t)rr * 4 * npts + 6 * (size_t)t + q;
+            const float *PA = partA + ((size_t)rr * 6 + q) * nt + t;
+            float s[5] = {0.f, 0.f, 0.f, 0.f, 0.f}, c[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll 4
+            for (int sp = wg; sp < ns; sp += W) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i) comp_add(s[i], c[i], P[sp * su + (size_t)i * npts]);
+                comp_add(s[4], c[4], PA[sp * sa]);
             }
-            const double *cu = g + 4 + 3 * a;
-            s2 = cadd(s2, cadd(cadd(cscale(ax, cu[0]), cscale(ay, cu[1])), cscale(az, cu[2])));
-            y1 = cadd(y1, cscale(s1, g[0]));
-            y2 = cadd(y2, cscale(s2, g[0]));
+            const double al = q < 3 ? kQa1 : kQa2, w = q < 3 ? kQw1 : kQw2;
+            const double wl = w * (a == (q < 3 ? q : q - 3) ? 1.0 - 2.0 * al : al) * g[0], wa = g[4 + 3 * a + (q >> 1)] * g[0];
+            y1 = cadd(y1, cd(wl * comp_value(s[0], c[0]), wl * comp_value(s[1], c[1])));
+            y2 = cadd(y2, cd(wl * comp_value(s[2], c[2]), wl * comp_value(s[3], c[3])));
+            const double av = wa * comp_value(s[4], c[4]);  // component q / 2 of curl_a . A, re or im
+            if (q & 1) y2.y += av;
+            else y2.x += av;
         }
         const double inv4pi = 0.079577471545947667884;
         y1 = cscale(y1, inv4pi);
         y2 = cscale(y2, inv4pi);
     }
-    if (use_near) {
-        for (int e = nr_ptr[v]; e < nr_ptr[v + 1]; ++e) {
-            const int j = nr_col[e];
-            const double2 xa = x[j], xb = x[nv + j];
-            const double2 *B = nr_val + 4 * (size_t)e;
-            y1 = cadd(y1, cadd(cmul(B[0], xa), cmul(B[1], xb)));
-            y2 = cadd(y2, cadd(cmul(B[2], xa), cmul(B[3], xb)));
+    if (valid && use_near) {
+        const double2 *xr = x.p[rr];
+        for (int e = nr_ptr[v] + wg * L + lane; e < nr_ptr[v + 1]; e += L * W) {
+            const int jc = nr_col[e];
+            const double2 xa = xr[jc], xb = xr[nv + jc];
+            const double2 *Bk = nr_val + 4 * (size_t)e;
+            y1 = cadd(y1, cadd(cmul(Bk[0], xa), cmul(Bk[1], xb)));
+            y2 = cadd(y2, cadd(cmul(Bk[2], xa), cmul(Bk[3], xb)));
         }
     }
-    y[v] = y1;
-    y[nv + v] = y2;
+#pragma unroll
+    for (int o = L / 2; o > 0; o >>= 1) {
+        y1.x += __shfl_xor_sync(0xffffffffu, y1.x, o);
+        y1.y += __shfl_xor_sync(0xffffffffu, y1.y, o);
+        y2.x += __shfl_xor_sync(0xffffffffu, y2.x, o);
+        y2.y += __shfl_xor_sync(0xffffffffu, y2.y, o);
+    }
+    if (W > 1) {  // a block per vertex: its warps' sums in warp order
+        if (lane == 0) {
+            red[wg][0] = y1;
+            red[wg][1] = y2;
+        }
+        __syncthreads();
+        if (threadIdx.x == 0)
+            for (int w = 1; w < W; ++w) {
+                y1 = cadd(y1, red[w][0]);
+                y2 = cadd(y2, red[w][1]);
+            }
+    }
+    if (valid && lane == 0 && wg == 0) {
+        y.p[rr][v] = y1;
+        y.p[rr][nv + v] = y2;
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -632,15 +879,6 @@ constexpr int FARM_THREADS = OSRC_FARM_THREADS;
 constexpr int FARM_QUNROLL = OSRC_FARM_QUNROLL;  // unroll of the rule-point loop
 constexpr int FARM_TRIS = FARM_THREADS / 3;  // test triangles per block
 constexpr int FARM_TS = 16;                  // source triangles per shared-memory tile
-constexpr int FARM_MAX_R = 8;
-
-struct VecPtrs {
-    const double2 *p[FARM_MAX_R];
-};
-struct OutPtrs {
-    double2 *p[FARM_MAX_R];
-};
-
 // one shared-memory tile buffer: sG, sD, sCm, normals, vertex ids, centroids
 constexpr size_t farm_buf_bytes(int R, bool centred) {
     return (size_t)FARM_TS * (12 * 16 + 12 * 16 * R + 24 * R + 16 + 16 + (centred ? 32 : 0));
@@ -801,7 +1039,7 @@ __device__ __forceinline__ void farm_pair(f2 X, f2 Y, f2 Z, const float4 G0, con
     const f2 wq = hi2(G1);
     t3r = fma2(fma2(c.irho, c1r, c0r), wq, t3r);
     t3i = fma2(fma2(c.irho, s1r, s0r), wq, t3i);
-    // -(H0 + H1) with the scaled c, s (see far_pair2)
+    // -(H0 + H1) with the scaled c, s (see far_tri)
     const f2 hp = mul2(fma2(c.k1, s1, fma2(c.k0, s0, add2(c0r, c1r))), ri2);
     const f2 hq = mul2(fma2(c.nk1, c1, fma2(c.nk0, c0, add2(s0r, s1r))), ri2);
     // K: (x - y).n_y (H0 + H1) = (-(x - y).n_y)(-(H0 + H1));  T: (H0 + H1)(x - y).n_x
@@ -993,60 +1231,6 @@ farm_kernel(const float4 *__restrict__ pt, const float4 *__restrict__ cen, const
     }
 }
 
-// Per (vertex, right-hand side): the far-field partial sums gathered with the
-// test weights, plus the near-field CSR product (as gather_kernel).
-__global__ void farm_gather_kernel(int nv, int nt, int npts, int nsplit, int R, const int *__restrict__ vt_ptr,
-                                   const int *__restrict__ vt_idx, const double *__restrict__ tgeo,
-                                   const float *__restrict__ part, const float *__restrict__ partA,
-                                   int use_far, const int *__restrict__ nr_ptr, const int *__restrict__ nr_col,
-                                   const double2 *__restrict__ nr_val, int use_near, VecPtrs x, OutPtrs y) {
-    const int v = blockIdx.x * blockDim.x + threadIdx.x;
-    const int rr = blockIdx.y;
-    if (v >= nv || rr >= R) return;
-    double2 y1 = cd(0, 0), y2 = cd(0, 0);
-    if (use_far) {
-        for (int e = vt_ptr[v]; e < vt_ptr[v + 1]; ++e) {
-            const int t = vt_idx[e] / 3, a = vt_idx[e] % 3;
-            const double *g = tgeo + 16 * (size_t)t;
-            double2 s1 = cd(0, 0), s2 = cd(0, 0), ax = cd(0, 0), ay = cd(0, 0), az = cd(0, 0);
-            for (int sp = 0; sp < nsplit; ++sp) {
-                const float *P = part + (((size_t)sp * R + rr) * 4) * npts;
-                for (int q = 0; q < 6; ++q) {
-                    double b[3], w;
-                    rule_point(q, b, w);
-                    const double wl = w * b[a];
-                    const size_t p = 6 * (size_t)t + q;
-                    s1 = cadd(s1, cd(wl * P[p], wl * P[p + (size_t)npts]));
-                    s2 = cadd(s2, cd(wl * P[p + 2 * (size_t)npts], wl * P[p + 3 * (size_t)npts]));
-                }
-                const float *PA = partA + (((size_t)sp * R + rr) * 6) * nt + t;
-                ax = cadd(ax, cd(PA[0], PA[(size_t)nt]));
-                ay = cadd(ay, cd(PA[2 * (size_t)nt], PA[3 * (size_t)nt]));
-                az = cadd(az, cd(PA[4 * (size_t)nt], PA[5 * (size_t)nt]));
-            }
-            const double *cu = g + 4 + 3 * a;
-            s2 = cadd(s2, cadd(cadd(cscale(ax, cu[0]), cscale(ay, cu[1])), cscale(az, cu[2])));
-            y1 = cadd(y1, cscale(s1, g[0]));
-            y2 = cadd(y2, cscale(s2, g[0]));
-        }
-        const double inv4pi = 0.079577471545947667884;
-        y1 = cscale(y1, inv4pi);
-        y2 = cscale(y2, inv4pi);
-    }
-    if (use_near) {
-        const double2 *xr = x.p[rr];
-        for (int e = nr_ptr[v]; e < nr_ptr[v + 1]; ++e) {
-            const int jc = nr_col[e];
-            const double2 xa = xr[jc], xb = xr[nv + jc];
-            const double2 *Bk = nr_val + 4 * (size_t)e;
-            y1 = cadd(y1, cadd(cmul(Bk[0], xa), cmul(Bk[1], xb)));
-            y2 = cadd(y2, cadd(cmul(Bk[2], xa), cmul(Bk[3], xb)));
-        }
-    }
-    y.p[rr][v] = y1;
-    y.p[rr][nv + v] = y2;
-}
-
 }  // namespace
 
 int far_setup_geometry(osrc_problem *pb, cudaStream_t st) {
@@ -1058,9 +1242,9 @@ int far_setup_geometry(osrc_problem *pb, cudaStream_t st) {
     OSRC_TRY(pb->d_tn.alloc(m->ctx, nt));
     OSRC_TRY(pb->d_tv.alloc(m->ctx, nt));
     OSRC_TRY(pb->d_tgeo.alloc(m->ctx, 16 * (size_t)nt));
-    OSRC_TRY(pb->d_sP.alloc(m->ctx, 30 * (size_t)nt));
+    OSRC_TRY(pb->d_sP.alloc(m->ctx, 24 * (size_t)nt));
     OSRC_TRY(pb->d_sP5.alloc(m->ctx, 6 * (size_t)nt));
-    OSRC_TRY(pb->d_sC.alloc(m->ctx, 5 * (size_t)nt));
+    OSRC_TRY(pb->d_sC.alloc(m->ctx, 2 * (size_t)nt));
     far_geom_kernel<<<(nt + 127) / 128, 128, 0, st>>>(m->d_verts.p, m->d_tris.p, nt, pb->d_pt.p,
                                                       pb->d_poff.p, pb->d_cen.p, pb->d_tn.p,
                                                       pb->d_tv.p, pb->d_tgeo.p);
@@ -1084,22 +1268,33 @@ int far_setup_geometry(osrc_problem *pb, cudaStream_t st) {
         for (const ObjMat &o : pb->obj) kmax = fmax(kmax, o.k1);
         pb->far_reduce = kmax * diag > FAR_PLAIN_MAX_PHASE;
     }
-    // split the source range so that the grid covers the GPU several times
-    int dev = m->ctx->device, sms = 0, per_sm = 0;
+    // Test triangles per block and source splits.  Small meshes take few test
+    // triangles per block (the block's warps then share the sources); the
+    // splits, at least FAR_MIN_TPS source triangles each so that summing the
+    // partial sums stays small beside the pair work, fill the resident blocks
+    // four times over, and near that number the one with the fullest last
+    // wave is taken.
+    int dev = m->ctx->device, sms = 0;
     OSRC_CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    if (pb->far_reduce)
-        OSRC_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, far_kernel<true, false, false>, FAR_THREADS, 0));
-    else
-        OSRC_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, far_kernel<false, false, false>, FAR_THREADS, 0));
-    if (per_sm < 1) per_sm = 1;
-    const int bx = (pb->npts / 2 + FAR_THREADS - 1) / FAR_THREADS;
-    const int slots = sms * per_sm;
-    int ns = (4 * slots + bx - 1) / bx;
-    const int max_ns = (nt + FAR_TS - 1) / FAR_TS;
-    if (ns > max_ns) ns = max_ns;
-    if (ns < 1) ns = 1;
+    pb->far_tris = nt < FAR_TRIS32_NT ? 32 : nt < FAR_TRIS64_NT ? 64 : FAR_THREADS;
+    const int slots = sms * OSRC_FAR_MIN_BLOCKS;
+    const int bx = (nt + pb->far_tris - 1) / pb->far_tris;
+    const int max_ns = std::max(1, std::min(FAR_MAX_NS, nt / FAR_MIN_TPS));
+    const int ns0 = std::min(max_ns, std::max(1, (4 * slots + bx - 1) / bx));
+    int ns = ns0;
+    double best = -1.0;
+    for (int cand = std::max(1, ns0 / 2); cand <= std::min(max_ns, 2 * ns0); ++cand) {
+        const long long blocks = (long long)bx * cand;
+        const long long waves = (blocks + slots - 1) / slots;
+        const double eff = (double)blocks / (double)(waves * slots);
+        if (eff > best + 1e-9) {
+            best = eff;
+            ns = cand;
+        }
+    }
     pb->nsplit = ns;
-    OSRC_TRY(pb->d_part.alloc(m->ctx, (size_t)ns * 10 * pb->npts));
+    OSRC_TRY(pb->d_part.alloc(m->ctx, (size_t)ns * 4 * pb->npts));
+    OSRC_TRY(pb->d_partA1.alloc(m->ctx, (size_t)ns * 6 * nt));
     return OSRC_OK;
 }
 
@@ -1117,6 +1312,25 @@ int far_prof_collect(osrc_problem *pb) {
     return OSRC_OK;
 }
 
+static int gather_launch(osrc_problem *pb, int ns, int R, const float *part, const float *partA, int use_far,
+                         int use_near, const VecPtrs &x, const OutPtrs &y, cudaStream_t st) {
+    osrc_mesh *m = pb->mesh;
+    const int nv = pb->nv;
+    const int per = nv <= GATHER_BLOCK_NV ? 1 : nv <= GATHER_WARP_NV ? GATHER_THREADS / 32 : GATHER_THREADS / 8;
+    const dim3 grid((nv + per - 1) / per, R);
+#define OSRC_GATHER_LAUNCH(LL, WW)                                                                             \
+    gather_kernel<LL, WW><<<grid, GATHER_THREADS, 0, st>>>(nv, pb->nt, pb->npts, ns, R, m->d_vt_ptr.p, m->d_vt_idx.p, \
+                                                       pb->d_tgeo.p, part, partA, use_far, pb->d_nr_ptr.p,       \
+                                                       pb->d_nr_col.p, pb->d_nr_val.p, use_near, x, y)
+    if (nv <= GATHER_BLOCK_NV) OSRC_GATHER_LAUNCH(32, 4);
+    else if (nv <= GATHER_WARP_NV) OSRC_GATHER_LAUNCH(32, 1);
+    else OSRC_GATHER_LAUNCH(8, 1);
+#undef OSRC_GATHER_LAUNCH
+    pb->launches++;
+    OSRC_CK(cudaGetLastError());
+    return OSRC_OK;
+}
+
 int far_apply(osrc_problem *pb, const double2 *x, double2 *y, int part, cudaStream_t st) {
     osrc_mesh *m = pb->mesh;
     const int nt = pb->nt, nv = pb->nv, npts = pb->npts;
@@ -1124,7 +1338,7 @@ int far_apply(osrc_problem *pb, const double2 *x, double2 *y, int part, cudaStre
     const int use_near = (part & OSRC_PART_NEAR) ? 1 : 0;
     if (use_far) {
         const float4 *src_pts = pb->far_reduce ? pb->d_poff.p : pb->d_pt.p;
-        far_prep_kernel<<<(nt + 127) / 128, 128, 0, st>>>(x, nv, nt, m->d_tris.p, src_pts,
+        far_prep_kernel<<<(npts + 127) / 128, 128, 0, st>>>(x, nv, nt, m->d_tris.p, src_pts,
                                                           pb->d_tgeo.p, pb->d_sP.p, pb->d_sP5.p,
                                                           pb->d_sC.p);
         pb->launches++;
@@ -1146,7 +1360,7 @@ int far_apply(osrc_problem *pb, const double2 *x, double2 *y, int part, cudaStre
         const float4 kff = make_float4(q0h, (float)(q0 - (double)q0h), q1h, (float)(q1 - (double)q1h));
         const int ns = pb->nsplit;
         const int tps = (nt + ns - 1) / ns;
-        dim3 grid((npts / 2 + FAR_THREADS - 1) / FAR_THREADS, ns);
+        dim3 grid((nt + pb->far_tris - 1) / pb->far_tris, ns);
         if (pb->prof_on) {
             OSRC_TRY(far_prof_collect(pb));
             OSRC_CK(cudaEventRecord(pb->prof_ev[0], st));
@@ -1157,8 +1371,9 @@ int far_apply(osrc_problem *pb, const double2 *x, double2 *y, int part, cudaStre
         float *prt = pb->d_part.p;
         const bool ab = pb->absorb;
 #define OSRC_FAR_LAUNCH(C, M, A)                                                                               \
-    far_kernel<C, M, A><<<grid, FAR_THREADS, 0, st>>>(pts, pb->d_cen.p, pb->d_tn.p, pb->d_tv.p, pb->d_sP.p,      \
-                                                      pb->d_sP5.p, pb->d_sC.p, nt, npts, tps, c, kff, tc, fo, prt)
+    far_kernel<C, M, A><<<grid, FAR_THREADS, 0, st>>>(pts, pb->d_cen.p, pb->d_tn.p, pb->d_tv.p, pb->d_sP.p,  \
+                                                          pb->d_sP5.p, pb->d_sC.p, nt, npts, tps, pb->far_tris, c, kff, tc, fo, \
+                                                          prt, pb->d_partA1.p)
         if (pb->far_reduce && pb->far_obj && ab) OSRC_FAR_LAUNCH(true, true, true);
         else if (pb->far_reduce && pb->far_obj) OSRC_FAR_LAUNCH(true, true, false);
         else if (pb->far_reduce) OSRC_FAR_LAUNCH(true, false, false);
@@ -1172,12 +1387,11 @@ int far_apply(osrc_problem *pb, const double2 *x, double2 *y, int part, cudaStre
             pb->prof_pending = true;
         }
     }
-    gather_kernel<<<(nv + 127) / 128, 128, 0, st>>>(
-        nv, npts, pb->nsplit, m->d_vt_ptr.p, m->d_vt_idx.p, pb->d_tgeo.p, pb->d_part.p, use_far,
-        pb->d_nr_ptr.p, pb->d_nr_col.p, pb->d_nr_val.p, use_near, x, y);
-    pb->launches++;
-    OSRC_CK(cudaGetLastError());
-    return OSRC_OK;
+    VecPtrs xp{};
+    OutPtrs yp{};
+    xp.p[0] = x;
+    yp.p[0] = y;
+    return gather_launch(pb, pb->nsplit, 1, pb->d_part.p, pb->d_partA1.p, use_far, use_near, xp, yp, st);
 }
 
 // ---------------------------------------------------------------------------
@@ -1319,12 +1533,7 @@ static int farm_launch(osrc_problem *pb, const double2 *const *xs, double2 *cons
             pb->prof_rhs_pending = R;
         }
     }
-    farm_gather_kernel<<<dim3((nv + 127) / 128, R), 128, 0, st>>>(
-        nv, nt, npts, ns, R, m->d_vt_ptr.p, m->d_vt_idx.p, pb->d_tgeo.p, pb->d_partm.p, pb->d_partA.p, use_far,
-        pb->d_nr_ptr.p, pb->d_nr_col.p, pb->d_nr_val.p, use_near, xp, yp);
-    pb->launches++;
-    OSRC_CK(cudaGetLastError());
-    return OSRC_OK;
+    return gather_launch(pb, ns, R, pb->d_partm.p, pb->d_partA.p, use_far, use_near, xp, yp, st);
 }
 
 // OSRC_TIMEOUT if a several-right-hand-side far kernel gave up a bounded

@@ -961,6 +961,7 @@ int problem_clone(osrc_problem *m, osrc_problem **out) {
     c->nt = m->nt;
     c->npts = m->npts;
     c->nsplit = m->nsplit;
+    c->far_tris = m->far_tris;
     c->far_reduce = m->far_reduce;
     c->near_pairs = m->near_pairs;
     c->near_nnz = m->near_nnz;
@@ -999,9 +1000,10 @@ int problem_clone(osrc_problem *m, osrc_problem **out) {
     const int nt = m->nt, nv = m->nv;
     const int nsys = 2 * m->p.n_pade + 2;
     int s = OSRC_OK;
-    if ((s = c->d_sP.alloc(ctx, 30 * (size_t)nt)) || (s = c->d_sP5.alloc(ctx, 6 * (size_t)nt)) ||
-        (s = c->d_sC.alloc(ctx, 5 * (size_t)nt)) ||
-        (s = c->d_part.alloc(ctx, (size_t)c->nsplit * 10 * c->npts)) ||
+    if ((s = c->d_sP.alloc(ctx, 24 * (size_t)nt)) || (s = c->d_sP5.alloc(ctx, 6 * (size_t)nt)) ||
+        (s = c->d_sC.alloc(ctx, 2 * (size_t)nt)) ||
+        (s = c->d_part.alloc(ctx, (size_t)c->nsplit * 4 * c->npts)) ||
+        (s = c->d_partA1.alloc(ctx, (size_t)c->nsplit * 6 * nt)) ||
         (s = c->d_kry.alloc(ctx, 5 * (size_t)nsys * nv)) ||
         (s = c->d_kry_rhs.alloc(ctx, (size_t)(2 + nsys) * nv)) || (s = c->d_kry_stat.alloc(ctx, 40)) ||
         (s = c->d_kry_res.alloc(ctx, 40)) || (s = c->d_tmp2.alloc(ctx, 4 * (size_t)nv)) ||
@@ -1030,9 +1032,11 @@ size_t estimate_problem_bytes(int nv, int nt, const osrc_params &p) {
 size_t estimate_work_bytes(int nv, int nt, const osrc_params &p, int maxit) {
     const size_t nsys = 2 * (size_t)p.n_pade + 2;
     size_t b = 0;
-    b += (size_t)nt * (30 * 16 + 6 * 8 + 5 * 16);      // far source data
-    const size_t ns = std::min<size_t>(64, (size_t)(nt + 63) / 64);
-    b += ns * 10 * 6 * (size_t)nt * 4;                  // far partial sums
+    b += (size_t)nt * (24 * 16 + 6 * 8 + 2 * 16);      // far source data
+    // far partial sums: 4 floats per test point and 6 per triangle for each of
+    // at most 64 source splits (far_setup_geometry)
+    const size_t ns = std::min<size_t>(64, (size_t)(nt + 5) / 6);
+    b += ns * (4 * 6 + 6) * (size_t)nt * 4;
     b += nsys * nv * (5 + 1) * 16 + 2 * (size_t)nv * 16 + 4 * (size_t)nv * 16;  // inner solves
     b += (size_t)(maxit + 1) * 2 * nv * 16 + (size_t)(maxit + 1) * maxit * 16;   // Krylov basis
     b += (size_t)5 * 2 * nv * 16 + 6 * (size_t)(maxit + 1) * 16;

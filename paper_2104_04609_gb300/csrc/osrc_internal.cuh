@@ -181,13 +181,14 @@ struct osrc_problem {
     DBuf<float4> d_poff; // [6nt]  point minus triangle centroid, quadrature weight * area
     DBuf<float4> d_cen;  // [2nt]  triangle centroid as float pairs (hi, lo)
     DBuf<float4> d_tn;   // [nt]   outward normal, plane offset n.P0
-    DBuf<int4> d_tv;     // [nt]   vertex indices
+    DBuf<int4> d_tv;     // [nt]   vertex indices, offset bits of the first rule point (far_geom_kernel)
     // ---- far field: per-apply workspace ----------------------------------
-    DBuf<float4> d_sP;   // [6nt][5] source points: -y, psi, phi with both signs, duplicated pairs
+    DBuf<float4> d_sP;   // [6nt][4] source points: -y, psi, phi as duplicated pairs
     DBuf<float2> d_sP5;  // [6nt] (-phi.im, -phi.im)
-    DBuf<float4> d_sC;   // [nt][5] c_sigma components with both signs, duplicated pairs
-    DBuf<float> d_part;       // [nsplit][6nt][10] per test point partial sums
-    int nsplit = 1;
+    DBuf<float4> d_sC;   // [nt][2] c_sigma components
+    DBuf<float> d_part;       // [nsplit][4][6nt] per test point partial sums
+    DBuf<float> d_partA1;     // [nsplit][6][nt] curl-term partial sums per test triangle
+    int nsplit = 1, far_tris = 128;  // far kernel: source splits, test triangles per block
     // ---- far field, several right-hand sides per launch (k_far.cu farm_*) ----
     DBuf<float4> d_sG;        // [6nt][2] static source geometry (coordinates, rule weight)
     DBuf<float4> d_sD;        // [nt][6][R][2] densities of R right-hand sides

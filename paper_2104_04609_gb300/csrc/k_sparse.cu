@@ -16,9 +16,10 @@
 // Jacobi-preconditioned and stop at |r| <= tol |f|.  All loops are bounded by
 // the iteration cap; every CTA of a cluster takes the same branch because
 // the decisions are made from cluster-reduced values summed in rank order.
-// Two kernels share this layout: kmix_kernel (FP32 inner solves refined in
-// FP64, used whenever a CTA's rows and FP32 entries fit) and kry_kernel
-// (all FP64: larger meshes, in-place systems, the allocation-free entry).
+// Two kernels: kmix_kernel (FP32 inner solves refined in FP64, used whenever
+// a CTA's rows fit its registers; its vectors cross the cluster through
+// distributed shared memory) and kry_kernel (all FP64, the layout above:
+// larger meshes, in-place systems, the allocation-free entry).
 #include <cooperative_groups.h>
 #include <cuda.h>
 
@@ -62,7 +63,8 @@ __global__ void csr_sum_kernel(int nnz, const int *__restrict__ cptr, const int 
 }
 
 constexpr int KRY_THREADS = 256;
-constexpr int KRY_MAX_SYS = 40;
+constexpr int KRY_MAX_SYS = 128;  // systems per launch
+constexpr int KRY_STAT = 40;      // status words of one problem (2 * 16 + 2 systems at most)
 
 struct KrySys {
     double2 alpha, beta;  // system matrix alpha M + beta S
@@ -72,6 +74,8 @@ struct KrySys {
     // disjoint objects: row i uses beta * bscale[vcomp[i]] (S has no entries
     // between objects, so the matrix stays complex symmetric); null: beta
     const double2 *bscale;
+    int *stat;    // kmix_kernel: iteration count / status and relative residual
+    double *res;
 };
 
 struct KryBatch {
@@ -141,7 +145,7 @@ __device__ void cluster_sum3(cg::cluster_group &cl, double v0, double v1, double
 }
 
 __global__ void __launch_bounds__(KRY_THREADS)
-kry_kernel(KryBatch batch, int n, const int *__restrict__ ptr, const int *__restrict__ col,
+kry_kernel(const __grid_constant__ KryBatch batch, int n, const int *__restrict__ ptr, const int *__restrict__ col,
            const double *__restrict__ M, const double *__restrict__ S, double2 *__restrict__ work,
            double tol, int maxit, int *__restrict__ stat, double *__restrict__ res_out) {
     __shared__ double red[3 * 32];
@@ -261,76 +265,171 @@ kry_kernel(KryBatch batch, int n, const int *__restrict__ ptr, const int *__rest
 }
 
 // ---- mixed-precision refinement ---------------------------------------------
-// The same systems (alpha M + beta S) w = f, solved by iterative refinement
-// in the same cluster layout: an FP32 Jacobi-CG/COCG solve of A d = r, with
-// the FP32 copy of A built once per launch in shared memory and r scaled to
-// unit norm, reduces the residual by KMIX_INNER_TOL; then the FP64 solution
-// is updated, x += d, and the FP64 residual r = f - A x decides: stop when
-// |r| <= tol |f| (the criterion of kry_kernel, here on the true residual),
-// else refine again.  Most arithmetic runs on the FP32 pipe, which on this
-// part issues 64 times the FP64 rate; a refinement costs one FP64 product.
-// Refinement converges while cond(D^-1 A) * 2^-24 stays well below one (the
-// OSRC and mass systems sit near cond 10..100); a refinement that fails to
-// halve the residual norm ends the solve as not converged.
-constexpr int KMIX_THREADS = 512;          // at most, per CTA (two CTAs per SM)
-constexpr int KMIX_ROWS_PER_THREAD = 2;    // rows a thread owns, at most
-constexpr float KMIX_INNER_TOL = 1e-5f;    // residual reduction of one FP32 solve
+// The same systems (alpha M + beta S) w = f, solved by iterative refinement:
+// an FP32 Jacobi-CG/COCG solve of A d = r, with r scaled to unit norm, reduces
+// the residual by up to 2e-6; then the FP64 solution is updated, x += d,
+// and the FP64 residual r = f - A x decides: stop when |r| <= tol |f| (the
+// criterion of kry_kernel, here on the true residual), else refine again.
+// Most arithmetic runs on the FP32 pipe, which on this part issues 64 times
+// the FP64 rate; a refinement costs one FP64 product.  Refinement converges
+// while cond(D^-1 A) * 2^-24 stays well below one (the OSRC and mass systems
+// sit near cond 10..100); a refinement that fails to halve the residual norm
+// ends the solve as not converged.
+//
+// An iteration is latency: about 15 flops per matrix entry between
+// cluster-wide sums.  So a thread keeps one row (RPT rows) of A in registers,
+// every CTA holds z = D^-1 r of the rows that its columns name in its own
+// shared memory, and an iteration has two waits, those of its two sums: z is
+// sent with the sum (r, z), and after it q = A p follows from A z and the
+// recurrences p = z + beta p, q = A z + beta q, so the search direction is
+// never sent.  What crosses between CTAs (z of the rows that another CTA's
+// columns name, the CTAs' sums) goes by st.async, whose bytes the receiver's
+// mbarrier counts: no fence and no cluster barrier in the iteration (a release
+// at cluster scope cost 1000 to 2000 cycles a sum).  Rows are numbered by
+// reverse Cuthill-McKee (d_ms_perm), so that a CTA's columns lie mostly in
+// itself and its neighbours.  A system that fits one CTA needs no cluster.
+// One preconditioner apply (10 systems; before: three cluster barriers an
+// iteration, the search direction in L2, entries in shared memory): 10242
+// vertices 0.37 ms (0.66), 2562 0.26 (0.59), 642 0.20 (0.37), 150 0.13 (0.29).
+constexpr int KMIX_E = 8;                  // matrix entries of a row kept in registers
+constexpr int KMIX_THREADS1 = 768;         // most threads with one row each (80 registers)
+constexpr int KMIX_THREADS2 = 640;         // and with two (96)
+constexpr float KMIX_MIN_TOL = 2e-6f;      // most a FP32 solve reduces the residual by
 constexpr int KMIX_MAX_REFINE = 40;
-constexpr size_t KMIX_SMEM_MAX = 200 * 1024;
+constexpr int KMIX_SMEM_MAX = 200 * 1024;  // bytes of z
+constexpr int KMIX_MAX_N = KMIX_SMEM_MAX / 8;  // rows (also below 2^16: the column places are 16 bits)
 
-// Cluster-wide sums of NV values, identical in every thread of every CTA of
-// the cluster: butterflies within each warp, the warp sums added by a
-// butterfly in warp 0, then the CTA sums of all ranks (lane r reads rank r's
-// slot through distributed shared memory) added by a butterfly in warp 0.
-// IEEE addition is commutative, so every lane of a butterfly ends with the
-// same bits, and every CTA adds the same rank-ordered values.  A slot may be
-// written again once every CTA has passed one more cluster barrier.
+// Sum of NV <= 4 values over the warp by halving (each exchange hands half of
+// the values to the other lane: 6 shuffles for 3 or 4 values instead of 5 per
+// value): lane l < 4 ends with value kmix_slot(l).
+__device__ __forceinline__ int kmix_slot(int lane) { return 2 * (lane & 1) + ((lane >> 1) & 1); }
+
 template <typename T, int NV>
-__device__ __forceinline__ void kmix_csum(cg::cluster_group &cl, T (&v)[NV], T *wred, T *slot, T *out) {
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-        for (int k = 0; k < NV; ++k) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
-    if (lane == 0)
-#pragma unroll
-        for (int k = 0; k < NV; ++k) wred[NV * wid + k] = v[k];
-    __syncthreads();
-    if (wid == 0) {
-        T w[NV];
-#pragma unroll
-        for (int k = 0; k < NV; ++k) w[k] = lane < nw ? wred[NV * lane + k] : T(0);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-            for (int k = 0; k < NV; ++k) w[k] += __shfl_xor_sync(0xffffffffu, w[k], o);
-        if (lane == 0)
-#pragma unroll
-            for (int k = 0; k < NV; ++k) slot[k] = w[k];
+__device__ __forceinline__ T kmix_wsum(const T (&v)[NV], int lane) {
+    const T v0 = v[0], v1 = NV > 1 ? v[NV > 1 ? 1 : 0] : T(0), v2 = NV > 2 ? v[NV > 2 ? 2 : 0] : T(0);
+    T a;
+    if (NV > 2) {  // lane bit 0: values {2, 3} (3 is zero), else {0, 1}
+        const bool o = lane & 1, h = lane & 2;
+        const T k0 = (o ? v2 : v0) + __shfl_xor_sync(0xffffffffu, o ? v0 : v2, 1);
+        const T k1 = (o ? T(0) : v1) + __shfl_xor_sync(0xffffffffu, o ? v1 : T(0), 1);
+        a = (h ? k1 : k0) + __shfl_xor_sync(0xffffffffu, h ? k0 : k1, 2);
+    } else if (NV == 2) {  // lane bit 1: value 1
+        const bool h = lane & 2;
+        a = (h ? v1 : v0) + __shfl_xor_sync(0xffffffffu, h ? v0 : v1, 2);
+        a += __shfl_xor_sync(0xffffffffu, a, 1);
+    } else {
+        a = v0 + __shfl_xor_sync(0xffffffffu, v0, 1);
+        a += __shfl_xor_sync(0xffffffffu, a, 2);
     }
-    cl.sync();
-    if (wid == 0) {
-        const unsigned cs = cl.num_blocks();
-        T w[NV];
-        if ((unsigned)lane < cs) {
-            const T *rem = cl.map_shared_rank(slot, lane);
-#pragma unroll
-            for (int k = 0; k < NV; ++k) w[k] = rem[k];
-        } else {
-#pragma unroll
-            for (int k = 0; k < NV; ++k) w[k] = T(0);
+    a += __shfl_xor_sync(0xffffffffu, a, 4);
+    a += __shfl_xor_sync(0xffffffffu, a, 8);
+    a += __shfl_xor_sync(0xffffffffu, a, 16);
+    return a;
+}
+
+// One cluster-wide sum's mailbox: warp 0 of every CTA sends the CTA's sums to
+// slot[.][its rank] of each CTA of the cluster (st.async, counted in bytes by
+// that CTA's mbarrier); every thread waits for its own CTA's mbarrier, whose
+// one arrival is thread 0's with the bytes expected.  A box is used again only
+// after another box's sum, which every CTA enters after it has read this one.
+template <typename T, int NV>
+struct KmixBox {
+    uint64_t bar;
+    T slot[NV][16];
+    T wred[NV][32];  // the CTA's warp sums
+};
+
+constexpr unsigned long long KMIX_TIMEOUT_NS = 2000000000ULL;
+
+// waits for phase `parity`, at most KMIX_TIMEOUT_NS of global time
+__device__ __forceinline__ bool kmix_wait(uint32_t bar, uint32_t parity) {
+    unsigned long long t0 = 0;
+    for (int i = 0;; ++i) {
+        uint32_t done;
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+            "selp.u32 %0, 1, 0, p;\n\t}"
+            : "=r"(done)
+            : "r"(bar), "r"(parity)
+            : "memory");
+        if (done) return true;
+        if ((i & 1023) == 1023) {
+            unsigned long long t;
+            asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+            if (!t0) t0 = t;
+            else if (t - t0 > KMIX_TIMEOUT_NS) return false;
         }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-            for (int k = 0; k < NV; ++k) w[k] += __shfl_xor_sync(0xffffffffu, w[k], o);
-        if (lane == 0)
-#pragma unroll
-            for (int k = 0; k < NV; ++k) out[k] = w[k];
     }
+}
+
+// store to the cluster's shared memory, its bytes counted by the mbarrier bar
+// of the same CTA
+__device__ __forceinline__ void kmix_send(uint32_t a, uint32_t bar, float v) {
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];" ::"r"(a),
+                 "r"(__float_as_uint(v)), "r"(bar)
+                 : "memory");
+}
+__device__ __forceinline__ void kmix_send(uint32_t a, uint32_t bar, double v) {
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.b64 [%0], %1, [%2];" ::"r"(a),
+                 "l"(__double_as_longlong(v)), "r"(bar)
+                 : "memory");
+}
+__device__ __forceinline__ void kmix_send(uint32_t a, uint32_t bar, float2 v) {
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.b32 [%0], {%1, %2}, [%3];" ::"r"(a),
+                 "r"(__float_as_uint(v.x)), "r"(__float_as_uint(v.y)), "r"(bar)
+                 : "memory");
+}
+__device__ __forceinline__ uint32_t kmix_mapa(uint32_t a, uint32_t rank) {
+    uint32_t r;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
+    return r;
+}
+
+// Sums of NV values over the cluster (CL) or CTA, identical in every thread of
+// every CTA: the warps' sums meet in shared memory, warp 0 (CL; else every
+// warp) adds them, and the ranks' sums are added in the same order everywhere.
+// parity: phase of the box's next use, flipped here; extra: bytes that other
+// CTAs send with this sum besides the sums.  *dead is set when a wait gave up;
+// the waits after it are skipped.
+template <bool CL, typename T, int NV>
+__device__ __forceinline__ void kmix_csum(unsigned cs, unsigned rank, T (&v)[NV], KmixBox<T, NV> *box, uint32_t &parity,
+                                          uint32_t extra, volatile int *dead) {
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const int k = kmix_slot(lane);
+    T a = kmix_wsum<T, NV>(v, lane);
+    if (lane < 4 && k < NV) box->wred[k][wid] = a;
     __syncthreads();
+    if (!CL || wid == 0) {
 #pragma unroll
-    for (int k = 0; k < NV; ++k) v[k] = out[k];
+        for (int i = 0; i < NV; ++i) v[i] = lane < nw ? box->wred[i][lane] : T(0);
+        a = kmix_wsum<T, NV>(v, lane);
+    }
+    if (CL) {
+        const uint32_t bar = (uint32_t)__cvta_generic_to_shared(&box->bar);
+        if (wid == 0) {
+            if (lane == 0)
+                asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar),
+                             "r"((uint32_t)(cs * NV * sizeof(T)) + extra)
+                             : "memory");
+            const uint32_t to = min((unsigned)lane, cs - 1);
+            const uint32_t rbar = kmix_mapa(bar, to);
+            const uint32_t rslot = kmix_mapa((uint32_t)__cvta_generic_to_shared(&box->slot[0][rank]), to);
+#pragma unroll
+            for (int i = 0; i < NV; ++i) {
+                const T w = __shfl_sync(0xffffffffu, a, (i >> 1) | ((i & 1) << 1));
+                if ((unsigned)lane < cs) kmix_send(rslot + (uint32_t)(i * 16 * sizeof(T)), rbar, w);
+            }
+        }
+        if (!*dead && !kmix_wait(bar, parity)) *dead = 1;
+        __syncwarp();
+        parity ^= 1u;
+#pragma unroll
+        for (int i = 0; i < NV; ++i) v[i] = (unsigned)lane < cs ? box->slot[i][lane] : T(0);
+        a = kmix_wsum<T, NV>(v, lane);
+    }
+#pragma unroll
+    for (int i = 0; i < NV; ++i) v[i] = __shfl_sync(0xffffffffu, a, (i >> 1) | ((i & 1) << 1));
 }
 
 __device__ __forceinline__ float2 f2mul(float2 a, float2 b) {
@@ -339,75 +438,151 @@ __device__ __forceinline__ float2 f2mul(float2 a, float2 b) {
 __device__ __forceinline__ float2 f2dot(float2 a, float2 b, int conj) {
     return conj ? make_float2(a.x * b.x + a.y * b.y, a.x * b.y - a.y * b.x) : f2mul(a, b);
 }
+// a / b with an approximate reciprocal (PTX rcp.approx, 1 ulp: the same bits in
+// every CTA; an iteration's scalars need no more)
 __device__ __forceinline__ float2 f2div(float2 a, float2 b) {
-    const float den = b.x * b.x + b.y * b.y;
-    return make_float2((a.x * b.x + a.y * b.y) / den, (a.y * b.x - a.x * b.y) / den);
+    float ri;
+    asm("rcp.approx.f32 %0, %1;" : "=f"(ri) : "f"(b.x * b.x + b.y * b.y));
+    return make_float2((a.x * b.x + a.y * b.y) * ri, (a.y * b.x - a.x * b.y) * ri);
+}
+// a b + c
+__device__ __forceinline__ float2 f2fma(float2 a, float2 b, float2 c) {
+    return make_float2(fmaf(a.x, b.x, fmaf(-a.y, b.y, c.x)), fmaf(a.x, b.y, fmaf(a.y, b.x, c.y)));
 }
 
-// One cluster per system, rows [r0, r1) per CTA, row r0 + tid + k blockDim.x
-// for k < RPT per thread.  Dynamic shared memory: the CTA's CSR entries of
-// A in FP32 (float2) followed by their columns.  work32: n float2 per
-// system, the published FP32 search direction.  sy.x holds the published
-// FP64 solution.  Status and residual as kry_kernel; the iteration count is
-// the number of FP32 iterations over all refinements.
-template <int RPT>
-__global__ void __launch_bounds__(KMIX_THREADS, 2)
-kmix_kernel(KryBatch batch, int n, const int *__restrict__ ptr, const int *__restrict__ col,
-            const double *__restrict__ M, const double *__restrict__ S, float2 *__restrict__ work32,
-            double tol, int maxit, int *__restrict__ stat, double *__restrict__ res_out) {
-    extern __shared__ __align__(16) unsigned char kmix_dyn[];
-    __shared__ float wredf[3 * 32];
-    __shared__ double wredd[32];
-    __shared__ float slotP[2], slotR[3], slotI[3], outf[3];
-    __shared__ double slotD[1], slotB[1], outd[1];
+// One cluster (CL) or CTA per system; CTA rank r owns the rows perm[r rows ..
+// (r + 1) rows).  Dynamic shared memory: z by row number (the CTA's own rows
+// and those its columns name).  sy.x holds
+// the published FP64 solution.  Status and residual as kry_kernel; the
+// iteration count is the number of FP32 iterations over all refinements.
+template <int RPT, bool CL>
+__global__ void __launch_bounds__(RPT == 1 ? KMIX_THREADS1 : KMIX_THREADS2, 1)
+kmix_kernel(const __grid_constant__ KryBatch batch, int n, const int *__restrict__ ptr, const int *__restrict__ col,
+            const double *__restrict__ M, const double *__restrict__ S, const int *__restrict__ perm,
+            const int *__restrict__ inv, double tol, int maxit) {
+    extern __shared__ __align__(16) float2 zs[];
+    // the sums of an iteration, of a refinement's start, of its end and of the
+    // start: boxes of their own, so that none is written before the barrier
+    // after its last reading
+    __shared__ KmixBox<float, 2> boxP;
+    __shared__ KmixBox<float, 3> boxR, boxI;
+    __shared__ KmixBox<double, 1> boxD, boxB;
+    __shared__ int s_dead, s_cnt;
+    volatile int *dead = &s_dead;
+    uint32_t phP = 0, phR = 0, phI = 0, phD = 0, phB = 0;
     cg::cluster_group cl = cg::this_cluster();
-    const unsigned cs = cl.num_blocks();
-    const unsigned rank = cl.block_rank();
-    const int sid = blockIdx.x / cs;
-    const KrySys sy = batch.s[sid];
-    const int rows = (n + cs - 1) / cs;
+    const unsigned cs = CL ? cl.num_blocks() : 1u, rank = CL ? cl.block_rank() : 0u;
+    const KrySys &sy = batch.s[blockIdx.x / cs];
+    const int rows = (n + (int)cs - 1) / (int)cs;
     const int r0 = min(n, (int)rank * rows), r1 = min(n, r0 + rows);
-    const int ebase = r0 < n ? ptr[r0] : 0;
-    const int ne = r0 < r1 ? ptr[r1] - ebase : 0;
-    float2 *As = reinterpret_cast<float2 *>(kmix_dyn);
-    int *Cs = reinterpret_cast<int *>(kmix_dyn + sizeof(float2) * (size_t)((ne + 1) & ~1));
-    float2 *pg = work32 + (size_t)sid * n;
     double2 *xg = sy.x;
     const int cj = sy.conj;
+    if (threadIdx.x == 0) {
+        s_dead = 0;
+        if (CL) {
+            uint64_t *bars[5] = {&boxP.bar, &boxR.bar, &boxI.bar, &boxD.bar, &boxB.bar};
+            for (uint64_t *b : bars)
+                asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"((uint32_t)__cvta_generic_to_shared(b)),
+                             "r"(1));
+            asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        }
+    }
+    if (CL) cl.sync();  // every CTA of the cluster runs, its barriers initialised
+    else __syncthreads();
+    const uint32_t zbase = (uint32_t)__cvta_generic_to_shared(zs);
+    const uint32_t barR = (uint32_t)__cvta_generic_to_shared(&boxR.bar);
+    const uint32_t barI = (uint32_t)__cvta_generic_to_shared(&boxI.bar);
+    const float2 al0 = make_float2((float)sy.alpha.x, (float)sy.alpha.y);
 
-    // per row: the FP64 residual and the FP32 state (the FP64 solution
-    // lives in sy.x, the right-hand side is read again when needed)
-    int row[RPT];
+    // per row: the FP64 residual, the FP32 state and the row of A with the
+    // places of its columns' z (the FP64 solution lives in sy.x, the right-hand
+    // side is read again when needed); who: the other ranks that need its z,
+    // which are the owners of its columns (the pattern is symmetric)
+    int row[RPT], deg[RPT];
+    uint32_t who[RPT];
     bool ok[RPT];
     double2 r64[RPT];
+    float2 a[RPT][KMIX_E], be0[RPT];
+    uint16_t ad[RPT][KMIX_E];
     float2 dinv[RPT], d[RPT], r[RPT], z[RPT], p[RPT], q[RPT];
+    for (int i = threadIdx.x; i < n; i += blockDim.x) zs[i] = make_float2(0.f, 0.f);
+    __syncthreads();
     double bb = 0.0;
 #pragma unroll
     for (int k = 0; k < RPT; ++k) {
-        row[k] = r0 + threadIdx.x + k * blockDim.x;
-        ok[k] = row[k] < r1;
+        const int li = threadIdx.x + k * blockDim.x, i = r0 + li;
+        ok[k] = i < r1;
+        row[k] = ok[k] ? perm[i] : 0;
+        deg[k] = 0;
         r64[k] = cd(0.0, 0.0);
-        dinv[k] = make_float2(0.f, 0.f);
+        dinv[k] = be0[k] = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int e = 0; e < KMIX_E; ++e) {
+            a[k][e] = make_float2(0.f, 0.f);
+            ad[k][e] = 0;
+        }
+        who[k] = 0;
         if (ok[k]) {
-            const int i = row[k];
-            const double2 bi = sy.bscale ? cmul(sy.beta, sy.bscale[batch.vcomp[i]]) : sy.beta;
-            double2 dg = cd(0.0, 0.0);
-            for (int e = ptr[i]; e < ptr[i + 1]; ++e) {
-                const double2 a = cadd(cscale(sy.alpha, M[e]), cscale(bi, S[e]));
-                As[e - ebase] = make_float2((float)a.x, (float)a.y);
-                Cs[e - ebase] = col[e];
-                if (col[e] == i) dg = a;
+            const double2 b64 = sy.bscale ? cmul(sy.beta, sy.bscale[batch.vcomp[row[k]]]) : sy.beta;
+            be0[k] = make_float2((float)b64.x, (float)b64.y);
+            const int p0 = ptr[row[k]];
+            deg[k] = ptr[row[k] + 1] - p0;
+            float2 dg = make_float2(0.f, 0.f);
+#pragma unroll
+            for (int e = 0; e < KMIX_E; ++e)
+                if (e < deg[k]) {
+                    const int c = col[p0 + e];
+                    const float m = (float)M[p0 + e], s = (float)S[p0 + e];
+                    a[k][e] = make_float2(fmaf(be0[k].x, s, al0.x * m), fmaf(be0[k].y, s, al0.y * m));
+                    const int ci = inv[c];
+                    ad[k][e] = (uint16_t)ci;
+                    who[k] |= 1u << (ci / rows);
+                    if (CL && ci / rows != (int)rank) zs[ci].x = 1.f;  // mark: sent by its owner
+                    if (c == row[k]) dg = a[k][e];
+                }
+            for (int e = KMIX_E; e < deg[k]; ++e) {
+                const int ci = inv[col[p0 + e]];
+                who[k] |= 1u << (ci / rows);
+                if (CL && ci / rows != (int)rank) zs[ci].x = 1.f;
+                if (col[p0 + e] == row[k]) {
+                    const float m = (float)M[p0 + e], s = (float)S[p0 + e];
+                    dg = make_float2(fmaf(be0[k].x, s, al0.x * m), fmaf(be0[k].y, s, al0.y * m));
+                }
             }
-            const double2 di = cdiv(cd(1.0, 0.0), dg);
-            dinv[k] = make_float2((float)di.x, (float)di.y);
-            r64[k] = sy.f[i];
+            who[k] &= ~(1u << rank);
+            dinv[k] = f2div(make_float2(1.f, 0.f), dg);
+            r64[k] = sy.f[row[k]];
             bb += cabs2(r64[k]);
-            xg[i] = cd(0.0, 0.0);
         }
     }
-    {
+    // bytes of z that the other CTAs send with each sum (r, z)
+    uint32_t zbytes = 0;
+    if (CL) {
+        __syncthreads();
+        int cnt = 0;
+        for (int i = threadIdx.x; i < n; i += blockDim.x) {
+            cnt += zs[i].x != 0.f;
+            zs[i] = make_float2(0.f, 0.f);
+        }
+        if (threadIdx.x == 0) s_cnt = 0;
+        __syncthreads();
+        if (cnt) atomicAdd(&s_cnt, cnt);
+        __syncthreads();
+        zbytes = 8u * (uint32_t)s_cnt;
+    }
+    // z of row k to the CTA's own copy and to the CTAs that need it
+    auto publish = [&](int k, uint32_t bar) {
+        const int ci = r0 + threadIdx.x + k * blockDim.x;
+        zs[ci] = z[k];
+        if (CL)
+            for (uint32_t w = who[k]; w; w &= w - 1) {
+                const uint32_t to = __ffs(w) - 1;
+                kmix_send(kmix_mapa(zbase + 8u * (uint32_t)ci, to), kmix_mapa(bar, to), z[k]);
+            }
+    };
+    {   // its wait also ends the other CTAs' clearing of their copies
         double v[1] = {bb};
-        kmix_csum<double, 1>(cl, v, wredd, slotB, outd);  // its barrier also orders the shared-memory fill
+        kmix_csum<CL, double, 1>(cs, rank, v, &boxB, phB, 0u, dead);
         bb = v[0];
     }
     double rr = bb;
@@ -417,85 +592,94 @@ kmix_kernel(KryBatch batch, int n, const int *__restrict__ ptr, const int *__res
         for (int ref = 0; ref < KMIX_MAX_REFINE && its < maxit; ++ref) {
             // FP32 solve of A d = r / |r|
             const double sc = 1.0 / sqrt(rr);
+            // the reduction still needed, taken in one solve where FP32 can
+            // reach it (with a margin, so that the FP64 residual passes), else
+            // split evenly between this solve and the next
+            const double need = tol * sqrt(bb) * sc;
+            const float itol = (float)(need >= 1e-5 ? fmin(0.3 * need, 0.5) : fmax((double)KMIX_MIN_TOL, 0.5 * sqrt(need)));
             float v3[3] = {0.f, 0.f, 0.f};
 #pragma unroll
             for (int k = 0; k < RPT; ++k) {
                 r[k] = make_float2((float)(r64[k].x * sc), (float)(r64[k].y * sc));
                 z[k] = f2mul(dinv[k], r[k]);
-                p[k] = z[k];
-                d[k] = make_float2(0.f, 0.f);
+                p[k] = q[k] = d[k] = make_float2(0.f, 0.f);
                 if (ok[k]) {
-                    pg[row[k]] = p[k];
+                    publish(k, barI);
                     const float2 t = f2dot(r[k], z[k], cj);
                     v3[0] += t.x;
                     v3[1] += t.y;
                     v3[2] += r[k].x * r[k].x + r[k].y * r[k].y;
                 }
             }
-            kmix_csum<float, 3>(cl, v3, wredf, slotI, outf);  // also publishes p
-            float2 rho = make_float2(v3[0], v3[1]);
+            kmix_csum<CL, float, 3>(cs, rank, v3, &boxI, phI, zbytes, dead);  // also publishes z
+            float2 rho = make_float2(v3[0], v3[1]), be = make_float2(0.f, 0.f);
             const float rr0 = v3[2];
             bool brk = false;
             while (its < maxit) {
+                // p = z + beta p, q = A z + beta q
                 float v2[2] = {0.f, 0.f};
 #pragma unroll
                 for (int k = 0; k < RPT; ++k) {
-                    float2 acc = make_float2(0.f, 0.f);
-                    if (ok[k]) {
-                        const int eb = ptr[row[k]] - ebase, ee = ptr[row[k] + 1] - ebase;
-#pragma unroll 4
-                        for (int e = eb; e < ee; ++e) {
-                            const float2 a = As[e], pj = __ldcg(&pg[Cs[e]]);
-                            acc.x = fmaf(a.x, pj.x, fmaf(-a.y, pj.y, acc.x));
-                            acc.y = fmaf(a.x, pj.y, fmaf(a.y, pj.x, acc.y));
+                    p[k] = f2fma(be, p[k], z[k]);
+                    float2 s0 = make_float2(0.f, 0.f), s1 = s0;
+#pragma unroll
+                    for (int e = 0; e < KMIX_E; e += 2) {
+                        s0 = f2fma(a[k][e], zs[ad[k][e]], s0);
+                        s1 = f2fma(a[k][e + 1], zs[ad[k][e + 1]], s1);
+                    }
+                    if (deg[k] > KMIX_E) {  // entries past the registers
+                        const int p0 = ptr[row[k]];
+                        for (int e = KMIX_E; e < deg[k]; ++e) {
+                            const float m = (float)M[p0 + e], s = (float)S[p0 + e];
+                            const float2 ae = make_float2(fmaf(be0[k].x, s, al0.x * m), fmaf(be0[k].y, s, al0.y * m));
+                            s0 = f2fma(ae, zs[inv[col[p0 + e]]], s0);
                         }
-                        const float2 t = f2dot(p[k], acc, cj);
+                    }
+                    q[k] = f2fma(be, q[k], make_float2(s0.x + s1.x, s0.y + s1.y));
+                    if (ok[k]) {
+                        const float2 t = f2dot(p[k], q[k], cj);
                         v2[0] += t.x;
                         v2[1] += t.y;
                     }
-                    q[k] = acc;
                 }
-                kmix_csum<float, 2>(cl, v2, wredf, slotP, outf);
+                kmix_csum<CL, float, 2>(cs, rank, v2, &boxP, phP, 0u, dead);  // every CTA has read its columns
                 const float2 pq = make_float2(v2[0], v2[1]);
                 if (!(pq.x * pq.x + pq.y * pq.y > 0.f)) { brk = true; break; }
-                const float2 al = f2div(rho, pq);
+                const float2 al = f2div(rho, pq), mal = make_float2(-al.x, -al.y);
                 float w3[3] = {0.f, 0.f, 0.f};
 #pragma unroll
                 for (int k = 0; k < RPT; ++k) {
-                    d[k] = make_float2(fmaf(al.x, p[k].x, fmaf(-al.y, p[k].y, d[k].x)),
-                                       fmaf(al.x, p[k].y, fmaf(al.y, p[k].x, d[k].y)));
-                    r[k] = make_float2(fmaf(-al.x, q[k].x, fmaf(al.y, q[k].y, r[k].x)),
-                                       fmaf(-al.x, q[k].y, fmaf(-al.y, q[k].x, r[k].y)));
+                    d[k] = f2fma(al, p[k], d[k]);
+                    r[k] = f2fma(mal, q[k], r[k]);
                     z[k] = f2mul(dinv[k], r[k]);
                     if (ok[k]) {
+                        publish(k, barR);
                         const float2 t = f2dot(r[k], z[k], cj);
                         w3[0] += t.x;
                         w3[1] += t.y;
                         w3[2] += r[k].x * r[k].x + r[k].y * r[k].y;
                     }
                 }
-                kmix_csum<float, 3>(cl, w3, wredf, slotR, outf);
+                kmix_csum<CL, float, 3>(cs, rank, w3, &boxR, phR, zbytes, dead);
                 ++its;
-                if (w3[2] <= KMIX_INNER_TOL * KMIX_INNER_TOL * rr0) break;
+                if (CL && *dead) { brk = true; break; }
+                if (w3[2] <= itol * itol * rr0) break;
                 if (!(rho.x * rho.x + rho.y * rho.y > 0.f)) { brk = true; break; }
                 const float2 rz = make_float2(w3[0], w3[1]);
-                const float2 be = f2div(rz, rho);
+                be = f2div(rz, rho);
                 rho = rz;
-#pragma unroll
-                for (int k = 0; k < RPT; ++k) {
-                    p[k] = make_float2(fmaf(be.x, p[k].x, fmaf(-be.y, p[k].y, z[k].x)),
-                                       fmaf(be.x, p[k].y, fmaf(be.y, p[k].x, z[k].y)));
-                    if (ok[k]) pg[row[k]] = p[k];
-                }
-                cl.sync();  // p published
             }
             if (brk) { status = 2; break; }
             // FP64 update and residual
             const double back = sqrt(rr);
 #pragma unroll
             for (int k = 0; k < RPT; ++k)
-                if (ok[k]) xg[row[k]] = cadd(xg[row[k]], cd((double)d[k].x * back, (double)d[k].y * back));
-            cl.sync();  // x published
+                if (ok[k]) {
+                    const double2 dx = cd((double)d[k].x * back, (double)d[k].y * back);
+                    xg[row[k]] = ref ? cadd(xg[row[k]], dx) : dx;
+                }
+            if (CL) cl.sync();  // x published
+            else __syncthreads();
             double rn = 0.0;
 #pragma unroll
             for (int k = 0; k < RPT; ++k) {
@@ -515,7 +699,7 @@ kmix_kernel(KryBatch batch, int n, const int *__restrict__ ptr, const int *__res
                 rn += cabs2(r64[k]);
             }
             double v[1] = {rn};
-            kmix_csum<double, 1>(cl, v, wredd, slotD, outd);
+            kmix_csum<CL, double, 1>(cs, rank, v, &boxD, phD, 0u, dead);
             const double rprev = rr;
             rr = v[0];
             if (rr <= tol * tol * bb) { status = 0; break; }
@@ -523,11 +707,14 @@ kmix_kernel(KryBatch batch, int n, const int *__restrict__ ptr, const int *__res
         }
     } else {
         rr = 0.0;
+#pragma unroll
+        for (int k = 0; k < RPT; ++k)
+            if (ok[k]) xg[row[k]] = cd(0.0, 0.0);
     }
-    cl.sync();  // keep shared memory alive until every CTA has read it
+    if (CL) cl.sync();  // keep shared memory alive until every CTA has read it
     if (rank == 0 && threadIdx.x == 0) {
-        stat[sid] = status == 0 ? its : (status == 1 ? -its : -1000000 - its);
-        res_out[sid] = bb > 0.0 ? sqrt(rr / bb) : 0.0;
+        *sy.stat = status == 0 ? its : (status == 1 ? -its : -1000000 - its);
+        *sy.res = bb > 0.0 ? sqrt(rr / bb) : 0.0;
     }
 }
 
@@ -558,21 +745,34 @@ struct OsrcComb {
     double2 g[16];
 };
 
+constexpr int OSRC_COMB_RUNS = 16;  // workspaces per launch
+struct OsrcCombRuns {
+    const double2 *sol[OSRC_COMB_RUNS];
+    double2 *z[OSRC_COMB_RUNS];
+};
+
 // sol[0] = u1 = M^-1 y1, sol[1..np] = v_j, sol[np+1] = v'_0, sol[np+2..2np+1] = v'_j:
-//   z1 = i k [(C0 + sum_j A_j/B_j) u1 - sum_j (A_j/B_j) v_j]
-//   z2 = [g0 v'_0 + sum_j g_j v'_j] / (i k)
-__global__ void osrc_combine_kernel(int n, OsrcComb c, const double2 *__restrict__ sol,
-                                    double2 *__restrict__ z) {
+//   z1 = i k [(C0 + sum_j A_j/B_j) u1 - sum_j (A_j/B_j) v_j]   (blockIdx.y 0)
+//   z2 = [g0 v'_0 + sum_j g_j v'_j] / (i k)                   (blockIdx.y 1)
+// One thread per entry and block row, small blocks: FP64 chains are slow on
+// this part, and a thread with both block rows in blocks of 256 took 8.4 us
+// on 642 vertices.
+__global__ void osrc_combine_kernel(int n, const __grid_constant__ OsrcComb c, const __grid_constant__ OsrcCombRuns v) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
-    double2 a = cmul(c.cu, sol[i]);
-    for (int j = 0; j < c.np; ++j) a = csub(a, cmul(c.a[j], sol[(size_t)(1 + j) * n + i]));
-    double2 b = cmul(c.g0, sol[(size_t)(c.np + 1) * n + i]);
-    for (int j = 0; j < c.np; ++j) b = cadd(b, cmul(c.g[j], sol[(size_t)(c.np + 2 + j) * n + i]));
+    const double2 *sol = v.sol[blockIdx.z];
+    double2 *z = v.z[blockIdx.z];
     const double2 ik = c.ik_obj ? c.ik_obj[c.vcomp[i]] : c.ik;
-    const double2 iik = c.ik_obj ? cdiv(cd(1.0, 0.0), ik) : c.iik;
-    z[i] = cmul(ik, a);
-    z[n + i] = cmul(iik, b);
+    if (blockIdx.y == 0) {
+        double2 a = cmul(c.cu, sol[i]);
+        for (int j = 0; j < c.np; ++j) a = csub(a, cmul(c.a[j], sol[(size_t)(1 + j) * n + i]));
+        z[i] = cmul(ik, a);
+    } else {
+        const double2 iik = c.ik_obj ? cdiv(cd(1.0, 0.0), ik) : c.iik;
+        double2 b = cmul(c.g0, sol[(size_t)(c.np + 1) * n + i]);
+        for (int j = 0; j < c.np; ++j) b = cadd(b, cmul(c.g[j], sol[(size_t)(c.np + 2 + j) * n + i]));
+        z[n + i] = cmul(iik, b);
+    }
 }
 
 // Largest cluster the kernels may use on each device: 16 CTAs (a
@@ -613,48 +813,32 @@ int cluster_size_for(int n) {
     return cs;
 }
 
-template <int RPT>
-int kmix_attrs() {
-    OSRC_CK(cudaFuncSetAttribute(kmix_kernel<RPT>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-    OSRC_CK(cudaFuncSetAttribute(kmix_kernel<RPT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)KMIX_SMEM_MAX));
-    return OSRC_OK;
-}
+// Launch shape of kmix_kernel for nsys systems of n rows: cluster size, rows
+// per thread, threads; cs = 0: not usable (too many rows, or no cluster of that
+// shape fits the device).  Among the cluster sizes the one with the smallest
+// estimate is taken: the time of an iteration, measured as 0.85 us (one CTA) or
+// 1.85 us (cluster) of sums plus 1.3 ns per row of a CTA, times the load of the
+// device beyond one wave (the average system takes about 0.6 of the hardest
+// one's iterations and the hardest start first).
+struct KmixPlan {
+    int nsys = 0, cs = 0, rpt = 0, threads = 0;
+};
 
-// Decides once per problem whether the mixed-precision kernel serves its
-// systems: every CTA's rows within KMIX_THREADS x KMIX_ROWS_PER_THREAD, its
-// FP32 entries within KMIX_SMEM_MAX, and the device able to hold one cluster
-// of that shape.
-int kmix_decide(osrc_problem *pb, int cs) {
-    if (pb->kmix_state >= 0) return OSRC_OK;
-    pb->kmix_state = 0;
-    const int n = pb->nv;
-    if ((int)pb->ms_ptr_h.size() != n + 1) return OSRC_OK;
-    const int rows = (n + cs - 1) / cs;
-    const int rpt = (rows + KMIX_THREADS - 1) / KMIX_THREADS;
-    if (rpt < 1 || rpt > KMIX_ROWS_PER_THREAD) return OSRC_OK;
-    size_t smem = 0;
-    for (int k = 0; k < cs; ++k) {
-        const int r0 = std::min(n, k * rows), r1 = std::min(n, r0 + rows);
-        const size_t ne = (size_t)(pb->ms_ptr_h[r1] - pb->ms_ptr_h[r0]);
-        smem = std::max(smem, sizeof(float2) * ((ne + 1) & ~(size_t)1) + sizeof(int) * ne);
-    }
-    if (smem > KMIX_SMEM_MAX) return OSRC_OK;
-    const int threads = ((rows + rpt - 1) / rpt + 31) / 32 * 32;
-    static PerDeviceOnce once;
-    const int attr_status = per_device_once(once, [](int) -> int {
-        int st = kmix_attrs<1>();
-        if (st == OSRC_OK) st = kmix_attrs<2>();
-        return st;
-    });
-    if (attr_status != OSRC_OK) {  // no opt-in on this device: the FP64 kernel serves
-        (void)cudaGetLastError();
-        return OSRC_OK;
-    }
+template <int RPT, bool CL>
+int kmix_active_clusters(int n, int cs, int threads, int *count) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(cs, 1, 1);
     cfg.blockDim = dim3(threads, 1, 1);
-    cfg.dynamicSmemBytes = smem;
+    cfg.dynamicSmemBytes = (size_t)n * sizeof(float2);
+    if (!CL) {
+        int per_sm = 0, dev = 0, sms = 0;
+        OSRC_CK(cudaGetDevice(&dev));
+        OSRC_CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+        OSRC_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kmix_kernel<RPT, CL>, threads,
+                                                              cfg.dynamicSmemBytes));
+        *count = per_sm * sms;
+        return OSRC_OK;
+    }
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = cs;
@@ -662,18 +846,85 @@ int kmix_decide(osrc_problem *pb, int cs) {
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    int nclusters = 0;
-    const cudaError_t e = rpt == 1 ? cudaOccupancyMaxActiveClusters(&nclusters, kmix_kernel<1>, &cfg)
-                                   : cudaOccupancyMaxActiveClusters(&nclusters, kmix_kernel<2>, &cfg);
-    if (e != cudaSuccess) {
+    if (cudaOccupancyMaxActiveClusters(count, kmix_kernel<RPT, CL>, &cfg) != cudaSuccess) {
         (void)cudaGetLastError();
-        return OSRC_OK;
+        *count = 0;
     }
-    if (nclusters < 1) return OSRC_OK;
-    pb->kmix_state = 1;
-    pb->kmix_rpt = rpt;
-    pb->kmix_threads = threads;
-    pb->kmix_smem = smem;
+    return OSRC_OK;
+}
+
+int kmix_plan(osrc_problem *pb, int nsys, KmixPlan *out) {
+    *out = KmixPlan{};
+    const int n = pb->nv;
+    if (!pb->d_ms_perm.p || n > KMIX_MAX_N) return OSRC_OK;
+    for (const auto &q : pb->kmix_plans)
+        if (q[0] == nsys) {
+            out->nsys = q[0];
+            out->cs = q[1];
+            out->rpt = q[2];
+            out->threads = q[3];
+            return OSRC_OK;
+        }
+    static PerDeviceOnce once;
+    static int max_cluster[OSRC_MAX_DEVICES] = {};
+    OSRC_TRY(per_device_once(once, [](int dev) -> int {
+        max_cluster[dev] = 8;
+        OSRC_CK(cudaFuncSetAttribute(kmix_kernel<1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, KMIX_SMEM_MAX));
+        OSRC_CK(cudaFuncSetAttribute(kmix_kernel<2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, KMIX_SMEM_MAX));
+        if (cudaFuncSetAttribute(kmix_kernel<1, true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+            cudaFuncSetAttribute(kmix_kernel<2, true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess)
+            max_cluster[dev] = 16;
+        (void)cudaGetLastError();
+        return (int)OSRC_OK;
+    }));
+    int dev = 0;
+    OSRC_CK(cudaGetDevice(&dev));
+    KmixPlan best;
+    best.nsys = nsys;
+    double cost = 1e300;
+    for (int cs = 1; cs <= max_cluster[dev]; ++cs) {
+        const int rows = (n + cs - 1) / cs;
+        const int rpt = rows <= KMIX_THREADS1 ? 1 : 2;
+        const int threads = ((rows + rpt - 1) / rpt + 31) / 32 * 32;
+        if (rpt == 2 && threads > KMIX_THREADS2) continue;
+        int count = 0;
+        auto active = cs == 1 ? (rpt == 1 ? kmix_active_clusters<1, false> : kmix_active_clusters<2, false>)
+                              : (rpt == 1 ? kmix_active_clusters<1, true> : kmix_active_clusters<2, true>);
+        OSRC_TRY(active(n, cs, threads, &count));
+        if (count < 1) continue;
+        const double load = std::max(1.0, 0.6 * nsys / count);
+        const double t = load * ((cs == 1 ? 0.85 : 1.85) + 1.3e-3 * rows);
+        if (t < cost * (1.0 - 1e-9)) {
+            cost = t;
+            best.cs = cs;
+            best.rpt = rpt;
+            best.threads = threads;
+        }
+    }
+    if (pb->kmix_plans.size() < 16) pb->kmix_plans.push_back({best.nsys, best.cs, best.rpt, best.threads});
+    *out = best;
+    return OSRC_OK;
+}
+
+template <int RPT, bool CL>
+int kmix_launch(osrc_problem *pb, const KryBatch &batch, const KmixPlan &pl, cudaStream_t st) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(batch.nsys * pl.cs, 1, 1);
+    cfg.blockDim = dim3(pl.threads, 1, 1);
+    cfg.dynamicSmemBytes = (size_t)pb->nv * sizeof(float2);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = pl.cs;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = CL ? 1 : 0;
+    OSRC_CK(cudaLaunchKernelEx(&cfg, kmix_kernel<RPT, CL>, batch, pb->nv, (const int *)pb->d_ms_ptr.p,
+                               (const int *)pb->d_ms_col.p, (const double *)pb->d_M.p, (const double *)pb->d_S.p,
+                               (const int *)pb->d_ms_perm.p, (const int *)(pb->d_ms_perm.p + pb->nv),
+                               pb->p.inner_tol, pb->p.inner_maxit));
+    pb->launches++;
     return OSRC_OK;
 }
 
@@ -681,40 +932,24 @@ static bool ranges_overlap(const double2 *a, const double2 *b, int n) {
     return a < b + n && b < a + n;
 }
 
-int launch_kry(osrc_problem *pb, const KryBatch &batch, cudaStream_t st) {
-    OSRC_TRY(kry_opt_in());
+// One launch for the batch.  kmix_kernel starts the hardest systems (largest
+// |beta|: closest to the stiffness matrix) first; kry_kernel, whose status
+// words go by system number, takes the systems of one workspace in order.
+int launch_kry(osrc_problem *pb, KryBatch &batch, cudaStream_t st) {
     const int n = pb->nv;
-    const int cs = cluster_size_for(n);
-    OSRC_TRY(kmix_decide(pb, cs));
-    bool mix = pb->kmix_state == 1;
+    KmixPlan pl;
+    OSRC_TRY(kmix_plan(pb, batch.nsys, &pl));
+    bool mix = pl.cs > 0;
     for (int k = 0; k < batch.nsys && mix; ++k)  // in-place systems stay on the FP64 kernel
         if (ranges_overlap(batch.s[k].f, batch.s[k].x, n)) mix = false;
     if (mix) {
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(batch.nsys * cs, 1, 1);
-        cfg.blockDim = dim3(pb->kmix_threads, 1, 1);
-        cfg.dynamicSmemBytes = pb->kmix_smem;
-        cfg.stream = st;
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = cs;
-        attr[0].val.clusterDim.y = 1;
-        attr[0].val.clusterDim.z = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
-        float2 *w32 = reinterpret_cast<float2 *>(pb->d_kry.p);
-        const int *ptr = pb->d_ms_ptr.p, *col = pb->d_ms_col.p;
-        if (pb->kmix_rpt == 1)
-            OSRC_CK(cudaLaunchKernelEx(&cfg, kmix_kernel<1>, batch, n, ptr, col, (const double *)pb->d_M.p,
-                                       (const double *)pb->d_S.p, w32, pb->p.inner_tol, pb->p.inner_maxit,
-                                       pb->d_kry_stat.p, pb->d_kry_res.p));
-        else
-            OSRC_CK(cudaLaunchKernelEx(&cfg, kmix_kernel<2>, batch, n, ptr, col, (const double *)pb->d_M.p,
-                                       (const double *)pb->d_S.p, w32, pb->p.inner_tol, pb->p.inner_maxit,
-                                       pb->d_kry_stat.p, pb->d_kry_res.p));
-        pb->launches++;
-        return OSRC_OK;
+        std::stable_sort(batch.s, batch.s + batch.nsys,
+                         [](const KrySys &a, const KrySys &c) { return cabs2(a.beta) > cabs2(c.beta); });
+        if (pl.cs == 1) return pl.rpt == 1 ? kmix_launch<1, false>(pb, batch, pl, st) : kmix_launch<2, false>(pb, batch, pl, st);
+        return pl.rpt == 1 ? kmix_launch<1, true>(pb, batch, pl, st) : kmix_launch<2, true>(pb, batch, pl, st);
     }
+    OSRC_TRY(kry_opt_in());
+    const int cs = cluster_size_for(n);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(batch.nsys * cs, 1, 1);
     cfg.blockDim = dim3(KRY_THREADS, 1, 1);
@@ -738,7 +973,7 @@ int launch_kry(osrc_problem *pb, const KryBatch &batch, cudaStream_t st) {
 // Reads back the inner solver status (one small copy; the caller's stream is
 // synchronised) and turns non-convergence into a status code.
 int check_kry(osrc_problem *pb, int nsys, cudaStream_t st) {
-    int stat[KRY_MAX_SYS];
+    int stat[KRY_STAT];
     OSRC_CK(cudaMemcpyAsync(stat, pb->d_kry_stat.p, nsys * sizeof(int), cudaMemcpyDeviceToHost, st));
     OSRC_CK(cudaStreamSynchronize(st));
     return kry_status_host(pb, stat, nsys);
@@ -772,24 +1007,16 @@ int ms_build(osrc_problem *pb, const std::vector<int> &cptr, const std::vector<i
     const int nsys = 2 * pb->p.n_pade + 2;
     OSRC_TRY(pb->d_kry.alloc(ctx, 5 * (size_t)nsys * pb->nv));
     OSRC_TRY(pb->d_kry_rhs.alloc(ctx, (size_t)(2 + nsys) * pb->nv));
-    OSRC_TRY(pb->d_kry_stat.alloc(ctx, KRY_MAX_SYS));
-    OSRC_TRY(pb->d_kry_res.alloc(ctx, KRY_MAX_SYS));
+    OSRC_TRY(pb->d_kry_stat.alloc(ctx, KRY_STAT));
+    OSRC_TRY(pb->d_kry_res.alloc(ctx, KRY_STAT));
     OSRC_CK(cudaStreamSynchronize(st));
     return OSRC_OK;
 }
 
+static int mass_solve_async(osrc_problem *pb, const double2 *y, double2 *z, bool swap, cudaStream_t st);
+
 int mass_solve(osrc_problem *pb, const double2 *x, double2 *y, cudaStream_t st) {
-    const int n = pb->nv;
-    KryBatch b{};
-    b.nsys = 2;
-    for (int k = 0; k < 2; ++k) {
-        b.s[k].alpha = cd(1.0, 0.0);
-        b.s[k].beta = cd(0.0, 0.0);
-        b.s[k].f = x + (size_t)k * n;
-        b.s[k].x = y + (size_t)k * n;
-        b.s[k].conj = 1;
-    }
-    OSRC_TRY(launch_kry(pb, b, st));
+    OSRC_TRY(mass_solve_async(pb, x, y, false, st));
     return check_kry(pb, 2, st);
 }
 
@@ -805,17 +1032,24 @@ int osrc_precond_nsys(const osrc_problem *pb) {
 }
 
 // both block rows of M^-1 y; rows swapped in the output when swap is set
-static int mass_solve_async(osrc_problem *pb, const double2 *y, double2 *z, bool swap, cudaStream_t st) {
+static void mass_systems(osrc_problem *pb, const double2 *y, double2 *z, bool swap, KryBatch &b) {
     const int n = pb->nv;
-    KryBatch b{};
-    b.nsys = 2;
     for (int k = 0; k < 2; ++k) {
-        b.s[k].alpha = cd(1.0, 0.0);
-        b.s[k].beta = cd(0.0, 0.0);
-        b.s[k].f = y + (size_t)k * n;
-        b.s[k].x = z + (size_t)(swap ? 1 - k : k) * n;
-        b.s[k].conj = 1;
+        KrySys &s = b.s[b.nsys++];
+        s = KrySys{};
+        s.alpha = cd(1.0, 0.0);
+        s.beta = cd(0.0, 0.0);
+        s.f = y + (size_t)k * n;
+        s.x = z + (size_t)(swap ? 1 - k : k) * n;
+        s.conj = 1;
+        s.stat = pb->d_kry_stat.p + k;
+        s.res = pb->d_kry_res.p + k;
     }
+}
+
+static int mass_solve_async(osrc_problem *pb, const double2 *y, double2 *z, bool swap, cudaStream_t st) {
+    KryBatch b{};
+    mass_systems(pb, y, z, swap, b);
     return launch_kry(pb, b, st);
 }
 
@@ -835,62 +1069,72 @@ int osrc_precond_fused(osrc_problem *pb, const double2 *y, double2 *z, cudaStrea
     return check_kry(pb, osrc_precond_nsys(pb), st);
 }
 
-int osrc_precond_fused_async(osrc_problem *pb, const double2 *y, double2 *z, cudaStream_t st) {
+// the 2 N_Pade + 2 systems of P M^-1 y, solutions after the weak-form input in
+// d_kry_rhs
+static void osrc_systems(osrc_problem *pb, const double2 *y, KryBatch &b) {
     const int n = pb->nv, np = pb->p.n_pade;
-    if (pb->p.precond == OSRC_PRECOND_MASS) return mass_solve_async(pb, y, z, false, st);
-    if (pb->p.precond == OSRC_PRECOND_CALDERON) {
-        // z = M^-1 B Pi M^-1 y: the first mass solve writes its rows swapped
-        double2 *t = pb->d_kry_rhs.p + 2 * (size_t)n, *w = pb->d_tmp2.p + 2 * (size_t)n;
-        OSRC_TRY(mass_solve_async(pb, y, t, true, st));
-        if (pb->p.precision == OSRC_FP64_DENSE) OSRC_TRY(dense_apply(pb, t, w, st));
-        else OSRC_TRY(far_apply(pb, t, w, OSRC_PART_ALL, st));
-        return mass_solve_async(pb, w, z, false, st);
-    }
     const double2 ke2 = cmul(pb->k_eps, pb->k_eps);
     // disjoint objects: 1/k_eps^2 of each row's object via KrySys::bscale
     const double2 inv_ke2 = pb->multi ? cd(1.0, 0.0) : cdiv(cd(1.0, 0.0), ke2);
     const double2 *bscale = pb->multi ? pb->d_obj_ike.p + pb->mesh->ncomp : nullptr;
     double2 *sol = pb->d_kry_rhs.p + 2 * (size_t)n;
     const double2 *y1 = y, *y2 = y + n;
-    KryBatch b{};
-    b.nsys = 2 * np + 2;
     b.vcomp = pb->mesh->d_vcomp.p;
-    {   // M u1 = y1 (Hermitian CG)
-        KrySys &s = b.s[0];
+    // solution k: 0 M u1 = y1 (Hermitian CG); 1..np DtN (M - B_j S / k_eps^2) v_j = y1;
+    // np + 1 NtD (M - S / k_eps^2) v'_0 = y2; then NtD (M - B_j S / k_eps^2) v'_j = y2
+    for (int k = 0; k < 2 * np + 2; ++k) {
+        KrySys &s = b.s[b.nsys++];
+        s = KrySys{};
         s.alpha = cd(1.0, 0.0);
-        s.beta = cd(0.0, 0.0);
-        s.f = y1;
-        s.x = sol;
-        s.conj = 1;
+        const int j = k <= np ? k - 1 : k - np - 2;  // Pade term (-1: none)
+        s.beta = k == 0 ? cd(0.0, 0.0) : cscale(j < 0 ? inv_ke2 : cmul(pb->B[j], inv_ke2), -1.0);
+        s.bscale = k == 0 ? nullptr : bscale;
+        s.f = k <= np ? y1 : y2;
+        s.x = sol + (size_t)k * n;
+        s.conj = k == 0 ? 1 : 0;
+        s.stat = pb->d_kry_stat.p + k;
+        s.res = pb->d_kry_res.p + k;
     }
-    for (int j = 0; j < np; ++j) {  // DtN: (M - B_j S / k_eps^2) v_j = y1
-        KrySys &s = b.s[1 + j];
-        s.alpha = cd(1.0, 0.0);
-        s.beta = cscale(cmul(pb->B[j], inv_ke2), -1.0);
-        s.bscale = bscale;
-        s.f = y1;
-        s.x = sol + (size_t)(1 + j) * n;
-        s.conj = 0;
+}
+
+// z_r = P M^-1 y_r for nrun workspaces (the problem itself or clones of one
+// problem): the systems of all of them in as few launches as they fit
+// (KRY_MAX_SYS), so that the lockstep solve's right-hand sides fill the GPU
+// together instead of one after the other.
+int osrc_precond_fused_multi(osrc_problem *const *pbs, const double2 *const *ys, double2 *const *zs, int nrun,
+                             cudaStream_t st) {
+    osrc_problem *pb = pbs[0];
+    const int n = pb->nv, np = pb->p.n_pade;
+    if (pb->p.precond == OSRC_PRECOND_CALDERON) {
+        // z = M^-1 B Pi M^-1 y: the first mass solve writes its rows swapped
+        for (int r = 0; r < nrun; ++r) {
+            osrc_problem *q = pbs[r];
+            double2 *t = q->d_kry_rhs.p + 2 * (size_t)n, *w = q->d_tmp2.p + 2 * (size_t)n;
+            OSRC_TRY(mass_solve_async(q, ys[r], t, true, st));
+            if (q->p.precision == OSRC_FP64_DENSE) OSRC_TRY(dense_apply(q, t, w, st));
+            else OSRC_TRY(far_apply(q, t, w, OSRC_PART_ALL, st));
+            OSRC_TRY(mass_solve_async(q, w, zs[r], false, st));
+        }
+        return OSRC_OK;
     }
-    {   // NtD: (M - S / k_eps^2) v'_0 = y2
-        KrySys &s = b.s[np + 1];
-        s.alpha = cd(1.0, 0.0);
-        s.beta = cscale(inv_ke2, -1.0);
-        s.bscale = bscale;
-        s.f = y2;
-        s.x = sol + (size_t)(np + 1) * n;
-        s.conj = 0;
+    const bool mass = pb->p.precond == OSRC_PRECOND_MASS;
+    const int per = mass ? 2 : 2 * np + 2;
+    int group = std::max(1, std::min(nrun, KRY_MAX_SYS / per));
+    if (group > 1) {  // only the mixed kernel takes systems of several workspaces
+        KmixPlan pl;
+        OSRC_TRY(kmix_plan(pb, per * group, &pl));
+        if (pl.cs == 0) group = 1;
     }
-    for (int j = 0; j < np; ++j) {  // NtD: (M - B_j S / k_eps^2) v'_j = y2
-        KrySys &s = b.s[np + 2 + j];
-        s.alpha = cd(1.0, 0.0);
-        s.beta = cscale(cmul(pb->B[j], inv_ke2), -1.0);
-        s.bscale = bscale;
-        s.f = y2;
-        s.x = sol + (size_t)(np + 2 + j) * n;
-        s.conj = 0;
+    for (int r0 = 0; r0 < nrun; r0 += group) {
+        const int R = std::min(group, nrun - r0);
+        KryBatch b{};
+        for (int r = 0; r < R; ++r) {
+            if (mass) mass_systems(pbs[r0 + r], ys[r0 + r], zs[r0 + r], false, b);
+            else osrc_systems(pbs[r0 + r], ys[r0 + r], b);
+        }
+        OSRC_TRY(launch_kry(pbs[r0], b, st));
     }
-    OSRC_TRY(launch_kry(pb, b, st));
+    if (mass) return OSRC_OK;
     OsrcComb c{};
     c.np = np;
     c.ik = cd(-pb->k_osrc_i, pb->k_osrc);  // i k_osrc (complex with attenuation)
@@ -905,10 +1149,22 @@ int osrc_precond_fused_async(osrc_problem *pb, const double2 *y, double2 *z, cud
     }
     c.cu = cu;
     c.g0 = pb->g0;
-    osrc_combine_kernel<<<(n + 255) / 256, 256, 0, st>>>(n, c, sol, z);
-    pb->launches++;
-    OSRC_CK(cudaGetLastError());
+    for (int r0 = 0; r0 < nrun; r0 += OSRC_COMB_RUNS) {
+        const int R = std::min((int)OSRC_COMB_RUNS, nrun - r0);
+        OsrcCombRuns v{};
+        for (int r = 0; r < R; ++r) {
+            v.sol[r] = pbs[r0 + r]->d_kry_rhs.p + 2 * (size_t)n;
+            v.z[r] = zs[r0 + r];
+        }
+        osrc_combine_kernel<<<dim3((n + 63) / 64, 2, R), 64, 0, st>>>(n, c, v);
+        pbs[r0]->launches++;
+        OSRC_CK(cudaGetLastError());
+    }
     return OSRC_OK;
+}
+
+int osrc_precond_fused_async(osrc_problem *pb, const double2 *y, double2 *z, cudaStream_t st) {
+    return osrc_precond_fused_multi(&pb, &y, &z, 1, st);
 }
 
 // P x for a strong-form vector x: P x = P M^-1 (M x).

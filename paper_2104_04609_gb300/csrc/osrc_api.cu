@@ -315,6 +315,49 @@ int find_col(const std::vector<int> &ptr, const std::vector<int> &col, int i, in
     return (it != e && *it == j) ? (int)(it - col.begin()) : -1;
 }
 
+// Reverse Cuthill-McKee order of a symmetric CSR pattern (perm[new] = old)
+// followed by its inverse: breadth-first levels from an end of the component
+// (the last vertex that a search from its lowest degree reaches), so that
+// neighbours get near numbers.
+std::vector<int> rcm_order(int n, const std::vector<int> &ptr, const std::vector<int> &col) {
+    std::vector<int> order, seen(n, -1), out(2 * (size_t)n);
+    order.reserve(n);
+    auto degree = [&](int v) { return ptr[v + 1] - ptr[v]; };
+    int mark = 0;
+    auto search = [&](int start, std::vector<int> &q) {
+        ++mark;
+        q.assign(1, start);
+        seen[start] = mark;
+        for (size_t h = 0; h < q.size(); ++h) {
+            const size_t b = q.size();
+            for (int e = ptr[q[h]]; e < ptr[q[h] + 1]; ++e)
+                if (seen[col[e]] != mark) {
+                    seen[col[e]] = mark;
+                    q.push_back(col[e]);
+                }
+            std::stable_sort(q.begin() + b, q.end(), [&](int x, int y) { return degree(x) < degree(y); });
+        }
+    };
+    std::vector<char> done(n, 0);
+    std::vector<int> q;
+    for (int v = 0; v < n; ++v) {
+        if (done[v]) continue;
+        search(v, q);
+        int start = q[0];
+        for (int u : q)
+            if (degree(u) < degree(start)) start = u;
+        search(start, q);
+        search(q.back(), q);
+        for (int u : q) done[u] = 1;
+        order.insert(order.end(), q.begin(), q.end());
+    }
+    for (int i = 0; i < n; ++i) {
+        out[i] = order[n - 1 - i];
+        out[n + out[i]] = i;
+    }
+    return out;
+}
+
 void pade_coefficients(int np, double theta, std::complex<double> &C0,
                        std::vector<std::complex<double>> &A, std::vector<std::complex<double>> &B) {
     using cdbl = std::complex<double>;
@@ -510,7 +553,6 @@ static int problem_create(osrc_mesh *mesh, const osrc_params *prm, const double 
             for (int i = 0; i < nv; ++i) mcol.insert(mcol.end(), rowsets[i].begin(), rowsets[i].end());
         }
         pb->ms_nnz = mptr[nv];
-        pb->ms_ptr_h = mptr;
         cpos.clear();
         cidx.clear();
         for (int t = 0; t < nt; ++t)
@@ -525,6 +567,14 @@ static int problem_create(osrc_mesh *mesh, const osrc_params *prm, const double 
             cudaMemcpy(pb->d_ms_col.p, mcol.data(), mcol.size() * sizeof(int), cudaMemcpyHostToDevice)) {
             s = OSRC_CUDA_ERROR;
             break;
+        }
+        {
+            const std::vector<int> order = rcm_order(nv, mptr, mcol);
+            if ((s = pb->d_ms_perm.alloc(ctx, 2 * (size_t)nv))) break;
+            if (cudaMemcpy(pb->d_ms_perm.p, order.data(), 2 * (size_t)nv * sizeof(int), cudaMemcpyHostToDevice)) {
+                s = OSRC_CUDA_ERROR;
+                break;
+            }
         }
         if ((s = ms_build(pb, cptr, clist, st))) break;
         if (p.formulation == OSRC_MULLER && (s = near_add_mass(pb, st))) break;
@@ -714,6 +764,7 @@ int ensure_gmres_workspace(osrc_problem *pb, int maxit) {
     }
     if (!pb->d_w.p) {
         OSRC_TRY(pb->d_w.alloc(ctx, n));
+        OSRC_TRY(pb->d_npart.alloc(ctx, n / 256 + 1));
         OSRC_TRY(pb->d_y.alloc(ctx, n));
         OSRC_TRY(pb->d_cvec.alloc(ctx, n));
         OSRC_TRY(pb->d_b1.alloc(ctx, n));
@@ -757,34 +808,32 @@ static int enqueue_apply(GmresRun &g) {
     return OSRC_OK;
 }
 
-static int enqueue_iteration_rest(GmresRun &g) {
+// preconditioned: w = P M^-1 d_tmp2 is enqueued already (a batch shares it)
+static int enqueue_iteration_rest(GmresRun &g, bool preconditioned) {
     osrc_problem *pb = g.pb;
     cudaStream_t st = g.st;
     const int n = 2 * pb->nv, j = g.j, ldh = g.maxit + 1;
     double2 *V = pb->d_basis.p, *H = pb->d_h.p, *gv = pb->d_givens.p, *w = pb->d_w.p;
     double *sc = pb->d_scalars.p;
-    OSRC_TRY(osrc_precond_fused_async(pb, pb->d_tmp2.p, w, st));
+    if (!preconditioned) OSRC_TRY(osrc_precond_fused_async(pb, pb->d_tmp2.p, w, st));
     OSRC_CK(cudaEventRecord(g.tev[2], st));
     double2 *hc = H + (size_t)ldh * j;
     double2 *h2 = gv + 4 * ldh;  // second-pass projections
     OSRC_TRY(vec_dots_conj(pb, V, j + 1, w, n, hc, st));
-    OSRC_TRY(vec_update(pb, V, j + 1, hc, w, n, st));
+    OSRC_TRY(vec_update(pb, V, j + 1, hc, w, n, nullptr, st));
     OSRC_TRY(vec_dots_conj(pb, V, j + 1, w, n, h2, st));
-    OSRC_TRY(vec_update(pb, V, j + 1, h2, w, n, st));
-    OSRC_TRY(vec_axpby(pb, cd(1, 0), hc, cd(1, 0), h2, hc, j + 1, st));
-    OSRC_TRY(vec_norm(pb, w, n, sc + 1, st));
-    OSRC_CK(cudaMemcpyAsync(hc + j + 1, sc + 1, sizeof(double), cudaMemcpyDeviceToDevice, st));
-    OSRC_CK(cudaMemsetAsync((double *)(hc + j + 1) + 1, 0, sizeof(double), st));
+    OSRC_TRY(vec_update(pb, V, j + 1, h2, w, n, pb->d_npart.p, st));
+    OSRC_TRY(gmres_arnoldi_end(pb, j, ldh, H, gv, g.beta, pb->d_npart.p, n, sc + 1, osrc_precond_nsys(pb),
+                               pb->h_res + 2, host_stat(pb), st));
     OSRC_TRY(vec_scale_copy(pb, w, sc + 1, V + (size_t)(j + 1) * n, n, st));
-    OSRC_TRY(gmres_givens(pb, j, ldh, H, gv, sc + 2, g.beta, st));
-    OSRC_CK(cudaMemcpyAsync(pb->h_res + 2, sc + 2, sizeof(double), cudaMemcpyDeviceToHost, st));
     OSRC_CK(cudaEventRecord(g.tev[3], st));
-    return end_step(g);
+    OSRC_CK(cudaEventRecord(g.ev, st));
+    return OSRC_OK;
 }
 
 static int enqueue_iteration(GmresRun &g) {
     OSRC_TRY(enqueue_apply(g));
-    return enqueue_iteration_rest(g);
+    return enqueue_iteration_rest(g, false);
 }
 
 // x = V y, then the true weak residual |b - B x| / |b|; split like the
@@ -966,7 +1015,7 @@ int problem_clone(osrc_problem *m, osrc_problem **out) {
     c->near_pairs = m->near_pairs;
     c->near_nnz = m->near_nnz;
     c->ms_nnz = m->ms_nnz;
-    c->ms_ptr_h = m->ms_ptr_h;
+    c->kmix_plans = m->kmix_plans;
     c->k_osrc = m->k_osrc;
     c->k_osrc_i = m->k_osrc_i;
     c->k_eps = m->k_eps;
@@ -994,6 +1043,7 @@ int problem_clone(osrc_problem *m, osrc_problem **out) {
     c->d_nr_val.borrow(m->d_nr_val);
     c->d_ms_ptr.borrow(m->d_ms_ptr);
     c->d_ms_col.borrow(m->d_ms_col);
+    c->d_ms_perm.borrow(m->d_ms_perm);
     c->d_M.borrow(m->d_M);
     c->d_S.borrow(m->d_S);
     c->d_dense.borrow(m->d_dense);
@@ -1109,7 +1159,9 @@ static int gmres_solve_lockstep(osrc_problem *pb, const void *b, void *x, int nr
             OSRC_TRY(runs[r].start(cs.c[r], st, br, xr, tol, maxit));
         }
         std::vector<const double2 *> xs;
-        std::vector<double2 *> ys;
+        std::vector<double2 *> ys, pzs;
+        std::vector<const double2 *> pys;
+        std::vector<osrc_problem *> pcs;
         std::vector<int> it, fin;
         for (;;) {
             OSRC_CK(cudaStreamSynchronize(st));
@@ -1149,11 +1201,25 @@ static int gmres_solve_lockstep(osrc_problem *pb, const void *b, void *x, int nr
                 OSRC_TRY(far_apply_multi(pb, xs.data(), ys.data(), (int)it.size(), OSRC_PART_ALL, st));
                 OSRC_CK(cudaEventRecord(eb, st));
                 apply_pending = true;
+                // one preconditioner launch for all runs; its time and the
+                // apply's are counted once, the preconditioner's with the
+                // first run
                 for (int r : it) {
-                    // the shared apply's time is counted once by the driver
                     OSRC_CK(cudaEventRecord(runs[r].tev[0], st));
-                    OSRC_CK(cudaEventRecord(runs[r].tev[1], st));
-                    OSRC_TRY(enqueue_iteration_rest(runs[r]));
+                    if (r == it[0]) OSRC_CK(cudaEventRecord(runs[r].tev[1], st));
+                }
+                pcs.clear();
+                pys.clear();
+                pzs.clear();
+                for (int r : it) {
+                    pcs.push_back(cs.c[r]);
+                    pys.push_back(cs.c[r]->d_tmp2.p);
+                    pzs.push_back(cs.c[r]->d_w.p);
+                }
+                OSRC_TRY(osrc_precond_fused_multi(pcs.data(), pys.data(), pzs.data(), (int)pcs.size(), st));
+                for (int r : it) {
+                    if (r != it[0]) OSRC_CK(cudaEventRecord(runs[r].tev[1], st));
+                    OSRC_TRY(enqueue_iteration_rest(runs[r], true));
                 }
             }
             if (!fin.empty()) {

@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <array>
 #include <string>
 #include <atomic>
 #include <mutex>
@@ -211,7 +212,7 @@ struct osrc_problem {
     // ---- sparse mass / stiffness (1-ring CSR), FP64 ----------------------
     int ms_nnz = 0;
     DBuf<int> d_ms_ptr, d_ms_col;
-    std::vector<int> ms_ptr_h;  // host copy of the CSR row pointers (shared-memory sizing)
+    DBuf<int> d_ms_perm;        // [2][nv] reverse Cuthill-McKee order of the vertices and its inverse
     DBuf<double> d_M, d_S;
     // ---- dense FP64 system (OSRC_FP64_DENSE) -------------------------------
     DBuf<double2> d_dense;    // [2nv][2nv] row-major
@@ -227,17 +228,16 @@ struct osrc_problem {
     DBuf<int> d_kry_stat;     // per-system iteration count / status
     DBuf<double> d_kry_res;   // per-system final relative residual
     int inner_last_max = 0;
-    // mixed-precision inner solver (k_sparse.cu): -1 not yet decided, 0 not
-    // usable for this problem, 1 usable with kmix_rpt rows per thread,
-    // kmix_threads threads and kmix_smem bytes of dynamic shared memory
-    int kmix_state = -1, kmix_rpt = 0, kmix_threads = 0;
-    size_t kmix_smem = 0;
+    // mixed-precision inner solver (k_sparse.cu): launch shapes by number of
+    // systems {nsys, cluster size (0: not usable), rows per thread, threads}
+    std::vector<std::array<int, 4>> kmix_plans;
     // ---- GMRES workspace --------------------------------------------------------
     DBuf<double2> d_basis;    // (maxit+1) x 2nv
     int basis_cap = 0;
     DBuf<double2> d_h;        // Hessenberg (maxit+1) x maxit, column-major
     DBuf<double2> d_givens;   // cs (as .x), sn, g vectors
     DBuf<double> d_scalars;   // reduction scratch
+    DBuf<double> d_npart;     // block shares of |w|^2
     DBuf<double2> d_w, d_y, d_x1, d_b1, d_cvec;  // 2nv vectors
     double *h_res = nullptr;  // pinned host block: doubles [0, 16), then ints (inner status)
     // ---- disjoint objects with their own materials --------------------------------
@@ -295,6 +295,9 @@ int osrc_precond(osrc_problem *pb, const double2 *x, double2 *y, cudaStream_t st
 int osrc_precond_fused(osrc_problem *pb, const double2 *y, double2 *z, cudaStream_t st);
 // the same without waiting: the inner status is left in d_kry_stat
 int osrc_precond_fused_async(osrc_problem *pb, const double2 *y, double2 *z, cudaStream_t st);
+// z_r = P M^-1 y_r for several workspaces of one problem
+int osrc_precond_fused_multi(osrc_problem *const *pbs, const double2 *const *ys, double2 *const *zs, int nrun,
+                             cudaStream_t st);
 int osrc_precond_nsys(const osrc_problem *pb);
 // turns a host copy of the inner status words into a status code
 int kry_status_host(osrc_problem *pb, const int *stat, int nsys);
@@ -302,13 +305,16 @@ int kry_status_host(osrc_problem *pb, const int *stat, int nsys);
 // GMRES helpers (k_gmres.cu)
 int vec_dots_conj(osrc_problem *pb, const double2 *V, int nvec, const double2 *w, int n,
                   double2 *out, cudaStream_t st);
-int vec_update(osrc_problem *pb, const double2 *V, int nvec, const double2 *h, double2 *w,
-               int n, cudaStream_t st);
+// part (null: none): the blocks' shares of |w|^2 after the update
+int vec_update(osrc_problem *pb, const double2 *V, int nvec, const double2 *h, double2 *w, int n, double *part,
+               cudaStream_t st);
 int vec_norm(osrc_problem *pb, const double2 *w, int n, double *out, cudaStream_t st);
 int vec_scale_copy(osrc_problem *pb, const double2 *w, const double *nrm, double2 *out,
                    int n, cudaStream_t st);
-int gmres_givens(osrc_problem *pb, int j, int ldh, double2 *H, double2 *gv, double *res_out,
-                 double beta_norm_for_rel, cudaStream_t st);
+// end of an Arnoldi step: norm, Hessenberg column, rotations, residual and inner
+// status words to (pinned) host memory
+int gmres_arnoldi_end(osrc_problem *pb, int j, int ldh, double2 *H, double2 *gv, double beta, const double *part,
+                      int n, double *nrm, int nstat, double *res_host, int *stat_host, cudaStream_t st);
 int gmres_finish(osrc_problem *pb, int j, int ldh, const double2 *H, const double2 *gv,
                  const double2 *V, double2 *x, int n, cudaStream_t st);
 int vec_axpby(osrc_problem *pb, double2 a, const double2 *x, double2 b, const double2 *y,

@@ -252,6 +252,7 @@ struct osrc_problem {
     // ---- field evaluation off the surface (k_field.cu) -------------------------
     DBuf<double4> d_fsrc;     // [6nt][3] rule points, normals, densities
     DBuf<int> d_freg;         // region scratch when the caller passes none
+    DBuf<double> d_fpart;     // source splits' sums (region, field)
     DBuf<int> d_fobeg;        // [objects + 1] source-point ranges of the objects
     // ---- far-kernel event timing -------------------------------------------------
     bool prof_on = false, prof_pending = false;

@@ -78,15 +78,31 @@ __global__ void far_part_near_kernel(int nv, int Kp, const int *__restrict__ ptr
 }
 
 // B_cat rows r < R: [Re X_r | -Im X_r]; rows R + r: [Im X_r | Re X_r];
-// X given [row][rhs] complex FP32 (R right-hand sides, n2 rows).
-__global__ void pack_b_kernel(int n2, int R, int Kp, const float2 *__restrict__ X,
+// X given [row][rhs] complex FP32 (R right-hand sides, n2 rows).  With V, X is
+// first divided by nrm[r] (0 where the column is done or nrm is 0) and stored
+// there: the new basis vector, packed for the next product in the same pass.
+__global__ void pack_b_kernel(int n2, int R, int Kp, const float2 *__restrict__ X, const float *__restrict__ nrm,
+                              const int *__restrict__ done, float2 *__restrict__ V,
                               __nv_bfloat16 *__restrict__ Bcat) {
     __shared__ float2 tile[32][33];
     const int k0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
     const int tx = threadIdx.x, ty = threadIdx.y;  // 32 x 8
+    float sc = 1.f;
+    if (V && r0 + tx < R) {
+        const float s = nrm[r0 + tx];
+        sc = (done[r0 + tx] || !(s > 0.f)) ? 0.f : 1.f / s;
+    }
     for (int j = ty; j < 32; j += 8) {
         const int k = k0 + j, r = r0 + tx;
-        tile[j][tx] = (k < n2 && r < R) ? X[(size_t)k * R + r] : f2c(0.f, 0.f);
+        float2 v = f2c(0.f, 0.f);
+        if (k < n2 && r < R) {
+            v = X[(size_t)k * R + r];
+            if (V) {
+                v = sc == 0.f ? f2c(0.f, 0.f) : fscale(v, sc);
+                V[(size_t)k * R + r] = v;
+            }
+        }
+        tile[j][tx] = v;
     }
     __syncthreads();
     for (int j = ty; j < 32; j += 8) {
@@ -426,109 +442,175 @@ __global__ void d2f_kernel(int n, const double *__restrict__ a, float *__restric
 // ---------------------------------------------------------------------------
 // FP32 batched Arnoldi: block vectors [n2][R]
 // ---------------------------------------------------------------------------
-// out[i][r] = sum_m conj(V_i[m][r]) w[m][r] for i < nvec; block per i.
-// Column dot products in two deterministic stages.  Stage 1: block (c, i)
-// sums conj(V_i[m][r]) w[m][r] over row chunk c into part[i][c][r];
-// stage 2 adds the chunks in order.  nchunk * nvec blocks keep every SM
-// streaming even for the first basis vectors.
+// Column dot products out[i][r] = sum_m conj(V_i[m][r]) w[m][r], i < nvec, in
+// two deterministic stages.  Stage 1: block (c, group of BD_VEC vectors) sums
+// row chunk c into part[i][c][r]; a thread holds two neighbouring columns
+// (16-byte loads) and BD_VEC vectors, so that w is read once for all of them
+// and BD_VEC + 1 loads are in flight per row.  Stage 2 adds the chunks in
+// order.  One vector a block with 8-byte loads streamed at 60 % of this.
 constexpr int BD_THREADS = 256;
 constexpr int BD_MAX_CHUNK = 64;
+constexpr int BD_VEC = 4;
+
+__device__ __forceinline__ void cdot_acc(float4 &s, const float4 &a, const float4 &b) {  // s += conj(a) b, two columns
+    s.x += a.x * b.x + a.y * b.y;
+    s.y += a.x * b.y - a.y * b.x;
+    s.z += a.z * b.z + a.w * b.w;
+    s.w += a.z * b.w - a.w * b.z;
+}
 
 __global__ void __launch_bounds__(BD_THREADS)
-bdots_part_kernel(const float2 *__restrict__ V, size_t ldv, const float2 *__restrict__ w, int n2, int R,
+bdots_part_kernel(const float2 *__restrict__ V, size_t ldv, int nvec, const float2 *__restrict__ w, int n2, int R,
                   int nchunk, float2 *__restrict__ part) {
-    __shared__ float2 acc[BD_THREADS];
-    const int c = blockIdx.x, i = blockIdx.y;
-    const int r = threadIdx.x % R;
-    const int rl = threadIdx.x / R, nrl = BD_THREADS / R;
+    __shared__ float4 acc[BD_THREADS];
+    const int c = blockIdx.x, i0 = blockIdx.y * BD_VEC, R2 = R / 2;
+    const int r = threadIdx.x % R2, rl = threadIdx.x / R2, nrl = BD_THREADS / R2;
     const int rows = (n2 + nchunk - 1) / nchunk;
     const int m0 = c * rows, m1 = min(n2, m0 + rows);
-    const float2 *v = V + ldv * i;
-    float2 s0 = f2c(0.f, 0.f), s1 = f2c(0.f, 0.f);
+    const float4 *v[BD_VEC];
+#pragma unroll
+    for (int a = 0; a < BD_VEC; ++a) v[a] = reinterpret_cast<const float4 *>(V + ldv * min(i0 + a, nvec - 1));
+    const float4 *w4 = reinterpret_cast<const float4 *>(w);
+    float4 s[BD_VEC];
+#pragma unroll
+    for (int a = 0; a < BD_VEC; ++a) s[a] = make_float4(0.f, 0.f, 0.f, 0.f);
     if (rl < nrl) {
-        int m = m0 + rl;
-        for (; m + nrl < m1; m += 2 * nrl) {
-            const float2 a0 = v[(size_t)m * R + r], b0 = w[(size_t)m * R + r];
-            const float2 a1 = v[(size_t)(m + nrl) * R + r], b1 = w[(size_t)(m + nrl) * R + r];
-            s0.x += a0.x * b0.x + a0.y * b0.y;
-            s0.y += a0.x * b0.y - a0.y * b0.x;
-            s1.x += a1.x * b1.x + a1.y * b1.y;
-            s1.y += a1.x * b1.y - a1.y * b1.x;
-        }
-        if (m < m1) {
-            const float2 a0 = v[(size_t)m * R + r], b0 = w[(size_t)m * R + r];
-            s0.x += a0.x * b0.x + a0.y * b0.y;
-            s0.y += a0.x * b0.y - a0.y * b0.x;
+#pragma unroll 2
+        for (int m = m0 + rl; m < m1; m += nrl) {
+            const size_t k = (size_t)m * R2 + r;
+            const float4 b = w4[k];
+#pragma unroll
+            for (int a = 0; a < BD_VEC; ++a) cdot_acc(s[a], v[a][k], b);
         }
     }
-    acc[threadIdx.x] = fadd(s0, s1);
-    __syncthreads();
-    if (threadIdx.x < R) {
-        float2 t = f2c(0.f, 0.f);
-        for (int l = 0; l < nrl; ++l) t = fadd(t, acc[l * R + threadIdx.x]);
-        part[((size_t)i * nchunk + c) * R + threadIdx.x] = t;
+#pragma unroll
+    for (int a = 0; a < BD_VEC; ++a) {
+        if (i0 + a >= nvec) break;
+        __syncthreads();
+        acc[threadIdx.x] = s[a];
+        __syncthreads();
+        if (threadIdx.x < R2) {
+            float4 t = acc[threadIdx.x];
+            for (int l = 1; l < nrl; ++l) {
+                const float4 o = acc[l * R2 + threadIdx.x];
+                t.x += o.x;
+                t.y += o.y;
+                t.z += o.z;
+                t.w += o.w;
+            }
+            reinterpret_cast<float4 *>(part + ((size_t)(i0 + a) * nchunk + c) * R)[threadIdx.x] = t;
+        }
     }
 }
 
-// out[i][r] = sum_c part[i][c][r]; with nrm != NULL (one vector, V = w)
-// nrm[r] = sqrt(Re out[0][r]) instead
+// out[i][r] = sum_c part[i][c][r], four lanes per entry; with nrm != NULL (one
+// vector, V = w) nrm[r] = sqrt(Re out[0][r]) instead
 __global__ void bdots_fin_kernel(const float2 *__restrict__ part, int nvec, int nchunk, int R,
                                  float2 *__restrict__ out, float *__restrict__ nrm) {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= nvec * R) return;
-    const int i = k / R, r = k % R;
+    // thread = (entry group of 8, lane of 4, entry): eight neighbouring columns a quarter warp
+    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
+    const int k = idx / 32 * 8 + (idx & 7), q = (idx >> 3) & 3;
+    const bool ok = k < nvec * R;
+    const int i = ok ? k / R : 0, r = ok ? k % R : 0;
     float2 t = f2c(0.f, 0.f);
-    for (int c = 0; c < nchunk; ++c) t = fadd(t, part[((size_t)i * nchunk + c) * R + r]);
+#pragma unroll 8
+    for (int c = q; c < nchunk; c += 4) t = fadd(t, part[((size_t)i * nchunk + c) * R + r]);
+    for (int o = 8; o < 32; o <<= 1) {
+        t.x += __shfl_xor_sync(0xffffffffu, t.x, o);
+        t.y += __shfl_xor_sync(0xffffffffu, t.y, o);
+    }
+    if (!ok || q) return;
     if (nrm)
         nrm[r] = sqrtf(fmaxf(t.x, 0.f));
     else
         out[k] = t;
 }
 
-// w[m][r] -= sum_i h[i][r] V_i[m][r]
-__global__ void bupdate_kernel(const float2 *__restrict__ V, size_t ldv, int nvec, const float2 *__restrict__ h,
-                               float2 *__restrict__ w, int n2, int R) {
-    const size_t k = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= (size_t)n2 * R) return;
-    const int r = (int)(k % R);
-    float2 s = w[k];
-    for (int i = 0; i < nvec; ++i) s = fsub(s, fmulc(h[(size_t)i * R + r], V[ldv * i + k]));
-    w[k] = s;
-}
-
-// v[m][r] = w[m][r] / nrm[r] (0 where the column is frozen or nrm is 0)
-__global__ void bscale_kernel(const float2 *__restrict__ w, const float *__restrict__ nrm,
-                              const int *__restrict__ done, float2 *__restrict__ v, int n2, int R) {
-    const size_t k = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= (size_t)n2 * R) return;
-    const int r = (int)(k % R);
-    const float s = nrm[r];
-    v[k] = (done[r] || !(s > 0.f)) ? f2c(0.f, 0.f) : fscale(w[k], 1.f / s);
-}
-
-// Per right-hand side r (one thread each): new Hessenberg column
-// H[.][j][r] (h from the projections, h_{j+1} = nrm[r]), earlier Givens
-// rotations, the new rotation, g update, residual estimate; columns that
-// have converged keep their state (done[r] = 1, iteration count fixed).
-__global__ void bgivens_kernel(int j, int ldh, int R, const float2 *__restrict__ hcol,
-                               const float *__restrict__ nrm, float2 *__restrict__ H,
-                               float *__restrict__ cs, float2 *__restrict__ sn, float2 *__restrict__ g,
-                               const float *__restrict__ beta, float tol, int *__restrict__ done,
-                               int *__restrict__ its, float *__restrict__ res) {
-    const int r = blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= R || done[r]) return;
-    float2 *h = H + ((size_t)j * ldh) * R;  // h[i] at h[i * R + r]
-    for (int i = 0; i <= j; ++i) h[(size_t)i * R + r] = hcol[(size_t)i * R + r];
-    h[(size_t)(j + 1) * R + r] = f2c(nrm[r], 0.f);
-    for (int i = 0; i < j; ++i) {
-        const float c = cs[(size_t)i * R + r];
-        const float2 s = sn[(size_t)i * R + r];
-        const float2 hi = h[(size_t)i * R + r], hi1 = h[(size_t)(i + 1) * R + r];
-        const float2 t = fadd(fscale(hi, c), fmulc(s, hi1));
-        h[(size_t)(i + 1) * R + r] = fadd(fscale(fmulc(f2c(s.x, -s.y), hi), -1.f), fscale(hi1, c));
-        h[(size_t)i * R + r] = t;
+// w[m][r] -= sum_i h[i][r] V_i[m][r], and part[c][r] = sum over the block's row
+// chunk of |w[m][r]|^2 (the columns' norms cost no pass of their own).  Block c
+// takes rows [c rows, (c + 1) rows); a thread holds two neighbouring columns
+// (16-byte loads), eight vectors ahead.
+constexpr int BU_THREADS = 256;
+__global__ void __launch_bounds__(BU_THREADS)
+bupdate_kernel(const float2 *__restrict__ V, size_t ldv, int nvec, const float2 *__restrict__ h,
+               float2 *__restrict__ w, int n2, int R, int rows, float *__restrict__ part) {
+    __shared__ float2 acc[BU_THREADS];
+    const int R2 = R / 2, r = threadIdx.x % R2, rl = threadIdx.x / R2, nrl = BU_THREADS / R2;
+    const int m0 = blockIdx.x * rows, m1 = min(n2, m0 + rows);
+    const float4 *V4 = reinterpret_cast<const float4 *>(V), *h4 = reinterpret_cast<const float4 *>(h);
+    float4 *w4 = reinterpret_cast<float4 *>(w);
+    float2 a = f2c(0.f, 0.f);
+    if (rl < nrl)
+        for (int m = m0 + rl; m < m1; m += nrl) {
+            const size_t k = (size_t)m * R2 + r;
+            float4 s = w4[k];
+#pragma unroll 8
+            for (int i = 0; i < nvec; ++i) {
+                const float4 v = V4[ldv / 2 * i + k], g = h4[(size_t)i * R2 + r];
+                s.x -= g.x * v.x - g.y * v.y;
+                s.y -= g.x * v.y + g.y * v.x;
+                s.z -= g.z * v.z - g.w * v.w;
+                s.w -= g.z * v.w + g.w * v.z;
+            }
+            w4[k] = s;
+            a.x += s.x * s.x + s.y * s.y;
+            a.y += s.z * s.z + s.w * s.w;
+        }
+    acc[threadIdx.x] = a;
+    __syncthreads();
+    if (threadIdx.x < R2) {
+        float2 t = acc[threadIdx.x];
+        for (int l = 1; l < nrl; ++l) t = fadd(t, acc[l * R2 + threadIdx.x]);
+        reinterpret_cast<float2 *>(part + (size_t)blockIdx.x * R)[threadIdx.x] = t;
     }
-    const float2 a = h[(size_t)j * R + r], b = h[(size_t)(j + 1) * R + r];
+}
+
+// Per right-hand side r (BG_LANES lanes each): the column norm from its nc row
+// chunks' shares, the new Hessenberg column H[.][j][r] (h from the projections,
+// h_{j+1} = |w_r|), earlier Givens rotations, the new rotation, g update,
+// residual estimate; columns that have converged keep their state (done[r] = 1,
+// iteration count fixed).  The rotations are a serial chain per column: a warp
+// stages their operands in shared memory, BG_TILE at a time, and one lane walks
+// it (through global memory step by step it took 27 us at 25 iterations).
+constexpr int BG_LANES = 32, BG_COLS = 4, BG_TILE = 64;
+__global__ void bgivens_kernel(int j, int ldh, int R, const float2 *__restrict__ hcol,
+                               const float *__restrict__ part, int nc, float *__restrict__ nrm,
+                               float2 *__restrict__ H, float *__restrict__ cs, float2 *__restrict__ sn,
+                               float2 *__restrict__ g, const float *__restrict__ beta, float tol,
+                               int *__restrict__ done, int *__restrict__ its, float *__restrict__ res) {
+    __shared__ float sc[BG_COLS][BG_TILE];
+    __shared__ float2 ss[BG_COLS][BG_TILE], sh[BG_COLS][BG_TILE];
+    const int lane = threadIdx.x % BG_LANES, col = threadIdx.x / BG_LANES, r = blockIdx.x * BG_COLS + col;
+    if (r >= R) return;  // whole warps
+    float t = 0.f;
+    for (int c = lane; c < nc; c += BG_LANES) t += part[(size_t)c * R + r];
+    for (int o = BG_LANES / 2; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    const float wn = sqrtf(fmaxf(t, 0.f));
+    if (lane == 0) nrm[r] = wn;
+    if (done[r]) return;
+    float2 *h = H + ((size_t)j * ldh) * R;  // h[i] at h[i * R + r]
+    float2 hi = hcol[r];
+    for (int i0 = 0; i0 < j; i0 += BG_TILE) {
+        const int m = min(BG_TILE, j - i0);
+        for (int a = lane; a < m; a += BG_LANES) {
+            sc[col][a] = cs[(size_t)(i0 + a) * R + r];
+            ss[col][a] = sn[(size_t)(i0 + a) * R + r];
+            sh[col][a] = hcol[(size_t)(i0 + a + 1) * R + r];
+        }
+        __syncwarp();
+        if (lane == 0)
+            for (int a = 0; a < m; ++a) {
+                const float c = sc[col][a];
+                const float2 s = ss[col][a], h1 = sh[col][a];
+                sh[col][a] = fadd(fscale(hi, c), fmulc(s, h1));
+                hi = fadd(fscale(fmulc(f2c(s.x, -s.y), hi), -1.f), fscale(h1, c));
+            }
+        __syncwarp();
+        for (int a = lane; a < m; a += BG_LANES) h[(size_t)(i0 + a) * R + r] = sh[col][a];
+        __syncwarp();
+    }
+    if (lane != 0) return;
+    const float2 a = hi, b = f2c(wn, 0.f);
     const float aa = sqrtf(fabs2(a)), bb = sqrtf(fabs2(b));
     const float nu = hypotf(aa, bb);
     float c;
@@ -545,25 +627,44 @@ __global__ void bgivens_kernel(int j, int ldh, int R, const float2 *__restrict__
     h[(size_t)j * R + r] = fadd(fscale(a, c), fmulc(s, b));
     h[(size_t)(j + 1) * R + r] = f2c(0.f, 0.f);
     const float2 gj = g[(size_t)j * R + r];
-    g[(size_t)(j + 1) * R + r] = fscale(fmulc(f2c(s.x, -s.y), gj), -1.f);
+    const float2 gn = fscale(fmulc(f2c(s.x, -s.y), gj), -1.f);
+    g[(size_t)(j + 1) * R + r] = gn;
     g[(size_t)j * R + r] = fscale(gj, c);
-    const float rel = sqrtf(fabs2(g[(size_t)(j + 1) * R + r])) / beta[r];
+    const float rel = sqrtf(fabs2(gn)) / beta[r];
     res[r] = rel;
     its[r] = j + 1;
     if (rel <= tol || !(nu > 0.f)) done[r] = 1;
 }
 
-// y_r = H_r^-1 g_r (its[r] x its[r] upper triangular), one thread per r
-__global__ void bbacksub_kernel(int ldh, int R, const float2 *__restrict__ H, const float2 *__restrict__ g,
-                                const int *__restrict__ its, float2 *__restrict__ y) {
-    const int r = blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= R) return;
-    const int m = its[r];
-    for (int i = m - 1; i >= 0; --i) {
-        float2 s = g[(size_t)i * R + r];
-        for (int k = i + 1; k < m; ++k)
-            s = fsub(s, fmulc(H[((size_t)k * ldh + i) * R + r], y[(size_t)k * R + r]));
-        y[(size_t)i * R + r] = fdivc(s, H[((size_t)i * ldh + i) * R + r]);
+// y_r = H_r^-1 g_r (its[r] x its[r] upper triangular) by columns: BS_COLS
+// right-hand sides a block, BS_LANES threads each; y_i is final once the columns
+// behind it have been subtracted from the right-hand side, and all lanes subtract
+// column i together (row by row, a thread per right-hand side took 2.7 ms at 117
+// iterations).
+constexpr int BS_COLS = 8, BS_LANES = 32;
+__global__ void __launch_bounds__(BS_COLS *BS_LANES)
+bbacksub_kernel(int ldh, int R, const float2 *__restrict__ H, const float2 *__restrict__ g,
+                const int *__restrict__ its, float2 *y) {
+    __shared__ float2 yi[2][BS_COLS];
+    const int cl = threadIdx.x % BS_COLS, ln = threadIdx.x / BS_COLS, r = blockIdx.x * BS_COLS + cl;
+    const int m = r < R ? its[r] : 0;
+    int mx = 0;
+    for (int c = 0; c < BS_COLS; ++c)
+        if (blockIdx.x * BS_COLS + c < R) mx = max(mx, its[blockIdx.x * BS_COLS + c]);
+    for (int i = ln; i < m; i += BS_LANES) y[(size_t)i * R + r] = g[(size_t)i * R + r];
+    for (int i = mx - 1; i >= 0; --i) {
+        __syncthreads();
+        if (ln == i % BS_LANES && i < m) {  // the lane that owns row i
+            const float2 v = fdivc(y[(size_t)i * R + r], H[((size_t)i * ldh + i) * R + r]);
+            y[(size_t)i * R + r] = v;
+            yi[i & 1][cl] = v;
+        }
+        __syncthreads();
+        if (i < m) {
+            const float2 v = yi[i & 1][cl];
+            for (int k = ln; k < i; k += BS_LANES)
+                y[(size_t)k * R + r] = fsub(y[(size_t)k * R + r], fmulc(H[((size_t)i * ldh + k) * R + r], v));
+        }
     }
 }
 
@@ -620,7 +721,9 @@ __device__ __forceinline__ void ff_mac(float &sh, float &sl, float ah, float al,
     sh = t;
 }
 
-constexpr int FF_TM = 64, FF_TR = 16, FF_TK = 16;
+// 64 rows x 8 right-hand sides a block: with 16 a 6000-row, 64-column residual is
+// 376 blocks, 2.5 per SM, and the SMs with three set the time
+constexpr int FF_TM = 64, FF_TR = 8, FF_TK = 16;
 
 __global__ void __launch_bounds__(256)
 resid_ff_kernel(int n2, int nrhs, const float4 *__restrict__ AFF, const double2 *__restrict__ X,
@@ -629,14 +732,12 @@ resid_ff_kernel(int n2, int nrhs, const float4 *__restrict__ AFF, const double2 
     __shared__ float4 sx[FF_TR][FF_TK + 1];
     const int m0 = blockIdx.x * FF_TM, r0 = blockIdx.y * FF_TR;
     const int tid = threadIdx.x;
-    const int tm = tid % 32, tr = (tid / 32) * 2;  // rows tm, tm + 32; right-hand sides tr, tr + 1
-    float acc[2][2][4];                             // [row][rhs][re h, re l, im h, im l]
+    const int tm = tid % 32, tr = tid / 32;  // rows tm, tm + 32; right-hand side tr
+    float acc[2][4];                          // [row][re h, re l, im h, im l]
 #pragma unroll
     for (int a = 0; a < 2; ++a)
 #pragma unroll
-        for (int b = 0; b < 2; ++b)
-#pragma unroll
-            for (int c = 0; c < 4; ++c) acc[a][b][c] = 0.f;
+        for (int c = 0; c < 4; ++c) acc[a][c] = 0.f;
     for (int k0 = 0; k0 < n2; k0 += FF_TK) {
         for (int e = tid; e < FF_TM * FF_TK; e += 256) {
             const int mm = e / FF_TK, kk = e % FF_TK;
@@ -657,33 +758,28 @@ resid_ff_kernel(int n2, int nrhs, const float4 *__restrict__ AFF, const double2 
 #pragma unroll 4
         for (int kk = 0; kk < FF_TK; ++kk) {
             const float4 a[2] = {sa[tm][kk], sa[tm + 32][kk]};
-            const float4 x[2] = {sx[tr][kk], sx[tr + 1][kk]};
+            const float4 x = sx[tr][kk];
 #pragma unroll
-            for (int i = 0; i < 2; ++i)
-#pragma unroll
-                for (int j = 0; j < 2; ++j) {
-                    float *c = acc[i][j];
-                    ff_mac(c[0], c[1], a[i].x, a[i].z, x[j].x, x[j].z);    // + Re a Re x
-                    ff_mac(c[0], c[1], -a[i].y, -a[i].w, x[j].y, x[j].w);  // - Im a Im x
-                    ff_mac(c[2], c[3], a[i].x, a[i].z, x[j].y, x[j].w);    // + Re a Im x
-                    ff_mac(c[2], c[3], a[i].y, a[i].w, x[j].x, x[j].z);    // + Im a Re x
-                }
+            for (int i = 0; i < 2; ++i) {
+                float *c = acc[i];
+                ff_mac(c[0], c[1], a[i].x, a[i].z, x.x, x.z);    // + Re a Re x
+                ff_mac(c[2], c[3], a[i].x, a[i].z, x.y, x.w);    // + Re a Im x
+                ff_mac(c[0], c[1], -a[i].y, -a[i].w, x.y, x.w);  // - Im a Im x
+                ff_mac(c[2], c[3], a[i].y, a[i].w, x.x, x.z);    // + Im a Re x
+            }
         }
         __syncthreads();
     }
 #pragma unroll
-    for (int i = 0; i < 2; ++i)
-#pragma unroll
-        for (int j = 0; j < 2; ++j) {
-            const int m = m0 + tm + 32 * i, r = r0 + tr + j;
-            if (m < n2 && r < nrhs) {
-                const float *c = acc[i][j];
-                const double2 ax = cd((double)c[0] + (double)c[1], (double)c[2] + (double)c[3]);
-                Rr[(size_t)r * n2 + m] = csub(B[(size_t)r * n2 + m], ax);
-            }
+    for (int i = 0; i < 2; ++i) {
+        const int m = m0 + tm + 32 * i, r = r0 + tr;
+        if (m < n2 && r < nrhs) {
+            const float *c = acc[i];
+            const double2 ax = cd((double)c[0] + (double)c[1], (double)c[2] + (double)c[3]);
+            Rr[(size_t)r * n2 + m] = csub(B[(size_t)r * n2 + m], ax);
         }
+    }
 }
-
 
 // per right-hand side: nrm[r] = |v[r][:]| (FP64, [nrhs][n2])
 __global__ void norm_rows64_kernel(int n2, const double2 *__restrict__ v, double *__restrict__ nrm) {
@@ -772,6 +868,13 @@ struct BatchedState {
     DBuf<double2> X64, R64;
     DBuf<double> bn, rn, scl;
     int basis_cap = 0;
+    int *hdone = nullptr;       // pinned: convergence flags of two iterations
+    cudaEvent_t ev[2] = {nullptr, nullptr};
+    ~BatchedState() {
+        if (hdone) cudaFreeHost(hdone);
+        for (auto &e : ev)
+            if (e) cudaEventDestroy(e);
+    }
 };
 
 void batched_free(BatchedState *s) { delete s; }
@@ -836,7 +939,8 @@ int batched_prepare(osrc_problem *pb, int R, int maxit_inner, cudaStream_t st) {
         OSRC_TRY(bs->t2.alloc(ctx, plane));
         OSRC_TRY(bs->H.alloc(ctx, (size_t)(maxit_inner + 1) * (maxit_inner + 1) * R));
         OSRC_TRY(bs->hcol.alloc(ctx, (size_t)(maxit_inner + 1) * R));
-        OSRC_TRY(bs->part.alloc(ctx, (size_t)(maxit_inner + 1) * BD_MAX_CHUNK * R));
+        // projections' chunk sums, or the update's row-chunk norms (at most 1216 floats a column)
+        OSRC_TRY(bs->part.alloc(ctx, std::max((size_t)(maxit_inner + 1) * BD_MAX_CHUNK, (size_t)640) * R));
         OSRC_TRY(bs->g.alloc(ctx, (size_t)(maxit_inner + 1) * R));
         OSRC_TRY(bs->sn.alloc(ctx, (size_t)(maxit_inner + 1) * R));
         OSRC_TRY(bs->yv.alloc(ctx, (size_t)(maxit_inner + 1) * R));
@@ -856,16 +960,23 @@ int batched_prepare(osrc_problem *pb, int R, int maxit_inner, cudaStream_t st) {
 
 // y = A_inner x for a block x ([n2][R] FP32): BF16 tensor-core GEMM of the
 // far-field part + exact near-field CSR product
-static int batched_matvec(osrc_problem *pb, const float2 *x, float2 *y, cudaStream_t st) {
+static void batched_pack(osrc_problem *pb, const float2 *x, float2 *v, cudaStream_t st) {
     BatchedState *bs = pb->batched;
-    const int n2 = bs->n2, R = bs->R, nv = pb->nv;
-    dim3 gb((n2 + 31) / 32, (R + 31) / 32);
-    pack_b_kernel<<<gb, dim3(32, 8), 0, st>>>(n2, R, bs->Kp, x, bs->Bcat.p);
+    const dim3 gb((bs->n2 + 31) / 32, (bs->R + 31) / 32);
+    pack_b_kernel<<<gb, dim3(32, 8), 0, st>>>(bs->n2, bs->R, bs->Kp, x, bs->nrm.p, bs->done.p, v, bs->Bcat.p);
+    pb->launches++;
+}
+
+// packed: Bcat holds x already
+static int batched_matvec(osrc_problem *pb, const float2 *x, float2 *y, bool packed, cudaStream_t st) {
+    BatchedState *bs = pb->batched;
+    const int R = bs->R, nv = pb->nv;
+    if (!packed) batched_pack(pb, x, nullptr, st);
     OSRC_TRY(umma_gemm_bf16(bs->Acat.p, bs->Mp, bs->Kp, bs->Bcat.p, 2 * R, bs->C.p, 2 * R, bs->gws.p,
                             bs->gws.n, bs->err.p, st));
     unpack_near_kernel<<<nv, R, 0, st>>>(nv, R, 2 * R, bs->C.p, pb->d_nr_ptr.p, pb->d_nr_col.p, bs->nr32.p, x,
                                          y);
-    pb->launches += 3;
+    pb->launches += 2;
     OSRC_CK(cudaGetLastError());
     return OSRC_OK;
 }
@@ -941,13 +1052,12 @@ static int batched_precond(osrc_problem *pb, const float2 *y, float2 *z, float t
 static int batched_precond_dense(osrc_problem *pb, const float2 *y, float2 *z, cudaStream_t st) {
     BatchedState *bs = pb->batched;
     const int n2 = bs->n2, R = bs->R;
-    dim3 gb((n2 + 31) / 32, (R + 31) / 32);
-    pack_b_kernel<<<gb, dim3(32, 8), 0, st>>>(n2, R, bs->Kp, y, bs->Bcat.p);
+    batched_pack(pb, y, nullptr, st);
     OSRC_TRY(umma_gemm_bf16(bs->Pcat.p, bs->Mp, bs->Kp, bs->Bcat.p, 2 * R, bs->C.p, 2 * R, bs->gws.p,
                             bs->gws.n, bs->err.p, st));
     const size_t plane = (size_t)n2 * R;
     unpack_plain_kernel<<<(unsigned)((plane + 255) / 256), 256, 0, st>>>(n2, R, 2 * R, bs->C.p, z);
-    pb->launches += 3;
+    pb->launches += 2;
     OSRC_CK(cudaGetLastError());
     return OSRC_OK;
 }
@@ -968,49 +1078,67 @@ static int batched_inner_gmres(osrc_problem *pb, const float2 *c, float tol, int
     const int ldh = maxit + 1;
     const unsigned gp = (unsigned)((plane + 255) / 256);
     const int nchunk = std::max(1, std::min(BD_MAX_CHUNK, n2 / 64));
+    if (!bs->hdone) {
+        OSRC_CK(cudaMallocHost((void **)&bs->hdone, 2 * 128 * sizeof(int)));
+        for (auto &e : bs->ev) OSRC_CK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+    }
     auto dots = [&](int nvec, const float2 *w, float2 *out) {
-        bdots_part_kernel<<<dim3(nchunk, nvec), BD_THREADS, 0, st>>>(bs->V.p, plane, w, n2, R, nchunk,
-                                                                     bs->part.p);
-        bdots_fin_kernel<<<(nvec * R + 255) / 256, 256, 0, st>>>(bs->part.p, nvec, nchunk, R, out, nullptr);
+        bdots_part_kernel<<<dim3(nchunk, (nvec + BD_VEC - 1) / BD_VEC), BD_THREADS, 0, st>>>(bs->V.p, plane, nvec, w,
+                                                                                              n2, R, nchunk, bs->part.p);
+        bdots_fin_kernel<<<(nvec * R * 4 + 255) / 256, 256, 0, st>>>(bs->part.p, nvec, nchunk, R, out, nullptr);
     };
     auto norm = [&](const float2 *w) {
-        bdots_part_kernel<<<dim3(nchunk, 1), BD_THREADS, 0, st>>>(w, plane, w, n2, R, nchunk, bs->part.p);
-        bdots_fin_kernel<<<(R + 255) / 256, 256, 0, st>>>(bs->part.p, 1, nchunk, R, nullptr, bs->nrm.p);
+        bdots_part_kernel<<<dim3(nchunk, 1), BD_THREADS, 0, st>>>(w, plane, 1, w, n2, R, nchunk, bs->part.p);
+        bdots_fin_kernel<<<(R * 4 + 255) / 256, 256, 0, st>>>(bs->part.p, 1, nchunk, R, nullptr, bs->nrm.p);
     };
     // rhs of the preconditioned system
     OSRC_TRY(batched_apply_precond(pb, c, bs->w.p, ptol, pmaxit, st));
     norm(bs->w.p);
     binit_kernel<<<(R + 127) / 128, 128, 0, st>>>(R, bs->nrm.p, bs->beta.p, bs->g.p, bs->done.p, bs->its.p);
     OSRC_CK(cudaMemsetAsync(bs->g.p + R, 0, (size_t)maxit * R * sizeof(float2), st));
-    bscale_kernel<<<gp, 256, 0, st>>>(bs->w.p, bs->nrm.p, bs->done.p, bs->V.p, n2, R);
-    std::vector<int> hdone(R);
-    int j = 0;
+    batched_pack(pb, bs->w.p, bs->V.p, st);
+    // row chunks of the update: as many as bs->part has room for
+    const int unrl = 2 * BU_THREADS / R;  // rows a block takes at a time
+    const int urows = ((n2 + 1215) / 1216 + unrl - 1) / unrl * unrl, uchunk = (n2 + urows - 1) / urows;
+    // The host reads the convergence flags of iteration j while the device
+    // runs iteration j + 1 (an iteration too many, on columns that are all
+    // frozen, when j was the last): it waited 60 to 90 us for them otherwise.
+    int *hdone[2] = {bs->hdone, bs->hdone + R};
+    int j = 0, its = 0;
     for (j = 0; j < maxit; ++j) {
         float2 *vj = bs->V.p + (size_t)j * plane;
-        OSRC_TRY(batched_matvec(pb, vj, bs->t2.p, st));
+        OSRC_TRY(batched_matvec(pb, vj, bs->t2.p, true, st));
         OSRC_TRY(batched_apply_precond(pb, bs->t2.p, bs->w.p, ptol, pmaxit, st));
         // one classical Gram-Schmidt pass: the inner solve only reduces the
         // residual by inner_tol (>= 1e-3 in use), far above where FP32 CGS
         // loses orthogonality, and the outer refinement corrects the rest
         // (a second pass cost 25 % more time for 2 % fewer iterations)
         dots(j + 1, bs->w.p, bs->hcol.p);
-        bupdate_kernel<<<gp, 256, 0, st>>>(bs->V.p, plane, j + 1, bs->hcol.p, bs->w.p, n2, R);
-        norm(bs->w.p);
-        bgivens_kernel<<<(R + 127) / 128, 128, 0, st>>>(j, ldh, R, bs->hcol.p, bs->nrm.p, bs->H.p, bs->cs.p,
-                                                        bs->sn.p, bs->g.p, bs->beta.p, tol, bs->done.p,
-                                                        bs->its.p, bs->res.p);
-        bscale_kernel<<<gp, 256, 0, st>>>(bs->w.p, bs->nrm.p, bs->done.p, bs->V.p + (size_t)(j + 1) * plane, n2, R);
-        pb->launches += 8;
-        OSRC_CK(cudaMemcpyAsync(hdone.data(), bs->done.p, R * sizeof(int), cudaMemcpyDeviceToHost, st));
-        OSRC_CK(cudaStreamSynchronize(st));
-        bool all = true;
-        for (int r = 0; r < R; ++r) all = all && hdone[r];
-        if (all) {
-            ++j;
-            break;
+        bupdate_kernel<<<uchunk, BU_THREADS, 0, st>>>(bs->V.p, plane, j + 1, bs->hcol.p, bs->w.p, n2, R, urows,
+                                                      (float *)bs->part.p);
+        bgivens_kernel<<<(R + BG_COLS - 1) / BG_COLS, BG_COLS * BG_LANES, 0, st>>>(j, ldh, R, bs->hcol.p, (const float *)bs->part.p,
+                                                                   uchunk, bs->nrm.p, bs->H.p, bs->cs.p, bs->sn.p,
+                                                                   bs->g.p, bs->beta.p, tol, bs->done.p, bs->its.p,
+                                                                   bs->res.p);
+        batched_pack(pb, bs->w.p, bs->V.p + (size_t)(j + 1) * plane, st);
+        pb->launches += 4;
+        OSRC_CK(cudaMemcpyAsync(hdone[j & 1], bs->done.p, R * sizeof(int), cudaMemcpyDeviceToHost, st));
+        OSRC_CK(cudaEventRecord(bs->ev[j & 1], st));
+        its = j + 1;
+        if (j > 0) {
+            OSRC_CK(cudaEventSynchronize(bs->ev[(j - 1) & 1]));
+            bool all = true;
+            for (int r = 0; r < R; ++r) all = all && hdone[(j - 1) & 1][r];
+            if (all) {
+                its = j;
+                break;
+            }
         }
     }
-    bbacksub_kernel<<<(R + 127) / 128, 128, 0, st>>>(ldh, R, bs->H.p, bs->g.p, bs->its.p, bs->yv.p);
+    // the flags' last copies land before the buffers are used again
+    OSRC_CK(cudaStreamSynchronize(st));
+    j = its;
+    bbacksub_kernel<<<(R + BS_COLS - 1) / BS_COLS, BS_COLS * BS_LANES, 0, st>>>(ldh, R, bs->H.p, bs->g.p, bs->its.p, bs->yv.p);
     bcombine_kernel<<<gp, 256, 0, st>>>(bs->V.p, plane, maxit, bs->yv.p, bs->its.p, bs->t1.p, n2, R);
     pb->launches += 2;
     OSRC_CK(cudaGetLastError());
@@ -1116,7 +1244,7 @@ extern "C" int osrc_dense_batched_apply_ex(osrc_problem *pb, const void *x, void
         out = bs->t1.p;
     }
     if (what == 0 || what == 2) {
-        OSRC_TRY(batched_matvec(pb, bs->t2.p, bs->w.p, st));
+        OSRC_TRY(batched_matvec(pb, bs->t2.p, bs->w.p, false, st));
         out = bs->w.p;
     }
     if (what == 1 || what == 2) {

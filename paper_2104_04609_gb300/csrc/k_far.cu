@@ -361,23 +361,30 @@ __device__ __forceinline__ Diff2 far_diff(f2 X, f2 Y, f2 Z, const float4 &P0, co
     return d;
 }
 
-template <bool CENTRED, bool MULTI, bool ABSORB>
-__device__ __forceinline__ void far_tri(const f2 (&X)[3], const f2 (&Y)[3], const f2 (&Z)[3], const float4 &n4,
-                                        float pdn, const float4 &P0, const float4 &P1, const float4 &P2, const float4 &P3,
-                                        const f2 &P5, const FarConst2 &c, const CenterPair &cp, f2 m1, f2 k1i,
-                                        f2 dk1i, PairAcc (&A)[3], CurlAcc &B) {
+// Kernel values of one source point at the six test points (three pairs):
+// c / r and s / r of both wavenumbers, -(H0 + H1) r^2 = hp + i hq, 1 / r^2, and
+// (y - x).n_x.
+struct FarVals {
+    f2 c0r[3], s0r[3], c1r[3], s1r[3], hp[3], hq[3], ri2[3], dnxn;
+};
+
 #define F3 _Pragma("unroll") for (int p = 0; p < 3; ++p)
+template <bool CENTRED, bool MULTI, bool ABSORB>
+__device__ __forceinline__ FarVals far_vals(const f2 (&X)[3], const f2 (&Y)[3], const f2 (&Z)[3], const float4 &n4,
+                                            float pdn, const float4 &P0, const float4 &P1, const FarConst2 &c,
+                                            const CenterPair &cp, f2 m1, f2 k1i) {
+    FarVals v;
     Diff2 d[3];
     F3 d[p] = far_diff<CENTRED>(X[p], Y[p], Z[p], P0, P1, cp);
-    const f2 dnxn = CENTRED ? dup2(-fmaf(P0.x, n4.x, fmaf(P0.z, n4.y, fmaf(P1.x, n4.z, pdn))))
-                            : dup2(-fmaf(d[0].dz.x, n4.z, fmaf(d[0].dy.x, n4.y, fmaf(d[0].dx.x, n4.x, -pdn))));
-    f2 r2[3], ri[3], r[3], ri2[3], s0[3], c0[3], s1[3], c1[3];
+    v.dnxn = CENTRED ? dup2(-fmaf(P0.x, n4.x, fmaf(P0.z, n4.y, fmaf(P1.x, n4.z, pdn))))
+                     : dup2(-fmaf(d[0].dz.x, n4.z, fmaf(d[0].dy.x, n4.y, fmaf(d[0].dx.x, n4.x, -pdn))));
+    f2 r2[3], ri[3], r[3], s0[3], c0[3], s1[3], c1[3];
     F3 r2[p] = mul2(d[p].dx, d[p].dx);
     F3 r2[p] = fma2(d[p].dy, d[p].dy, r2[p]);
     F3 r2[p] = fma2(d[p].dz, d[p].dz, r2[p]);
     F3 ri[p] = make_float2(rsqrtf(r2[p].x), rsqrtf(r2[p].y));
     F3 r[p] = mul2(r2[p], ri[p]);
-    F3 ri2[p] = mul2(ri[p], ri[p]);
+    F3 v.ri2[p] = mul2(ri[p], ri[p]);
     if (CENTRED) {
         f2 num[3], dd[3];
         F3 num[p] = mul2(d[p].ddx, d[p].ddx);
@@ -417,64 +424,73 @@ __device__ __forceinline__ void far_tri(const f2 (&X)[3], const f2 (&Y)[3], cons
             s1[p] = mul2(s1[p], damp);
         }
     }
-    const f2 psr = hi2(P1), psi = lo2(P2), mpsi = hi2(P2), phr = lo2(P3), phi = hi2(P3), mphi = P5;
     // cos and sin scaled by 1/r once: G = (c + i s)/r for every kernel below
-    f2 c0r[3], s0r[3], c1r[3], s1r[3], ga[3], gb[3], hp[3], hq[3];
-    F3 c0r[p] = mul2(c0[p], ri[p]);
-    F3 s0r[p] = mul2(s0[p], ri[p]);
-    F3 c1r[p] = mul2(c1[p], ri[p]);
-    F3 s1r[p] = mul2(s1[p], ri[p]);
+    F3 v.c0r[p] = mul2(c0[p], ri[p]);
+    F3 v.s0r[p] = mul2(s0[p], ri[p]);
+    F3 v.c1r[p] = mul2(c1[p], ri[p]);
+    F3 v.s1r[p] = mul2(s1[p], ri[p]);
     // -(H0 + H1) r^2, H = e^{ikr} (i k r - 1) / r^3, with the scaled c, s:
     //   re = c0/r + c1/r + k0 s0 + k1 s1,  im = s0/r + s1/r - k0 c0 - k1 c1
-    F3 hp[p] = add2(c0r[p], c1r[p]);
-    F3 hq[p] = add2(s0r[p], s1r[p]);
-    F3 hp[p] = fma2(c.k0, s0[p], hp[p]);
-    F3 hp[p] = fma2(c.k1, s1[p], hp[p]);
-    F3 hq[p] = fma2(c.nk0, c0[p], hq[p]);
-    F3 hq[p] = fma2(c.nk1, c1[p], hq[p]);
+    F3 v.hp[p] = add2(v.c0r[p], v.c1r[p]);
+    F3 v.hq[p] = add2(v.s0r[p], v.s1r[p]);
+    F3 v.hp[p] = fma2(c.k0, s0[p], v.hp[p]);
+    F3 v.hp[p] = fma2(c.k1, s1[p], v.hp[p]);
+    F3 v.hq[p] = fma2(c.nk0, c0[p], v.hq[p]);
+    F3 v.hq[p] = fma2(c.nk1, c1[p], v.hq[p]);
     if (absorb) {  // (i k1 r - 1) with Im k1: + k1i r (c1, s1) / r
-        F3 hp[p] = fma2(k1i, c1[p], hp[p]);
-        F3 hq[p] = fma2(k1i, s1[p], hq[p]);
+        F3 v.hp[p] = fma2(k1i, c1[p], v.hp[p]);
+        F3 v.hq[p] = fma2(k1i, s1[p], v.hq[p]);
     }
+    return v;
+}
+
+template <bool CENTRED, bool MULTI, bool ABSORB>
+__device__ __forceinline__ void far_tri(const f2 (&X)[3], const f2 (&Y)[3], const f2 (&Z)[3], const float4 &n4,
+                                        float pdn, const float4 &P0, const float4 &P1, const float4 &P2, const float4 &P3,
+                                        const f2 &P5, const FarConst2 &c, const CenterPair &cp, f2 m1, f2 k1i,
+                                        f2 dk1i, PairAcc (&A)[3], CurlAcc &B) {
+    constexpr bool absorb = MULTI && ABSORB;
+    FarVals v = far_vals<CENTRED, MULTI, ABSORB>(X, Y, Z, n4, pdn, P0, P1, c, cp, m1, k1i);
+    const f2 psr = hi2(P1), psi = lo2(P2), mpsi = hi2(P2), phr = lo2(P3), phi = hi2(P3), mphi = P5;
+    f2 ga[3], gb[3];
     // D curl term: sums of G0 and G1, weighted and combined by the caller
-    F3 B.g0r = add2(B.g0r, c0r[p]);
-    F3 B.g0i = add2(B.g0i, s0r[p]);
-    F3 B.g1r = add2(B.g1r, c1r[p]);
-    F3 B.g1i = add2(B.g1i, s1r[p]);
+    F3 B.g0r = add2(B.g0r, v.c0r[p]);
+    F3 B.g0i = add2(B.g0i, v.s0r[p]);
+    F3 B.g1r = add2(B.g1r, v.c1r[p]);
+    F3 B.g1i = add2(B.g1i, v.s1r[p]);
     // V block (G0 + rho G1) psi, without 1/(4 pi)
-    F3 ga[p] = fma2(c.rho, c1r[p], c0r[p]);
-    F3 gb[p] = fma2(c.rho, s1r[p], s0r[p]);
+    F3 ga[p] = fma2(c.rho, v.c1r[p], v.c0r[p]);
+    F3 gb[p] = fma2(c.rho, v.s1r[p], v.s0r[p]);
     F3 A[p].u1r = fma2(gb[p], mpsi, A[p].u1r);
     F3 A[p].u1i = fma2(gb[p], psr, A[p].u1i);
     F3 A[p].u1r = fma2(ga[p], psr, A[p].u1r);
     F3 A[p].u1i = fma2(ga[p], psi, A[p].u1i);
     // D normal term (k0^2 G0 + k1^2/rho G1) phi, as (G0 + dk1 G1) phi; the
     // scale dks is applied per source triangle
-    F3 ga[p] = fma2(c.dk1, c1r[p], c0r[p]);
-    F3 gb[p] = fma2(c.dk1, s1r[p], s0r[p]);
+    F3 ga[p] = fma2(c.dk1, v.c1r[p], v.c0r[p]);
+    F3 gb[p] = fma2(c.dk1, v.s1r[p], v.s0r[p]);
     if (absorb) {  // complex k1^2 / (rho dks)
-        F3 ga[p] = fma2(mul2(dk1i, s1r[p]), dup2(-1.f), ga[p]);
-        F3 gb[p] = fma2(dk1i, c1r[p], gb[p]);
+        F3 ga[p] = fma2(mul2(dk1i, v.s1r[p]), dup2(-1.f), ga[p]);
+        F3 gb[p] = fma2(dk1i, v.c1r[p], gb[p]);
     }
     F3 A[p].ur = fma2(gb[p], mphi, A[p].ur);
     F3 A[p].ui = fma2(gb[p], phr, A[p].ui);
     F3 A[p].ur = fma2(ga[p], phr, A[p].ur);
     F3 A[p].ui = fma2(ga[p], phi, A[p].ui);
     // T1n = -sum Hs phi
-    F3 hp[p] = mul2(hp[p], ri2[p]);
-    F3 hq[p] = mul2(hq[p], ri2[p]);
-    F3 A[p].t1r = fma2(hq[p], mphi, A[p].t1r);
-    F3 A[p].t1i = fma2(hq[p], phr, A[p].t1i);
-    F3 A[p].t1r = fma2(hp[p], phr, A[p].t1r);
-    F3 A[p].t1i = fma2(hp[p], phi, A[p].t1i);
+    F3 v.hp[p] = mul2(v.hp[p], v.ri2[p]);
+    F3 v.hq[p] = mul2(v.hq[p], v.ri2[p]);
+    F3 A[p].t1r = fma2(v.hq[p], mphi, A[p].t1r);
+    F3 A[p].t1i = fma2(v.hq[p], phr, A[p].t1i);
+    F3 A[p].t1r = fma2(v.hp[p], phr, A[p].t1r);
+    F3 A[p].t1i = fma2(v.hp[p], phi, A[p].t1i);
     // T block: (H0 + H1)(x - y).n_x psi = (-(H0 + H1)) (y - x).n_x psi
-    F3 hp[p] = mul2(hp[p], dnxn);
-    F3 hq[p] = mul2(hq[p], dnxn);
-    F3 A[p].u2r = fma2(hq[p], mpsi, A[p].u2r);
-    F3 A[p].u2i = fma2(hq[p], psr, A[p].u2i);
-    F3 A[p].u2r = fma2(hp[p], psr, A[p].u2r);
-    F3 A[p].u2i = fma2(hp[p], psi, A[p].u2i);
-#undef F3
+    F3 v.hp[p] = mul2(v.hp[p], v.dnxn);
+    F3 v.hq[p] = mul2(v.hq[p], v.dnxn);
+    F3 A[p].u2r = fma2(v.hq[p], mpsi, A[p].u2r);
+    F3 A[p].u2i = fma2(v.hq[p], psr, A[p].u2i);
+    F3 A[p].u2r = fma2(v.hp[p], psr, A[p].u2r);
+    F3 A[p].u2i = fma2(v.hp[p], psi, A[p].u2i);
 }
 
 // One thread per test triangle: its six points are three pairs (p, p + 3)
@@ -723,12 +739,14 @@ far_kernel(const float4 *__restrict__ pt, const float4 *__restrict__ cen,
 
 // ---------------------------------------------------------------------------
 // Gather: L lanes per (vertex, right-hand side).  Far field, over the
-// incident (triangle t, local index a):
+// incident (triangle t, local index a), from far_kernel's sums:
 //   y1_v = (1/4pi) sum |t| sum_q w_q lambda_a(q) u1(t,q)
 //   y2_v = (1/4pi) sum |t| [sum_q w_q lambda_a(q) u2(t,q) + curl_a . A(t)]
+// or from farm_kernel's (E), which hold the test weights already:
+//   y1_v = (1/4pi) sum |t| E1(t,a),  y2_v = (1/4pi) sum |t| [E2(t,a) + curl_a . A(t)]
 // plus the near-field CSR rows (2x2 complex blocks) applied to x.  Partial
-// sums as far_kernel and farm_kernel leave them: part [ns][R][4][npts],
-// partA [ns][R][6][nt].
+// sums: part [ns][R][4][npts] and partA [ns][R][6][nt], or (E) part
+// [ns][R][18][nt], u1 (re, im) and u2 (re, im) of the corners 0, 1, 2, then A.
 // The lanes share the (triangle, point) items and the CSR entries.  The
 // source splits are added in FP32 with their rounding errors carried along
 // (Knuth's TwoSum: the sum to about 48 bits), because FP64 issues at 1/64 of
@@ -756,7 +774,7 @@ __device__ __forceinline__ double comp_value(float s, float e) {
     return isfinite(s) ? (double)s + (double)e : (double)s;
 }
 
-template <int L, int W>
+template <int L, int W, bool E>
 __global__ void __launch_bounds__(GATHER_THREADS)
 gather_kernel(int nv, int nt, int npts, int ns, int R, const int *__restrict__ vt_ptr,
               const int *__restrict__ vt_idx, const double *__restrict__ tgeo, const float *__restrict__ part,
@@ -771,7 +789,26 @@ gather_kernel(int nv, int nt, int npts, int ns, int R, const int *__restrict__ v
     const int rr = blockIdx.y;
     const bool valid = v < nv;  // every lane takes part in the shuffles below
     double2 y1 = cd(0, 0), y2 = cd(0, 0);
-    if (valid && use_far) {
+    if (E && valid && use_far) {
+        const int e0 = vt_ptr[v], items = 5 * (vt_ptr[v + 1] - e0);
+        const size_t su = (size_t)R * 18 * nt;
+        for (int it = lane; it < items; it += L) {
+            const int e = it / 5, q = it - 5 * e;  // q: u1, u2, A.x, A.y, A.z (complex)
+            const int ta = vt_idx[e0 + e], t = ta / 3, a = ta - 3 * t;
+            const double *g = tgeo + 16 * (size_t)t;
+            const float *P = part + ((size_t)rr * 18 + (q < 2 ? 4 * a + 2 * q : 8 + 2 * q)) * nt + t;
+            float s[2] = {0.f, 0.f}, c[2] = {0.f, 0.f};
+#pragma unroll 4
+            for (int sp = wg; sp < ns; sp += W) {
+                comp_add(s[0], c[0], P[sp * su]);
+                comp_add(s[1], c[1], P[sp * su + nt]);
+            }
+            const double w = 0.079577471545947667884 * g[0] * (q < 2 ? 1.0 : g[4 + 3 * a + (q - 2)]);
+            const double2 val = cd(w * comp_value(s[0], c[0]), w * comp_value(s[1], c[1]));
+            if (q == 0) y1 = cadd(y1, val);
+            else y2 = cadd(y2, val);
+        }
+    } else if (valid && use_far) {
         const int e0 = vt_ptr[v], items = 6 * (vt_ptr[v + 1] - e0);
         const size_t su = (size_t)R * 4 * npts, sa = (size_t)R * 6 * nt;
         for (int it = lane; it < items; it += L) {
@@ -836,400 +873,282 @@ gather_kernel(int nv, int nt, int npts, int ns, int R, const int *__restrict__ v
 
 // ---------------------------------------------------------------------------
 // Multi-right-hand-side far field: one launch applies B_far to R vectors.
-// Everything that depends only on the point pair (distance, 1/r, the four
-// sine / cosine values, the kernel combinations) is computed once and shared
-// by the R right-hand sides; only the accumulations scale with R.  To keep
-// per-right-hand-side state small, the per-source-triangle factors of the
-// K and D-normal terms ((x - y).n_y and n_x.n_y) are folded into the pair's
-// kernel values, so each right-hand side has just the two complex sums
-//   u1 = sum [ (G0 + rho G1) psi_q + (x - y).n_y (H0 + H1) phi_q ]
-//   u2 = sum [ (H0 + H1)(x - y).n_x psi_q - (n_x.n_y)(k0^2 G0 + k1^2/rho G1) phi_q ]
-// per test point, kept in registers over the whole source range.  The D
-// curl term A = sum_s (sum_q w_q (G0 + G1/rho)) c_s needs only
-// W(tau, s) = sum_p w_p sum_q w_q (G0 + G1/rho), which does not depend on the
-// right-hand side: each thread's share of it goes to shared memory per
-// source triangle, and after each tile the three threads of a test triangle
-// contract it with the right-hand sides' curl sources c_s (each thread a
-// third of the right-hand sides).
+// The densities are linear on a triangle and the test functions its three hat
+// functions, so what a pair of triangles contributes is, for any number of
+// right-hand sides, four complex 3 x 3 matrices [test corner b][source corner a]:
+//   S = sum_pq w_p w_q L_b(x_p) L_a(y_q) (G0 + rho G1),   K: (x - y).n_y (H0 + H1),
+//   T: (H0 + H1)(x - y).n_x,   N: -(n_x.n_y)(k0^2 G0 + k1^2/rho G1)
+// and the scalar W = sum_pq w_p w_q (G0 + G1/rho) of the curl term.  A pair of
+// points costs its kernel values and their share of the matrices; a
+// right-hand side costs 4 multiply-adds a point pair (144 a triangle pair,
+// u1_b += S psi + K phi, u2_b += T psi + N phi) instead of the 16 of sums point
+// by point.  The matrices come from sums M0, M1 of G0 and G1 (S, N and W are
+// combinations of them, formed once per triangle pair), and the rule's two
+// classes of three points with barycentric (alpha, beta, beta) give
+// sum_q v_q L_a(y_q) = beta sum_q v_q + (alpha - beta) v_a per class.
 //
-// Block: FARM_THREADS = 384 threads = 128 test triangles, thread j holds test
-// points 2 (j mod 3), 2 (j mod 3) + 1 of triangle j / 3 packed in FP32x2
-// lanes.  Source data (per point, duplicated pairs for the packed lanes):
-//   sG [6nt][2]   (-y.x, -y.x, -y.y, -y.y), (-y.z, -y.z, w_q, w_q)   (static)
-//   sD [nt][6][R][2]  (psi.re, psi.re, psi.im, psi.im), (phi.re, ..., phi.im)
-//   sCm [nt][R][3]    c_s components (complex)
-// Outputs (no atomics; gridDim.y splits the source range):
-//   part  [ns][R][4][npts]  u1 (re, im), u2 (re, im) per test point
-//   partA [ns][R][6][nt]    sum_p w_p A(x_p) per test triangle (x, y, z; re, im)
+// Source data (the points duplicated into pairs for the packed lanes):
+//   sG [6nt][2]   (-y.x, -y.x, -y.y, -y.y), (-y.z, -y.z, 0, 0)   (static)
+//   sD [nt][R][5] corner a: |s| (psi_a, phi_a); then c_s (three complex, 0, 0)
+// Output (no atomics; gridDim.y splits the source range):
+//   part [ns][R][18][nt]  u1 (re, im), u2 (re, im) of corners 0, 1, 2; then
+//                         A = sum_s W c_s (x, y, z; re, im)
 // ---------------------------------------------------------------------------
-// 384 threads = 12 warps, 3 on each of the SM's four schedulers (a block
-// whose warps spread unevenly over the schedulers waits at every tile
-// barrier for its most crowded scheduler); one block per SM at <= 170
-// registers per thread
-#ifndef OSRC_FARM_THREADS
-#define OSRC_FARM_THREADS 384
-#endif
-constexpr int FARM_THREADS = OSRC_FARM_THREADS;
-#ifndef OSRC_FARM_MIN_BLOCKS
-#define OSRC_FARM_MIN_BLOCKS 1
-#endif
-#ifndef OSRC_FARM_QUNROLL
-#define OSRC_FARM_QUNROLL 2
-#endif
-constexpr int FARM_QUNROLL = OSRC_FARM_QUNROLL;  // unroll of the rule-point loop
-constexpr int FARM_TRIS = FARM_THREADS / 3;  // test triangles per block
-constexpr int FARM_TS = 16;                  // source triangles per shared-memory tile
-// one shared-memory tile buffer: sG, sD, sCm, normals, vertex ids, centroids
-constexpr size_t farm_buf_bytes(int R, bool centred) {
-    return (size_t)FARM_TS * (12 * 16 + 12 * 16 * R + 24 * R + 16 + 16 + (centred ? 32 : 0));
-}
+constexpr int FARM_TS = 32;  // source triangles per shared-memory tile
+constexpr int FARM_MIN_BLOCKS = 2;
 
-size_t farm_smem_bytes(int R, bool centred) {
-    return 2 * farm_buf_bytes(R, centred) + (size_t)FARM_TS * FARM_THREADS * sizeof(float2) + 2 * sizeof(uint64_t);
-}
-
-constexpr unsigned long long FARM_TIMEOUT_NS = 2000000000ULL;
-
-__device__ __forceinline__ uint32_t farm_saddr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ unsigned long long farm_ns() {
-    unsigned long long t;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-    return t;
-}
-
-// waits for phase `parity` of the mbarrier, at most FARM_TIMEOUT_NS of global time
-__device__ __forceinline__ bool farm_wait(uint64_t *bar, uint32_t parity) {
-    const unsigned long long t0 = farm_ns();
-    while (true) {
-        uint32_t done;
-        asm volatile(
-            "{\n\t.reg .pred p;\n\t"
-            "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-            "selp.u32 %0, 1, 0, p;\n\t}"
-            : "=r"(done)
-            : "r"(farm_saddr(bar)), "r"(parity)
-            : "memory");
-        if (done) return true;
-        if (farm_ns() - t0 > FARM_TIMEOUT_NS) return false;
-    }
-}
-
-// 1-D bulk copy global -> shared (16-byte aligned addresses, size a multiple
-// of 16), completion counted on the mbarrier
-__device__ __forceinline__ void farm_bulk(void *dst, const void *src, uint32_t bytes, uint64_t *bar) {
-    asm volatile(
-        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-            farm_saddr(dst)),
-        "l"((uint64_t)src), "r"(bytes), "r"(farm_saddr(bar))
-        : "memory");
+constexpr size_t farm_smem_bytes(int R) {
+    return (size_t)FARM_TS * (12 * 16 + 5 * 16 * R + 16 + 16 + 32) + (size_t)FAR_THREADS * 72 * R;
 }
 
 // static source geometry of the multi kernel: coordinates (absolute, or
 // offsets from the triangle centroid for the centred variant) negated and
-// duplicated, and the rule weight w_q
+// duplicated
 __global__ void farm_geom_kernel(const float4 *__restrict__ pts, int npts, float4 *__restrict__ sG) {
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= npts) return;
     const float4 p = pts[k];
-    const int q = k % 6;
-    const float w = (float)(q < 3 ? kQw1 : kQw2);
     sG[2 * (size_t)k] = make_float4(-p.x, -p.x, -p.y, -p.y);
-    sG[2 * (size_t)k + 1] = make_float4(-p.z, -p.z, w, w);
+    sG[2 * (size_t)k + 1] = make_float4(-p.z, -p.z, 0.f, 0.f);
 }
 
-// densities of R right-hand sides at the source rule points and the curl
-// sources c_s, one thread per (source triangle, right-hand side)
+// corner densities of R right-hand sides times the triangle's area and the
+// curl sources c_s, one thread per (source triangle, right-hand side)
 __global__ void farm_prep_kernel(VecPtrs x, int R, int nv, int nt, const int *__restrict__ tris,
-                                 const double *__restrict__ tgeo, float4 *__restrict__ sD,
-                                 float2 *__restrict__ sCm) {
+                                 const double *__restrict__ tgeo, float4 *__restrict__ sD) {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     const int r = blockIdx.y;
     if (t >= nt || r >= R) return;
     const double2 *xr = x.p[r];
-    double2 ps[3], ph[3];
-    for (int a = 0; a < 3; ++a) {
-        const int v = tris[3 * t + a];
-        ps[a] = xr[v];
-        ph[a] = xr[nv + v];
-    }
     const double *g = tgeo + 16 * (size_t)t;
     const double area = g[0];
-    for (int q = 0; q < 6; ++q) {
-        double b[3], w;
-        rule_point(q, b, w);
-        const double W = w * area;
-        double2 sv = cd(0, 0), fv = cd(0, 0);
-        for (int a = 0; a < 3; ++a) {
-            sv = cadd(sv, cscale(ps[a], b[a]));
-            fv = cadd(fv, cscale(ph[a], b[a]));
-        }
-        const float psr = (float)(W * sv.x), psi = (float)(W * sv.y);
-        const float phr = (float)(W * fv.x), phi = (float)(W * fv.y);
-        float4 *d = sD + 2 * ((6 * (size_t)t + q) * R + r);
-        d[0] = make_float4(psr, psr, psi, psi);
-        d[1] = make_float4(phr, phr, phi, phi);
+    float4 *d = sD + 5 * ((size_t)t * R + r);
+    double2 cv[3] = {cd(0, 0), cd(0, 0), cd(0, 0)};
+    for (int a = 0; a < 3; ++a) {
+        const int v = tris[3 * t + a];
+        const double2 ps = cscale(xr[v], area), ph = cscale(xr[nv + v], area);
+        d[a] = make_float4((float)ps.x, (float)ps.y, (float)ph.x, (float)ph.y);
+        for (int j = 0; j < 3; ++j) cv[j] = cadd(cv[j], cscale(ph, g[4 + 3 * a + j]));
     }
-    for (int j = 0; j < 3; ++j) {
-        double2 cv = cd(0, 0);
-        for (int a = 0; a < 3; ++a) cv = cadd(cv, cscale(ph[a], g[4 + 3 * a + j]));
-        sCm[3 * ((size_t)t * R + r) + j] = make_float2((float)(cv.x * area), (float)(cv.y * area));
-    }
+    d[3] = make_float4((float)cv[0].x, (float)cv[0].y, (float)cv[1].x, (float)cv[1].y);
+    d[4] = make_float4((float)cv[2].x, (float)cv[2].y, 0.f, 0.f);
 }
 
-// One source point against the thread's two test points, R right-hand sides.
-template <int R, bool CENTRED>
-__device__ __forceinline__ void farm_pair(f2 X, f2 Y, f2 Z, const float4 G0, const float4 G1,
-                                          const float4 *__restrict__ D, f2 mnx, f2 mny, f2 mnz, f2 xnyn,
-                                          f2 nn, const FarConst2 &c, const CenterPair &cp, f2 &t3r,
-                                          f2 &t3i, f2 (&u1r)[R], f2 (&u1i)[R], f2 (&u2r)[R],
-                                          f2 (&u2i)[R]) {
-    f2 dx, dy, dz, ddx, ddy, ddz;
-    if (CENTRED) {
-        ddx = add2(X, lo2(G0));
-        ddy = add2(Y, hi2(G0));
-        ddz = add2(Z, lo2(G1));
-        dx = add2(ddx, cp.Dx);
-        dy = add2(ddy, cp.Dy);
-        dz = add2(ddz, cp.Dz);
-    } else {
-        dx = add2(X, lo2(G0));
-        dy = add2(Y, hi2(G0));
-        dz = add2(Z, lo2(G1));
-    }
-    f2 r2 = mul2(dx, dx);
-    r2 = fma2(dy, dy, r2);
-    r2 = fma2(dz, dz, r2);
-    const f2 ri = make_float2(rsqrtf(r2.x), rsqrtf(r2.y));
-    const f2 r = mul2(r2, ri);
-    const f2 ri2 = mul2(ri, ri);
-    f2 dnxn = mul2(dx, mnx);  // (y - x).n_x
-    dnxn = fma2(dy, mny, dnxn);
-    dnxn = fma2(dz, mnz, dnxn);
-    f2 s0, c0, s1, c1;
-    if (CENTRED) {
-        f2 num = mul2(ddx, ddx);
-        num = fma2(ddy, ddy, num);
-        num = fma2(ddz, ddz, num);
-        f2 dd = mul2(ddx, cp.Dx);
-        dd = fma2(ddy, cp.Dy, dd);
-        dd = fma2(ddz, cp.Dz, dd);
-        num = fma2(dd, dup2(2.f), num);
-        const f2 den = add2(r, cp.rc);
-        const f2 dlt = mul2(num, make_float2(rcp_approx(den.x), rcp_approx(den.y)));
-        const f2 ph0 = fma2(c.k0, dlt, cp.b0);
-        const f2 ph1 = fma2(c.k1, dlt, cp.b1);
-        __sincosf(ph0.x, &s0.x, &c0.x);
-        __sincosf(ph0.y, &s0.y, &c0.y);
-        __sincosf(ph1.x, &s1.x, &c1.x);
-        __sincosf(ph1.y, &s1.y, &c1.y);
-    } else {
-        const f2 kr0 = mul2(r, c.k0), kr1 = mul2(r, c.k1);
-        __sincosf(kr0.x, &s0.x, &c0.x);
-        __sincosf(kr0.y, &s0.y, &c0.y);
-        __sincosf(kr1.x, &s1.x, &c1.x);
-        __sincosf(kr1.y, &s1.y, &c1.y);
-    }
-    const f2 c0r = mul2(c0, ri), s0r = mul2(s0, ri), c1r = mul2(c1, ri), s1r = mul2(s1, ri);
-    // V: G0 + rho G1
-    const f2 gpr = fma2(c.rho, c1r, c0r), gpi = fma2(c.rho, s1r, s0r);
-    // D normal: (-n_x.n_y) dks (G0 + dk1 G1), nn = -n_x.n_y dks
-    const f2 gkr = mul2(nn, fma2(c.dk1, c1r, c0r)), gki = mul2(nn, fma2(c.dk1, s1r, s0r));
-    // D curl weight: sum_q w_q (G0 + G1/rho)
-    const f2 wq = hi2(G1);
-    t3r = fma2(fma2(c.irho, c1r, c0r), wq, t3r);
-    t3i = fma2(fma2(c.irho, s1r, s0r), wq, t3i);
-    // -(H0 + H1) with the scaled c, s (see far_tri)
-    const f2 hp = mul2(fma2(c.k1, s1, fma2(c.k0, s0, add2(c0r, c1r))), ri2);
-    const f2 hq = mul2(fma2(c.nk1, c1, fma2(c.nk0, c0, add2(s0r, s1r))), ri2);
-    // K: (x - y).n_y (H0 + H1) = (-(x - y).n_y)(-(H0 + H1));  T: (H0 + H1)(x - y).n_x
-    const f2 kr = mul2(xnyn, hp), ki = mul2(xnyn, hq);
-    const f2 tr = mul2(dnxn, hp), ti = mul2(dnxn, hq);
-    const f2 m1 = dup2(-1.f);
-    const f2 ngpi = mul2(gpi, m1), nki = mul2(ki, m1), nti = mul2(ti, m1), ngki = mul2(gki, m1);
-#pragma unroll
-    for (int rr = 0; rr < R; ++rr) {
-        const float4 Ps = D[2 * rr], Ph = D[2 * rr + 1];
-        const f2 psr = lo2(Ps), psi = hi2(Ps), phr = lo2(Ph), phi = hi2(Ph);
-        u1r[rr] = fma2(gpr, psr, fma2(ngpi, psi, fma2(kr, phr, fma2(nki, phi, u1r[rr]))));
-        u1i[rr] = fma2(gpr, psi, fma2(gpi, psr, fma2(kr, phi, fma2(ki, phr, u1i[rr]))));
-        u2r[rr] = fma2(tr, psr, fma2(nti, psi, fma2(gkr, phr, fma2(ngki, phi, u2r[rr]))));
-        u2i[rr] = fma2(tr, psi, fma2(ti, psr, fma2(gkr, phi, fma2(gki, phr, u2i[rr]))));
-    }
-}
-
-template <int R, bool CENTRED>
-struct FarmBuf {
-    float4 *G;   // [TS*6][2]
-    float4 *D;   // [TS*6][R][2]
-    float2 *C;   // [TS][R][3]
-    float4 *N;   // [TS] normal, plane offset
-    int4 *V;     // [TS] vertex ids
-    float4 *Cen; // [2 TS] (centred)
-    __device__ FarmBuf(unsigned char *base) {
-        G = reinterpret_cast<float4 *>(base);
-        D = G + FARM_TS * 12;
-        C = reinterpret_cast<float2 *>(D + FARM_TS * 12 * R);
-        N = reinterpret_cast<float4 *>(C + FARM_TS * 3 * R);
-        V = reinterpret_cast<int4 *>(N + FARM_TS);
-        Cen = reinterpret_cast<float4 *>(V + FARM_TS);
-    }
-};
-
-// Source tiles are staged by 1-D TMA bulk copies (cp.async.bulk) into a
-// two-buffer shared-memory ring: thread 0 issues tile k + 1 while every
-// thread computes tile k, and an mbarrier per buffer counts the bytes in.
-// Every wait is bounded (FARM_TIMEOUT_NS of global time); a thread that
-// gives up sets *err, stops waiting, and writes NaN instead of its sums, and
-// thread 0 waits (bounded) for the copies it issued before the block exits.
-template <int R, bool CENTRED>
-__global__ void __launch_bounds__(FARM_THREADS, OSRC_FARM_MIN_BLOCKS)
+// One thread per test triangle, on far_kernel's grid (blocks of block_tris test
+// triangles, the warps of a block sharing its source tiles when that is less
+// than FAR_THREADS).  The matrices stay in registers (72, and 24 sums; 255
+// registers, two blocks per SM); the right-hand sides' sums, 18 floats each,
+// are in shared memory, a thread's own column, so R costs no registers and one
+// kernel takes every R up to FARM_MAX_R.  After each tile they move to part:
+// short sums keep their rounding errors (1.2 to 2 times less than without on
+// 3000 to 5000 vertices) for 2 % of the time, the old values of an entry's 18
+// being loaded together.
+// Bound by the FP32 pipe: an apply at 10242 vertices is 26.9 ms of kernel
+// values and matrices and 2.7 ms a right-hand side (R 2: 32.5 ms, 4: 38.0,
+// 8: 48.8), where point-by-point sums took 24 + 9.9 (43.6, 65.1, 102.7).  R = 1
+// would take 29.6 against far_kernel's 25.9.  Tensor cores do not help: TF32
+// pieces with the kernel values as an operand took 64.7 ms at R 2 and 80.8 at
+// 8, mma.sync and packed FMA not overlapping.
+template <bool CENTRED>
+__global__ void __launch_bounds__(FAR_THREADS, FARM_MIN_BLOCKS)
 farm_kernel(const float4 *__restrict__ pt, const float4 *__restrict__ cen, const float4 *__restrict__ tn,
-            const int4 *__restrict__ tv, const float4 *__restrict__ sG, const float4 *__restrict__ sD,
-            const float2 *__restrict__ sCm, int nt, int npts, int tris_per_split, FarConst2 c,
-            float4 kff, float *__restrict__ part, float *__restrict__ partA, int *__restrict__ err) {
+            const int4 *__restrict__ tv, const float4 *__restrict__ sG, const float4 *__restrict__ sD, int R,
+            int nt, int tris_per_split, int block_tris, FarConst2 c, float4 kff, float *__restrict__ part) {
     extern __shared__ __align__(16) unsigned char farm_smem[];
-    constexpr size_t BUF = farm_buf_bytes(R, CENTRED);
-    float2 *shW = reinterpret_cast<float2 *>(farm_smem + 2 * BUF);  // [TS][threads]
-    uint64_t *bar = reinterpret_cast<uint64_t *>(shW + FARM_TS * FARM_THREADS);
+    float4 *acc4 = reinterpret_cast<float4 *>(farm_smem);                            // [R][4][threads]
+    float2 *acc2 = reinterpret_cast<float2 *>(acc4 + (size_t)R * 4 * FAR_THREADS);   // [R][threads]
+    float4 *shG = reinterpret_cast<float4 *>(acc2 + (size_t)R * FAR_THREADS);        // [TS][6][2]
+    float4 *shD = shG + FARM_TS * 12;                                                // [TS][R][5]
+    float4 *shN = shD + FARM_TS * 5 * R;                                             // [TS] (-n, n.P0)
+    int4 *shV = reinterpret_cast<int4 *>(shN + FARM_TS);                             // [TS]
+    float4 *shCen = reinterpret_cast<float4 *>(shV + FARM_TS);                       // [TS][2] (centred)
 
-    const int j = threadIdx.x;
-    const int lt = j / 3, sub = j - 3 * (j / 3);
-    const int tau_raw = blockIdx.x * FARM_TRIS + lt;
-    const bool active = tau_raw < nt;
-    const int tau = active ? tau_raw : 0;
-    const int p0 = 6 * tau + 2 * sub;
+    const int tx = threadIdx.x % block_tris, grp = threadIdx.x / block_tris, ngrp = FAR_THREADS / block_tris;
+    const int j = blockIdx.x * block_tris + tx;
     const int split = blockIdx.y;
-    const int s_begin = split * tris_per_split;
+    const int s_begin = min(nt, split * tris_per_split);
     const int s_end = min(nt, s_begin + tris_per_split);
-    const int ntiles = s_end > s_begin ? (s_end - s_begin + FARM_TS - 1) / FARM_TS : 0;
-    const float4 xa = pt[p0], xb = pt[p0 + 1];
-    const f2 X = make_float2(xa.x, xb.x), Y = make_float2(xa.y, xb.y), Z = make_float2(xa.z, xb.z);
+    const int tau = j < nt ? j : 0;
+    f2 X[3], Y[3], Z[3];
+#pragma unroll
+    for (int p = 0; p < 3; ++p) {
+        const float4 xa = pt[6 * tau + p], xb = pt[6 * tau + p + 3];
+        X[p] = make_float2(xa.x, xb.x);
+        Y[p] = make_float2(xa.y, xb.y);
+        Z[p] = make_float2(xa.z, xb.z);
+    }
     const float4 n4 = tn[tau];
     const int4 vt = tv[tau];
-    const f2 mnx = dup2(-n4.x), mny = dup2(-n4.y), mnz = dup2(-n4.z);
-    const float wa = (float)(2 * sub < 3 ? kQw1 : kQw2), wb = (float)(2 * sub + 1 < 3 ? kQw1 : kQw2);
+    // the rule's classes: weights times beta, and times alpha - beta
+    constexpr float WB1 = (float)(kQw1 * kQa1), WB2 = (float)(kQw2 * kQa2);
+    constexpr float WG1 = (float)(kQw1 * (1.0 - 3.0 * kQa1)), WG2 = (float)(kQw2 * (1.0 - 3.0 * kQa2));
+    const f2 wb = make_float2(WB1, WB2), wg = make_float2(WG1, WG2);
     float4 cth = make_float4(0.f, 0.f, 0.f, 0.f), ctl = cth;
     if (CENTRED) {
         cth = cen[2 * tau];
         ctl = cen[2 * tau + 1];
     }
-    f2 u1r[R], u1i[R], u2r[R], u2i[R];
-#pragma unroll
-    for (int rr = 0; rr < R; ++rr) u1r[rr] = u1i[rr] = u2r[rr] = u2i[rr] = make_float2(0.f, 0.f);
+    float *const out = part + (size_t)split * R * 18 * nt;
+    for (int i = threadIdx.x; i < R * 18 * FAR_THREADS; i += FAR_THREADS) reinterpret_cast<float *>(acc4)[i] = 0.f;
 
-    // thread 0: the copies of tile k into buffer k & 1
-    auto issue = [&](int k) {
-        const int t0 = s_begin + k * FARM_TS;
+    for (int t0 = s_begin; t0 < s_end; t0 += FARM_TS) {
         const int cnt = min(FARM_TS, s_end - t0);
-        FarmBuf<R, CENTRED> fb(farm_smem + (k & 1) * BUF);
-        uint64_t *mb = &bar[k & 1];
-        const uint32_t bytes = (uint32_t)cnt * (12 * 16 + 12 * 16 * R + 24 * R + 16 + 16 + (CENTRED ? 32 : 0));
-        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(farm_saddr(mb)), "r"(bytes)
-                     : "memory");
-        farm_bulk(fb.G, sG + 12 * (size_t)t0, (uint32_t)cnt * 12 * 16, mb);
-        farm_bulk(fb.D, sD + 12 * (size_t)R * t0, (uint32_t)cnt * 12 * 16 * R, mb);
-        farm_bulk(fb.C, sCm + 3 * (size_t)R * t0, (uint32_t)cnt * 24 * R, mb);
-        farm_bulk(fb.N, tn + t0, (uint32_t)cnt * 16, mb);
-        farm_bulk(fb.V, tv + t0, (uint32_t)cnt * 16, mb);
-        if (CENTRED) farm_bulk(fb.Cen, cen + 2 * (size_t)t0, (uint32_t)cnt * 32, mb);
-    };
-    if (j == 0) {
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(farm_saddr(&bar[0])));
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(farm_saddr(&bar[1])));
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
-    __syncthreads();
-    if (j == 0 && ntiles > 0) issue(0);
-    bool dead = false;      // a bounded wait gave up
-    int issued = ntiles > 0 ? 1 : 0;  // tiles issued (thread 0)
+        for (int i = threadIdx.x; i < cnt * 12; i += FAR_THREADS) shG[i] = sG[12 * (size_t)t0 + i];
+        for (int i = threadIdx.x; i < cnt * 5 * R; i += FAR_THREADS) shD[i] = sD[5 * (size_t)R * t0 + i];
+        for (int i = threadIdx.x; i < cnt; i += FAR_THREADS) {
+            const float4 ns = tn[t0 + i];
+            shN[i] = make_float4(-ns.x, -ns.y, -ns.z, ns.w);
+            shV[i] = tv[t0 + i];
+        }
+        if (CENTRED)
+            for (int i = threadIdx.x; i < 2 * cnt; i += FAR_THREADS) shCen[i] = cen[2 * (size_t)t0 + i];
+        __syncthreads();
 
-    for (int k = 0; k < ntiles; ++k) {
-        const int t0 = s_begin + k * FARM_TS;
-        const int cnt = min(FARM_TS, s_end - t0);
-        FarmBuf<R, CENTRED> fb(farm_smem + (k & 1) * BUF);
-        if (!dead && !farm_wait(&bar[k & 1], (uint32_t)(k >> 1) & 1u)) {
-            dead = true;
-            atomicExch(err, 1);
-        }
-        // the other buffer held tile k - 1, released by the barrier that ended it
-        if (j == 0 && !dead && k + 1 < ntiles) {
-            issue(k + 1);
-            issued = k + 2;
-        }
-        for (int s = 0; s < cnt; ++s) {
-            const int4 vs = fb.V[s];
+        for (int s = grp; s < cnt; s += ngrp) {
+            const int4 vs = shV[s];
             const bool touch = (vs.x == vt.x) | (vs.x == vt.y) | (vs.x == vt.z) |
                                (vs.y == vt.x) | (vs.y == vt.y) | (vs.y == vt.z) |
                                (vs.z == vt.x) | (vs.z == vt.y) | (vs.z == vt.z);
-            if (touch) {
-                shW[s * FARM_THREADS + j] = make_float2(0.f, 0.f);
-                continue;
-            }
-            const float4 ns = fb.N[s];
-            const float4 mns = make_float4(-ns.x, -ns.y, -ns.z, ns.w);
+            if (touch) continue;
             CenterPair cp;
-            f2 xnyn;
+            float pdn = __int_as_float(vt.w);
+            const float4 mns = shN[s];
+            float dn = mns.w;
             if (CENTRED) {
-                cp = center_pair(cth, ctl, fb.Cen[2 * s], fb.Cen[2 * s + 1], kff.x, kff.y, kff.z, kff.w);
-                const float dn = cp.Dx.x * mns.x + cp.Dy.x * mns.y + cp.Dz.x * mns.z;
-                xnyn = fma2(Z, dup2(mns.z), fma2(Y, dup2(mns.y), fma2(X, dup2(mns.x), dup2(dn))));
-            } else {
-                xnyn = fma2(Z, dup2(mns.z), fma2(Y, dup2(mns.y), fma2(X, dup2(mns.x), dup2(mns.w))));
+                cp = center_pair(cth, ctl, shCen[2 * s], shCen[2 * s + 1], kff.x, kff.y, kff.z, kff.w);
+                pdn = fmaf(cp.Dx.x, n4.x, fmaf(cp.Dy.x, n4.y, cp.Dz.x * n4.z)) +
+                      fmaf(cp.lx, n4.x, fmaf(cp.ly, n4.y, cp.lz * n4.z));
+                dn = cp.Dx.x * mns.x + cp.Dy.x * mns.y + cp.Dz.x * mns.z;
             }
-            const f2 nn = dup2((n4.x * mns.x + n4.y * mns.y + n4.z * mns.z) * c.dk0.x);
-            f2 t3r = make_float2(0.f, 0.f), t3i = t3r;
-#pragma unroll FARM_QUNROLL
-            for (int q = 0; q < 6; ++q)
-                farm_pair<R, CENTRED>(X, Y, Z, fb.G[12 * s + 2 * q], fb.G[12 * s + 2 * q + 1],
-                                      &fb.D[2 * R * (6 * s + q)], mnx, mny, mnz, xnyn, nn, c, cp, t3r,
-                                      t3i, u1r, u1i, u2r, u2i);
-            shW[s * FARM_THREADS + j] = make_float2(wa * t3r.x + wb * t3r.y, wa * t3i.x + wb * t3i.y);
-        }
-        __syncthreads();
-        // curl term of this tile: thread (lt, sub) takes right-hand sides sub, sub + 3, ...
-        if (active) {
-            for (int rr = sub; rr < R; rr += 3) {
-                float ar[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-                for (int s = 0; s < cnt; ++s) {
-                    const float2 *w3 = shW + s * FARM_THREADS + 3 * lt;
-                    const float wr = w3[0].x + w3[1].x + w3[2].x, wi = w3[0].y + w3[1].y + w3[2].y;
-                    const float2 *cc = fb.C + 3 * (s * R + rr);
+            f2 kb[3], kg[3];  // the test weights times -(x - y).n_y
+            F3 {
+                const f2 xnyn = fma2(Z[p], dup2(mns.z), fma2(Y[p], dup2(mns.y), fma2(X[p], dup2(mns.x), dup2(dn))));
+                kb[p] = mul2(wb, xnyn);
+                kg[p] = mul2(wg, xnyn);
+            }
+            // E[v][b][a], v = M0, M1, T, K (re, im): class 0 stores, class 1 adds; bs: the beta parts
+            float E[8][3][3], bs[8][3];
 #pragma unroll
-                    for (int d = 0; d < 3; ++d) {
-                        const float2 cv = cc[d];
-                        ar[2 * d] += wr * cv.x - wi * cv.y;
-                        ar[2 * d + 1] += wr * cv.y + wi * cv.x;
+            for (int q = 0; q < 6; ++q) {
+                const float4 P0 = shG[12 * s + 2 * q], P1 = shG[12 * s + 2 * q + 1];
+                FarVals v = far_vals<CENTRED, false, false>(X, Y, Z, n4, pdn, P0, P1, c, cp, dup2(1.f), dup2(0.f));
+                F3 v.hp[p] = mul2(v.hp[p], v.ri2[p]);
+                F3 v.hq[p] = mul2(v.hq[p], v.ri2[p]);
+                const float wgq = q < 3 ? WG1 : WG2, wbq = q < 3 ? WB1 : WB2;
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const f2(&u)[3] = i == 0 ? v.c0r : i == 1 ? v.s0r : i == 2 ? v.c1r : i == 3 ? v.s1r
+                                      : (i & 1) ? v.hq : v.hp;
+                    const f2 sum = i < 6 ? mul2(wb, add2(add2(u[0], u[1]), u[2]))
+                                         : fma2(kb[2], u[2], fma2(kb[1], u[1], mul2(kb[0], u[0])));
+#pragma unroll
+                    for (int b = 0; b < 3; ++b) {
+                        const f2 tb = fma2(i < 6 ? wg : kg[b], u[b], sum);
+                        float t = tb.x + tb.y;
+                        if (i == 4 || i == 5) t *= v.dnxn.x;  // T: (y - x).n_x is the source point's alone
+                        E[i][b][q % 3] = q < 3 ? wgq * t : fmaf(wgq, t, E[i][b][q % 3]);
+                        bs[i][b] = q == 0 ? wbq * t : fmaf(wbq, t, bs[i][b]);
                     }
                 }
-                float *pa = partA + (((size_t)split * R + rr) * 6) * nt + tau;
+            }
+            float w0 = 0.f, w1 = 0.f, w2 = 0.f, w3 = 0.f;
 #pragma unroll
-                for (int d = 0; d < 6; ++d) pa[(size_t)d * nt] = k == 0 ? ar[d] : pa[(size_t)d * nt] + ar[d];
+            for (int b = 0; b < 3; ++b)
+#pragma unroll
+                for (int a = 0; a < 3; ++a) {
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) E[i][b][a] += bs[i][b];
+                    w0 += E[0][b][a];
+                    w1 += E[1][b][a];
+                    w2 += E[2][b][a];
+                    w3 += E[3][b][a];
+                }
+            const float wr = fmaf(c.irho.x, w2, w0), wi = fmaf(c.irho.x, w3, w1);
+            const float nn = (n4.x * mns.x + n4.y * mns.y + n4.z * mns.z) * c.dk0.x;  // -(n_x.n_y) dks
+            // M0, M1 -> S and N
+#pragma unroll
+            for (int b = 0; b < 3; ++b)
+#pragma unroll
+                for (int a = 0; a < 3; ++a) {
+                    const float g0 = E[0][b][a], g1 = E[1][b][a], g2 = E[2][b][a], g3 = E[3][b][a];
+                    E[0][b][a] = fmaf(c.rho.x, g2, g0);
+                    E[1][b][a] = fmaf(c.rho.x, g3, g1);
+                    E[2][b][a] = nn * fmaf(c.dk1.x, g2, g0);
+                    E[3][b][a] = nn * fmaf(c.dk1.x, g3, g1);
+                }
+#pragma unroll 1
+            for (int r = 0; r < R; ++r) {
+                const float4 *D = shD + 5 * (s * R + r);
+                float4 *o4 = acc4 + (size_t)r * 4 * FAR_THREADS + threadIdx.x;
+                float4 u[3];
+#pragma unroll
+                for (int b = 0; b < 3; ++b) u[b] = o4[b * FAR_THREADS];
+#pragma unroll
+                for (int a = 0; a < 3; ++a) {
+                    const float4 d = D[a];
+#pragma unroll
+                    for (int b = 0; b < 3; ++b) {
+                        u[b].x = fmaf(E[0][b][a], d.x, fmaf(-E[1][b][a], d.y, fmaf(E[6][b][a], d.z, fmaf(-E[7][b][a], d.w, u[b].x))));
+                        u[b].y = fmaf(E[0][b][a], d.y, fmaf(E[1][b][a], d.x, fmaf(E[6][b][a], d.w, fmaf(E[7][b][a], d.z, u[b].y))));
+                        u[b].z = fmaf(E[4][b][a], d.x, fmaf(-E[5][b][a], d.y, fmaf(E[2][b][a], d.z, fmaf(-E[3][b][a], d.w, u[b].z))));
+                        u[b].w = fmaf(E[4][b][a], d.y, fmaf(E[5][b][a], d.x, fmaf(E[2][b][a], d.w, fmaf(E[3][b][a], d.z, u[b].w))));
+                    }
+                }
+#pragma unroll
+                for (int b = 0; b < 3; ++b) o4[b * FAR_THREADS] = u[b];
+                const float4 C0 = D[3], C1 = D[4];
+                float4 A = o4[3 * FAR_THREADS];
+                float2 *o2 = acc2 + (size_t)r * FAR_THREADS + threadIdx.x, Az = *o2;
+                A.x = fmaf(wr, C0.x, fmaf(-wi, C0.y, A.x));
+                A.y = fmaf(wr, C0.y, fmaf(wi, C0.x, A.y));
+                A.z = fmaf(wr, C0.z, fmaf(-wi, C0.w, A.z));
+                A.w = fmaf(wr, C0.w, fmaf(wi, C0.z, A.w));
+                Az.x = fmaf(wr, C1.x, fmaf(-wi, C1.y, Az.x));
+                Az.y = fmaf(wr, C1.y, fmaf(wi, C1.x, Az.y));
+                o4[3 * FAR_THREADS] = A;
+                *o2 = Az;
             }
         }
         __syncthreads();
-    }
-    if (j == 0 && dead) {  // copies still in flight land before the block exits: the
-                           // last tile issued into each buffer
-        for (int k = max(0, issued - 2); k < issued; ++k)
-            if (!farm_wait(&bar[k & 1], (uint32_t)(k >> 1) & 1u)) break;
-    }
-    if (active) {
-        f2 *pp = reinterpret_cast<f2 *>(part);
-        const f2 nan2 = make_float2(__int_as_float(0x7fc00000), __int_as_float(0x7fc00000));
+        // the tile's sums of all groups to part (the first tile stores, later
+        // ones add; the same thread has the same entries each time)
+        const bool first = t0 == s_begin;
+        for (int i = threadIdx.x; i < R * block_tris; i += FAR_THREADS) {
+            const int r = i / block_tris, jj = i - r * block_tris, jt = blockIdx.x * block_tris + jj;
+            float *o = out + (size_t)r * 18 * nt + jt;
+            float v[18];
 #pragma unroll
-        for (int rr = 0; rr < R; ++rr) {
-            const size_t base = (((size_t)split * R + rr) * 4) * npts + p0;
-            pp[base / 2] = dead ? nan2 : u1r[rr];
-            pp[(base + (size_t)npts) / 2] = dead ? nan2 : u1i[rr];
-            pp[(base + 2 * (size_t)npts) / 2] = dead ? nan2 : u2r[rr];
-            pp[(base + 3 * (size_t)npts) / 2] = dead ? nan2 : u2i[rr];
+            for (int e = 0; e < 18; ++e) v[e] = first || jt >= nt ? 0.f : o[(size_t)e * nt];
+            for (int g = 0; g < ngrp; ++g) {
+                const int th = g * block_tris + jj;
+#pragma unroll
+                for (int f = 0; f < 4; ++f) {
+                    float4 *a = acc4 + ((size_t)r * 4 + f) * FAR_THREADS + th;
+                    const float4 w = *a;
+                    v[4 * f] += w.x;
+                    v[4 * f + 1] += w.y;
+                    v[4 * f + 2] += w.z;
+                    v[4 * f + 3] += w.w;
+                    *a = make_float4(0.f, 0.f, 0.f, 0.f);
+                }
+                float2 *a = acc2 + (size_t)r * FAR_THREADS + th;
+                v[16] += a->x;
+                v[17] += a->y;
+                *a = make_float2(0.f, 0.f);
+            }
+            if (jt < nt)
+#pragma unroll
+                for (int e = 0; e < 18; ++e) o[(size_t)e * nt] = v[e];
         }
-        if (ntiles == 0)  // empty split: zero curl sums
-            for (int rr = sub; rr < R; rr += 3)
-                for (int d = 0; d < 6; ++d) partA[(((size_t)split * R + rr) * 6 + d) * nt + tau] = 0.f;
+        __syncthreads();
     }
+    if (s_begin >= s_end)  // empty split: zero sums
+        for (int i = threadIdx.x; i < R * 18 * block_tris; i += FAR_THREADS) {
+            const int k = i / block_tris, jt = blockIdx.x * block_tris + i - k * block_tris;
+            if (jt < nt) out[(size_t)k * nt + jt] = 0.f;
+        }
 }
+#undef F3
 
 }  // namespace
 
@@ -1277,7 +1196,7 @@ int far_setup_geometry(osrc_problem *pb, cudaStream_t st) {
     int dev = m->ctx->device, sms = 0;
     OSRC_CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     pb->far_tris = nt < FAR_TRIS32_NT ? 32 : nt < FAR_TRIS64_NT ? 64 : FAR_THREADS;
-    const int slots = sms * OSRC_FAR_MIN_BLOCKS;
+    const int slots = sms * OSRC_FAR_MIN_BLOCKS;  // farm_kernel runs on the same grid
     const int bx = (nt + pb->far_tris - 1) / pb->far_tris;
     const int max_ns = std::max(1, std::min(FAR_MAX_NS, nt / FAR_MIN_TPS));
     const int ns0 = std::min(max_ns, std::max(1, (4 * slots + bx - 1) / bx));
@@ -1319,7 +1238,7 @@ static int gather_launch(osrc_problem *pb, int ns, int R, const float *part, con
     const int per = nv <= GATHER_BLOCK_NV ? 1 : nv <= GATHER_WARP_NV ? GATHER_THREADS / 32 : GATHER_THREADS / 8;
     const dim3 grid((nv + per - 1) / per, R);
 #define OSRC_GATHER_LAUNCH(LL, WW)                                                                             \
-    gather_kernel<LL, WW><<<grid, GATHER_THREADS, 0, st>>>(nv, pb->nt, pb->npts, ns, R, m->d_vt_ptr.p, m->d_vt_idx.p, \
+    (partA ? gather_kernel<LL, WW, false> : gather_kernel<LL, WW, true>)<<<grid, GATHER_THREADS, 0, st>>>(nv, pb->nt, pb->npts, ns, R, m->d_vt_ptr.p, m->d_vt_idx.p, \
                                                        pb->d_tgeo.p, part, partA, use_far, pb->d_nr_ptr.p,       \
                                                        pb->d_nr_col.p, pb->d_nr_val.p, use_near, x, y)
     if (nv <= GATHER_BLOCK_NV) OSRC_GATHER_LAUNCH(32, 4);
@@ -1396,27 +1315,17 @@ int far_apply(osrc_problem *pb, const double2 *x, double2 *y, int part, cudaStre
 
 // ---------------------------------------------------------------------------
 // multi-right-hand-side apply: y_r = B_far x_r (+ near) for r < nrhs, in
-// launches of up to FARM_MAX_R right-hand sides (chunks of 8, then 4, 2;
-// a last single vector takes the one-right-hand-side kernel)
+// launches of up to FARM_MAX_R right-hand sides (a last single vector takes
+// the one-right-hand-side kernel)
 // ---------------------------------------------------------------------------
-template <int R, bool C>
-static int farm_setup_kernel_attr(size_t smem) {
-    OSRC_CK(cudaFuncSetAttribute(farm_kernel<R, C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    return OSRC_OK;
-}
-
 static PerDeviceOnce g_farm_once;
 
-static int farm_prepare(osrc_problem *pb, int rmax, cudaStream_t st) {
+static int farm_prepare(osrc_problem *pb, cudaStream_t st) {
     OSRC_TRY(per_device_once(g_farm_once, [](int) {
-        int s = OSRC_OK;
-        if (!s) s = farm_setup_kernel_attr<2, false>(farm_smem_bytes(2, false));
-        if (!s) s = farm_setup_kernel_attr<4, false>(farm_smem_bytes(4, false));
-        if (!s) s = farm_setup_kernel_attr<8, false>(farm_smem_bytes(8, false));
-        if (!s) s = farm_setup_kernel_attr<2, true>(farm_smem_bytes(2, true));
-        if (!s) s = farm_setup_kernel_attr<4, true>(farm_smem_bytes(4, true));
-        if (!s) s = farm_setup_kernel_attr<8, true>(farm_smem_bytes(8, true));
-        return s;
+        const int smem = (int)farm_smem_bytes(FARM_MAX_R);
+        OSRC_CK(cudaFuncSetAttribute(farm_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+        OSRC_CK(cudaFuncSetAttribute(farm_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+        return OSRC_OK;
     }));
     osrc_ctx *ctx = pb->mesh->ctx;
     const int nt = pb->nt, npts = pb->npts;
@@ -1427,46 +1336,9 @@ static int farm_prepare(osrc_problem *pb, int rmax, cudaStream_t st) {
         pb->launches++;
         OSRC_CK(cudaGetLastError());
     }
-    if (pb->farm_cap < rmax) {
-        int dev = ctx->device, sms = 0, per_sm = 0;
-        OSRC_CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-        const size_t sm8 = farm_smem_bytes(8, pb->far_reduce);
-        if (pb->far_reduce)
-            OSRC_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, farm_kernel<8, true>, FARM_THREADS, sm8));
-        else
-            OSRC_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, farm_kernel<8, false>, FARM_THREADS, sm8));
-        if (per_sm < 1) per_sm = 1;
-        // source splits: at least four blocks per resident slot, and among
-        // the counts up to twice that, the one whose last wave is fullest
-        const int bx = (nt + FARM_TRIS - 1) / FARM_TRIS;
-        const int slots = sms * per_sm;
-        const int max_ns = std::max(1, (nt + 4 * FARM_TS - 1) / (4 * FARM_TS));
-        int ns0 = std::min(max_ns, std::max(1, (4 * slots + bx - 1) / bx));
-        int ns = ns0;
-        double best = -1.0;
-        for (int cand = ns0; cand <= std::min(max_ns, 2 * ns0); ++cand) {
-            const long long blocks = (long long)bx * cand;
-            const long long waves = (blocks + slots - 1) / slots;
-            const double eff = (double)blocks / (double)(waves * slots);
-            if (eff > best + 1e-9) {
-                best = eff;
-                ns = cand;
-            }
-        }
-        pb->farm_ns = ns;
-        pb->d_sD.release();
-        pb->d_sCm.release();
-        pb->d_partm.release();
-        pb->d_partA.release();
-        OSRC_TRY(pb->d_sD.alloc(ctx, 12 * (size_t)nt * FARM_MAX_R));
-        OSRC_TRY(pb->d_sCm.alloc(ctx, 3 * (size_t)nt * FARM_MAX_R));
-        OSRC_TRY(pb->d_partm.alloc(ctx, (size_t)ns * FARM_MAX_R * 4 * npts));
-        OSRC_TRY(pb->d_partA.alloc(ctx, (size_t)ns * FARM_MAX_R * 6 * nt));
-        if (!pb->d_farm_err.p) {
-            OSRC_TRY(pb->d_farm_err.alloc(ctx, 1));
-            OSRC_CK(cudaMemsetAsync(pb->d_farm_err.p, 0, sizeof(int), st));
-        }
-        pb->farm_cap = FARM_MAX_R;
+    if (!pb->d_partm.p) {
+        OSRC_TRY(pb->d_sD.alloc(ctx, 5 * (size_t)nt * FARM_MAX_R));
+        OSRC_TRY(pb->d_partm.alloc(ctx, (size_t)pb->nsplit * FARM_MAX_R * 18 * nt));
     }
     return OSRC_OK;
 }
@@ -1474,7 +1346,7 @@ static int farm_prepare(osrc_problem *pb, int rmax, cudaStream_t st) {
 static int farm_launch(osrc_problem *pb, const double2 *const *xs, double2 *const *ys, int R, int part,
                        cudaStream_t st) {
     osrc_mesh *m = pb->mesh;
-    const int nt = pb->nt, nv = pb->nv, npts = pb->npts;
+    const int nt = pb->nt, nv = pb->nv;
     const int use_far = (part & OSRC_PART_FAR) ? 1 : 0;
     const int use_near = (part & OSRC_PART_NEAR) ? 1 : 0;
     VecPtrs xp{};
@@ -1483,10 +1355,10 @@ static int farm_launch(osrc_problem *pb, const double2 *const *xs, double2 *cons
         xp.p[r] = xs[r];
         yp.p[r] = ys[r];
     }
-    const int ns = pb->farm_ns;
+    const int ns = pb->nsplit;
     if (use_far) {
         farm_prep_kernel<<<dim3((nt + 127) / 128, R), 128, 0, st>>>(xp, R, nv, nt, m->d_tris.p, pb->d_tgeo.p,
-                                                                   pb->d_sD.p, pb->d_sCm.p);
+                                                                   pb->d_sD.p);
         pb->launches++;
         const double k0 = pb->p.k_ext, k1 = pb->p.k_int, rho = pb->p.rho_ratio;
         const double inv2pi = 0.15915494309189533577;
@@ -1504,26 +1376,18 @@ static int farm_launch(osrc_problem *pb, const double2 *const *xs, double2 *cons
         const float q0h = (float)q0, q1h = (float)q1;
         const float4 kff = make_float4(q0h, (float)(q0 - (double)q0h), q1h, (float)(q1 - (double)q1h));
         const int tps = (nt + ns - 1) / ns;
-        dim3 grid((nt + FARM_TRIS - 1) / FARM_TRIS, ns);
+        dim3 grid((nt + pb->far_tris - 1) / pb->far_tris, ns);
         const float4 *pts = pb->far_reduce ? pb->d_poff.p : pb->d_pt.p;
-        const size_t smem = farm_smem_bytes(R, pb->far_reduce);
+        const size_t smem = farm_smem_bytes(R);
         if (pb->prof_on) {
             OSRC_TRY(far_prof_collect(pb));
             OSRC_CK(cudaEventRecord(pb->prof_ev[0], st));
         }
-#define OSRC_FARM_LAUNCH(RR, C)                                                                          \
-    farm_kernel<RR, C><<<grid, FARM_THREADS, smem, st>>>(pts, pb->d_cen.p, pb->d_tn.p, pb->d_tv.p, pb->d_sG.p, \
-                                                         pb->d_sD.p, pb->d_sCm.p, nt, npts, tps, c, kff,    \
-                                                         pb->d_partm.p, pb->d_partA.p, pb->d_farm_err.p)
-        if (pb->far_reduce) {
-            if (R == 8) OSRC_FARM_LAUNCH(8, true);
-            else if (R == 4) OSRC_FARM_LAUNCH(4, true);
-            else OSRC_FARM_LAUNCH(2, true);
-        } else {
-            if (R == 8) OSRC_FARM_LAUNCH(8, false);
-            else if (R == 4) OSRC_FARM_LAUNCH(4, false);
-            else OSRC_FARM_LAUNCH(2, false);
-        }
+#define OSRC_FARM_LAUNCH(C)                                                                                    \
+    farm_kernel<C><<<grid, FAR_THREADS, smem, st>>>(pts, pb->d_cen.p, pb->d_tn.p, pb->d_tv.p, pb->d_sG.p,      \
+                                                    pb->d_sD.p, R, nt, tps, pb->far_tris, c, kff, pb->d_partm.p)
+        if (pb->far_reduce) OSRC_FARM_LAUNCH(true);
+        else OSRC_FARM_LAUNCH(false);
 #undef OSRC_FARM_LAUNCH
         pb->launches++;
         OSRC_CK(cudaGetLastError());
@@ -1533,22 +1397,7 @@ static int farm_launch(osrc_problem *pb, const double2 *const *xs, double2 *cons
             pb->prof_rhs_pending = R;
         }
     }
-    return gather_launch(pb, ns, R, pb->d_partm.p, pb->d_partA.p, use_far, use_near, xp, yp, st);
-}
-
-// OSRC_TIMEOUT if a several-right-hand-side far kernel gave up a bounded
-// wait since the last check (the flag is cleared); synchronises the stream
-int far_multi_check(osrc_problem *pb, cudaStream_t st) {
-    if (!pb->d_farm_err.p) return OSRC_OK;
-    int h = 0;
-    OSRC_CK(cudaMemcpyAsync(&h, pb->d_farm_err.p, sizeof(int), cudaMemcpyDeviceToHost, st));
-    OSRC_CK(cudaStreamSynchronize(st));
-    if (h) {
-        OSRC_CK(cudaMemsetAsync(pb->d_farm_err.p, 0, sizeof(int), st));
-        osrc_set_error("far kernel: a bounded wait for a staged source tile gave up");
-        return OSRC_TIMEOUT;
-    }
-    return OSRC_OK;
+    return gather_launch(pb, ns, R, pb->d_partm.p, nullptr, use_far, use_near, xp, yp, st);
 }
 
 bool far_multi_supported(const osrc_problem *pb) {
@@ -1562,11 +1411,11 @@ int far_apply_multi(osrc_problem *pb, const double2 *const *xs, double2 *const *
         for (int r = 0; r < nrhs; ++r) OSRC_TRY(far_apply(pb, xs[r], ys[r], part, st));
         return OSRC_OK;
     }
-    OSRC_TRY(farm_prepare(pb, FARM_MAX_R, st));
+    OSRC_TRY(farm_prepare(pb, st));
     int r0 = 0;
     while (r0 < nrhs) {
         const int left = nrhs - r0;
-        const int R = left >= 8 ? 8 : left >= 4 ? 4 : left >= 2 ? 2 : 1;
+        const int R = std::min(left, FARM_MAX_R);
         if (R == 1) OSRC_TRY(far_apply(pb, xs[r0], ys[r0], part, st));
         else OSRC_TRY(farm_launch(pb, xs + r0, ys + r0, R, part, st));
         r0 += R;

@@ -1165,7 +1165,6 @@ static int gmres_solve_lockstep(osrc_problem *pb, const void *b, void *x, int nr
         std::vector<int> it, fin;
         for (;;) {
             OSRC_CK(cudaStreamSynchronize(st));
-            OSRC_TRY(far_multi_check(pb, st));
             if (pb->cancel && pb->cancel->load()) {
                 osrc_set_error("lockstep GMRES cancelled");
                 return OSRC_TIMEOUT;

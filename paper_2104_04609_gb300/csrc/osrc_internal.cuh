@@ -191,16 +191,12 @@ struct osrc_problem {
     DBuf<float> d_partA1;     // [nsplit][6][nt] curl-term partial sums per test triangle
     int nsplit = 1, far_tris = 128;  // far kernel: source splits, test triangles per block
     // ---- far field, several right-hand sides per launch (k_far.cu farm_*) ----
-    DBuf<float4> d_sG;        // [6nt][2] static source geometry (coordinates, rule weight)
-    DBuf<float4> d_sD;        // [nt][6][R][2] densities of R right-hand sides
-    DBuf<float2> d_sCm;       // [nt][R][3] curl sources
-    DBuf<float> d_partm;      // [ns][R][4][6nt] u1, u2 partial sums
-    DBuf<float> d_partA;      // [ns][R][6][nt] curl-term partial sums per test triangle
-    DBuf<int> d_farm_err;     // set when the kernel gave up a bounded wait
+    DBuf<float4> d_sG;        // [6nt][2] static source geometry (coordinates)
+    DBuf<float4> d_sD;        // [nt][R][5] corner densities and curl sources of R right-hand sides
+    DBuf<float> d_partm;      // [ns][R][18][nt] u1, u2 partial sums per corner, curl-term sums
     // when set and true, a lockstep GMRES on this problem stops at its next
     // iteration with OSRC_TIMEOUT (the serving loop's shutdown)
     const std::atomic<bool> *cancel = nullptr;
-    int farm_ns = 1, farm_cap = 0;
     bool far_reduce = false;  // centred far kernel with float-float phases (large k r)
     // ---- FP64 per-triangle geometry: area, normal, curls of the hat functions
     DBuf<double> d_tgeo;      // [nt][16]
@@ -276,7 +272,6 @@ int far_apply(osrc_problem *pb, const double2 *x, double2 *y, int part, cudaStre
 int far_apply_multi(osrc_problem *pb, const double2 *const *xs, double2 *const *ys, int nrhs, int part,
                     cudaStream_t st);
 bool far_multi_supported(const osrc_problem *pb);
-int far_multi_check(osrc_problem *pb, cudaStream_t st);
 
 // near field (k_near.cu)
 int near_build(osrc_problem *pb, const std::vector<NearPair> &pairs,

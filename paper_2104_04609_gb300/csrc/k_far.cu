@@ -5,12 +5,15 @@
 // Structure of one apply y = B_far x:
 //   1. far_prep_kernel   (per source rule point)  densities at the 6 source
 //      points and the surface-curl vector of the phi density, FP32;
-//   2. far_kernel        (per test triangle)       N-body sum over all source
-//      points staged through shared memory in tiles of triangles; both
+//   2. below SYM_MIN_NT triangles far_kernel (per test triangle), N-body sum
+//      over all source points staged through shared memory in tiles of triangles; both
 //      wavenumbers are evaluated from one distance; the source range is split
 //      over gridDim.y so that the grid fills every SM; partial sums per test
 //      point (u1, u2) and per test triangle (curl term) go to d_part, d_partA
-//      (no atomics);
+//      (no atomics); from SYM_MIN_NT on sym_kernel, which evaluates each pair of
+//      triangles once, as element matrices, for both directions, and takes
+//      several right-hand sides (farm_kernel: the same one-sided, for several
+//      right-hand sides on small meshes and more than SYM_MAX_R);
 //   3. gather_kernel     (a group of lanes per vertex)  sums the partials of
 //      the test points of the incident triangles with the test weights (FP64)
 //      and adds the near-field CSR product (touching pairs, Sauter-Schwab
@@ -68,6 +71,17 @@ constexpr int FAR_MIN_TPS = 16;  // fewest source triangles per split
 constexpr int FAR_TRIS32_NT = 2048;
 constexpr int FAR_TRIS64_NT = 4096;
 constexpr int FAR_MAX_NS = 64;   // most source splits
+// sym_kernel from this many triangles on (far_kernel / sym_kernel at 796
+// triangles 73 / 97 us, 1280: 144 / 145, 2048: 299 / 276, 2996: 618 / 506, 3996:
+// 1062 / 940, 20480: 25.9 / 17.3 ms; its work comes in tiles of 128 x 32
+// triangles, too few of them for small meshes)
+constexpr int SYM_MIN_NT = 2048;
+constexpr int SYM_MAX_SLOTS = 104;  // most partial sums of an apply (R = 1): 104 x 18 floats a triangle
+                                    // (70 or 200 measure the same within 1 %)
+// right-hand sides of a sym_kernel launch: what two blocks per SM have shared
+// memory for (8 as 5 + 3 would take 55 ms at 10242 vertices, farm_kernel 48.8)
+constexpr int SYM_MAX_R = 5;
+constexpr int SYM_MULTI_SLOTS = 96; // partial sums, times right-hand sides, of several-right-hand-side launches
 // lanes of the gather per vertex: a block up to GATHER_BLOCK_NV vertices, a
 // warp up to GATHER_WARP_NV, then 8 (150 vertices: block 38 us an apply, warp
 // 41; 642: warp 10.28 ms a solve, block 10.38, 8 lanes 10.60; 2568: 8 lanes
@@ -377,7 +391,7 @@ __device__ __forceinline__ FarVals far_vals(const f2 (&X)[3], const f2 (&Y)[3], 
     Diff2 d[3];
     F3 d[p] = far_diff<CENTRED>(X[p], Y[p], Z[p], P0, P1, cp);
     v.dnxn = CENTRED ? dup2(-fmaf(P0.x, n4.x, fmaf(P0.z, n4.y, fmaf(P1.x, n4.z, pdn))))
-                     : dup2(-fmaf(d[0].dz.x, n4.z, fmaf(d[0].dy.x, n4.y, fmaf(d[0].dx.x, n4.x, -pdn))));
+                     : dup2(-fmaf(d[0].dz.x, n4.z, fmaf(d[0].dy.x, n4.y, fmaf(d[0].dx.x, n4.x, pdn))));
     f2 r2[3], ri[3], r[3], s0[3], c0[3], s1[3], c1[3];
     F3 r2[p] = mul2(d[p].dx, d[p].dx);
     F3 r2[p] = fma2(d[p].dy, d[p].dy, r2[p]);
@@ -512,10 +526,9 @@ __device__ __forceinline__ void far_tri(const f2 (&X)[3], const f2 (&Y)[3], cons
 // and source points by plain adds, weighted per class and multiplied into c_s
 // once per triangle pair (10 cycles), the source
 // loads from shared memory (a third), and the centroid phases of the centred
-// variant (a third).  An apply at 10242 vertices: 25.9 ms (29.1 where a
-// thread held one pair of points), 20000 vertices centred 124 ms (147), four
-// objects of 642 vertices 2.19 ms (3.27).  255 registers and two blocks per
-// SM measured 1 to 4 % better than 168 and three.
+// variant (a third).  642 vertices: 0.144 ms an apply, 1.67 ms at 2562 (0.16 and
+// 1.85 where a thread held one pair of points; sym_kernel 0.145 and 1.31).  255
+// registers and two blocks per SM measured 1 to 4 % better than 168 and three.
 // Small meshes give a block 32 or 64 test triangles and split each source
 // tile between its warps, whose sums are added in shared memory: more warps
 // in flight for the same number of partial sums (see far_setup_geometry).
@@ -889,7 +902,7 @@ gather_kernel(int nv, int nt, int npts, int ns, int R, const int *__restrict__ v
 //
 // Source data (the points duplicated into pairs for the packed lanes):
 //   sG [6nt][2]   (-y.x, -y.x, -y.y, -y.y), (-y.z, -y.z, 0, 0)   (static)
-//   sD [nt][R][5] corner a: |s| (psi_a, phi_a); then c_s (three complex, 0, 0)
+//   sD [R][5][nt] corner a: |s| (psi_a, phi_a); then c_s (three complex, 0, 0)
 // Output (no atomics; gridDim.y splits the source range):
 //   part [ns][R][18][nt]  u1 (re, im), u2 (re, im) of corners 0, 1, 2; then
 //                         A = sum_s W c_s (x, y, z; re, im)
@@ -922,16 +935,150 @@ __global__ void farm_prep_kernel(VecPtrs x, int R, int nv, int nt, const int *__
     const double2 *xr = x.p[r];
     const double *g = tgeo + 16 * (size_t)t;
     const double area = g[0];
-    float4 *d = sD + 5 * ((size_t)t * R + r);
+    float4 *d = sD + 5 * (size_t)r * nt + t;
     double2 cv[3] = {cd(0, 0), cd(0, 0), cd(0, 0)};
     for (int a = 0; a < 3; ++a) {
         const int v = tris[3 * t + a];
         const double2 ps = cscale(xr[v], area), ph = cscale(xr[nv + v], area);
-        d[a] = make_float4((float)ps.x, (float)ps.y, (float)ph.x, (float)ph.y);
+        d[a * (size_t)nt] = make_float4((float)ps.x, (float)ps.y, (float)ph.x, (float)ph.y);
         for (int j = 0; j < 3; ++j) cv[j] = cadd(cv[j], cscale(ph, g[4 + 3 * a + j]));
     }
-    d[3] = make_float4((float)cv[0].x, (float)cv[0].y, (float)cv[1].x, (float)cv[1].y);
-    d[4] = make_float4((float)cv[2].x, (float)cv[2].y, 0.f, 0.f);
+    d[3 * (size_t)nt] = make_float4((float)cv[0].x, (float)cv[0].y, (float)cv[1].x, (float)cv[1].y);
+    d[4 * (size_t)nt] = make_float4((float)cv[2].x, (float)cv[2].y, 0.f, 0.f);
+}
+
+// The matrices of one triangle pair, [re, im of S, N, T, K][b][a], and W.
+struct ElemMat {
+    float E[8][3][3];
+    float wr, wi;
+};
+
+// mns = (-n_y, .), my0 = -y_0, dn: -(x - y).n_y = (X - y_0).mns + dn (centred:
+// X.mns + dn); load(q, P0, P1) gives source point q as duplicated pairs; m1, k1i, dk1i as in far_vals (MULTI, ABSORB).
+template <bool CENTRED, bool MULTI, bool ABSORB, typename L>
+__device__ __forceinline__ void elem_matrices(const f2 (&X)[3], const f2 (&Y)[3], const f2 (&Z)[3], const float4 &n4,
+                                              float pdn, const float4 &mns, const float4 &my0, float dn, const L &load,
+                                              const FarConst2 &c, const CenterPair &cp, f2 m1, f2 k1i, float dk1i,
+                                              ElemMat &M) {
+    // the rule's classes: weights times beta, and times alpha - beta
+    constexpr float WB1 = (float)(kQw1 * kQa1), WB2 = (float)(kQw2 * kQa2);
+    constexpr float WG1 = (float)(kQw1 * (1.0 - 3.0 * kQa1)), WG2 = (float)(kQw2 * (1.0 - 3.0 * kQa2));
+    const f2 wb = make_float2(WB1, WB2), wg = make_float2(WG1, WG2);
+    f2 kb[3], kg[3];  // the test weights times -(x - y).n_y
+    F3 {
+        const f2 dx = CENTRED ? X[p] : add2(X[p], dup2(my0.x)), dy = CENTRED ? Y[p] : add2(Y[p], dup2(my0.y)),
+                 dz = CENTRED ? Z[p] : add2(Z[p], dup2(my0.z));
+        const f2 xnyn = fma2(dz, dup2(mns.z), fma2(dy, dup2(mns.y), fma2(dx, dup2(mns.x), dup2(dn))));
+        kb[p] = mul2(wb, xnyn);
+        kg[p] = mul2(wg, xnyn);
+    }
+    // first M0, M1 (G0, G1), T, K; class 0 stores, class 1 adds; bs: the beta parts
+    float(&E)[8][3][3] = M.E;
+    float bs[8][3];
+#pragma unroll
+    for (int q = 0; q < 6; ++q) {
+        float4 P0, P1;
+        load(q, P0, P1);
+        FarVals v = far_vals<CENTRED, MULTI, ABSORB>(X, Y, Z, n4, pdn, P0, P1, c, cp, m1, k1i);
+        F3 v.hp[p] = mul2(v.hp[p], v.ri2[p]);
+        F3 v.hq[p] = mul2(v.hq[p], v.ri2[p]);
+        const float wgq = q < 3 ? WG1 : WG2, wbq = q < 3 ? WB1 : WB2;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const f2(&u)[3] = i == 0 ? v.c0r : i == 1 ? v.s0r : i == 2 ? v.c1r : i == 3 ? v.s1r : (i & 1) ? v.hq : v.hp;
+            const f2 sum = i < 6 ? mul2(wb, add2(add2(u[0], u[1]), u[2]))
+                                 : fma2(kb[2], u[2], fma2(kb[1], u[1], mul2(kb[0], u[0])));
+#pragma unroll
+            for (int b = 0; b < 3; ++b) {
+                const f2 tb = fma2(i < 6 ? wg : kg[b], u[b], sum);
+                float t = tb.x + tb.y;
+                if (i == 4 || i == 5) t *= v.dnxn.x;  // T: (y - x).n_x is the source point's alone
+                E[i][b][q % 3] = q < 3 ? wgq * t : fmaf(wgq, t, E[i][b][q % 3]);
+                bs[i][b] = q == 0 ? wbq * t : fmaf(wbq, t, bs[i][b]);
+            }
+        }
+    }
+    float w0 = 0.f, w1 = 0.f, w2 = 0.f, w3 = 0.f;
+#pragma unroll
+    for (int b = 0; b < 3; ++b)
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+#pragma unroll
+            for (int i = 0; i < 8; ++i) E[i][b][a] += bs[i][b];
+            w0 += E[0][b][a];
+            w1 += E[1][b][a];
+            w2 += E[2][b][a];
+            w3 += E[3][b][a];
+        }
+    M.wr = fmaf(c.irho.x, w2, w0);
+    M.wi = fmaf(c.irho.x, w3, w1);
+    const float nn = (n4.x * mns.x + n4.y * mns.y + n4.z * mns.z) * c.dk0.x;  // -(n_x.n_y) dks
+    // M0, M1 -> S and N
+#pragma unroll
+    for (int b = 0; b < 3; ++b)
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            const float g0 = E[0][b][a], g1 = E[1][b][a], g2 = E[2][b][a], g3 = E[3][b][a];
+            E[0][b][a] = fmaf(c.rho.x, g2, g0);
+            E[1][b][a] = fmaf(c.rho.x, g3, g1);
+            float nr = fmaf(c.dk1.x, g2, g0), ni = fmaf(c.dk1.x, g3, g1);
+            if (MULTI && ABSORB) {
+                nr = fmaf(-dk1i, g3, nr);
+                ni = fmaf(dk1i, g2, ni);
+            }
+            E[2][b][a] = nn * nr;
+            E[3][b][a] = nn * ni;
+        }
+}
+
+// u_b (u1 re, im, u2 re, im) += the matrices on the corner densities
+// d[a stride] (psi, phi).  REV: the pair seen from the source triangle.  S and N are symmetric;
+// the normals change places and x - y its sign, so K becomes -T^T and T -K^T.
+template <bool REV>
+__device__ __forceinline__ void elem_apply(const ElemMat &M, const float4 *d, size_t stride, float4 (&u)[3]) {
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        const float4 da = d[a * stride];
+#pragma unroll
+        for (int b = 0; b < 3; ++b) {
+            const int i = REV ? a : b, j = REV ? b : a;
+            const float sr = M.E[0][i][j], si = M.E[1][i][j], nr = M.E[2][i][j], ni = M.E[3][i][j];
+            const float tr = REV ? -M.E[6][i][j] : M.E[4][i][j], ti = REV ? -M.E[7][i][j] : M.E[5][i][j];
+            const float kr = REV ? -M.E[4][i][j] : M.E[6][i][j], ki = REV ? -M.E[5][i][j] : M.E[7][i][j];
+            u[b].x = fmaf(sr, da.x, fmaf(-si, da.y, fmaf(kr, da.z, fmaf(-ki, da.w, u[b].x))));
+            u[b].y = fmaf(sr, da.y, fmaf(si, da.x, fmaf(kr, da.w, fmaf(ki, da.z, u[b].y))));
+            u[b].z = fmaf(tr, da.x, fmaf(-ti, da.y, fmaf(nr, da.z, fmaf(-ni, da.w, u[b].z))));
+            u[b].w = fmaf(tr, da.y, fmaf(ti, da.x, fmaf(nr, da.w, fmaf(ni, da.z, u[b].w))));
+        }
+    }
+}
+
+// A += W c; with COMP the sums' rounding errors are carried along in *e4, *e2
+template <bool COMP>
+__device__ __forceinline__ void elem_curl(const ElemMat &M, float4 C0, float4 C1, float4 *a4, float2 *a2, float4 *e4, float2 *e2) {
+    float4 A = *a4;
+    float2 Z = *a2;
+    if (COMP) {
+        float4 E = *e4;
+        float2 F = *e2;
+        comp_add_fast(A.x, E.x, fmaf(M.wr, C0.x, -M.wi * C0.y));
+        comp_add_fast(A.y, E.y, fmaf(M.wr, C0.y, M.wi * C0.x));
+        comp_add_fast(A.z, E.z, fmaf(M.wr, C0.z, -M.wi * C0.w));
+        comp_add_fast(A.w, E.w, fmaf(M.wr, C0.w, M.wi * C0.z));
+        comp_add_fast(Z.x, F.x, fmaf(M.wr, C1.x, -M.wi * C1.y));
+        comp_add_fast(Z.y, F.y, fmaf(M.wr, C1.y, M.wi * C1.x));
+        *e4 = E;
+        *e2 = F;
+    } else {
+        A.x = fmaf(M.wr, C0.x, fmaf(-M.wi, C0.y, A.x));
+        A.y = fmaf(M.wr, C0.y, fmaf(M.wi, C0.x, A.y));
+        A.z = fmaf(M.wr, C0.z, fmaf(-M.wi, C0.w, A.z));
+        A.w = fmaf(M.wr, C0.w, fmaf(M.wi, C0.z, A.w));
+        Z.x = fmaf(M.wr, C1.x, fmaf(-M.wi, C1.y, Z.x));
+        Z.y = fmaf(M.wr, C1.y, fmaf(M.wi, C1.x, Z.y));
+    }
+    *a4 = A;
+    *a2 = Z;
 }
 
 // One thread per test triangle, on far_kernel's grid (blocks of block_tris test
@@ -943,10 +1090,9 @@ __global__ void farm_prep_kernel(VecPtrs x, int R, int nv, int nt, const int *__
 // short sums keep their rounding errors (1.2 to 2 times less than without on
 // 3000 to 5000 vertices) for 2 % of the time, the old values of an entry's 18
 // being loaded together.
-// Bound by the FP32 pipe: an apply at 10242 vertices is 26.9 ms of kernel
-// values and matrices and 2.7 ms a right-hand side (R 2: 32.5 ms, 4: 38.0,
-// 8: 48.8), where point-by-point sums took 24 + 9.9 (43.6, 65.1, 102.7).  R = 1
-// would take 29.6 against far_kernel's 25.9.  Tensor cores do not help: TF32
+// Bound by the FP32 pipe: an apply at 10242 vertices is 27.1 ms of kernel
+// values and matrices and 2.7 ms a right-hand side (R 8: 48.8 ms), where
+// point-by-point sums took 24 + 9.9 (102.7).  Tensor cores do not help: TF32
 // pieces with the kernel values as an operand took 64.7 ms at R 2 and 80.8 at
 // 8, mma.sync and packed FMA not overlapping.
 template <bool CENTRED>
@@ -958,7 +1104,7 @@ farm_kernel(const float4 *__restrict__ pt, const float4 *__restrict__ cen, const
     float4 *acc4 = reinterpret_cast<float4 *>(farm_smem);                            // [R][4][threads]
     float2 *acc2 = reinterpret_cast<float2 *>(acc4 + (size_t)R * 4 * FAR_THREADS);   // [R][threads]
     float4 *shG = reinterpret_cast<float4 *>(acc2 + (size_t)R * FAR_THREADS);        // [TS][6][2]
-    float4 *shD = shG + FARM_TS * 12;                                                // [TS][R][5]
+    float4 *shD = shG + FARM_TS * 12;                                                // [R][5][TS]
     float4 *shN = shD + FARM_TS * 5 * R;                                             // [TS] (-n, n.P0)
     int4 *shV = reinterpret_cast<int4 *>(shN + FARM_TS);                             // [TS]
     float4 *shCen = reinterpret_cast<float4 *>(shV + FARM_TS);                       // [TS][2] (centred)
@@ -979,10 +1125,6 @@ farm_kernel(const float4 *__restrict__ pt, const float4 *__restrict__ cen, const
     }
     const float4 n4 = tn[tau];
     const int4 vt = tv[tau];
-    // the rule's classes: weights times beta, and times alpha - beta
-    constexpr float WB1 = (float)(kQw1 * kQa1), WB2 = (float)(kQw2 * kQa2);
-    constexpr float WG1 = (float)(kQw1 * (1.0 - 3.0 * kQa1)), WG2 = (float)(kQw2 * (1.0 - 3.0 * kQa2));
-    const f2 wb = make_float2(WB1, WB2), wg = make_float2(WG1, WG2);
     float4 cth = make_float4(0.f, 0.f, 0.f, 0.f), ctl = cth;
     if (CENTRED) {
         cth = cen[2 * tau];
@@ -994,7 +1136,11 @@ farm_kernel(const float4 *__restrict__ pt, const float4 *__restrict__ cen, const
     for (int t0 = s_begin; t0 < s_end; t0 += FARM_TS) {
         const int cnt = min(FARM_TS, s_end - t0);
         for (int i = threadIdx.x; i < cnt * 12; i += FAR_THREADS) shG[i] = sG[12 * (size_t)t0 + i];
-        for (int i = threadIdx.x; i < cnt * 5 * R; i += FAR_THREADS) shD[i] = sD[5 * (size_t)R * t0 + i];
+#pragma unroll 1  // an unrolled copy's addresses would stay in registers the pair loop needs
+        for (int i = threadIdx.x; i < 5 * R * FARM_TS; i += FAR_THREADS) {
+            const int si = i % FARM_TS, k = i / FARM_TS;
+            if (si < cnt) shD[i] = sD[(size_t)k * nt + t0 + si];
+        }
         for (int i = threadIdx.x; i < cnt; i += FAR_THREADS) {
             const float4 ns = tn[t0 + i];
             shN[i] = make_float4(-ns.x, -ns.y, -ns.z, ns.w);
@@ -1013,100 +1159,33 @@ farm_kernel(const float4 *__restrict__ pt, const float4 *__restrict__ cen, const
             CenterPair cp;
             float pdn = __int_as_float(vt.w);
             const float4 mns = shN[s];
-            float dn = mns.w;
+            const float4 g0 = shG[12 * s], g1 = shG[12 * s + 1], my0 = make_float4(g0.x, g0.z, g1.x, 0.f);
+            float dn = __int_as_float(vs.w);  // n_y.(P0 - y_0), see far_geom_kernel
             if (CENTRED) {
                 cp = center_pair(cth, ctl, shCen[2 * s], shCen[2 * s + 1], kff.x, kff.y, kff.z, kff.w);
                 pdn = fmaf(cp.Dx.x, n4.x, fmaf(cp.Dy.x, n4.y, cp.Dz.x * n4.z)) +
                       fmaf(cp.lx, n4.x, fmaf(cp.ly, n4.y, cp.lz * n4.z));
                 dn = cp.Dx.x * mns.x + cp.Dy.x * mns.y + cp.Dz.x * mns.z;
             }
-            f2 kb[3], kg[3];  // the test weights times -(x - y).n_y
-            F3 {
-                const f2 xnyn = fma2(Z[p], dup2(mns.z), fma2(Y[p], dup2(mns.y), fma2(X[p], dup2(mns.x), dup2(dn))));
-                kb[p] = mul2(wb, xnyn);
-                kg[p] = mul2(wg, xnyn);
-            }
-            // E[v][b][a], v = M0, M1, T, K (re, im): class 0 stores, class 1 adds; bs: the beta parts
-            float E[8][3][3], bs[8][3];
-#pragma unroll
-            for (int q = 0; q < 6; ++q) {
-                const float4 P0 = shG[12 * s + 2 * q], P1 = shG[12 * s + 2 * q + 1];
-                FarVals v = far_vals<CENTRED, false, false>(X, Y, Z, n4, pdn, P0, P1, c, cp, dup2(1.f), dup2(0.f));
-                F3 v.hp[p] = mul2(v.hp[p], v.ri2[p]);
-                F3 v.hq[p] = mul2(v.hq[p], v.ri2[p]);
-                const float wgq = q < 3 ? WG1 : WG2, wbq = q < 3 ? WB1 : WB2;
-#pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    const f2(&u)[3] = i == 0 ? v.c0r : i == 1 ? v.s0r : i == 2 ? v.c1r : i == 3 ? v.s1r
-                                      : (i & 1) ? v.hq : v.hp;
-                    const f2 sum = i < 6 ? mul2(wb, add2(add2(u[0], u[1]), u[2]))
-                                         : fma2(kb[2], u[2], fma2(kb[1], u[1], mul2(kb[0], u[0])));
-#pragma unroll
-                    for (int b = 0; b < 3; ++b) {
-                        const f2 tb = fma2(i < 6 ? wg : kg[b], u[b], sum);
-                        float t = tb.x + tb.y;
-                        if (i == 4 || i == 5) t *= v.dnxn.x;  // T: (y - x).n_x is the source point's alone
-                        E[i][b][q % 3] = q < 3 ? wgq * t : fmaf(wgq, t, E[i][b][q % 3]);
-                        bs[i][b] = q == 0 ? wbq * t : fmaf(wbq, t, bs[i][b]);
-                    }
-                }
-            }
-            float w0 = 0.f, w1 = 0.f, w2 = 0.f, w3 = 0.f;
-#pragma unroll
-            for (int b = 0; b < 3; ++b)
-#pragma unroll
-                for (int a = 0; a < 3; ++a) {
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) E[i][b][a] += bs[i][b];
-                    w0 += E[0][b][a];
-                    w1 += E[1][b][a];
-                    w2 += E[2][b][a];
-                    w3 += E[3][b][a];
-                }
-            const float wr = fmaf(c.irho.x, w2, w0), wi = fmaf(c.irho.x, w3, w1);
-            const float nn = (n4.x * mns.x + n4.y * mns.y + n4.z * mns.z) * c.dk0.x;  // -(n_x.n_y) dks
-            // M0, M1 -> S and N
-#pragma unroll
-            for (int b = 0; b < 3; ++b)
-#pragma unroll
-                for (int a = 0; a < 3; ++a) {
-                    const float g0 = E[0][b][a], g1 = E[1][b][a], g2 = E[2][b][a], g3 = E[3][b][a];
-                    E[0][b][a] = fmaf(c.rho.x, g2, g0);
-                    E[1][b][a] = fmaf(c.rho.x, g3, g1);
-                    E[2][b][a] = nn * fmaf(c.dk1.x, g2, g0);
-                    E[3][b][a] = nn * fmaf(c.dk1.x, g3, g1);
-                }
+            ElemMat M;
+            elem_matrices<CENTRED, false, false>(
+                X, Y, Z, n4, pdn, mns, my0, dn, [&](int q, float4 &P0, float4 &P1) {
+                    P0 = shG[12 * s + 2 * q];
+                    P1 = shG[12 * s + 2 * q + 1];
+                },
+                c, cp, dup2(1.f), dup2(0.f), 0.f, M);
 #pragma unroll 1
             for (int r = 0; r < R; ++r) {
-                const float4 *D = shD + 5 * (s * R + r);
+                const float4 *D = shD + 5 * r * FARM_TS + s;
                 float4 *o4 = acc4 + (size_t)r * 4 * FAR_THREADS + threadIdx.x;
                 float4 u[3];
 #pragma unroll
                 for (int b = 0; b < 3; ++b) u[b] = o4[b * FAR_THREADS];
-#pragma unroll
-                for (int a = 0; a < 3; ++a) {
-                    const float4 d = D[a];
-#pragma unroll
-                    for (int b = 0; b < 3; ++b) {
-                        u[b].x = fmaf(E[0][b][a], d.x, fmaf(-E[1][b][a], d.y, fmaf(E[6][b][a], d.z, fmaf(-E[7][b][a], d.w, u[b].x))));
-                        u[b].y = fmaf(E[0][b][a], d.y, fmaf(E[1][b][a], d.x, fmaf(E[6][b][a], d.w, fmaf(E[7][b][a], d.z, u[b].y))));
-                        u[b].z = fmaf(E[4][b][a], d.x, fmaf(-E[5][b][a], d.y, fmaf(E[2][b][a], d.z, fmaf(-E[3][b][a], d.w, u[b].z))));
-                        u[b].w = fmaf(E[4][b][a], d.y, fmaf(E[5][b][a], d.x, fmaf(E[2][b][a], d.w, fmaf(E[3][b][a], d.z, u[b].w))));
-                    }
-                }
+                elem_apply<false>(M, D, FARM_TS, u);
 #pragma unroll
                 for (int b = 0; b < 3; ++b) o4[b * FAR_THREADS] = u[b];
-                const float4 C0 = D[3], C1 = D[4];
-                float4 A = o4[3 * FAR_THREADS];
-                float2 *o2 = acc2 + (size_t)r * FAR_THREADS + threadIdx.x, Az = *o2;
-                A.x = fmaf(wr, C0.x, fmaf(-wi, C0.y, A.x));
-                A.y = fmaf(wr, C0.y, fmaf(wi, C0.x, A.y));
-                A.z = fmaf(wr, C0.z, fmaf(-wi, C0.w, A.z));
-                A.w = fmaf(wr, C0.w, fmaf(wi, C0.z, A.w));
-                Az.x = fmaf(wr, C1.x, fmaf(-wi, C1.y, Az.x));
-                Az.y = fmaf(wr, C1.y, fmaf(wi, C1.x, Az.y));
-                o4[3 * FAR_THREADS] = A;
-                *o2 = Az;
+                elem_curl<false>(M, D[3 * FARM_TS], D[4 * FARM_TS], o4 + 3 * FAR_THREADS,
+                                 acc2 + (size_t)r * FAR_THREADS + threadIdx.x, nullptr, nullptr);
             }
         }
         __syncthreads();
@@ -1148,9 +1227,333 @@ farm_kernel(const float4 *__restrict__ pt, const float4 *__restrict__ cen, const
             if (jt < nt) out[(size_t)k * nt + jt] = 0.f;
         }
 }
+// ---------------------------------------------------------------------------
+// The same with each pair of triangles evaluated once for both directions
+// (elem_apply<true>): the kernel values and matrices, most of the work of few
+// right-hand sides, are halved.  The triangles are cut into N groups of 128; a
+// block takes test group I (a thread per triangle) against groups I + d mod N,
+// d = 0 (its own, every ordered pair, test side only) and d = 1 .. N/2 (for
+// even N the last only from I < N/2), which meets every two groups once.
+//
+// A source group is staged 32 triangles at a time.  At step i lane l of a warp
+// takes source triangle (i + l) mod 32, so the lanes' source-side sums, in
+// shared memory, a set per warp, never meet; after the 32 steps the four
+// warps' sums are added and leave for the slot of d (source side), the test
+// side's for the block's split.  A launch covers nsrc values of d, so no two
+// blocks write one entry; further launches add to it.  Everything is added in
+// a fixed order.
+//   part [ntst + nsrc][R][18][nt]  as farm_kernel's
+// One vector's curl sums carry their rounding errors along (COMP; several
+// vectors' are as accurate as point-by-point sums without).  Bound by the FP32
+// pipe at 8 warps per SM: an apply at 10242 vertices 17.3 ms (far_kernel 25.9),
+// 20000 vertices centred 78.6 (124), four objects of 642 vertices 1.69 (2.19);
+// R = 2: 19.9, 3: 23.0, 4: 28.4, 5: 32.0 (farm_kernel 32.5, 35.3, 38.0, 40.6).
+// ---------------------------------------------------------------------------
+constexpr int SYM_U = 32;  // source triangles per tile (one step each per lane)
+constexpr size_t sym_smem_bytes(int R, bool centred) {
+    return (size_t)R * (2 * 72 * FAR_THREADS + 80 * SYM_U) + (R == 1 ? 2 * 24 * FAR_THREADS : 0) +
+           (size_t)SYM_U * (96 + 16 + 16 + (centred ? 32 : 0) + 16);
+}
+
+template <bool CENTRED, bool MULTI, bool ABSORB, bool COMP>
+__global__ void __launch_bounds__(FAR_THREADS, FARM_MIN_BLOCKS)
+sym_kernel(const float4 *__restrict__ pt, const float4 *__restrict__ cen, const float4 *__restrict__ tn,
+           const int4 *__restrict__ tv, const float4 *__restrict__ sD, int R, int nt, int d_first, int d_count,
+           int units_per_split, int ntst, int accumulate, FarConst2 c0, float4 kff0, const int *__restrict__ tcomp,
+           const FarObj *__restrict__ fobj, float *__restrict__ part) {
+    extern __shared__ __align__(16) unsigned char sym_smem[];
+    float4 *acc4 = reinterpret_cast<float4 *>(sym_smem);           // [R][4][threads] test side
+    float4 *src4 = acc4 + (size_t)R * 4 * FAR_THREADS;             // [R][4][warp][32] source side
+    float2 *acc2 = reinterpret_cast<float2 *>(src4 + (size_t)R * 4 * FAR_THREADS);
+    float2 *src2 = acc2 + (size_t)R * FAR_THREADS;
+    // errors of the curl sums (COMP): [test, source][threads]
+    float4 *err4 = reinterpret_cast<float4 *>(src2 + (size_t)R * FAR_THREADS);
+    float2 *err2 = reinterpret_cast<float2 *>(err4 + (COMP ? 2 * FAR_THREADS : 0));
+    float4 *shP = reinterpret_cast<float4 *>(err2 + (COMP ? 2 * FAR_THREADS : 0));  // [6][32] -y
+    float4 *shD = shP + 6 * SYM_U;                                 // [R][5][32]
+    float4 *shN = shD + (size_t)5 * R * SYM_U;                     // [32] -n
+    int4 *shV = reinterpret_cast<int4 *>(shN + SYM_U);             // [32]
+    int *shComp = reinterpret_cast<int *>(shV + SYM_U);            // [32] (16 bytes each reserved)
+    float4 *shCen = reinterpret_cast<float4 *>(shV + 2 * SYM_U);   // [2][32] (centred)
+
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int N = (nt + FAR_THREADS - 1) / FAR_THREADS, I = blockIdx.x;
+    const int j = I * FAR_THREADS + threadIdx.x;
+    const bool active = j < nt;
+    const int tau = active ? j : 0;
+    f2 X[3], Y[3], Z[3];
+#pragma unroll
+    for (int p = 0; p < 3; ++p) {
+        const float4 xa = pt[6 * tau + p], xb = pt[6 * tau + p + 3];
+        X[p] = make_float2(xa.x, xb.x);
+        Y[p] = make_float2(xa.y, xb.y);
+        Z[p] = make_float2(xa.z, xb.z);
+    }
+    const float4 n4 = tn[tau];
+    const int4 vt = tv[tau];
+    FarConst2 c = c0;
+    float4 kff = kff0;
+    int ct = 0;
+    float sgn = 1.f, dk1i = 0.f;
+    f2 k1i = make_float2(0.f, 0.f);
+    if (MULTI) {
+        ct = tcomp[tau];
+        const FarObj o = fobj[ct];
+        c.k1 = dup2(o.k1);
+        c.nk1 = dup2(o.nk1);
+        c.rho = dup2(o.rho);
+        c.irho = dup2(o.irho);
+        c.dk1 = dup2(o.dk1);
+        kff.z = o.k1h;
+        kff.w = o.k1l;
+        sgn = o.sgn;
+        k1i = dup2(o.k1i);
+        dk1i = o.dk1i;
+    }
+    float4 cth = make_float4(0.f, 0.f, 0.f, 0.f), ctl = cth;
+    if (CENTRED) {
+        cth = cen[2 * tau];
+        ctl = cen[2 * tau + 1];
+    }
+    // both sides' sums: acc4 to err2 are contiguous
+    for (int i = threadIdx.x; i < (R * 36 + (COMP ? 12 : 0)) * FAR_THREADS; i += FAR_THREADS) reinterpret_cast<float *>(acc4)[i] = 0.f;
+
+    float *const tout = part + (size_t)blockIdx.y * R * 18 * nt + j;
+    const int u0 = blockIdx.y * units_per_split, u1 = min(4 * d_count, u0 + units_per_split);
+    bool stored = accumulate != 0, any = false;
+    for (int u = u0; u < u1; ++u) {
+        const int d = d_first + u / 4;
+        if (2 * d == N && I >= d) break;  // the other group of the pair has it
+        const int J = I + d < N ? I + d : I + d - N;
+        const int t0 = J * FAR_THREADS + (u % 4) * SYM_U, cnt = min(SYM_U, nt - t0);
+        if (cnt <= 0) continue;
+        const bool both = d != 0;
+        __syncthreads();
+        for (int i = threadIdx.x; i < 6 * SYM_U; i += FAR_THREADS) {
+            const int si = i / 6, q = i - 6 * si;
+            if (si < cnt) {
+                const float4 y = pt[6 * (size_t)t0 + i];
+                shP[q * SYM_U + si] = make_float4(-y.x, -y.y, -y.z, 0.f);
+            }
+        }
+        for (int i = threadIdx.x; i < 5 * R * SYM_U; i += FAR_THREADS) {
+            const int si = i % SYM_U, k = i / SYM_U;
+            if (si < cnt) shD[i] = sD[(size_t)k * nt + t0 + si];
+        }
+        if (threadIdx.x < cnt) {
+            const float4 ns = tn[t0 + threadIdx.x];
+            shN[threadIdx.x] = make_float4(-ns.x, -ns.y, -ns.z, ns.w);
+            shV[threadIdx.x] = tv[t0 + threadIdx.x];
+            if (MULTI) shComp[threadIdx.x] = tcomp[t0 + threadIdx.x];
+            if (CENTRED) {
+                shCen[threadIdx.x] = cen[2 * (size_t)(t0 + threadIdx.x)];
+                shCen[SYM_U + threadIdx.x] = cen[2 * (size_t)(t0 + threadIdx.x) + 1];
+            }
+        }
+        __syncthreads();
+#pragma unroll 1
+        for (int st = 0; st < SYM_U; ++st) {
+            const int s = (st + lane) & (SYM_U - 1);
+            const int4 vs = shV[s];
+            const bool touch = (vs.x == vt.x) | (vs.x == vt.y) | (vs.x == vt.z) |
+                               (vs.y == vt.x) | (vs.y == vt.y) | (vs.y == vt.z) |
+                               (vs.z == vt.x) | (vs.z == vt.y) | (vs.z == vt.z);
+            if (active && s < cnt && !touch) {
+                CenterPair cp;
+                float pdn = __int_as_float(vt.w);
+                const float4 mns = shN[s];
+                float dn;
+                if (CENTRED) {
+                    cp = center_pair(cth, ctl, shCen[s], shCen[SYM_U + s], kff.x, kff.y, kff.z, kff.w);
+                    pdn = fmaf(cp.Dx.x, n4.x, fmaf(cp.Dy.x, n4.y, cp.Dz.x * n4.z)) +
+                          fmaf(cp.lx, n4.x, fmaf(cp.ly, n4.y, cp.lz * n4.z));
+                    dn = fmaf(cp.Dx.x, mns.x, fmaf(cp.Dy.x, mns.y, cp.Dz.x * mns.z)) +
+                         fmaf(cp.lx, mns.x, fmaf(cp.ly, mns.y, cp.lz * mns.z));
+                } else {
+                    dn = __int_as_float(vs.w);  // n_y.(P0 - y_0), see far_geom_kernel
+                }
+                const f2 m1 = dup2(MULTI ? (shComp[s] != ct ? 0.f : sgn) : 1.f);
+                ElemMat M;
+                elem_matrices<CENTRED, MULTI, ABSORB>(
+                    X, Y, Z, n4, pdn, mns, shP[s], dn, [&](int q, float4 &P0, float4 &P1) {
+                        const float4 y = shP[q * SYM_U + s];
+                        P0 = make_float4(y.x, y.x, y.y, y.y);
+                        P1 = make_float4(y.z, y.z, 0.f, 0.f);
+                    },
+                    c, cp, m1, k1i, dk1i, M);
+#pragma unroll 1
+                for (int r = 0; r < R; ++r) {
+                    float4 v[3];
+                    const float4 *D = shD + 5 * r * SYM_U + s;
+                    float4 *o4 = acc4 + (size_t)r * 4 * FAR_THREADS + threadIdx.x;
+                    float2 *o2 = acc2 + (size_t)r * FAR_THREADS + threadIdx.x;
+#pragma unroll
+                    for (int b = 0; b < 3; ++b) v[b] = o4[b * FAR_THREADS];
+                    elem_apply<false>(M, D, SYM_U, v);
+#pragma unroll
+                    for (int b = 0; b < 3; ++b) o4[b * FAR_THREADS] = v[b];
+                    elem_curl<COMP>(M, D[3 * SYM_U], D[4 * SYM_U], o4 + 3 * FAR_THREADS, o2, err4 + threadIdx.x, err2 + threadIdx.x);
+                    if (both) {
+                        const float4 *T = sD + 5 * (size_t)r * nt + tau;
+                        o4 = src4 + (size_t)r * 4 * FAR_THREADS + warp * 32 + s;
+                        o2 = src2 + (size_t)r * FAR_THREADS + warp * 32 + s;
+#pragma unroll
+                        for (int b = 0; b < 3; ++b) v[b] = o4[b * FAR_THREADS];
+                        elem_apply<true>(M, T, nt, v);
+#pragma unroll
+                        for (int b = 0; b < 3; ++b) o4[b * FAR_THREADS] = v[b];
+                        elem_curl<COMP>(M, T[3 * (size_t)nt], T[4 * (size_t)nt], o4 + 3 * FAR_THREADS, o2,
+                                        err4 + FAR_THREADS + warp * 32 + s, err2 + FAR_THREADS + warp * 32 + s);
+                    }
+                }
+            }
+            __syncwarp();
+        }
+        __syncthreads();
+        // test side: the thread's own sums (the first tile stores, later ones
+        // add; compensated curl sums stay until the last)
+        constexpr int TE = COMP ? 12 : 18;
+        for (int r = 0; r < R; ++r) {
+            float *o = tout + (size_t)r * 18 * nt;
+            float v[TE];
+#pragma unroll
+            for (int e = 0; e < TE; ++e) v[e] = stored && active ? o[(size_t)e * nt] : 0.f;
+#pragma unroll
+            for (int f = 0; f < TE / 4; ++f) {
+                float4 *a = acc4 + ((size_t)r * 4 + f) * FAR_THREADS + threadIdx.x;
+                const float4 w = *a;
+                v[4 * f] += w.x;
+                v[4 * f + 1] += w.y;
+                v[4 * f + 2] += w.z;
+                v[4 * f + 3] += w.w;
+                *a = make_float4(0.f, 0.f, 0.f, 0.f);
+            }
+            if (!COMP) {
+                float2 *a = acc2 + (size_t)r * FAR_THREADS + threadIdx.x;
+                v[TE - 2] += a->x;
+                v[TE - 1] += a->y;
+                *a = make_float2(0.f, 0.f);
+            }
+            if (active)
+#pragma unroll
+                for (int e = 0; e < TE; ++e) o[(size_t)e * nt] = v[e];
+        }
+        stored = any = true;
+        // source side: the four warps' sums, in their order, to the slot of d
+        if (both) {
+            const int slot = ntst + (d - max(d_first, 1));
+#pragma unroll 1
+            for (int i = threadIdx.x; i < R * 5 * SYM_U; i += FAR_THREADS) {
+                const int si = i % SYM_U, k = i / SYM_U, r = k / 5, f = k - 5 * r;
+                float4 v = make_float4(0.f, 0.f, 0.f, 0.f), ve = v;
+                for (int w = 0; w < FAR_THREADS / 32; ++w) {
+                    if (f < 4) {
+                        float4 *a = src4 + ((size_t)r * 4 + f) * FAR_THREADS + w * 32 + si;
+                        comp_add(v.x, ve.x, a->x);
+                        comp_add(v.y, ve.y, a->y);
+                        comp_add(v.z, ve.z, a->z);
+                        comp_add(v.w, ve.w, a->w);
+                        *a = make_float4(0.f, 0.f, 0.f, 0.f);
+                        if (COMP && f == 3) {
+                            a = err4 + FAR_THREADS + w * 32 + si;
+                            ve.x += a->x;
+                            ve.y += a->y;
+                            ve.z += a->z;
+                            ve.w += a->w;
+                            *a = make_float4(0.f, 0.f, 0.f, 0.f);
+                        }
+                    } else {
+                        float2 *a = src2 + (size_t)r * FAR_THREADS + w * 32 + si;
+                        comp_add(v.x, ve.x, a->x);
+                        comp_add(v.y, ve.y, a->y);
+                        *a = make_float2(0.f, 0.f);
+                        if (COMP) {
+                            a = err2 + FAR_THREADS + w * 32 + si;
+                            ve.x += a->x;
+                            ve.y += a->y;
+                            *a = make_float2(0.f, 0.f);
+                        }
+                    }
+                }
+                if (si < cnt) {
+                    float *o = part + (((size_t)slot * R + r) * 18 + 4 * f) * nt + t0 + si;
+                    const float w4[4] = {v.x + ve.x, v.y + ve.y, v.z + ve.z, v.w + ve.w};
+#pragma unroll
+                    for (int e = 0; e < 4; ++e)
+                        if (f < 4 || e < 2) o[(size_t)e * nt] = accumulate ? o[(size_t)e * nt] + w4[e] : w4[e];
+                }
+            }
+        }
+    }
+    if (!stored && active)  // no tile: zero sums
+        for (int i = 0; i < R * 18; ++i) tout[(size_t)i * nt] = 0.f;
+    // (without a tile the sums have not met a barrier since they were cleared)
+    if (COMP && any && active) {
+        const float4 A = acc4[3 * FAR_THREADS + threadIdx.x], Ae = err4[threadIdx.x];
+        const float2 Az = acc2[threadIdx.x], Aze = err2[threadIdx.x];
+        const float v[6] = {A.x + Ae.x, A.y + Ae.y, A.z + Ae.z, A.w + Ae.w, Az.x + Aze.x, Az.y + Aze.y};
+#pragma unroll
+        for (int e = 0; e < 6; ++e) {
+            float *o = tout + (size_t)(12 + e) * nt;
+            *o = accumulate ? *o + v[e] : v[e];
+        }
+    }
+}
 #undef F3
 
 }  // namespace
+
+// Work split of sym_kernel: cuts the N / 2 offsets into launches of nsrc and a
+// launch's 32-triangle tiles over ntst blocks per test group, such that the
+// launches' waves of blocks, times the tiles of a block, are fewest, within
+// max_slots partial sums.
+static PerDeviceOnce g_sym_once;
+
+static FarSymPlan sym_plan(int nt, int sms, int max_slots) {
+    const int N = (nt + FAR_THREADS - 1) / FAR_THREADS, half = N / 2;
+    const long long slots = (long long)sms * FARM_MIN_BLOCKS;
+    FarSymPlan best;
+    double cost = -1.0;
+    for (int nsrc = half ? 1 : 0; nsrc <= std::min(half, max_slots - 1); ++nsrc) {
+        const int units = 4 * (nsrc + 1), launches = nsrc ? (half + nsrc - 1) / nsrc : 1;
+        for (int ups = 1; ups <= units; ++ups) {
+            const int ntst = (units + ups - 1) / ups;
+            if (ntst + nsrc > max_slots) continue;
+            const double c = launches * ((double)((N * (long long)ntst + slots - 1) / slots) * ups + 1.0);
+            if (cost < 0.0 || c < cost) {
+                cost = c;
+                best.nsrc = nsrc;
+                best.ntst = ntst;
+                best.ups = ups;
+            }
+        }
+    }
+    return best;
+}
+
+// partial sums times right-hand sides of the several-right-hand-side launches
+static size_t farm_slots(const osrc_problem *pb) {
+    const int s = pb->nsplit * FARM_MAX_R;
+    return pb->far_sym && !pb->mesh->ctx->budget ? std::max(s, SYM_MULTI_SLOTS) : std::max(s, 2 * FARM_MAX_R);
+}
+
+int far_workspace(osrc_problem *pb) {
+    osrc_ctx *ctx = pb->mesh->ctx;
+    const size_t nt = pb->nt;
+    if (pb->far_sym) {
+        int s = pb->d_sD.alloc(ctx, 5 * nt);
+        if (!s) s = pb->d_part.alloc(ctx, (size_t)(pb->sym[1].ntst + pb->sym[1].nsrc) * 18 * nt);
+        if (s != OSRC_OUT_OF_MEMORY) return s;
+        pb->d_sD.release();  // no room: the one-sided kernels' buffers may fit
+        pb->d_part.release();
+        pb->far_sym = false;
+    }
+    OSRC_TRY(pb->d_sP.alloc(ctx, 24 * nt));
+    OSRC_TRY(pb->d_sP5.alloc(ctx, 6 * nt));
+    OSRC_TRY(pb->d_sC.alloc(ctx, 2 * nt));
+    OSRC_TRY(pb->d_part.alloc(ctx, (size_t)pb->nsplit * 4 * pb->npts));
+    return pb->d_partA1.alloc(ctx, (size_t)pb->nsplit * 6 * nt);
+}
 
 int far_setup_geometry(osrc_problem *pb, cudaStream_t st) {
     osrc_mesh *m = pb->mesh;
@@ -1161,9 +1564,6 @@ int far_setup_geometry(osrc_problem *pb, cudaStream_t st) {
     OSRC_TRY(pb->d_tn.alloc(m->ctx, nt));
     OSRC_TRY(pb->d_tv.alloc(m->ctx, nt));
     OSRC_TRY(pb->d_tgeo.alloc(m->ctx, 16 * (size_t)nt));
-    OSRC_TRY(pb->d_sP.alloc(m->ctx, 24 * (size_t)nt));
-    OSRC_TRY(pb->d_sP5.alloc(m->ctx, 6 * (size_t)nt));
-    OSRC_TRY(pb->d_sC.alloc(m->ctx, 2 * (size_t)nt));
     far_geom_kernel<<<(nt + 127) / 128, 128, 0, st>>>(m->d_verts.p, m->d_tris.p, nt, pb->d_pt.p,
                                                       pb->d_poff.p, pb->d_cen.p, pb->d_tn.p,
                                                       pb->d_tv.p, pb->d_tgeo.p);
@@ -1193,7 +1593,8 @@ int far_setup_geometry(osrc_problem *pb, cudaStream_t st) {
     // partial sums stays small beside the pair work, fill the resident blocks
     // four times over, and near that number the one with the fullest last
     // wave is taken.
-    int dev = m->ctx->device, sms = 0;
+    int dev = m->ctx->device;
+    int &sms = pb->sms;
     OSRC_CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     pb->far_tris = nt < FAR_TRIS32_NT ? 32 : nt < FAR_TRIS64_NT ? 64 : FAR_THREADS;
     const int slots = sms * OSRC_FAR_MIN_BLOCKS;  // farm_kernel runs on the same grid
@@ -1212,8 +1613,87 @@ int far_setup_geometry(osrc_problem *pb, cudaStream_t st) {
         }
     }
     pb->nsplit = ns;
-    OSRC_TRY(pb->d_part.alloc(m->ctx, (size_t)ns * 4 * pb->npts));
-    OSRC_TRY(pb->d_partA1.alloc(m->ctx, (size_t)ns * 6 * nt));
+    pb->far_sym = nt >= SYM_MIN_NT;
+    static_assert(SYM_MAX_R < sizeof(pb->sym) / sizeof(pb->sym[0]), "a plan for every R");
+    // on a context with a memory budget no more than far_kernel's buffers
+    const int one = m->ctx->budget ? std::max(2, std::min(SYM_MAX_SLOTS, (30 * ns + 116) / 18)) : SYM_MAX_SLOTS;
+    if (pb->far_sym)
+        for (int r = 1; r <= SYM_MAX_R; ++r)
+            pb->sym[r] = sym_plan(nt, sms, r == 1 ? one : (int)farm_slots(pb) / r);
+    OSRC_TRY(per_device_once(g_sym_once, [](int) {
+        const int sp = (int)sym_smem_bytes(SYM_MAX_R, false), sc = (int)sym_smem_bytes(SYM_MAX_R, true);
+        const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
+        OSRC_CK(cudaFuncSetAttribute(sym_kernel<false, false, false, false>, attr, sp));
+        OSRC_CK(cudaFuncSetAttribute(sym_kernel<true, false, false, false>, attr, sc));
+        return OSRC_OK;
+    }));
+    return far_workspace(pb);
+}
+
+int far_prof_collect(osrc_problem *pb);
+
+static FarConst2 far_consts(const osrc_problem *pb, float4 &kff) {
+    const double k0 = pb->p.k_ext, k1 = pb->p.k_int, rho = pb->p.rho_ratio;
+    const double inv2pi = 0.15915494309189533577;
+    auto d2 = [](double v) { return make_float2((float)v, (float)v); };
+    FarConst2 c;
+    c.k0 = d2(k0);
+    c.k1 = d2(k1);
+    c.nk0 = d2(-k0);
+    c.nk1 = d2(-k1);
+    c.rho = d2(rho);
+    c.irho = d2(1.0 / rho);
+    c.dk0 = d2(pb->far_dks);
+    c.dk1 = d2(k1 * k1 / rho / pb->far_dks);
+    // k / (2 pi) as float pairs (hi, lo) for the float-float phases
+    const double q0 = k0 * inv2pi, q1 = k1 * inv2pi;
+    const float q0h = (float)q0, q1h = (float)q1;
+    kff = make_float4(q0h, (float)(q0 - (double)q0h), q1h, (float)(q1 - (double)q1h));
+    return c;
+}
+
+// sD from the vectors and the launches of sym_kernel over all offsets
+static int sym_launch(osrc_problem *pb, const VecPtrs &xp, int R, const FarSymPlan &pl, float *part, cudaStream_t st) {
+    osrc_mesh *m = pb->mesh;
+    const int nt = pb->nt, N = (nt + FAR_THREADS - 1) / FAR_THREADS, half = N / 2;
+    farm_prep_kernel<<<dim3((nt + 127) / 128, R), 128, 0, st>>>(xp, R, pb->nv, nt, m->d_tris.p, pb->d_tgeo.p,
+                                                               pb->d_sD.p);
+    pb->launches++;
+    float4 kff;
+    const FarConst2 c = far_consts(pb, kff);
+    const size_t smem = sym_smem_bytes(R, pb->far_reduce);
+    const float4 *pts = pb->far_reduce ? pb->d_poff.p : pb->d_pt.p;
+    if (pb->prof_on) {
+        OSRC_TRY(far_prof_collect(pb));
+        OSRC_CK(cudaEventRecord(pb->prof_ev[0], st));
+    }
+    // even N in one launch: the lower half of the groups has no sums of the last offset
+    if (half && 2 * half == N && pl.nsrc >= half)
+        OSRC_CK(cudaMemsetAsync(part + (size_t)(pl.ntst + half - 1) * R * 18 * nt, 0, (size_t)R * 18 * nt * sizeof(float), st));
+    for (int d = 0; d <= half; d += d ? pl.nsrc : pl.nsrc + 1) {
+        const int count = d ? std::min(pl.nsrc, half + 1 - d) : pl.nsrc + 1;
+        const dim3 grid(N, (4 * count + pl.ups - 1) / pl.ups);
+#define OSRC_SYM_LAUNCH(C, M, A, E)                                                                                \
+    sym_kernel<C, M, A, E><<<grid, FAR_THREADS, smem, st>>>(pts, pb->d_cen.p, pb->d_tn.p, pb->d_tv.p, pb->d_sD.p, R, \
+                                                            nt, d, count, pl.ups, pl.ntst, d ? 1 : 0, c, kff,       \
+                                                            m->d_tcomp.p, pb->d_fobj.p, part)
+        if (pb->far_reduce && pb->far_obj && pb->absorb) OSRC_SYM_LAUNCH(true, true, true, true);
+        else if (pb->far_reduce && pb->far_obj) OSRC_SYM_LAUNCH(true, true, false, true);
+        else if (pb->far_reduce && R == 1) OSRC_SYM_LAUNCH(true, false, false, true);
+        else if (pb->far_reduce) OSRC_SYM_LAUNCH(true, false, false, false);
+        else if (pb->far_obj && pb->absorb) OSRC_SYM_LAUNCH(false, true, true, true);
+        else if (pb->far_obj) OSRC_SYM_LAUNCH(false, true, false, true);
+        else if (R == 1) OSRC_SYM_LAUNCH(false, false, false, true);
+        else OSRC_SYM_LAUNCH(false, false, false, false);
+#undef OSRC_SYM_LAUNCH
+        pb->launches++;
+        OSRC_CK(cudaGetLastError());
+    }
+    if (pb->prof_on) {
+        OSRC_CK(cudaEventRecord(pb->prof_ev[1], st));
+        pb->prof_pending = true;
+        pb->prof_rhs_pending = R;
+    }
     return OSRC_OK;
 }
 
@@ -1255,28 +1735,23 @@ int far_apply(osrc_problem *pb, const double2 *x, double2 *y, int part, cudaStre
     const int nt = pb->nt, nv = pb->nv, npts = pb->npts;
     const int use_far = (part & OSRC_PART_FAR) ? 1 : 0;
     const int use_near = (part & OSRC_PART_NEAR) ? 1 : 0;
+    VecPtrs xp{};
+    OutPtrs yp{};
+    xp.p[0] = x;
+    yp.p[0] = y;
+    if (use_far && !pb->d_part.p) OSRC_TRY(far_workspace(pb));  // a clone made without it
+    if (use_far && pb->far_sym) {
+        OSRC_TRY(sym_launch(pb, xp, 1, pb->sym[1], pb->d_part.p, st));
+        return gather_launch(pb, pb->sym[1].ntst + pb->sym[1].nsrc, 1, pb->d_part.p, nullptr, use_far, use_near, xp, yp, st);
+    }
     if (use_far) {
         const float4 *src_pts = pb->far_reduce ? pb->d_poff.p : pb->d_pt.p;
         far_prep_kernel<<<(npts + 127) / 128, 128, 0, st>>>(x, nv, nt, m->d_tris.p, src_pts,
                                                           pb->d_tgeo.p, pb->d_sP.p, pb->d_sP5.p,
                                                           pb->d_sC.p);
         pb->launches++;
-        const double k0 = pb->p.k_ext, k1 = pb->p.k_int, rho = pb->p.rho_ratio;
-        const double inv2pi = 0.15915494309189533577;
-        auto d2 = [](double v) { return make_float2((float)v, (float)v); };
-        FarConst2 c;
-        c.k0 = d2(k0);
-        c.k1 = d2(k1);
-        c.nk0 = d2(-k0);
-        c.nk1 = d2(-k1);
-        c.rho = d2(rho);
-        c.irho = d2(1.0 / rho);
-        c.dk0 = d2(pb->far_dks);
-        c.dk1 = d2(k1 * k1 / rho / pb->far_dks);
-        // k / (2 pi) as float pairs (hi, lo) for the float-float phases
-        const double q0 = k0 * inv2pi, q1 = k1 * inv2pi;
-        const float q0h = (float)q0, q1h = (float)q1;
-        const float4 kff = make_float4(q0h, (float)(q0 - (double)q0h), q1h, (float)(q1 - (double)q1h));
+        float4 kff;
+        const FarConst2 c = far_consts(pb, kff);
         const int ns = pb->nsplit;
         const int tps = (nt + ns - 1) / ns;
         dim3 grid((nt + pb->far_tris - 1) / pb->far_tris, ns);
@@ -1306,10 +1781,6 @@ int far_apply(osrc_problem *pb, const double2 *x, double2 *y, int part, cudaStre
             pb->prof_pending = true;
         }
     }
-    VecPtrs xp{};
-    OutPtrs yp{};
-    xp.p[0] = x;
-    yp.p[0] = y;
     return gather_launch(pb, pb->nsplit, 1, pb->d_part.p, pb->d_partA1.p, use_far, use_near, xp, yp, st);
 }
 
@@ -1338,7 +1809,7 @@ static int farm_prepare(osrc_problem *pb, cudaStream_t st) {
     }
     if (!pb->d_partm.p) {
         OSRC_TRY(pb->d_sD.alloc(ctx, 5 * (size_t)nt * FARM_MAX_R));
-        OSRC_TRY(pb->d_partm.alloc(ctx, (size_t)pb->nsplit * FARM_MAX_R * 18 * nt));
+        OSRC_TRY(pb->d_partm.alloc(ctx, farm_slots(pb) * 18 * nt));
     }
     return OSRC_OK;
 }
@@ -1356,25 +1827,17 @@ static int farm_launch(osrc_problem *pb, const double2 *const *xs, double2 *cons
         yp.p[r] = ys[r];
     }
     const int ns = pb->nsplit;
+    if (use_far && pb->far_sym && R <= SYM_MAX_R) {
+        const FarSymPlan pl = pb->sym[R];
+        OSRC_TRY(sym_launch(pb, xp, R, pl, pb->d_partm.p, st));
+        return gather_launch(pb, pl.ntst + pl.nsrc, R, pb->d_partm.p, nullptr, use_far, use_near, xp, yp, st);
+    }
     if (use_far) {
         farm_prep_kernel<<<dim3((nt + 127) / 128, R), 128, 0, st>>>(xp, R, nv, nt, m->d_tris.p, pb->d_tgeo.p,
                                                                    pb->d_sD.p);
         pb->launches++;
-        const double k0 = pb->p.k_ext, k1 = pb->p.k_int, rho = pb->p.rho_ratio;
-        const double inv2pi = 0.15915494309189533577;
-        auto d2 = [](double v) { return make_float2((float)v, (float)v); };
-        FarConst2 c;
-        c.k0 = d2(k0);
-        c.k1 = d2(k1);
-        c.nk0 = d2(-k0);
-        c.nk1 = d2(-k1);
-        c.rho = d2(rho);
-        c.irho = d2(1.0 / rho);
-        c.dk0 = d2(pb->far_dks);
-        c.dk1 = d2(k1 * k1 / rho / pb->far_dks);
-        const double q0 = k0 * inv2pi, q1 = k1 * inv2pi;
-        const float q0h = (float)q0, q1h = (float)q1;
-        const float4 kff = make_float4(q0h, (float)(q0 - (double)q0h), q1h, (float)(q1 - (double)q1h));
+        float4 kff;
+        const FarConst2 c = far_consts(pb, kff);
         const int tps = (nt + ns - 1) / ns;
         dim3 grid((nt + pb->far_tris - 1) / pb->far_tris, ns);
         const float4 *pts = pb->far_reduce ? pb->d_poff.p : pb->d_pt.p;

@@ -1000,7 +1000,7 @@ int GmresRun::run_to_completion() {
 // ---------------------------------------------------------------------------
 // problem clones: shared resident state, own workspace (serving slots)
 // ---------------------------------------------------------------------------
-int problem_clone(osrc_problem *m, osrc_problem **out) {
+int problem_clone(osrc_problem *m, osrc_problem **out, bool far) {
     *out = nullptr;
     osrc_ctx *ctx = m->mesh->ctx;
     osrc_problem *c = new osrc_problem;
@@ -1011,6 +1011,9 @@ int problem_clone(osrc_problem *m, osrc_problem **out) {
     c->npts = m->npts;
     c->nsplit = m->nsplit;
     c->far_tris = m->far_tris;
+    c->far_sym = m->far_sym;
+    for (int r = 0; r < 6; ++r) c->sym[r] = m->sym[r];
+    c->sms = m->sms;
     c->far_reduce = m->far_reduce;
     c->near_pairs = m->near_pairs;
     c->near_nnz = m->near_nnz;
@@ -1047,14 +1050,10 @@ int problem_clone(osrc_problem *m, osrc_problem **out) {
     c->d_M.borrow(m->d_M);
     c->d_S.borrow(m->d_S);
     c->d_dense.borrow(m->d_dense);
-    const int nt = m->nt, nv = m->nv;
+    const int nv = m->nv;
     const int nsys = 2 * m->p.n_pade + 2;
     int s = OSRC_OK;
-    if ((s = c->d_sP.alloc(ctx, 24 * (size_t)nt)) || (s = c->d_sP5.alloc(ctx, 6 * (size_t)nt)) ||
-        (s = c->d_sC.alloc(ctx, 2 * (size_t)nt)) ||
-        (s = c->d_part.alloc(ctx, (size_t)c->nsplit * 4 * c->npts)) ||
-        (s = c->d_partA1.alloc(ctx, (size_t)c->nsplit * 6 * nt)) ||
-        (s = c->d_kry.alloc(ctx, 5 * (size_t)nsys * nv)) ||
+    if ((far && (s = far_workspace(c))) || (s = c->d_kry.alloc(ctx, 5 * (size_t)nsys * nv)) ||
         (s = c->d_kry_rhs.alloc(ctx, (size_t)(2 + nsys) * nv)) || (s = c->d_kry_stat.alloc(ctx, 40)) ||
         (s = c->d_kry_res.alloc(ctx, 40)) || (s = c->d_tmp2.alloc(ctx, 4 * (size_t)nv)) ||
         (s = c->d_scalars.alloc(ctx, 64))) {
@@ -1119,7 +1118,7 @@ static int gmres_solve_lockstep(osrc_problem *pb, const void *b, void *x, int nr
     const int G = std::min(nrhs, kBatchRuns);
     CloneSet cs;
     cs.c.assign(G, nullptr);
-    for (int g = 0; g < G; ++g) OSRC_TRY(problem_clone(pb, &cs.c[g]));
+    for (int g = 0; g < G; ++g) OSRC_TRY(problem_clone(pb, &cs.c[g], false));
     DBuf<double2> db, dx;
     if (host) {
         OSRC_TRY(db.alloc(pb->mesh->ctx, (size_t)G * n));

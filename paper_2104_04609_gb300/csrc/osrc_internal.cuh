@@ -119,6 +119,12 @@ struct DBuf {
     ~DBuf() { release(); }
 };
 
+// Work split of the far field's symmetric kernel: offsets per launch, blocks per
+// test group, tiles per block.
+struct FarSymPlan {
+    int nsrc = 0, ntst = 1, ups = 4;
+};
+
 struct osrc_mesh {
     osrc_ctx *ctx = nullptr;
     int nv = 0, nt = 0;
@@ -190,6 +196,9 @@ struct osrc_problem {
     DBuf<float> d_part;       // [nsplit][4][6nt] per test point partial sums
     DBuf<float> d_partA1;     // [nsplit][6][nt] curl-term partial sums per test triangle
     int nsplit = 1, far_tris = 128;  // far kernel: source splits, test triangles per block
+    bool far_sym = false;     // pairs of triangles evaluated once for both directions
+    FarSymPlan sym[6];        // its work split by right-hand sides of a launch
+    int sms = 1;
     // ---- far field, several right-hand sides per launch (k_far.cu farm_*) ----
     DBuf<float4> d_sG;        // [6nt][2] static source geometry (coordinates)
     DBuf<float4> d_sD;        // [nt][R][5] corner densities and curl sources of R right-hand sides
@@ -266,6 +275,7 @@ int far_prof_collect(osrc_problem *pb);
 // ---------------------------------------------------------------------------
 // far field (k_far.cu)
 int far_setup_geometry(osrc_problem *pb, cudaStream_t st);
+int far_workspace(osrc_problem *pb);
 int far_apply(osrc_problem *pb, const double2 *x, double2 *y, int part, cudaStream_t st);
 // y_r = B x_r for nrhs vectors (far part of several right-hand sides per launch
 // where the problem allows it: one object, PMCHWT, lossless interior)
@@ -356,8 +366,9 @@ struct GmresRun {
 
 int ensure_gmres_workspace(osrc_problem *pb, int maxit);
 // a problem that borrows the resident state of `master` and owns a fresh
-// workspace (per-apply, inner-solver and GMRES buffers)
-int problem_clone(osrc_problem *master, osrc_problem **out);
+// workspace (per-apply, inner-solver and GMRES buffers); far: with the far
+// field's per-apply buffers (a lockstep solve applies B through the master)
+int problem_clone(osrc_problem *master, osrc_problem **out, bool far = true);
 // device bytes of the resident state and of one workspace (estimates used
 // for admission by device memory)
 size_t estimate_problem_bytes(int nv, int nt, const osrc_params &p);

@@ -5,28 +5,40 @@
 // preconditioner matrix.
 //
 // GEMM: C[M x N] = A[M x K] * B[N x K]^T, A and B BF16 and K-major (row-major
-// with K contiguous), C FP32.  The product is cut into 128-row tiles and
-// 64-wide K slices.  The tile x slice iterations are dealt out in equal
-// contiguous ranges to a persistent grid of one CTA per SM (stream-K), so
-// every SM works to the end even when the number of tiles is not a multiple
-// of the SM count (the 16000-row product of the 8000-vertex system has 125
-// tiles for 152 SMs).  Per CTA of 192 threads:
+// with K contiguous), C FP32.  The product is cut into tiles of 256 rows and
+// 64-wide K slices, a tile to a pair of CTAs (cta_group::2, a cluster on the
+// two SMs of a TPC); up to UM_PAIR_N columns 128 rows and one CTA, which then
+// plays both parts below.  The tile x slice iterations are dealt out in equal
+// contiguous ranges to a persistent grid of one pair per two SMs (stream-K),
+// so every SM works to the end even when the number of tiles is not a multiple
+// of the pairs (the 16000-row product of the 8000-vertex system has 63 tiles
+// for 76 pairs).  CTA r of a pair holds rows 128 r .. of the A tile and half
+// of the columns' B rows; the pair's MMA reads both halves.  Per CTA of 192
+// threads:
 //   - lane 0 of warp 4 issues TMA loads (128-byte swizzle) of the K slices of
-//     A (evict-first in L2: it is streamed once) and B (evict-last: every CTA
-//     re-reads it) into a shared-memory ring of as many stages as fit;
-//   - lane 0 of warp 5 issues tcgen05.mma (kind::f16, M 128, N, K 16) into
-//     one of two FP32 accumulators in tensor memory, releases each stage with
-//     tcgen05.commit and signals the end of each tile segment;
-//   - warps 0-3 read the accumulator of a finished segment (tcgen05.ld, warp
-//     w owns lanes 32w..32w+31, a thread one row) and store it as 16-byte
-//     vectors while the MMAs of the next segment fill the other accumulator.
-// A CTA range that covers a whole tile writes C directly.  A tile split
-// between CTAs has its pieces written to a workspace (slot 2c for the first
-// segment of CTA c, 2c + 1 for its last) and summed by a second kernel in CTA
-// order, so C is the same bit for bit from run to run (no atomics).
+//     its part of A (evict-first in L2: it is streamed once) and B (evict-last:
+//     every pair re-reads it) into a shared-memory ring of as many stages as
+//     fit; the bytes of both CTAs are counted on CTA 0's barrier;
+//   - lane 0 of warp 5 of CTA 0 issues tcgen05.mma (kind::f16, M 256, N, K 16)
+//     into one of two FP32 accumulators in the pair's tensor memory, releases
+//     each stage of both CTAs with tcgen05.commit and signals the end of each
+//     tile segment;
+//   - warps 0-3 read their half of the accumulator of a finished segment
+//     (tcgen05.ld, warp w owns lanes 32w..32w+31, a thread one row) and store
+//     it as 16-byte vectors while the MMAs of the next segment fill the other.
+// A pair's range that covers a whole tile writes C directly.  A tile split
+// between pairs has its pieces written to a workspace (slot 2c for the first
+// segment of pair c, 2c + 1 for its last) and summed by a second kernel in
+// pair order, so C is the same bit for bit from run to run (no atomics).
 // Every mbarrier wait is bounded (2 s of global time): on timeout the kernel
 // records an error flag, stops waiting, waits (bounded) for its own TMA loads
-// and MMAs in flight, frees its tensor memory and returns.
+// and MMAs in flight, frees its tensor memory and returns; the pair leaves
+// together (a cluster barrier that every thread reaches).
+//
+// Bound by A's one pass through HBM.  A pair of CTAs shares B, which halves its
+// traffic from L2 and the shared memory it takes (N 256: 7 stages of 32 KB where
+// one CTA per tile had 4 of 48): 16000 x 32000 x 256 220 -> 203 us, against
+// 178 us for N = 16, which is all A; 6016 x 12032 x 128 unchanged, 46.
 //
 // Complex products use the real embedding: with A_cat = [Re A | Im A]
 // (M x 2K) and, for right-hand sides X_r, B rows [Re X_r | -Im X_r] (first
@@ -43,14 +55,21 @@
 
 namespace {
 
-constexpr int UM_BM = 128;              // rows of a tile (one tensor-memory lane per row)
+constexpr int UM_BM = 128;              // rows of a CTA's half tile (one tensor-memory lane per row)
 constexpr int UM_NBUF = 2;              // accumulators in tensor memory (2 x N <= 512 columns)
 constexpr int UM_BK = 64;               // 64 BF16 = one 128-byte swizzle row
 constexpr int UM_THREADS = 192;         // warps 0-3 epilogue, warp 4 TMA, warp 5 MMA
-constexpr int UM_MIN_ITERS = 48;        // fewest K slices per CTA
-constexpr int UM_MAX_STAGES = 8;
+// fewest K slices per CTA or pair: 48 / 24 / 12 take, at 512 x 1024 x 128, 37 / 23
+// / 21 us, 1408 x 2816 x 256 41 / 33 / 31, 3072 x 6144 x 256 38 / 33 / 42; larger
+// products have more
+constexpr int UM_MIN_ITERS = 24;
+constexpr int UM_MAX_STAGES = 8;        // 4 cost 10 %, 13 (of small N) gain nothing
 constexpr size_t UM_SMEM_MAX = 230400;  // dynamic shared memory per CTA (227 KB less the static part)
 constexpr size_t UM_SMEM_FIXED = 1024 + 256;  // alignment slack, barriers
+// columns above which a pair of CTAs takes a tile: it costs a launch 2 us (cluster
+// barriers) and pays where B's traffic counts (16000 x 32000: N 256 220 -> 203
+// us, 192 205 -> 196, 128 189 -> 183; 6016 x 12032 x 128 in a solve 31.8 -> 33.5)
+constexpr int UM_PAIR_N = 128;
 constexpr int UM_FIX_ROWS = 8;                  // rows of a split tile per block of the summing kernel
 constexpr unsigned long long UM_TIMEOUT_NS = 2000000000ULL;
 
@@ -73,34 +92,86 @@ __device__ __forceinline__ void mbar_expect_tx(uint64_t *bar, uint32_t bytes) {
                  : "memory");
 }
 
-__device__ __forceinline__ void mbar_arrive(uint64_t *bar) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
+// address of the same variable in CTA 0 of the pair
+template <bool PAIR>
+__device__ __forceinline__ uint32_t smem_cta0(const void *p) {
+    if (!PAIR) return smem_u32(p);
+    uint32_t a;
+    asm("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(a) : "r"(smem_u32(p)));
+    return a;
+}
+
+template <bool PAIR>
+__device__ __forceinline__ void mbar_arrive_cta0(uint64_t *bar) {
+    if (PAIR)
+        asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(smem_cta0<true>(bar)) : "memory");
+    else
+        asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
+
+// releases the barrier (of both CTAs) when the MMAs issued so far are done
+template <bool PAIR>
+__device__ __forceinline__ void commit(uint64_t *bar) {
+    if (PAIR)
+        asm volatile(
+            "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(
+                smem_u32(bar)),
+            "h"((uint16_t)3)
+            : "memory");
+    else
+        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
+                     : "memory");
+}
+
+__device__ __forceinline__ void cluster_barrier() {
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
 // Waits for the completion of phase `parity`; false after the time limit.
+// CLUSTER: the arrivals came from both CTAs.
+template <bool CLUSTER = false>
 __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity) {
     const unsigned long long t0 = global_ns();
     while (true) {
         uint32_t done;
-        asm volatile(
-            "{\n\t.reg .pred p;\n\t"
-            "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-            "selp.u32 %0, 1, 0, p;\n\t}"
-            : "=r"(done)
-            : "r"(smem_u32(bar)), "r"(parity)
-            : "memory");
+        if (CLUSTER)
+            asm volatile(
+                "{\n\t.reg .pred p;\n\t"
+                "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+                "selp.u32 %0, 1, 0, p;\n\t}"
+                : "=r"(done)
+                : "r"(smem_u32(bar)), "r"(parity)
+                : "memory");
+        else
+            asm volatile(
+                "{\n\t.reg .pred p;\n\t"
+                "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+                "selp.u32 %0, 1, 0, p;\n\t}"
+                : "=r"(done)
+                : "r"(smem_u32(bar)), "r"(parity)
+                : "memory");
         if (done) return true;
         if (global_ns() - t0 > UM_TIMEOUT_NS) return false;
     }
 }
 
-__device__ __forceinline__ void tma_load_2d(void *dst, const CUtensorMap *map, int x, int y, uint64_t *bar,
+// into this CTA's shared memory, the bytes counted on CTA 0's barrier
+template <bool PAIR>
+__device__ __forceinline__ void tma_load_2d(void *dst, const CUtensorMap *map, int x, int y, uint32_t bar,
                                             uint64_t policy) {
-    asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint"
-        " [%0], [%1, {%2, %3}], [%4], %5;" ::"r"(smem_u32(dst)),
-        "l"((uint64_t)map), "r"(x), "r"(y), "r"(smem_u32(bar)), "l"(policy)
-        : "memory");
+    if (PAIR)
+        asm volatile(
+            "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint"
+            " [%0], [%1, {%2, %3}], [%4], %5;" ::"r"(smem_u32(dst)),
+            "l"((uint64_t)map), "r"(x), "r"(y), "r"(bar), "l"(policy)
+            : "memory");
+    else
+        asm volatile(
+            "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint"
+            " [%0], [%1, {%2, %3}], [%4], %5;" ::"r"(smem_u32(dst)),
+            "l"((uint64_t)map), "r"(x), "r"(y), "r"(bar), "l"(policy)
+            : "memory");
 }
 
 // Shared-memory matrix descriptor: K-major, 128-byte swizzle, 8-row atoms of
@@ -122,15 +193,17 @@ __host__ __device__ constexpr uint32_t instr_desc(int m, int n) {
 }
 
 // ncols = tensor-memory columns of one accumulator (a power of two >= N);
-// two accumulators alternate between the tile segments of a CTA.
+// two accumulators alternate between the tile segments of a pair.
+// PAIR: a pair of CTAs (a cluster of two) per tile, else one.
+template <bool PAIR>
 __global__ void __launch_bounds__(UM_THREADS, 1)
 umma_sk_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b, int M,
                int N, int KB, long long iters, int stages, uint32_t ncols, float *__restrict__ C, int ldc,
                float *__restrict__ ws, int *__restrict__ err) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char *base = (unsigned char *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    constexpr int nbuf = UM_NBUF;
-    const uint32_t a_bytes = UM_BM * UM_BK * 2, b_bytes = (uint32_t)N * UM_BK * 2;
+    constexpr int nbuf = UM_NBUF, CG = PAIR ? 2 : 1, TM = CG * UM_BM;
+    const uint32_t a_bytes = UM_BM * UM_BK * 2, b_bytes = (uint32_t)N / CG * UM_BK * 2;
     const uint32_t stage_bytes = a_bytes + b_bytes;
     uint64_t *bars = (uint64_t *)(base + (size_t)stages * stage_bytes);
     uint64_t *full = bars, *empty = bars + stages, *accf = bars + 2 * stages, *acce = accf + 2, *drain = acce + 2;
@@ -139,8 +212,8 @@ umma_sk_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     volatile int *vto = &timed_out;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int G = gridDim.x, cta = blockIdx.x;
-    const long long it_begin = sk_begin(cta, iters, G), it_end = sk_begin(cta + 1, iters, G);
+    const int G = gridDim.x / CG, pair = blockIdx.x / CG, rank = blockIdx.x % CG;
+    const long long it_begin = sk_begin(pair, iters, G), it_end = sk_begin(pair + 1, iters, G);
     const uint32_t tcols = (uint32_t)nbuf * ncols;
 
     if (threadIdx.x == 0) {
@@ -151,18 +224,25 @@ umma_sk_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         }
         for (int b = 0; b < 2; ++b) {
             mbar_init(&accf[b], 1);
-            mbar_init(&acce[b], 4 * 32);
+            mbar_init(&acce[b], CG * 4 * 32);  // CTA 0's: the epilogues of both CTAs
         }
         mbar_init(drain, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 0) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
-                     "r"(tcols));
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+        if (PAIR) {
+            asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
+                         "r"(tcols));
+            asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;");
+        } else {
+            asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
+                         "r"(tcols));
+            asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+        }
     }
     asm volatile("tcgen05.fence::before_thread_sync;");
     __syncthreads();
+    if (PAIR) cluster_barrier();  // barriers and tensor memory of both CTAs are ready
     asm volatile("tcgen05.fence::after_thread_sync;");
     const uint32_t tmem = *tmem_slot;
 
@@ -188,24 +268,26 @@ umma_sk_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
                     }
                     unsigned char *sa = base + (size_t)s * stage_bytes, *sb = sa + a_bytes;
                     const int kx = (sg.kb0 + j) * UM_BK;
-                    mbar_expect_tx(&full[s], stage_bytes);
-                    tma_load_2d(sa, &map_a, kx, sg.tile * UM_BM, &full[s], pol_a);
-                    tma_load_2d(sb, &map_b, kx, 0, &full[s], pol_b);
+                    const uint32_t fb = smem_cta0<PAIR>(&full[s]);
+                    if (rank == 0) mbar_expect_tx(&full[s], CG * stage_bytes);
+                    tma_load_2d<PAIR>(sa, &map_a, kx, sg.tile * TM + rank * UM_BM, fb, pol_a);
+                    tma_load_2d<PAIR>(sb, &map_b, kx, rank * (N / CG), fb, pol_b);
                     ++g;
                 }
                 it += sg.n;
             }
             if (!ok) {
                 *vto = 1;
-                // let the loads already issued land before the CTA exits
-                for (uint32_t j = g > (uint32_t)stages ? g - stages : 0; j < g; ++j)
+                // let the loads already issued land before the pair exits (CTA 0's
+                // barriers count both CTAs')
+                for (uint32_t j = g > (uint32_t)stages ? g - stages : 0; j < g && rank == 0; ++j)
                     mbar_wait(&full[j % stages], (j / stages) & 1);
             }
         }
     } else if (warp == 5) {
-        if (lane == 0) {
-            // MMA issuer
-            const uint32_t idesc = instr_desc(UM_BM, N);
+        if (lane == 0 && rank == 0) {
+            // MMA issuer of the pair
+            const uint32_t idesc = instr_desc(TM, N);
             uint32_t g = 0;
             int seg = 0;
             bool ok = true;
@@ -213,7 +295,7 @@ umma_sk_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
                 const SkSeg sg = sk_next(it, it_end, KB);
                 const int b = seg % nbuf;
                 const uint32_t use = (uint32_t)(seg / nbuf);
-                if (seg >= nbuf && !mbar_wait(&acce[b], (use - 1) & 1)) {
+                if (seg >= nbuf && !mbar_wait<PAIR>(&acce[b], (use - 1) & 1)) {
                     ok = false;
                     break;
                 }
@@ -232,28 +314,28 @@ umma_sk_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
                     for (int k = 0; k < UM_BK / 16; ++k) {
                         // 16 BF16 = 32 bytes along K inside the swizzled rows
                         const uint32_t accum = (j | k) ? 1u : 0u;
-                        asm volatile(
-                            "{\n\t.reg .pred p;\n\t"
-                            "setp.ne.b32 p, %4, 0;\n\t"
-                            "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(acc),
-                            "l"(da + (uint64_t)(2 * k)), "l"(db + (uint64_t)(2 * k)), "r"(idesc), "r"(accum));
+                        if (PAIR)
+                            asm volatile(
+                                "{\n\t.reg .pred p;\n\t"
+                                "setp.ne.b32 p, %4, 0;\n\t"
+                                "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(acc),
+                                "l"(da + (uint64_t)(2 * k)), "l"(db + (uint64_t)(2 * k)), "r"(idesc), "r"(accum));
+                        else
+                            asm volatile(
+                                "{\n\t.reg .pred p;\n\t"
+                                "setp.ne.b32 p, %4, 0;\n\t"
+                                "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(acc),
+                                "l"(da + (uint64_t)(2 * k)), "l"(db + (uint64_t)(2 * k)), "r"(idesc), "r"(accum));
                     }
-                    asm volatile(
-                        "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                            smem_u32(&empty[s]))
-                        : "memory");
+                    commit<PAIR>(&empty[s]);
                 }
                 if (!ok) break;
-                asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                                 smem_u32(&accf[b]))
-                             : "memory");
+                commit<PAIR>(&accf[b]);
                 it += sg.n;
             }
             if (!ok) *vto = 1;
             // every MMA issued has finished before the tensor memory is freed
-            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                             smem_u32(drain))
-                         : "memory");
+            commit<PAIR>(drain);
             if (!mbar_wait(drain, 0)) *vto = 1;
         }
     } else {
@@ -273,12 +355,13 @@ umma_sk_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
             int ld, rows;
             bool vec;
             if (sg.kb0 == 0 && sg.n == KB) {
-                dst = C + (size_t)sg.tile * UM_BM * ldc;
+                const int row0 = sg.tile * TM + rank * UM_BM;
+                dst = C + (size_t)row0 * ldc;
                 ld = ldc;
-                rows = M - sg.tile * UM_BM;
+                rows = M - row0;  // the last tile of an odd number of halves: none for CTA 1
                 vec = (ldc & 3) == 0 && ((uintptr_t)C & 15) == 0;
             } else {
-                dst = ws + (size_t)sk_slot(cta, seg) * UM_BM * N;
+                dst = ws + ((size_t)sk_slot(pair, seg) * TM + rank * UM_BM) * N;
                 ld = N;
                 rows = UM_BM;
                 vec = true;
@@ -320,19 +403,23 @@ umma_sk_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
                 }
             }
             asm volatile("tcgen05.fence::before_thread_sync;");
-            mbar_arrive(&acce[b]);
+            mbar_arrive_cta0<PAIR>(&acce[b]);
             it += sg.n;
         }
     }
     asm volatile("tcgen05.fence::before_thread_sync;");
     __syncthreads();
+    if (PAIR) cluster_barrier();  // neither CTA's shared or tensor memory goes while the other's work may use it
     asm volatile("tcgen05.fence::after_thread_sync;");
-    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(tcols));
+    if (warp == 0) {
+        if (PAIR) asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(tcols));
+        else asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(tcols));
+    }
     if (threadIdx.x == 0 && timed_out) atomicExch(err, 1);
 }
 
-// Sums the pieces of every tile split between CTAs, in CTA order, into C.
-// CTA c owns iterations [c I / G, (c + 1) I / G); the CTAs that touch tile t
+// Sums the pieces of every tile split between pairs, in their order, into C.
+// Pair c owns iterations [c I / G, (c + 1) I / G); the pairs that touch tile t
 // are those owning its first and last iteration and the ones between.
 // Block (t, y) takes rows UM_FIX_ROWS y .. of tile t, one float4 column group
 // per thread.
@@ -341,7 +428,7 @@ __global__ void umma_sk_fixup_kernel(int M, int N, int bmt, int KB, long long it
     const int tile = blockIdx.x;
     int c_lo, c_hi;
     sk_tile_ctas(tile, KB, iters, G, &c_lo, &c_hi);
-    if (c_lo == c_hi) return;  // one CTA covered the tile and wrote C itself
+    if (c_lo == c_hi) return;  // one pair covered the tile and wrote C itself
     const int rows = min(bmt, M - tile * bmt), n4 = N / 4;
     const int rbeg = blockIdx.y * UM_FIX_ROWS, rend = min(rows, rbeg + UM_FIX_ROWS);
     for (int e = threadIdx.x; e < (rend - rbeg) * n4; e += blockDim.x) {
@@ -414,7 +501,7 @@ int sm_count(int *n) {
 // Launch plan of one product: persistent grid, ring depth, accumulator
 // columns and workspace (the pieces of split tiles).
 struct UmmaPlan {
-    int tiles = 0, KB = 0, grid = 0, stages = 0;
+    int cg = 1, tiles = 0, KB = 0, grid = 0, stages = 0;  // grid: ranges (CTAs or pairs)
     uint32_t ncols = 32;
     long long iters = 0;
     bool split = false;
@@ -425,7 +512,7 @@ static bool umma_shape_ok(int M, int N, int K) {
     return M > 0 && M % UM_BM == 0 && K > 0 && K % UM_BK == 0 && N >= 16 && N <= 256 && N % 16 == 0;
 }
 
-// One CTA per SM, but at least UM_MIN_ITERS K slices each.
+// One pair of CTAs per two SMs, but at least UM_MIN_ITERS K slices each.
 static int umma_plan(int M, int N, int K, UmmaPlan *p) {
     if (!umma_shape_ok(M, N, K)) {
         osrc_set_error("umma_gemm_bf16: unsupported shape");
@@ -434,21 +521,23 @@ static int umma_plan(int M, int N, int K, UmmaPlan *p) {
     int nsm = 0;
     OSRC_TRY(sm_count(&nsm));
     UmmaPlan q;
-    q.tiles = M / UM_BM;
+    q.cg = N > UM_PAIR_N ? 2 : 1;
+    const int tm = q.cg * UM_BM;
+    q.tiles = (M + tm - 1) / tm;
     q.KB = K / UM_BK;
     q.iters = (long long)q.tiles * q.KB;
     long long g = q.iters / UM_MIN_ITERS;
-    if (g > nsm) g = nsm;
+    if (g > nsm / q.cg) g = nsm / q.cg;
     if (g < 1) g = 1;
     q.grid = (int)g;
     while (q.ncols < (uint32_t)N) q.ncols <<= 1;
-    const size_t stage = (size_t)UM_BM * UM_BK * 2 + (size_t)N * UM_BK * 2;
+    const size_t stage = (size_t)UM_BM * UM_BK * 2 + (size_t)N / q.cg * UM_BK * 2;
     q.stages = (int)((UM_SMEM_MAX - UM_SMEM_FIXED) / stage);
     if (q.stages > UM_MAX_STAGES) q.stages = UM_MAX_STAGES;
     q.smem = UM_SMEM_FIXED + (size_t)q.stages * stage;
     for (int c = 1; c < q.grid && !q.split; ++c)
         if (sk_begin(c, q.iters, q.grid) % q.KB) q.split = true;
-    q.ws_floats = q.split ? (size_t)2 * q.grid * UM_BM * N : 0;
+    q.ws_floats = q.split ? (size_t)2 * q.grid * tm * N : 0;
     *p = q;
     return OSRC_OK;
 }
@@ -474,20 +563,39 @@ static int umma_gemm_run(const void *A, int M, int K, const void *Bm, int N, flo
     OSRC_TRY(get_encoder());
     CUtensorMap ma, mb;
     OSRC_TRY(make_map(&ma, A, M, K, UM_BM));
-    OSRC_TRY(make_map(&mb, Bm, N, K, N));
+    OSRC_TRY(make_map(&mb, Bm, N, K, N / p.cg));
     static PerDeviceOnce once;
     OSRC_TRY(per_device_once(once, [](int) -> int {
-        OSRC_CK(cudaFuncSetAttribute(umma_sk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        OSRC_CK(cudaFuncSetAttribute(umma_sk_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)UM_SMEM_MAX));
+        OSRC_CK(cudaFuncSetAttribute(umma_sk_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)UM_SMEM_MAX));
         return OSRC_OK;
     }));
-    umma_sk_kernel<<<p.grid, UM_THREADS, p.smem, st>>>(ma, mb, M, N, p.KB, p.iters, p.stages, p.ncols, C, ldc,
-                                                       ws, err);
+    if (p.cg == 2) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(2 * p.grid, 1, 1);
+        cfg.blockDim = dim3(UM_THREADS, 1, 1);
+        cfg.dynamicSmemBytes = p.smem;
+        cfg.stream = st;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = 2;
+        attr[0].val.clusterDim.y = 1;
+        attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        OSRC_CK(cudaLaunchKernelEx(&cfg, umma_sk_kernel<true>, ma, mb, M, N, p.KB, p.iters, p.stages, p.ncols, C, ldc,
+                                   ws, err));
+    } else {
+        umma_sk_kernel<false><<<p.grid, UM_THREADS, p.smem, st>>>(ma, mb, M, N, p.KB, p.iters, p.stages, p.ncols, C, ldc,
+                                                                 ws, err);
+    }
     OSRC_CK(cudaGetLastError());
     if (p.split) {
-        const dim3 fg(p.tiles, UM_BM / UM_FIX_ROWS);
+        const dim3 fg(p.tiles, p.cg * UM_BM / UM_FIX_ROWS);
         const bool vec = (ldc & 3) == 0 && ((uintptr_t)C & 15) == 0;
-        umma_sk_fixup_kernel<<<fg, 256, 0, st>>>(M, N, UM_BM, p.KB, p.iters, p.grid, ws, C, ldc, vec);
+        umma_sk_fixup_kernel<<<fg, 256, 0, st>>>(M, N, p.cg * UM_BM, p.KB, p.iters, p.grid, ws, C, ldc, vec);
         OSRC_CK(cudaGetLastError());
     }
     return OSRC_OK;

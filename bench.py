@@ -34,24 +34,24 @@ WORKLOAD = "sphere10242"
 METRIC = "OSRC-PMCHWT solves/s to 1e-5 residual"
 UNIT = "solves/s"
 TOL = 1e-5
-# FP32 flops (FMA = 2) of one far-field point pair, both wavenumbers, as the
-# factored evaluation of the far kernel performs it: 32 FMA, 14 MUL, 5 ADD
-# (distance, 1/r and 1/r^2, (y - x).n_x, k r for both k, cos and sin of both
-# phases scaled by 1/r, then the V, D-normal (scale k0^2 taken out per source
-# triangle), D-curl, H and T/K accumulations); 5 MUFU operations (1 rsqrt,
-# 2 sin, 2 cos) and their argument scaling come on top and are not counted.
-FLOPS_PER_PAIR = 83
+# executed FP32 flops (FMA = 2) of one ordered far-field point pair, both
+# wavenumbers, of the symmetric far kernel (meshes of 2048 triangles and more):
+# an unordered pair is evaluated once for both directions at 28 for its kernel
+# values (distance, 1/r and 1/r^2, k r for both k, cos and sin of both phases
+# scaled by 1/r, H), 46 for its share of the element matrices' contractions over
+# the two rules, 6 for finishing the matrices (per triangle pair / 36) and 8.7
+# per direction for applying them; 5 MUFU operations (1 rsqrt, 2 sin, 2 cos)
+# and their argument scaling come on top and are not counted.
+FLOPS_PER_PAIR = 49
 # nominal count for a per-operator evaluation (V, K, T, D separately per
 # wavenumber), reported beside the main figure
 FLOPS_PER_PAIR_NOMINAL = 176
-# executed FP32 flops per far point pair of the several-right-hand-side far
-# kernel: shared per pair (distance, 1/r, 1/r^2, (y - x).n_x, k r, scaled cos
-# and sin, the V / D-normal / D-curl / H combinations with the K and D-normal
-# triangle factors folded in, and negated imaginary parts: 16 FMA, 22 MUL,
-# 5 ADD), plus per right-hand side the four complex multiply-adds into u1, u2
-# (16 FMA)
-FLOPS_PER_PAIR_MULTI_SHARED = 59
-FLOPS_PER_PAIR_MULTI_RHS = 32
+# executed FP32 flops per ordered far point pair of the one-sided several-right-
+# hand-side kernel (launches of 6 to 8 vectors): kernel values and element
+# matrices, and per right-hand side their application; launches of up to 5
+# vectors share the first part between both directions of a pair
+FLOPS_PER_PAIR_MULTI_SHARED = 80.5
+FLOPS_PER_PAIR_MULTI_RHS = 8.7
 # GMRES iterations of this workload (measured on the GPU path; the oracle's
 # unrestarted GMRES needs the same count within +-2 at smaller sizes): used
 # to turn the oracle's sampled matvec rate into solves/s
@@ -774,11 +774,12 @@ def run_field(S, x, W, B):
 # --------------------------------------------------------------------------
 SMALL_WORKLOAD = "sphere642"
 LARGE_WORKLOAD = "bumpy80000"
-# FP32 flops per far point pair of the large-ka (centred) variant: the 83 of the
-# plain kernel less its 2 MUL for k r, plus 21 for the phase from the centroid
-# distance (3 ADD for the offsets, r^2 - r_c^2 in 2 x (1 MUL + 2 FMA) + 1 FMA,
-# 1 ADD and 1 MUL for r - r_c, one FMA per wavenumber for the phase)
-FLOPS_PER_PAIR_CENTRED = 102
+# executed FP32 flops per ordered far point pair of the large-ka (centred)
+# variant: half of 19 more per unordered pair (less 2 MUL for k r, plus 21 for
+# the phase from the centroid distance: 3 ADD for the offsets, r^2 - r_c^2 in
+# 2 x (1 MUL + 2 FMA) + 1 FMA, 1 ADD and 1 MUL for r - r_c, one FMA per
+# wavenumber for the phase)
+FLOPS_PER_PAIR_CENTRED = 58
 
 
 def run_small_dense(device):

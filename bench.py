@@ -56,11 +56,12 @@ FLOPS_PER_PAIR_MULTI_RHS = 8.7
 # unrestarted GMRES needs the same count within +-2 at smaller sizes): used
 # to turn the oracle's sampled matvec rate into solves/s
 REF_ITERATIONS = 47
-# DRAM bytes (read + write) of one far_kernel<0, 0, 0> launch at this
-# workload, from one ncu capture of this command (dram__bytes_read.sum
-# 15,393,536 + dram__bytes_write.sum 2,816, the ncu summary of the far kernel
-# kept with the profiles); to be retaken whenever the far kernel changes
-FAR_TRAFFIC_BYTES = 15396352
+# DRAM bytes (read + write) of one apply's two sym_kernel launches at this
+# workload, from one ncu capture (dram__bytes_read.sum 4,550,400 + 142,337,280,
+# dram__bytes_write.sum 81,699,072 + 75,492,096: the partial sums; the ncu
+# summary of the kernel is kept with the profiles); to be retaken whenever the
+# far kernel changes
+FAR_TRAFFIC_BYTES = 304078848
 
 
 def parse():
@@ -391,7 +392,7 @@ def run_ours(args, D):
         "roofline": {
             "bound": "alu", "kernel": "far_kernel",
             "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
-            "traffic": FAR_TRAFFIC_BYTES, "traffic_unit": "bytes per launch (ncu)",
+            "traffic": FAR_TRAFFIC_BYTES, "traffic_unit": "bytes per apply (ncu)",
             "flops_per_unit": FLOPS_PER_PAIR, "units_per_launch": far_pairs,
             "unit_def": "far point pair (test point, source point of triangles sharing no "
                         "vertex), both wavenumbers",

@@ -9,7 +9,7 @@
 //      over all source points staged through shared memory in tiles of triangles; both
 //      wavenumbers are evaluated from one distance; the source range is split
 //      over gridDim.y so that the grid fills every SM; partial sums per test
-//      point (u1, u2) and per test triangle (curl term) go to d_part, d_partA
+//      point (u1, u2) and per test triangle (curl term) go to d_part, d_partA1
 //      (no atomics); from SYM_MIN_NT on sym_kernel, which evaluates each pair of
 //      triangles once, as element matrices, for both directions, and takes
 //      several right-hand sides (farm_kernel: the same one-sided, for several

@@ -95,13 +95,15 @@ struct DBuf {
     size_t n = 0;
     osrc_ctx *ctx = nullptr;
     bool owned = true;
+    // on failure the buffer is empty (p null, n 0), whatever it held before
     int alloc(osrc_ctx *c, size_t count) {
         release();
         ctx = c;
-        n = count;
         owned = true;
         if (count == 0) return OSRC_OK;
-        return ctx_alloc(ctx, (void **)&p, count * sizeof(T));
+        const int s = ctx_alloc(ctx, (void **)&p, count * sizeof(T));
+        if (s == OSRC_OK) n = count;
+        return s;
     }
     void borrow(const DBuf &o) {
         release();

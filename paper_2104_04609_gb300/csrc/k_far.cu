@@ -1537,6 +1537,12 @@ static size_t farm_slots(const osrc_problem *pb) {
     return pb->far_sym && !pb->mesh->ctx->budget ? std::max(s, SYM_MULTI_SLOTS) : std::max(s, 2 * FARM_MAX_R);
 }
 
+// every buffer of the one-vector apply's path is there
+static bool far_workspace_made(const osrc_problem *pb) {
+    return pb->far_sym ? pb->d_sD.p && pb->d_part.p
+                       : pb->d_sP.p && pb->d_sP5.p && pb->d_sC.p && pb->d_part.p && pb->d_partA1.p;
+}
+
 int far_workspace(osrc_problem *pb) {
     osrc_ctx *ctx = pb->mesh->ctx;
     const size_t nt = pb->nt;
@@ -1616,7 +1622,7 @@ int far_setup_geometry(osrc_problem *pb, cudaStream_t st) {
     pb->far_sym = nt >= SYM_MIN_NT;
     static_assert(SYM_MAX_R < sizeof(pb->sym) / sizeof(pb->sym[0]), "a plan for every R");
     // on a context with a memory budget no more than far_kernel's buffers
-    const int one = m->ctx->budget ? std::max(2, std::min(SYM_MAX_SLOTS, (30 * ns + 116) / 18)) : SYM_MAX_SLOTS;
+    const int one = m->ctx->budget ? std::max(2, std::min(SYM_MAX_SLOTS, (30 * ns + 96) / 18)) : SYM_MAX_SLOTS;
     if (pb->far_sym)
         for (int r = 1; r <= SYM_MAX_R; ++r)
             pb->sym[r] = sym_plan(nt, sms, r == 1 ? one : (int)farm_slots(pb) / r);
@@ -1653,11 +1659,11 @@ static FarConst2 far_consts(const osrc_problem *pb, float4 &kff) {
 }
 
 // sD from the vectors and the launches of sym_kernel over all offsets
-static int sym_launch(osrc_problem *pb, const VecPtrs &xp, int R, const FarSymPlan &pl, float *part, cudaStream_t st) {
+static int sym_launch(osrc_problem *pb, const VecPtrs &xp, int R, const FarSymPlan &pl, float4 *sD, float *part,
+                      cudaStream_t st) {
     osrc_mesh *m = pb->mesh;
     const int nt = pb->nt, N = (nt + FAR_THREADS - 1) / FAR_THREADS, half = N / 2;
-    farm_prep_kernel<<<dim3((nt + 127) / 128, R), 128, 0, st>>>(xp, R, pb->nv, nt, m->d_tris.p, pb->d_tgeo.p,
-                                                               pb->d_sD.p);
+    farm_prep_kernel<<<dim3((nt + 127) / 128, R), 128, 0, st>>>(xp, R, pb->nv, nt, m->d_tris.p, pb->d_tgeo.p, sD);
     pb->launches++;
     float4 kff;
     const FarConst2 c = far_consts(pb, kff);
@@ -1674,7 +1680,7 @@ static int sym_launch(osrc_problem *pb, const VecPtrs &xp, int R, const FarSymPl
         const int count = d ? std::min(pl.nsrc, half + 1 - d) : pl.nsrc + 1;
         const dim3 grid(N, (4 * count + pl.ups - 1) / pl.ups);
 #define OSRC_SYM_LAUNCH(C, M, A, E)                                                                                \
-    sym_kernel<C, M, A, E><<<grid, FAR_THREADS, smem, st>>>(pts, pb->d_cen.p, pb->d_tn.p, pb->d_tv.p, pb->d_sD.p, R, \
+    sym_kernel<C, M, A, E><<<grid, FAR_THREADS, smem, st>>>(pts, pb->d_cen.p, pb->d_tn.p, pb->d_tv.p, sD, R, \
                                                             nt, d, count, pl.ups, pl.ntst, d ? 1 : 0, c, kff,       \
                                                             m->d_tcomp.p, pb->d_fobj.p, part)
         if (pb->far_reduce && pb->far_obj && pb->absorb) OSRC_SYM_LAUNCH(true, true, true, true);
@@ -1739,9 +1745,9 @@ int far_apply(osrc_problem *pb, const double2 *x, double2 *y, int part, cudaStre
     OutPtrs yp{};
     xp.p[0] = x;
     yp.p[0] = y;
-    if (use_far && !pb->d_part.p) OSRC_TRY(far_workspace(pb));  // a clone made without it
+    if (use_far && !far_workspace_made(pb)) OSRC_TRY(far_workspace(pb));  // a clone made without it
     if (use_far && pb->far_sym) {
-        OSRC_TRY(sym_launch(pb, xp, 1, pb->sym[1], pb->d_part.p, st));
+        OSRC_TRY(sym_launch(pb, xp, 1, pb->sym[1], pb->d_sD.p, pb->d_part.p, st));
         return gather_launch(pb, pb->sym[1].ntst + pb->sym[1].nsrc, 1, pb->d_part.p, nullptr, use_far, use_near, xp, yp, st);
     }
     if (use_far) {
@@ -1807,10 +1813,10 @@ static int farm_prepare(osrc_problem *pb, cudaStream_t st) {
         pb->launches++;
         OSRC_CK(cudaGetLastError());
     }
-    if (!pb->d_partm.p) {
-        OSRC_TRY(pb->d_sD.alloc(ctx, 5 * (size_t)nt * FARM_MAX_R));
-        OSRC_TRY(pb->d_partm.alloc(ctx, farm_slots(pb) * 18 * nt));
-    }
+    // buffers of its own: one-vector applies, also captured ones and those on
+    // another stream, keep d_sD and d_part whatever happens here
+    if (!pb->d_sDm.p) OSRC_TRY(pb->d_sDm.alloc(ctx, 5 * (size_t)nt * FARM_MAX_R));
+    if (!pb->d_partm.p) OSRC_TRY(pb->d_partm.alloc(ctx, farm_slots(pb) * 18 * nt));
     return OSRC_OK;
 }
 
@@ -1829,12 +1835,12 @@ static int farm_launch(osrc_problem *pb, const double2 *const *xs, double2 *cons
     const int ns = pb->nsplit;
     if (use_far && pb->far_sym && R <= SYM_MAX_R) {
         const FarSymPlan pl = pb->sym[R];
-        OSRC_TRY(sym_launch(pb, xp, R, pl, pb->d_partm.p, st));
+        OSRC_TRY(sym_launch(pb, xp, R, pl, pb->d_sDm.p, pb->d_partm.p, st));
         return gather_launch(pb, pl.ntst + pl.nsrc, R, pb->d_partm.p, nullptr, use_far, use_near, xp, yp, st);
     }
     if (use_far) {
         farm_prep_kernel<<<dim3((nt + 127) / 128, R), 128, 0, st>>>(xp, R, nv, nt, m->d_tris.p, pb->d_tgeo.p,
-                                                                   pb->d_sD.p);
+                                                                   pb->d_sDm.p);
         pb->launches++;
         float4 kff;
         const FarConst2 c = far_consts(pb, kff);
@@ -1848,7 +1854,7 @@ static int farm_launch(osrc_problem *pb, const double2 *const *xs, double2 *cons
         }
 #define OSRC_FARM_LAUNCH(C)                                                                                    \
     farm_kernel<C><<<grid, FAR_THREADS, smem, st>>>(pts, pb->d_cen.p, pb->d_tn.p, pb->d_tv.p, pb->d_sG.p,      \
-                                                    pb->d_sD.p, R, nt, tps, pb->far_tris, c, kff, pb->d_partm.p)
+                                                    pb->d_sDm.p, R, nt, tps, pb->far_tris, c, kff, pb->d_partm.p)
         if (pb->far_reduce) OSRC_FARM_LAUNCH(true);
         else OSRC_FARM_LAUNCH(false);
 #undef OSRC_FARM_LAUNCH

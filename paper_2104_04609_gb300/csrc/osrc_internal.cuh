@@ -195,6 +195,7 @@ struct osrc_problem {
     DBuf<float4> d_sP;   // [6nt][4] source points: -y, psi, phi as duplicated pairs
     DBuf<float2> d_sP5;  // [6nt] (-phi.im, -phi.im)
     DBuf<float4> d_sC;   // [nt][2] c_sigma components
+    DBuf<float4> d_sD;   // [5][nt] corner densities and curl source (far_sym)
     DBuf<float> d_part;       // [nsplit][4][6nt] per test point partial sums
     DBuf<float> d_partA1;     // [nsplit][6][nt] curl-term partial sums per test triangle
     int nsplit = 1, far_tris = 128;  // far kernel: source splits, test triangles per block
@@ -203,7 +204,7 @@ struct osrc_problem {
     int sms = 1;
     // ---- far field, several right-hand sides per launch (k_far.cu farm_*) ----
     DBuf<float4> d_sG;        // [6nt][2] static source geometry (coordinates)
-    DBuf<float4> d_sD;        // [nt][R][5] corner densities and curl sources of R right-hand sides
+    DBuf<float4> d_sDm;       // [R][5][nt] corner densities and curl sources of R right-hand sides
     DBuf<float> d_partm;      // [ns][R][18][nt] u1, u2 partial sums per corner, curl-term sums
     // when set and true, a lockstep GMRES on this problem stops at its next
     // iteration with OSRC_TIMEOUT (the serving loop's shutdown)

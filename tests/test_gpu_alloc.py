@@ -1,0 +1,132 @@
+"""Calls whose device memory runs out, on a context with a budget: they return
+OSRC_OUT_OF_MEMORY, again when repeated, and leave the handle as it was, so
+that an apply still gives the same bits and the call itself succeeds once
+there is room."""
+import contextlib
+
+import numpy as np
+import pytest
+
+from paper_2104_04609_gb300 import inputs
+
+pytestmark = pytest.mark.gpu
+
+BUDGET = 1 << 27
+
+
+@contextlib.contextmanager
+def _filled(B, S, leave):
+    """Takes up the context's budget but for about `leave` bytes (by meshes)."""
+    meshes = []
+    try:
+        for nv in (20000, 2000, 200, 20):
+            v, t = inputs.fibonacci_hull(nv)
+            while True:
+                before = B.osrc_mem_used(S.ctx)
+                if before + 160 * nv > BUDGET - leave:  # a mesh takes about 96 bytes a vertex
+                    break
+                meshes.append(B.osrc_mesh_create(S.ctx, v, t))
+                assert B.osrc_mem_used(S.ctx) - before <= 160 * nv
+        yield
+    finally:
+        for m in meshes:
+            B.osrc_mesh_destroy(m)
+
+
+def _runs_out(B, S, call, leave):
+    """call() fails twice with the budget nearly used up, the one-vector apply
+    is undisturbed in between, and afterwards call() succeeds."""
+    import torch
+
+    rng = np.random.default_rng(3)
+    n = 2 * S.nv
+    x = torch.from_numpy(rng.standard_normal((1, n)) + 1j * rng.standard_normal((1, n))).cuda()
+    ref = S.apply(x).cpu().numpy()
+    with _filled(B, S, leave):
+        for _ in range(2):
+            with pytest.raises(B.OsrcError) as e:
+                call()
+            assert e.value.status == B.OSRC_OUT_OF_MEMORY
+            assert np.array_equal(S.apply(x).cpu().numpy(), ref)
+    return call()
+
+
+@pytest.mark.parametrize("leave", [1 << 12, 1 << 18])
+def test_field(leave):
+    """Neither the source points' data (168 KB) nor the regions of 2e5 targets fit."""
+    import torch
+
+    import oracle as O
+    from paper_2104_04609_gb300 import binding as B
+
+    v, t = inputs.fibonacci_hull(150)
+    pts = np.random.default_rng(1).standard_normal((200000, 3))
+    pts *= 3.0 / np.linalg.norm(pts, axis=1)[:, None]
+    S = B.Solver(v, t, 2.0, 3.0, 1.5, mem_budget_bytes=BUDGET)
+    try:
+        x = torch.from_numpy(np.random.default_rng(2).standard_normal(2 * S.nv) + 0j).cuda()
+        p = torch.from_numpy(pts).cuda()
+        u = torch.zeros(len(pts), dtype=torch.complex128, device="cuda")
+        _runs_out(B, S, lambda: B.osrc_field_eval(S.pb, x, p, u, B.OSRC_INC_PLANEWAVE, [0, 0, 1.0]),
+                  leave)
+        got = u[:50].cpu().numpy()
+    finally:
+        S.close()
+    ref = O.field(v, t, 2.0, 3.0, 1.5, x.cpu().numpy(), pts[:50])[0]
+    assert np.abs(got - ref).max() < 1e-10 * np.abs(ref).max()
+
+
+# leave: nothing of the several-vector buffers, their densities only (1.5 MB),
+# all but the partial sums (44 MB)
+@pytest.mark.parametrize("leave", [1 << 14, 1 << 20, 3 << 20])
+@pytest.mark.parametrize("nv,nrhs", [(1155, 3), (1155, 8), (1155, 9)])
+def test_several_vectors(nv, nrhs, leave):
+    import torch
+
+    from paper_2104_04609_gb300 import binding as B
+
+    v, t = inputs.fibonacci_hull(nv)
+    rng = np.random.default_rng(nv + nrhs)
+    S = B.Solver(v, t, 3.0, 4.0, 1.5, mem_budget_bytes=BUDGET)
+    try:
+        x = torch.from_numpy(rng.standard_normal((nrhs, 2 * nv)) + 1j * rng.standard_normal((nrhs, 2 * nv))).cuda()
+        y = _runs_out(B, S, lambda: S.apply(x), leave).cpu().numpy()
+        one = np.concatenate([S.apply(x[r:r + 1]).cpu().numpy() for r in range(nrhs)])
+    finally:
+        S.close()
+    assert np.linalg.norm(y - one) < 1e-5 * np.linalg.norm(one)
+
+
+def test_one_vector_beside_several():
+    """A captured one-vector apply is replayed after the first several-vector
+    apply, and the two run on streams of their own: the same bits as alone."""
+    import torch
+
+    from paper_2104_04609_gb300 import binding as B
+
+    v, t = inputs.fibonacci_hull(1155)
+    rng = np.random.default_rng(5)
+    S = B.Solver(v, t, 3.0, 4.0, 1.5)
+    try:
+        x = torch.from_numpy(rng.standard_normal((4, 2 * S.nv)) + 1j * rng.standard_normal((4, 2 * S.nv))).cuda()
+        x1, y1 = x[:1].clone(), torch.empty_like(x[:1])
+        ref1 = S.apply(x1).cpu().numpy()
+        torch.cuda.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g):
+            B.osrc_pmchwt_apply(S.pb, x1, y1)
+        refm = S.apply(x).cpu().numpy()
+        g.replay()
+        assert np.array_equal(y1.cpu().numpy(), ref1)
+        s1, s2 = torch.cuda.Stream(), torch.cuda.Stream()
+        ym = torch.empty_like(x)
+        for _ in range(10):
+            y1.zero_()
+            ym.zero_()
+            torch.cuda.synchronize()
+            B.osrc_pmchwt_apply(S.pb, x, ym, 4, stream=s1)
+            B.osrc_pmchwt_apply(S.pb, x1, y1, 1, stream=s2)
+            torch.cuda.synchronize()
+            assert np.array_equal(ym.cpu().numpy(), refm) and np.array_equal(y1.cpu().numpy(), ref1)
+    finally:
+        S.close()

@@ -754,6 +754,7 @@ int ensure_gmres_workspace(osrc_problem *pb, int maxit) {
     osrc_ctx *ctx = pb->mesh->ctx;
     const size_t n = 2 * (size_t)pb->nv;
     if (pb->basis_cap < maxit) {
+        pb->basis_cap = 0;  // until all three are there
         pb->d_basis.release();
         pb->d_h.release();
         pb->d_givens.release();
@@ -762,14 +763,10 @@ int ensure_gmres_workspace(osrc_problem *pb, int maxit) {
         OSRC_TRY(pb->d_givens.alloc(ctx, 6 * (size_t)(maxit + 1)));
         pb->basis_cap = maxit;
     }
-    if (!pb->d_w.p) {
-        OSRC_TRY(pb->d_w.alloc(ctx, n));
-        OSRC_TRY(pb->d_npart.alloc(ctx, n / 256 + 1));
-        OSRC_TRY(pb->d_y.alloc(ctx, n));
-        OSRC_TRY(pb->d_cvec.alloc(ctx, n));
-        OSRC_TRY(pb->d_b1.alloc(ctx, n));
-        OSRC_TRY(pb->d_x1.alloc(ctx, n));
-    }
+    // each by itself: an earlier call may have run out of memory between two
+    for (DBuf<double2> *b : {&pb->d_w, &pb->d_y, &pb->d_cvec, &pb->d_b1, &pb->d_x1})
+        if (!b->p) OSRC_TRY(b->alloc(ctx, n));
+    if (!pb->d_npart.p) OSRC_TRY(pb->d_npart.alloc(ctx, n / 256 + 1));
     if (!pb->h_res)
         OSRC_CK(cudaMallocHost((void **)&pb->h_res, kHostDoubles * sizeof(double) + kHostInts * sizeof(int)));
     return OSRC_OK;

@@ -130,3 +130,29 @@ def test_one_vector_beside_several():
             assert np.array_equal(ym.cpu().numpy(), refm) and np.array_equal(y1.cpu().numpy(), ref1)
     finally:
         S.close()
+
+
+# the basis (101 KB) does not fit, or one of the vectors of 4800 bytes after it
+@pytest.mark.parametrize("leave", [1 << 12, 111000, 115000, 120000, 125000])
+def test_solve(leave):
+    import torch
+
+    from paper_2104_04609_gb300 import binding as B
+
+    v, t = inputs.fibonacci_hull(150)
+    S, T = (B.Solver(v, t, 2.0, 3.0, 1.5, mem_budget_bytes=b) for b in (BUDGET, 0))
+    try:
+        b = S.rhs_planewave([[0.0, 0.0, 1.0]])
+        x, info = _runs_out(B, S, lambda: S.solve(b, tol=1e-6, maxit=20, raise_on_nonconvergence=False), leave)
+        ref, _ = T.solve(b, tol=1e-6, maxit=20, raise_on_nonconvergence=False)
+        assert torch.equal(x, ref)
+        # growing the basis fails: the old one is gone, and the shorter solve makes it again
+        with _filled(B, S, 1 << 12):
+            with pytest.raises(B.OsrcError) as e:
+                S.solve(b, tol=1e-6, maxit=4000)
+            assert e.value.status == B.OSRC_OUT_OF_MEMORY
+            x, _ = S.solve(b, tol=1e-6, maxit=20, raise_on_nonconvergence=False)
+        assert torch.equal(x, ref)
+    finally:
+        S.close()
+        T.close()

@@ -21,6 +21,7 @@
 #include <algorithm>
 #include <chrono>
 #include <cmath>
+#include <memory>
 
 #include "osrc_internal.cuh"
 
@@ -882,10 +883,10 @@ void batched_free(BatchedState *s) { delete s; }
 int batched_prepare(osrc_problem *pb, int R, int maxit_inner, cudaStream_t st) {
     if (!pb->d_dense.p) return OSRC_UNSUPPORTED;
     osrc_ctx *ctx = pb->mesh->ctx;
-    BatchedState *&bs = pb->batched;
     const int nv = pb->nv, n2 = 2 * nv;
-    if (!bs) {
-        bs = new BatchedState;
+    if (!pb->batched) {
+        // the problem's only once it is complete (out of memory may end it anywhere)
+        std::unique_ptr<BatchedState> bs(new BatchedState);
         bs->n2 = n2;
         bs->Mp = (n2 + 127) / 128 * 128;
         bs->Kp = (2 * n2 + 63) / 64 * 64;
@@ -920,12 +921,13 @@ int batched_prepare(osrc_problem *pb, int R, int maxit_inner, cudaStream_t st) {
         OSRC_CK(cudaMemsetAsync(bs->err.p, 0, sizeof(int), st));
         pb->launches += 4;
         OSRC_CK(cudaGetLastError());
+        pb->batched = bs.release();
     }
+    BatchedState *bs = pb->batched;
     if (bs->R != R || bs->basis_cap < maxit_inner) {
         const size_t plane = (size_t)n2 * R, vplane = (size_t)nv * R;
         const int nsys = 2 * pb->p.n_pade + 2;
-        bs->R = R;
-        bs->basis_cap = maxit_inner;
+        bs->R = bs->basis_cap = 0;  // until all are there
         OSRC_TRY(bs->Bcat.alloc(ctx, (size_t)2 * R * bs->Kp));
         OSRC_CK(cudaMemsetAsync(bs->Bcat.p, 0, (size_t)2 * R * bs->Kp * sizeof(__nv_bfloat16), st));
         OSRC_TRY(bs->C.alloc(ctx, (size_t)bs->Mp * 2 * R));
@@ -954,6 +956,8 @@ int batched_prepare(osrc_problem *pb, int R, int maxit_inner, cudaStream_t st) {
         OSRC_TRY(bs->bn.alloc(ctx, R));
         OSRC_TRY(bs->rn.alloc(ctx, R));
         OSRC_TRY(bs->scl.alloc(ctx, R));
+        bs->R = R;
+        bs->basis_cap = maxit_inner;
     }
     return OSRC_OK;
 }
@@ -1078,10 +1082,9 @@ static int batched_inner_gmres(osrc_problem *pb, const float2 *c, float tol, int
     const int ldh = maxit + 1;
     const unsigned gp = (unsigned)((plane + 255) / 256);
     const int nchunk = std::max(1, std::min(BD_MAX_CHUNK, n2 / 64));
-    if (!bs->hdone) {
-        OSRC_CK(cudaMallocHost((void **)&bs->hdone, 2 * 128 * sizeof(int)));
-        for (auto &e : bs->ev) OSRC_CK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
-    }
+    if (!bs->hdone) OSRC_CK(cudaMallocHost((void **)&bs->hdone, 2 * 128 * sizeof(int)));
+    for (auto &e : bs->ev)
+        if (!e) OSRC_CK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
     auto dots = [&](int nvec, const float2 *w, float2 *out) {
         bdots_part_kernel<<<dim3(nchunk, (nvec + BD_VEC - 1) / BD_VEC), BD_THREADS, 0, st>>>(bs->V.p, plane, nvec, w,
                                                                                               n2, R, nchunk, bs->part.p);

@@ -156,3 +156,31 @@ def test_solve(leave):
     finally:
         S.close()
         T.close()
+
+
+# successive buffers of the packed system and of the block workspaces
+@pytest.mark.parametrize("leave", [1 << 14, 600000, 1960000, 2300000, 3000000, 3420000])
+def test_dense_batched(leave):
+    import torch
+
+    from paper_2104_04609_gb300 import binding as B
+
+    v, t = inputs.fibonacci_hull(150)
+    S, T = (B.Solver(v, t, 2.0, 3.0, 1.5, mem_budget_bytes=b, precision=B.OSRC_FP64_DENSE) for b in (BUDGET, 0))
+    try:
+        b = S.rhs_planewave(inputs.plane_wave_dirs(5, seed=2))
+        x, ref = torch.empty_like(b), torch.empty_like(b)
+        _runs_out(B, S, lambda: B.osrc_dense_batched_solve(S.pb, b, x, tol=1e-8, inner_maxit=40), leave)
+        B.osrc_dense_batched_solve(T.pb, b, ref, tol=1e-8, inner_maxit=40)
+        assert torch.equal(x, ref)
+        # a larger block fails: the next smaller one makes its workspace again
+        b2 = S.rhs_planewave(inputs.plane_wave_dirs(64, seed=3))
+        with _filled(B, S, 1 << 14):
+            with pytest.raises(B.OsrcError) as e:
+                B.osrc_dense_batched_solve(S.pb, b2, torch.empty_like(b2), tol=1e-8, inner_maxit=40)
+            assert e.value.status == B.OSRC_OUT_OF_MEMORY
+            B.osrc_dense_batched_solve(S.pb, b, x.zero_(), tol=1e-8, inner_maxit=40)
+        assert torch.equal(x, ref)
+    finally:
+        S.close()
+        T.close()

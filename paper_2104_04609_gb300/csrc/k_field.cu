@@ -31,6 +31,10 @@ constexpr int FT = 128;          // targets per block; source points per tile of
 constexpr int FTT = 16;          // source triangles per tile of the field pass
 constexpr int FIELD_TAB = 512;   // entries of the e^{i theta} table per turn
 constexpr int FIELD_MAX_SPLIT = 64;
+// most doubles of splits' sums (256 MB); beyond it, and where the memory is not
+// there, both passes run unsplit, which takes none (targets enough to reach it
+// fill the SMs without splits)
+constexpr size_t FIELD_MAX_SCRATCH = (size_t)1 << 25;
 
 // Source data per rule point (6 per triangle): {y, w |tau|}, {n, 0} and
 // {w psi_q re, im, w phi_q re, im} with w including the area.
@@ -60,15 +64,17 @@ __global__ void field_src_kernel(int nt, int nv, const int *__restrict__ tris, c
 
 // rtot[(split * nobj + m) * npts + i]: the split's share of the solid angle of
 // object m's surface at point i, sum_q w_q (y_q - x).n_q / r^3.  obeg:
-// [nobj + 1] source-point ranges of the objects.
+// [nobj + 1] source-point ranges of the objects.  One split (rtot null): the
+// regions themselves (see field_region).
 __global__ void __launch_bounds__(FT)
 field_region_kernel(int npts, const double *__restrict__ pts, int nobj, const int *__restrict__ obeg,
-                    const double4 *__restrict__ src, double *__restrict__ rtot) {
+                    const double4 *__restrict__ src, double *__restrict__ rtot, int *__restrict__ region) {
     __shared__ float4 sy[FT], sn[FT];
     const int i = blockIdx.x * FT + threadIdx.x;
     const bool valid = i < npts;
     const float x0 = valid ? (float)pts[3 * (size_t)i] : 0.f, x1 = valid ? (float)pts[3 * (size_t)i + 1] : 0.f,
                 x2 = valid ? (float)pts[3 * (size_t)i + 2] : 0.f;
+    int reg = 0;
     for (int m = 0; m < nobj; ++m) {
         const int b0 = obeg[m], b1 = obeg[m + 1];
         const long long tiles = (b1 - b0 + FT - 1) / FT;
@@ -93,8 +99,13 @@ field_region_kernel(int npts, const double *__restrict__ pts, int nobj, const in
             total += (double)acc;
             __syncthreads();
         }
-        if (valid) rtot[((size_t)blockIdx.y * nobj + m) * npts + i] = total;
+        if (!rtot) {
+            if (total * kFInv4Pi > 0.5) reg = m + 1;
+        } else if (valid) {
+            rtot[((size_t)blockIdx.y * nobj + m) * npts + i] = total;
+        }
     }
+    if (!rtot && valid) region[i] = reg;
 }
 
 // region of target i: the last object whose surface has a solid angle of more
@@ -144,8 +155,8 @@ field_kernel(int npts, const double *__restrict__ pts, int nt, int nobj, const i
     for (int j = threadIdx.x; j < FIELD_TAB; j += FT) sincospi(j * (2.0 / FIELD_TAB), &tab[j].y, &tab[j].x);
     const double x0 = valid ? pts[3 * (size_t)i] : 0.0, x1 = valid ? pts[3 * (size_t)i + 1] : 0.0,
                  x2 = valid ? pts[3 * (size_t)i + 2] : 0.0;
-    const int ins = valid ? field_region(i, npts, nobj, nrs, rtot) : 0;
-    if (valid && blockIdx.y == 0) region[i] = ins;
+    const int ins = !valid ? 0 : rtot ? field_region(i, npts, nobj, nrs, rtot) : region[i];
+    if (valid && rtot && blockIdx.y == 0) region[i] = ins;
     // outside: every source point, k0; inside object m: its own points, k_m
     const double k = ins ? obj[ins - 1].k1 : c.k0;
     const double ki = ins ? obj[ins - 1].k1i : 0.0;  // attenuation inside
@@ -225,10 +236,10 @@ field_kernel(int npts, const double *__restrict__ pts, int nt, int nobj, const i
     if (valid) part[(size_t)blockIdx.y * npts + i] = ins ? csub(cscale(S, obj[ins - 1].rho), D) : csub(D, S);
 }
 
-// u = sum of the splits / (4 pi), plus the incident field outside
-__global__ void field_finish_kernel(int npts, const double *__restrict__ pts, int nsplit,
-                                    const double2 *__restrict__ part, const int *__restrict__ region, FieldConst c,
-                                    double2 *__restrict__ u) {
+// u = sum of the splits / (4 pi), plus the incident field outside; a single
+// split's sums are in u already (part = u)
+__global__ void field_finish_kernel(int npts, const double *__restrict__ pts, int nsplit, const double2 *part,
+                                    const int *__restrict__ region, FieldConst c, double2 *u) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= npts) return;
     double2 out = cd(0, 0);
@@ -300,14 +311,21 @@ extern "C" int osrc_field_eval(osrc_problem *pb, const void *x, const double *pt
     auto fk = pb->absorb ? field_kernel<true> : field_kernel<false>;
     OSRC_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_r, field_region_kernel, FT, 0));
     OSRC_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_f, fk, FT, 0));
-    const int nrs = field_splits(nb, (ns / m->ncomp + FT - 1) / FT, sms * std::max(1, per_r), 1);
-    const int nfs = field_splits(nb, (nt + FTT - 1) / FTT, sms * std::max(1, per_f), 3);
+    int nrs = field_splits(nb, (ns / m->ncomp + FT - 1) / FT, sms * std::max(1, per_r), 1);
+    int nfs = field_splits(nb, (nt + FTT - 1) / FTT, sms * std::max(1, per_f), 3);
     // splits' sums: region [nrs][objects][npts], field [nfs][npts] complex
-    const size_t nr = (size_t)nrs * m->ncomp * npts, np = nr + (nr & 1) + 2 * (size_t)nfs * npts;
-    if (pb->d_fpart.n < np) OSRC_TRY(pb->d_fpart.alloc(m->ctx, np));
-    double *rtot = pb->d_fpart.p;
-    double2 *part = (double2 *)(rtot + nr + (nr & 1));
-    field_region_kernel<<<dim3(nb, nrs), FT, 0, st>>>(npts, pts, m->ncomp, pb->d_fobeg.p, pb->d_fsrc.p, rtot);
+    const size_t nr = nrs > 1 ? (size_t)nrs * m->ncomp * npts : 0;
+    const size_t np = nr + (nr & 1) + (nfs > 1 ? 2 * (size_t)nfs * npts : 0);
+    bool split = np <= FIELD_MAX_SCRATCH;
+    if (split && pb->d_fpart.n < np) {
+        const int s = pb->d_fpart.alloc(m->ctx, np);
+        if (s != OSRC_OK && s != OSRC_OUT_OF_MEMORY) return s;
+        split = s == OSRC_OK;
+    }
+    if (!split) nrs = nfs = 1;
+    double *rtot = nrs > 1 ? pb->d_fpart.p : nullptr;
+    double2 *part = nfs > 1 ? (double2 *)(pb->d_fpart.p + nr + (nr & 1)) : (double2 *)u;
+    field_region_kernel<<<dim3(nb, nrs), FT, 0, st>>>(npts, pts, m->ncomp, pb->d_fobeg.p, pb->d_fsrc.p, rtot, reg);
     FieldConst c{pb->p.k_ext, inc_kind, 0.0, 0.0, 0.0};
     if (inc_kind) {
         c.s0 = inc_param[0];

@@ -184,3 +184,37 @@ def test_dense_batched(leave):
     finally:
         S.close()
         T.close()
+
+
+@pytest.mark.parametrize("objects", [1, 2])
+@pytest.mark.parametrize("npts", [1, 1000, 20000])
+def test_field_without_room_for_splits(npts, objects):
+    """Room for the source points only: the field is evaluated without splits
+    over the sources, the regions the same and the values to FP64 rounding of
+    sums of up to 3528 terms (3528 x 1.1e-16 of their size, 4e-13)."""
+    import torch
+
+    from paper_2104_04609_gb300 import binding as B
+
+    v, t = inputs.fibonacci_hull(150)
+    obj = None
+    if objects == 2:
+        v, t = np.concatenate([v - [2.0, 0, 0], v + [2.0, 0, 0]]), np.concatenate([t, t + len(v)]).astype(np.int32)
+        obj = ([3.0, 1.2], [1.5, 0.8])
+    rng = np.random.default_rng(npts)
+    pts = rng.standard_normal((npts, 3))
+    pts *= (np.where(rng.random(npts) < 0.5, 0.15, 6.0) / np.linalg.norm(pts, axis=1))[:, None]
+    if objects == 2:
+        pts[:, 0] += np.where(np.linalg.norm(pts, axis=1) < 1.0, rng.choice([-2.0, 2.0], npts), 0.0)
+    S, T = (B.Solver(v, t, 2.0, 3.0, 1.5, mem_budget_bytes=b, objects=obj) for b in (BUDGET, 0))
+    try:
+        x = torch.from_numpy(rng.standard_normal(2 * S.nv) + 1j * rng.standard_normal(2 * S.nv)).cuda()
+        p = torch.from_numpy(pts).cuda()
+        with _filled(B, S, 6 * len(t) * 96 + 64):
+            u, reg = S.field(x, p, B.OSRC_INC_PLANEWAVE, [0, 0, 1.0])
+        ref, regref = T.field(x, p, B.OSRC_INC_PLANEWAVE, [0, 0, 1.0])
+        assert torch.equal(reg, regref)
+        assert float((u - ref).abs().max() / ref.abs().max()) < 4e-13
+    finally:
+        S.close()
+        T.close()

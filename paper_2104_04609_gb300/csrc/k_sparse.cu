@@ -26,6 +26,7 @@
 #include <algorithm>
 #include <mutex>
 
+#include "bounded_wait.cuh"
 #include "osrc_internal.cuh"
 
 namespace cg = cooperative_groups;
@@ -339,28 +340,42 @@ struct KmixBox {
     T wred[NV][32];  // the CTA's warp sums
 };
 
-constexpr unsigned long long KMIX_TIMEOUT_NS = 2000000000ULL;
+#ifndef OSRC_KMIX_TIMEOUT_NS  // (tests of the give-up path set a short one)
+#define OSRC_KMIX_TIMEOUT_NS 2000000000ULL
+#endif
+constexpr unsigned long long KMIX_TIMEOUT_NS = OSRC_KMIX_TIMEOUT_NS;
+constexpr unsigned long long KMIX_DRAIN_NS = 1000000ULL;
 
-// waits for phase `parity`, at most KMIX_TIMEOUT_NS of global time
-__device__ __forceinline__ bool kmix_wait(uint32_t bar, uint32_t parity) {
-    unsigned long long t0 = 0;
-    for (int i = 0;; ++i) {
-        uint32_t done;
-        asm volatile(
-            "{\n\t.reg .pred p;\n\t"
-            "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
-            "selp.u32 %0, 1, 0, p;\n\t}"
-            : "=r"(done)
-            : "r"(bar), "r"(parity)
-            : "memory");
-        if (done) return true;
-        if ((i & 1023) == 1023) {
-            unsigned long long t;
-            asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-            if (!t0) t0 = t;
-            else if (t - t0 > KMIX_TIMEOUT_NS) return false;
-        }
-    }
+__device__ __forceinline__ unsigned long long kmix_ns() {
+    unsigned long long t;
+    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+    return t;
+}
+
+// the CTA's threads that have given up the present wait
+struct KmixCount {
+    int *p;
+    __device__ int load() const { return *(volatile int *)p; }
+    __device__ void add() const { atomicAdd(p, 1); }
+    __device__ bool cas(int e, int v) const { return atomicCAS(p, e, v) == e; }
+};
+
+// waits for phase `parity`, at most KMIX_TIMEOUT_NS of global time; the same
+// result in every thread of the CTA
+__device__ __forceinline__ bool kmix_wait(uint32_t bar, uint32_t parity, int *gave) {
+    return bounded_wait(
+        [&] {
+            uint32_t done;
+            asm volatile(
+                "{\n\t.reg .pred p;\n\t"
+                "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+                "selp.u32 %0, 1, 0, p;\n\t}"
+                : "=r"(done)
+                : "r"(bar), "r"(parity)
+                : "memory");
+            return done != 0;
+        },
+        kmix_ns, KmixCount{gave}, blockDim.x, KMIX_TIMEOUT_NS);
 }
 
 // store to the cluster's shared memory, its bytes counted by the mbarrier bar
@@ -390,11 +405,11 @@ __device__ __forceinline__ uint32_t kmix_mapa(uint32_t a, uint32_t rank) {
 // every CTA: the warps' sums meet in shared memory, warp 0 (CL; else every
 // warp) adds them, and the ranks' sums are added in the same order everywhere.
 // parity: phase of the box's next use, flipped here; extra: bytes that other
-// CTAs send with this sum besides the sums.  *dead is set when a wait gave up;
-// the waits after it are skipped.
+// CTAs send with this sum besides the sums.  False, in every thread of the CTA,
+// when the wait gave up: v is not a sum then, and the CTA goes to kmix_meet.
 template <bool CL, typename T, int NV>
-__device__ __forceinline__ void kmix_csum(unsigned cs, unsigned rank, T (&v)[NV], KmixBox<T, NV> *box, uint32_t &parity,
-                                          uint32_t extra, volatile int *dead) {
+__device__ __forceinline__ bool kmix_csum(unsigned cs, unsigned rank, T (&v)[NV], KmixBox<T, NV> *box, uint32_t &parity,
+                                          uint32_t extra, int *gave) {
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const int k = kmix_slot(lane);
     T a = kmix_wsum<T, NV>(v, lane);
@@ -418,11 +433,15 @@ __device__ __forceinline__ void kmix_csum(unsigned cs, unsigned rank, T (&v)[NV]
 #pragma unroll
             for (int i = 0; i < NV; ++i) {
                 const T w = __shfl_sync(0xffffffffu, a, (i >> 1) | ((i & 1) << 1));
+#ifdef OSRC_KMIX_MUTE  // tests: sums that a rank leaves out
+                if (OSRC_KMIX_MUTE(rank, to, i)) continue;
+#endif
                 if ((unsigned)lane < cs) kmix_send(rslot + (uint32_t)(i * 16 * sizeof(T)), rbar, w);
             }
         }
-        if (!*dead && !kmix_wait(bar, parity)) *dead = 1;
+        const bool here = kmix_wait(bar, parity, gave);
         __syncwarp();
+        if (!here) return false;
         parity ^= 1u;
 #pragma unroll
         for (int i = 0; i < NV; ++i) v[i] = (unsigned)lane < cs ? box->slot[i][lane] : T(0);
@@ -430,6 +449,26 @@ __device__ __forceinline__ void kmix_csum(unsigned cs, unsigned rank, T (&v)[NV]
     }
 #pragma unroll
     for (int i = 0; i < NV; ++i) v[i] = __shfl_sync(0xffffffffu, a, (i >> 1) | ((i & 1) << 1));
+    return true;
+}
+
+// A cluster barrier, the nth of this kernel, at which CTAs that go on (lost
+// false) learn of those that gave up a wait (lost true): true when any has.  The
+// latter leave n in every CTA's word `lost_at` before they arrive.  A CTA that
+// gives up has no further barrier before this one, and whichever the others come
+// to next (x published, the end; a CTA that waits for the lost one's sums gives
+// up itself) is the same nth, so all of them leave together, none writes to a CTA
+// that is gone, and a word written for a later barrier (n + 1 by a CTA that has
+// gone on already) is not taken for this one's.  Copies still on their way have
+// been issued by then: they get KMIX_DRAIN_NS, a thousand times a copy's latency,
+// to land before the CTAs exit.
+__device__ __forceinline__ bool kmix_meet(cg::cluster_group &cl, unsigned cs, int n, bool lost, int *lost_at) {
+    if (lost && threadIdx.x < cs) *(volatile int *)cl.map_shared_rank(lost_at, threadIdx.x) = n;
+    cl.sync();
+    const int at = *(volatile int *)lost_at;
+    if (at == 0 || at > n) return false;
+    for (const unsigned long long t0 = kmix_ns(); kmix_ns() - t0 < KMIX_DRAIN_NS;) {}
+    return true;
 }
 
 __device__ __forceinline__ float2 f2mul(float2 a, float2 b) {
@@ -467,8 +506,7 @@ kmix_kernel(const __grid_constant__ KryBatch batch, int n, const int *__restrict
     __shared__ KmixBox<float, 2> boxP;
     __shared__ KmixBox<float, 3> boxR, boxI;
     __shared__ KmixBox<double, 1> boxD, boxB;
-    __shared__ int s_dead, s_cnt;
-    volatile int *dead = &s_dead;
+    __shared__ int s_gave, s_lost, s_cnt;
     uint32_t phP = 0, phR = 0, phI = 0, phD = 0, phB = 0;
     cg::cluster_group cl = cg::this_cluster();
     const unsigned cs = CL ? cl.num_blocks() : 1u, rank = CL ? cl.block_rank() : 0u;
@@ -478,7 +516,7 @@ kmix_kernel(const __grid_constant__ KryBatch batch, int n, const int *__restrict
     double2 *xg = sy.x;
     const int cj = sy.conj;
     if (threadIdx.x == 0) {
-        s_dead = 0;
+        s_gave = s_lost = 0;
         if (CL) {
             uint64_t *bars[5] = {&boxP.bar, &boxR.bar, &boxI.bar, &boxD.bar, &boxB.bar};
             for (uint64_t *b : bars)
@@ -580,14 +618,16 @@ kmix_kernel(const __grid_constant__ KryBatch batch, int n, const int *__restrict
                 kmix_send(kmix_mapa(zbase + 8u * (uint32_t)ci, to), kmix_mapa(bar, to), z[k]);
             }
     };
+    bool lost = false, left = false;  // a wait gave up, here or (left) anywhere; both the same in the whole CTA
+    int meets = 0;
     {   // its wait also ends the other CTAs' clearing of their copies
         double v[1] = {bb};
-        kmix_csum<CL, double, 1>(cs, rank, v, &boxB, phB, 0u, dead);
+        lost = !kmix_csum<CL, double, 1>(cs, rank, v, &boxB, phB, 0u, &s_gave);
         bb = v[0];
     }
     double rr = bb;
     int its = 0, status = 0;  // 0 converged, 1 not converged, 2 breakdown
-    if (bb > 0.0) {
+    if (!lost && bb > 0.0) {
         status = 1;
         for (int ref = 0; ref < KMIX_MAX_REFINE && its < maxit; ++ref) {
             // FP32 solve of A d = r / |r|
@@ -611,7 +651,8 @@ kmix_kernel(const __grid_constant__ KryBatch batch, int n, const int *__restrict
                     v3[2] += r[k].x * r[k].x + r[k].y * r[k].y;
                 }
             }
-            kmix_csum<CL, float, 3>(cs, rank, v3, &boxI, phI, zbytes, dead);  // also publishes z
+            lost = !kmix_csum<CL, float, 3>(cs, rank, v3, &boxI, phI, zbytes, &s_gave);  // also publishes z
+            if (lost) break;
             float2 rho = make_float2(v3[0], v3[1]), be = make_float2(0.f, 0.f);
             const float rr0 = v3[2];
             bool brk = false;
@@ -642,7 +683,8 @@ kmix_kernel(const __grid_constant__ KryBatch batch, int n, const int *__restrict
                         v2[1] += t.y;
                     }
                 }
-                kmix_csum<CL, float, 2>(cs, rank, v2, &boxP, phP, 0u, dead);  // every CTA has read its columns
+                lost = !kmix_csum<CL, float, 2>(cs, rank, v2, &boxP, phP, 0u, &s_gave);  // every CTA has read its columns
+                if (lost) break;
                 const float2 pq = make_float2(v2[0], v2[1]);
                 if (!(pq.x * pq.x + pq.y * pq.y > 0.f)) { brk = true; break; }
                 const float2 al = f2div(rho, pq), mal = make_float2(-al.x, -al.y);
@@ -660,15 +702,16 @@ kmix_kernel(const __grid_constant__ KryBatch batch, int n, const int *__restrict
                         w3[2] += r[k].x * r[k].x + r[k].y * r[k].y;
                     }
                 }
-                kmix_csum<CL, float, 3>(cs, rank, w3, &boxR, phR, zbytes, dead);
+                lost = !kmix_csum<CL, float, 3>(cs, rank, w3, &boxR, phR, zbytes, &s_gave);
+                if (lost) break;
                 ++its;
-                if (CL && *dead) { brk = true; break; }
                 if (w3[2] <= itol * itol * rr0) break;
                 if (!(rho.x * rho.x + rho.y * rho.y > 0.f)) { brk = true; break; }
                 const float2 rz = make_float2(w3[0], w3[1]);
                 be = f2div(rz, rho);
                 rho = rz;
             }
+            if (lost) break;
             if (brk) { status = 2; break; }
             // FP64 update and residual
             const double back = sqrt(rr);
@@ -678,8 +721,8 @@ kmix_kernel(const __grid_constant__ KryBatch batch, int n, const int *__restrict
                     const double2 dx = cd((double)d[k].x * back, (double)d[k].y * back);
                     xg[row[k]] = ref ? cadd(xg[row[k]], dx) : dx;
                 }
-            if (CL) cl.sync();  // x published
-            else __syncthreads();
+            if (!CL) __syncthreads();
+            else if ((left = kmix_meet(cl, cs, ++meets, false, &s_lost))) break;  // x published
             double rn = 0.0;
 #pragma unroll
             for (int k = 0; k < RPT; ++k) {
@@ -699,21 +742,23 @@ kmix_kernel(const __grid_constant__ KryBatch batch, int n, const int *__restrict
                 rn += cabs2(r64[k]);
             }
             double v[1] = {rn};
-            kmix_csum<CL, double, 1>(cs, rank, v, &boxD, phD, 0u, dead);
+            lost = !kmix_csum<CL, double, 1>(cs, rank, v, &boxD, phD, 0u, &s_gave);
+            if (lost) break;
             const double rprev = rr;
             rr = v[0];
             if (rr <= tol * tol * bb) { status = 0; break; }
             if (!(rr <= 0.25 * rprev)) break;  // refinement stagnates (or NaN): not converged
         }
-    } else {
+    } else if (!lost) {
         rr = 0.0;
 #pragma unroll
         for (int k = 0; k < RPT; ++k)
             if (ok[k]) xg[row[k]] = cd(0.0, 0.0);
     }
-    if (CL) cl.sync();  // keep shared memory alive until every CTA has read it
+    // the end: shared memory stays until every CTA has read it
+    if (CL && !left) left = kmix_meet(cl, cs, ++meets, lost, &s_lost);
     if (rank == 0 && threadIdx.x == 0) {
-        *sy.stat = status == 0 ? its : (status == 1 ? -its : -1000000 - its);
+        *sy.stat = left ? KRY_LOST : status == 0 ? its : (status == 1 ? -its : -1000000 - its);
         *sy.res = bb > 0.0 ? sqrt(rr / bb) : 0.0;
     }
 }
@@ -1055,13 +1100,10 @@ static int mass_solve_async(osrc_problem *pb, const double2 *y, double2 *z, bool
 
 int kry_status_host(osrc_problem *pb, const int *stat, int nsys) {
     int worst = 0;
-    for (int i = 0; i < nsys; ++i) {
-        if (stat[i] <= -1000000) return OSRC_BREAKDOWN;
-        if (stat[i] < 0) return OSRC_NOT_CONVERGED;
-        if (stat[i] > worst) worst = stat[i];
-    }
-    if (worst > pb->inner_last_max) pb->inner_last_max = worst;
-    return OSRC_OK;
+    const int s = kry_stat_code(stat, nsys, &worst);
+    if (s == OSRC_TIMEOUT) osrc_set_error("inner solve: a bounded wait gave up");
+    if (s == OSRC_OK && worst > pb->inner_last_max) pb->inner_last_max = worst;
+    return s;
 }
 
 int osrc_precond_fused(osrc_problem *pb, const double2 *y, double2 *z, cudaStream_t st) {

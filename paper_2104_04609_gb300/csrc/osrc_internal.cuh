@@ -308,6 +308,19 @@ int osrc_precond_fused_async(osrc_problem *pb, const double2 *y, double2 *z, cud
 int osrc_precond_fused_multi(osrc_problem *const *pbs, const double2 *const *ys, double2 *const *zs, int nrun,
                              cudaStream_t st);
 int osrc_precond_nsys(const osrc_problem *pb);
+// a system's status word: iterations when it converged, -iterations when not,
+// -1000000 - iterations after a breakdown, KRY_LOST when a bounded wait gave up
+constexpr int KRY_LOST = INT32_MIN;
+// the first failure's status code, or OSRC_OK; *worst: the most iterations so far
+inline int kry_stat_code(const int *stat, int nsys, int *worst) {
+    for (int i = 0; i < nsys; ++i) {
+        if (stat[i] == KRY_LOST) return OSRC_TIMEOUT;
+        if (stat[i] <= -1000000) return OSRC_BREAKDOWN;
+        if (stat[i] < 0) return OSRC_NOT_CONVERGED;
+        if (stat[i] > *worst) *worst = stat[i];
+    }
+    return OSRC_OK;
+}
 // turns a host copy of the inner status words into a status code
 int kry_status_host(osrc_problem *pb, const int *stat, int nsys);
 

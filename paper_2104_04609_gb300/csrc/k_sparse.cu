@@ -292,13 +292,12 @@ kry_kernel(const __grid_constant__ KryBatch batch, int n, const int *__restrict_
 // One preconditioner apply (10 systems; before: three cluster barriers an
 // iteration, the search direction in L2, entries in shared memory): 10242
 // vertices 0.37 ms (0.66), 2562 0.26 (0.59), 642 0.20 (0.37), 150 0.13 (0.29).
-constexpr int KMIX_E = 8;                  // matrix entries of a row kept in registers
 constexpr int KMIX_THREADS1 = 768;         // most threads with one row each (80 registers)
 constexpr int KMIX_THREADS2 = 640;         // and with two (96)
 constexpr float KMIX_MIN_TOL = 2e-6f;      // most a FP32 solve reduces the residual by
 constexpr int KMIX_MAX_REFINE = 40;
-constexpr int KMIX_SMEM_MAX = 200 * 1024;  // bytes of z
-constexpr int KMIX_MAX_N = KMIX_SMEM_MAX / 8;  // rows (also below 2^16: the column places are 16 bits)
+constexpr int KMIX_MAX_N = 25600;          // rows (below 2^16: the column places are 16 bits)
+constexpr int KMIX_SMEM_MAX = 224 * 1024;  // bytes of z and of the long rows' entries
 
 // Sum of NV <= 4 values over the warp by halving (each exchange hands half of
 // the values to the other lane: 6 shuffles for 3 or 4 values instead of 5 per
@@ -491,22 +490,29 @@ __device__ __forceinline__ float2 f2fma(float2 a, float2 b, float2 c) {
 
 // One cluster (CL) or CTA per system; CTA rank r owns the rows perm[r rows ..
 // (r + 1) rows).  Dynamic shared memory: z by row number (the CTA's own rows
-// and those its columns name).  sy.x holds
-// the published FP64 solution.  Status and residual as kry_kernel; the
+// and those its columns name), then the entries of its rows past the KMIX_E
+// that a thread holds, and their columns' places (long_cap of each).  One such
+// row sets an iteration's time: a preconditioner apply on a UV sphere with poles
+// of degree 64 (1986 vertices) takes 1.37 ms with them in shared memory and took
+// 3.33 when each iteration read them from the FP64 matrices, a Menger sponge with
+// 40 % rows of 9 to 11 entries (896 vertices) 0.31 and 0.47.
+// sy.x holds the published FP64 solution.  Status and residual as kry_kernel; the
 // iteration count is the number of FP32 iterations over all refinements.
 template <int RPT, bool CL>
 __global__ void __launch_bounds__(RPT == 1 ? KMIX_THREADS1 : KMIX_THREADS2, 1)
 kmix_kernel(const __grid_constant__ KryBatch batch, int n, const int *__restrict__ ptr, const int *__restrict__ col,
             const double *__restrict__ M, const double *__restrict__ S, const int *__restrict__ perm,
-            const int *__restrict__ inv, double tol, int maxit) {
+            const int *__restrict__ inv, int long_cap, double tol, int maxit) {
     extern __shared__ __align__(16) float2 zs[];
+    float2 *la = zs + n;
+    uint16_t *lc = reinterpret_cast<uint16_t *>(la + long_cap);
     // the sums of an iteration, of a refinement's start, of its end and of the
     // start: boxes of their own, so that none is written before the barrier
     // after its last reading
     __shared__ KmixBox<float, 2> boxP;
     __shared__ KmixBox<float, 3> boxR, boxI;
     __shared__ KmixBox<double, 1> boxD, boxB;
-    __shared__ int s_gave, s_lost, s_cnt;
+    __shared__ int s_gave, s_lost, s_cnt, s_long;
     uint32_t phP = 0, phR = 0, phI = 0, phD = 0, phB = 0;
     cg::cluster_group cl = cg::this_cluster();
     const unsigned cs = CL ? cl.num_blocks() : 1u, rank = CL ? cl.block_rank() : 0u;
@@ -516,7 +522,7 @@ kmix_kernel(const __grid_constant__ KryBatch batch, int n, const int *__restrict
     double2 *xg = sy.x;
     const int cj = sy.conj;
     if (threadIdx.x == 0) {
-        s_gave = s_lost = 0;
+        s_gave = s_lost = s_long = 0;
         if (CL) {
             uint64_t *bars[5] = {&boxP.bar, &boxR.bar, &boxI.bar, &boxD.bar, &boxB.bar};
             for (uint64_t *b : bars)
@@ -536,11 +542,11 @@ kmix_kernel(const __grid_constant__ KryBatch batch, int n, const int *__restrict
     // places of its columns' z (the FP64 solution lives in sy.x, the right-hand
     // side is read again when needed); who: the other ranks that need its z,
     // which are the owners of its columns (the pattern is symmetric)
-    int row[RPT], deg[RPT];
+    int row[RPT], nlong[RPT], at[RPT];  // entries past KMIX_E, the first one's place in la, lc
     uint32_t who[RPT];
     bool ok[RPT];
     double2 r64[RPT];
-    float2 a[RPT][KMIX_E], be0[RPT];
+    float2 a[RPT][KMIX_E];
     uint16_t ad[RPT][KMIX_E];
     float2 dinv[RPT], d[RPT], r[RPT], z[RPT], p[RPT], q[RPT];
     for (int i = threadIdx.x; i < n; i += blockDim.x) zs[i] = make_float2(0.f, 0.f);
@@ -551,9 +557,9 @@ kmix_kernel(const __grid_constant__ KryBatch batch, int n, const int *__restrict
         const int li = threadIdx.x + k * blockDim.x, i = r0 + li;
         ok[k] = i < r1;
         row[k] = ok[k] ? perm[i] : 0;
-        deg[k] = 0;
+        nlong[k] = at[k] = 0;
         r64[k] = cd(0.0, 0.0);
-        dinv[k] = be0[k] = make_float2(0.f, 0.f);
+        dinv[k] = make_float2(0.f, 0.f);
 #pragma unroll
         for (int e = 0; e < KMIX_E; ++e) {
             a[k][e] = make_float2(0.f, 0.f);
@@ -562,29 +568,33 @@ kmix_kernel(const __grid_constant__ KryBatch batch, int n, const int *__restrict
         who[k] = 0;
         if (ok[k]) {
             const double2 b64 = sy.bscale ? cmul(sy.beta, sy.bscale[batch.vcomp[row[k]]]) : sy.beta;
-            be0[k] = make_float2((float)b64.x, (float)b64.y);
-            const int p0 = ptr[row[k]];
-            deg[k] = ptr[row[k] + 1] - p0;
+            const float2 be0 = make_float2((float)b64.x, (float)b64.y);
+            const int p0 = ptr[row[k]], deg = ptr[row[k] + 1] - p0;
             float2 dg = make_float2(0.f, 0.f);
 #pragma unroll
             for (int e = 0; e < KMIX_E; ++e)
-                if (e < deg[k]) {
+                if (e < deg) {
                     const int c = col[p0 + e];
                     const float m = (float)M[p0 + e], s = (float)S[p0 + e];
-                    a[k][e] = make_float2(fmaf(be0[k].x, s, al0.x * m), fmaf(be0[k].y, s, al0.y * m));
+                    a[k][e] = make_float2(fmaf(be0.x, s, al0.x * m), fmaf(be0.y, s, al0.y * m));
                     const int ci = inv[c];
                     ad[k][e] = (uint16_t)ci;
                     who[k] |= 1u << (ci / rows);
                     if (CL && ci / rows != (int)rank) zs[ci].x = 1.f;  // mark: sent by its owner
                     if (c == row[k]) dg = a[k][e];
                 }
-            for (int e = KMIX_E; e < deg[k]; ++e) {
-                const int ci = inv[col[p0 + e]];
-                who[k] |= 1u << (ci / rows);
-                if (CL && ci / rows != (int)rank) zs[ci].x = 1.f;
-                if (col[p0 + e] == row[k]) {
-                    const float m = (float)M[p0 + e], s = (float)S[p0 + e];
-                    dg = make_float2(fmaf(be0[k].x, s, al0.x * m), fmaf(be0[k].y, s, al0.y * m));
+            if (deg > KMIX_E) {
+                nlong[k] = deg - KMIX_E;
+                at[k] = atomicAdd(&s_long, nlong[k]);
+                for (int e = 0; e < nlong[k]; ++e) {
+                    const int pe = p0 + KMIX_E + e, ci = inv[col[pe]];
+                    const float m = (float)M[pe], s = (float)S[pe];
+                    const float2 ae = make_float2(fmaf(be0.x, s, al0.x * m), fmaf(be0.y, s, al0.y * m));
+                    la[at[k] + e] = ae;
+                    lc[at[k] + e] = (uint16_t)ci;
+                    who[k] |= 1u << (ci / rows);
+                    if (CL && ci / rows != (int)rank) zs[ci].x = 1.f;
+                    if (col[pe] == row[k]) dg = ae;
                 }
             }
             who[k] &= ~(1u << rank);
@@ -668,14 +678,8 @@ kmix_kernel(const __grid_constant__ KryBatch batch, int n, const int *__restrict
                         s0 = f2fma(a[k][e], zs[ad[k][e]], s0);
                         s1 = f2fma(a[k][e + 1], zs[ad[k][e + 1]], s1);
                     }
-                    if (deg[k] > KMIX_E) {  // entries past the registers
-                        const int p0 = ptr[row[k]];
-                        for (int e = KMIX_E; e < deg[k]; ++e) {
-                            const float m = (float)M[p0 + e], s = (float)S[p0 + e];
-                            const float2 ae = make_float2(fmaf(be0[k].x, s, al0.x * m), fmaf(be0[k].y, s, al0.y * m));
-                            s0 = f2fma(ae, zs[inv[col[p0 + e]]], s0);
-                        }
-                    }
+#pragma unroll 4
+                    for (int e = 0; e < nlong[k]; ++e) s0 = f2fma(la[at[k] + e], zs[lc[at[k] + e]], s0);
                     q[k] = f2fma(be, q[k], make_float2(s0.x + s1.x, s0.y + s1.y));
                     if (ok[k]) {
                         const float2 t = f2dot(p[k], q[k], cj);
@@ -865,16 +869,22 @@ int cluster_size_for(int n) {
 // 1.85 us (cluster) of sums plus 1.3 ns per row of a CTA, times the load of the
 // device beyond one wave (the average system takes about 0.6 of the hardest
 // one's iterations and the hardest start first).
+// Shared memory holds z and, where the mesh has rows of more than KMIX_E
+// entries, what a CTA's rows have beyond them.
 struct KmixPlan {
-    int nsys = 0, cs = 0, rpt = 0, threads = 0;
+    int nsys = 0, cs = 0, rpt = 0, threads = 0, long_cap = 0;
 };
 
+size_t kmix_smem(int n, int long_cap) {
+    return (size_t)n * sizeof(float2) + (size_t)long_cap * (sizeof(float2) + sizeof(uint16_t));
+}
+
 template <int RPT, bool CL>
-int kmix_active_clusters(int n, int cs, int threads, int *count) {
+int kmix_active_clusters(size_t smem, int cs, int threads, int *count) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(cs, 1, 1);
     cfg.blockDim = dim3(threads, 1, 1);
-    cfg.dynamicSmemBytes = (size_t)n * sizeof(float2);
+    cfg.dynamicSmemBytes = smem;
     if (!CL) {
         int per_sm = 0, dev = 0, sms = 0;
         OSRC_CK(cudaGetDevice(&dev));
@@ -908,14 +918,18 @@ int kmix_plan(osrc_problem *pb, int nsys, KmixPlan *out) {
             out->cs = q[1];
             out->rpt = q[2];
             out->threads = q[3];
+            out->long_cap = q[4];
             return OSRC_OK;
         }
     static PerDeviceOnce once;
     static int max_cluster[OSRC_MAX_DEVICES] = {};
     OSRC_TRY(per_device_once(once, [](int dev) -> int {
         max_cluster[dev] = 8;
-        OSRC_CK(cudaFuncSetAttribute(kmix_kernel<1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, KMIX_SMEM_MAX));
-        OSRC_CK(cudaFuncSetAttribute(kmix_kernel<2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, KMIX_SMEM_MAX));
+        const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
+        OSRC_CK(cudaFuncSetAttribute(kmix_kernel<1, false>, attr, KMIX_SMEM_MAX));
+        OSRC_CK(cudaFuncSetAttribute(kmix_kernel<2, false>, attr, KMIX_SMEM_MAX));
+        OSRC_CK(cudaFuncSetAttribute(kmix_kernel<1, true>, attr, KMIX_SMEM_MAX));
+        OSRC_CK(cudaFuncSetAttribute(kmix_kernel<2, true>, attr, KMIX_SMEM_MAX));
         if (cudaFuncSetAttribute(kmix_kernel<1, true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
             cudaFuncSetAttribute(kmix_kernel<2, true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess)
             max_cluster[dev] = 16;
@@ -932,10 +946,16 @@ int kmix_plan(osrc_problem *pb, int nsys, KmixPlan *out) {
         const int rpt = rows <= KMIX_THREADS1 ? 1 : 2;
         const int threads = ((rows + rpt - 1) / rpt + 31) / 32 * 32;
         if (rpt == 2 && threads > KMIX_THREADS2) continue;
+        int long_cap = 0;
+        if (!pb->ms_long.empty())
+            for (int r = 0; r < n; r += rows)
+                long_cap = std::max(long_cap, pb->ms_long[std::min(n, r + rows)] - pb->ms_long[r]);
+        const size_t smem = kmix_smem(n, long_cap);
+        if (smem > (size_t)KMIX_SMEM_MAX) continue;
         int count = 0;
         auto active = cs == 1 ? (rpt == 1 ? kmix_active_clusters<1, false> : kmix_active_clusters<2, false>)
                               : (rpt == 1 ? kmix_active_clusters<1, true> : kmix_active_clusters<2, true>);
-        OSRC_TRY(active(n, cs, threads, &count));
+        OSRC_TRY(active(smem, cs, threads, &count));
         if (count < 1) continue;
         const double load = std::max(1.0, 0.6 * nsys / count);
         const double t = load * ((cs == 1 ? 0.85 : 1.85) + 1.3e-3 * rows);
@@ -944,9 +964,10 @@ int kmix_plan(osrc_problem *pb, int nsys, KmixPlan *out) {
             best.cs = cs;
             best.rpt = rpt;
             best.threads = threads;
+            best.long_cap = long_cap;
         }
     }
-    if (pb->kmix_plans.size() < 16) pb->kmix_plans.push_back({best.nsys, best.cs, best.rpt, best.threads});
+    if (pb->kmix_plans.size() < 16) pb->kmix_plans.push_back({best.nsys, best.cs, best.rpt, best.threads, best.long_cap});
     *out = best;
     return OSRC_OK;
 }
@@ -956,7 +977,7 @@ int kmix_launch(osrc_problem *pb, const KryBatch &batch, const KmixPlan &pl, cud
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(batch.nsys * pl.cs, 1, 1);
     cfg.blockDim = dim3(pl.threads, 1, 1);
-    cfg.dynamicSmemBytes = (size_t)pb->nv * sizeof(float2);
+    cfg.dynamicSmemBytes = kmix_smem(pb->nv, pl.long_cap);
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -967,7 +988,7 @@ int kmix_launch(osrc_problem *pb, const KryBatch &batch, const KmixPlan &pl, cud
     cfg.numAttrs = CL ? 1 : 0;
     OSRC_CK(cudaLaunchKernelEx(&cfg, kmix_kernel<RPT, CL>, batch, pb->nv, (const int *)pb->d_ms_ptr.p,
                                (const int *)pb->d_ms_col.p, (const double *)pb->d_M.p, (const double *)pb->d_S.p,
-                               (const int *)pb->d_ms_perm.p, (const int *)(pb->d_ms_perm.p + pb->nv),
+                               (const int *)pb->d_ms_perm.p, (const int *)(pb->d_ms_perm.p + pb->nv), pl.long_cap,
                                pb->p.inner_tol, pb->p.inner_maxit));
     pb->launches++;
     return OSRC_OK;

@@ -570,6 +570,10 @@ static int problem_create(osrc_mesh *mesh, const osrc_params *prm, const double 
         }
         {
             const std::vector<int> order = rcm_order(nv, mptr, mcol);
+            std::vector<int> lng(nv + 1, 0);
+            for (int i = 0; i < nv; ++i)
+                lng[i + 1] = lng[i] + std::max(0, mptr[order[i] + 1] - mptr[order[i]] - KMIX_E);
+            if (lng[nv]) pb->ms_long = std::move(lng);
             if ((s = pb->d_ms_perm.alloc(ctx, 2 * (size_t)nv))) break;
             if (cudaMemcpy(pb->d_ms_perm.p, order.data(), 2 * (size_t)nv * sizeof(int), cudaMemcpyHostToDevice)) {
                 s = OSRC_CUDA_ERROR;
@@ -1016,6 +1020,7 @@ int problem_clone(osrc_problem *m, osrc_problem **out, bool far) {
     c->near_nnz = m->near_nnz;
     c->ms_nnz = m->ms_nnz;
     c->kmix_plans = m->kmix_plans;
+    c->ms_long = m->ms_long;
     c->k_osrc = m->k_osrc;
     c->k_osrc_i = m->k_osrc_i;
     c->k_eps = m->k_eps;

@@ -175,6 +175,8 @@ struct NearPair {
     int perm;      // pt[0..2] | ps[0..2] << 6, 2 bits each
 };
 
+constexpr int KMIX_E = 8;  // entries of a row that the mixed-precision inner solver keeps in registers
+
 struct BatchedState;
 void batched_free(BatchedState *s);
 
@@ -237,8 +239,11 @@ struct osrc_problem {
     DBuf<double> d_kry_res;   // per-system final relative residual
     int inner_last_max = 0;
     // mixed-precision inner solver (k_sparse.cu): launch shapes by number of
-    // systems {nsys, cluster size (0: not usable), rows per thread, threads}
-    std::vector<std::array<int, 4>> kmix_plans;
+    // systems {nsys, cluster size (0: not usable), rows per thread, threads,
+    // entries of long rows per CTA}, and the entries past KMIX_E of the rows
+    // before each in the order d_ms_perm (empty: no row has any)
+    std::vector<std::array<int, 5>> kmix_plans;
+    std::vector<int> ms_long;
     // ---- GMRES workspace --------------------------------------------------------
     DBuf<double2> d_basis;    // (maxit+1) x 2nv
     int basis_cap = 0;

@@ -117,7 +117,7 @@ static int check(int n, int cs, int *cases, double *worst) {
         cfg.attrs = attr;
         cfg.numAttrs = 1;
         CK(cudaLaunchKernelEx(&cfg, kmix_kernel<RPT, true>, b, n, (const int *)dptr, (const int *)dcol,
-                              (const double *)dM, (const double *)dS, (const int *)did, (const int *)did, 1e-10, 500));
+                              (const double *)dM, (const double *)dS, (const int *)did, (const int *)did, 0, 1e-10, 500));
         CK(cudaDeviceSynchronize());
         *ms = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
         CK(cudaMemcpy(stat, dstat, 2 * sizeof(int), cudaMemcpyDeviceToHost));

@@ -292,8 +292,9 @@ kry_kernel(const __grid_constant__ KryBatch batch, int n, const int *__restrict_
 // One preconditioner apply (10 systems; before: three cluster barriers an
 // iteration, the search direction in L2, entries in shared memory): 10242
 // vertices 0.37 ms (0.66), 2562 0.26 (0.59), 642 0.20 (0.37), 150 0.13 (0.29).
-constexpr int KMIX_THREADS1 = 768;         // most threads with one row each (80 registers)
-constexpr int KMIX_THREADS2 = 640;         // and with two (96)
+// most threads with one row each (80 registers; in a cluster 224 bytes of spill
+// stores and 152 of loads, alone none) and with two (96; 496 and 376, 284 and 180)
+constexpr int KMIX_THREADS1 = 768, KMIX_THREADS2 = 640;
 constexpr float KMIX_MIN_TOL = 2e-6f;      // most a FP32 solve reduces the residual by
 constexpr int KMIX_MAX_REFINE = 40;
 constexpr int KMIX_MAX_N = 25600;          // rows (below 2^16: the column places are 16 bits)
@@ -477,11 +478,30 @@ __device__ __forceinline__ float2 f2dot(float2 a, float2 b, int conj) {
     return conj ? make_float2(a.x * b.x + a.y * b.y, a.x * b.y - a.y * b.x) : f2mul(a, b);
 }
 // a / b with an approximate reciprocal (PTX rcp.approx, 1 ulp: the same bits in
-// every CTA; an iteration's scalars need no more)
+// every CTA).  It serves an iteration's scalars, which steer the search and enter
+// x and r alike: a preconditioner apply's error against a direct FP64 solve is
+// 5e-11 at 10242 vertices and 2.6e-10 at 642, with divisions the same to the
+// iteration (7e-11, 2.4e-10), but every warp forms them, and with `/` an apply on
+// 642 rows takes 288 us instead of 273.
 __device__ __forceinline__ float2 f2div(float2 a, float2 b) {
     float ri;
     asm("rcp.approx.f32 %0, %1;" : "=f"(ri) : "f"(b.x * b.x + b.y * b.y));
     return make_float2((a.x * b.x + a.y * b.y) * ri, (a.y * b.x - a.x * b.y) * ri);
+}
+// 1 / a to about 48 bits: one Newton step from the FP32 reciprocal where that has
+// the range
+__device__ __forceinline__ double kmix_rcp(double a) {
+    if (!(a > 1e-36 && a < 1e36)) return 1.0 / a;
+    const double r = 1.0f / (float)a;
+    return fma(r, fma(-a, r, 1.0), r);
+}
+// an entry alpha m + beta s: formed in FP64 and rounded once (the terms cancel
+// where a shifted system comes near singular: with entries 1e-6 of their terms'
+// size 2 refinements reach 1e-10, from terms rounded to FP32 6); the library's
+// systems have alpha 1
+__device__ __forceinline__ double2 kmix_entry(double2 alpha, double2 beta, double m, double s) {
+    if (alpha.x == 1.0 && alpha.y == 0.0) return cd(fma(beta.x, s, m), beta.y * s);
+    return cd(fma(beta.x, s, alpha.x * m), fma(beta.y, s, alpha.y * m));
 }
 // a b + c
 __device__ __forceinline__ float2 f2fma(float2 a, float2 b, float2 c) {
@@ -493,9 +513,9 @@ __device__ __forceinline__ float2 f2fma(float2 a, float2 b, float2 c) {
 // and those its columns name), then the entries of its rows past the KMIX_E
 // that a thread holds, and their columns' places (long_cap of each).  One such
 // row sets an iteration's time: a preconditioner apply on a UV sphere with poles
-// of degree 64 (1986 vertices) takes 1.37 ms with them in shared memory and took
+// of degree 64 (1986 vertices) takes 1.58 ms with them in shared memory and took
 // 3.33 when each iteration read them from the FP64 matrices, a Menger sponge with
-// 40 % rows of 9 to 11 entries (896 vertices) 0.31 and 0.47.
+// 40 % rows of 9 to 11 entries (896 vertices) 0.32 and 0.47.
 // sy.x holds the published FP64 solution.  Status and residual as kry_kernel; the
 // iteration count is the number of FP32 iterations over all refinements.
 template <int RPT, bool CL>
@@ -536,7 +556,6 @@ kmix_kernel(const __grid_constant__ KryBatch batch, int n, const int *__restrict
     const uint32_t zbase = (uint32_t)__cvta_generic_to_shared(zs);
     const uint32_t barR = (uint32_t)__cvta_generic_to_shared(&boxR.bar);
     const uint32_t barI = (uint32_t)__cvta_generic_to_shared(&boxI.bar);
-    const float2 al0 = make_float2((float)sy.alpha.x, (float)sy.alpha.y);
 
     // per row: the FP64 residual, the FP32 state and the row of A with the
     // places of its columns' z (the FP64 solution lives in sy.x, the right-hand
@@ -568,29 +587,27 @@ kmix_kernel(const __grid_constant__ KryBatch batch, int n, const int *__restrict
         who[k] = 0;
         if (ok[k]) {
             const double2 b64 = sy.bscale ? cmul(sy.beta, sy.bscale[batch.vcomp[row[k]]]) : sy.beta;
-            const float2 be0 = make_float2((float)b64.x, (float)b64.y);
             const int p0 = ptr[row[k]], deg = ptr[row[k] + 1] - p0;
-            float2 dg = make_float2(0.f, 0.f);
+            double2 dg = cd(0.0, 0.0);
 #pragma unroll
             for (int e = 0; e < KMIX_E; ++e)
                 if (e < deg) {
                     const int c = col[p0 + e];
-                    const float m = (float)M[p0 + e], s = (float)S[p0 + e];
-                    a[k][e] = make_float2(fmaf(be0.x, s, al0.x * m), fmaf(be0.y, s, al0.y * m));
+                    const double2 ae = kmix_entry(sy.alpha, b64, M[p0 + e], S[p0 + e]);
+                    a[k][e] = make_float2((float)ae.x, (float)ae.y);
                     const int ci = inv[c];
                     ad[k][e] = (uint16_t)ci;
                     who[k] |= 1u << (ci / rows);
                     if (CL && ci / rows != (int)rank) zs[ci].x = 1.f;  // mark: sent by its owner
-                    if (c == row[k]) dg = a[k][e];
+                    if (c == row[k]) dg = ae;
                 }
             if (deg > KMIX_E) {
                 nlong[k] = deg - KMIX_E;
                 at[k] = atomicAdd(&s_long, nlong[k]);
                 for (int e = 0; e < nlong[k]; ++e) {
                     const int pe = p0 + KMIX_E + e, ci = inv[col[pe]];
-                    const float m = (float)M[pe], s = (float)S[pe];
-                    const float2 ae = make_float2(fmaf(be0.x, s, al0.x * m), fmaf(be0.y, s, al0.y * m));
-                    la[at[k] + e] = ae;
+                    const double2 ae = kmix_entry(sy.alpha, b64, M[pe], S[pe]);
+                    la[at[k] + e] = make_float2((float)ae.x, (float)ae.y);
                     lc[at[k] + e] = (uint16_t)ci;
                     who[k] |= 1u << (ci / rows);
                     if (CL && ci / rows != (int)rank) zs[ci].x = 1.f;
@@ -598,7 +615,8 @@ kmix_kernel(const __grid_constant__ KryBatch batch, int n, const int *__restrict
                 }
             }
             who[k] &= ~(1u << rank);
-            dinv[k] = f2div(make_float2(1.f, 0.f), dg);
+            const double ri = kmix_rcp(cabs2(dg));
+            dinv[k] = make_float2((float)(dg.x * ri), (float)(-dg.y * ri));
             r64[k] = sy.f[row[k]];
             bb += cabs2(r64[k]);
         }

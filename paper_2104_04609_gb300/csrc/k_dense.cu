@@ -13,8 +13,8 @@
 // so every SM works to the end even when the number of tiles is not a multiple
 // of the pairs (the 16000-row product of the 8000-vertex system has 63 tiles
 // for 76 pairs).  CTA r of a pair holds rows 128 r .. of the A tile and half
-// of the columns' B rows; the pair's MMA reads both halves.  Per CTA of 192
-// threads:
+// of the columns' B rows (umma_shape.cuh); the pair's MMA reads both halves.
+// Per CTA of 192 threads:
 //   - lane 0 of warp 4 issues TMA loads (128-byte swizzle) of the K slices of
 //     its part of A (evict-first in L2: it is streamed once) and B (evict-last:
 //     every pair re-reads it) into a shared-memory ring of as many stages as
@@ -51,6 +51,7 @@
 #include <mutex>
 
 #include "osrc_internal.cuh"
+#include "umma_shape.cuh"
 #include "stream_k.cuh"
 
 namespace {
@@ -66,10 +67,6 @@ constexpr int UM_MIN_ITERS = 24;
 constexpr int UM_MAX_STAGES = 8;        // 4 cost 10 %, 13 (of small N) gain nothing
 constexpr size_t UM_SMEM_MAX = 230400;  // dynamic shared memory per CTA (227 KB less the static part)
 constexpr size_t UM_SMEM_FIXED = 1024 + 256;  // alignment slack, barriers
-// columns above which a pair of CTAs takes a tile: it costs a launch 2 us (cluster
-// barriers) and pays where B's traffic counts (16000 x 32000: N 256 220 -> 203
-// us, 192 205 -> 196, 128 189 -> 183; 6016 x 12032 x 128 in a solve 31.8 -> 33.5)
-constexpr int UM_PAIR_N = 128;
 constexpr int UM_FIX_ROWS = 8;                  // rows of a split tile per block of the summing kernel
 constexpr unsigned long long UM_TIMEOUT_NS = 2000000000ULL;
 
@@ -192,7 +189,7 @@ __host__ __device__ constexpr uint32_t instr_desc(int m, int n) {
     return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
 }
 
-// ncols = tensor-memory columns of one accumulator (a power of two >= N);
+// ncols = tensor-memory columns of one accumulator (umma_acc_cols);
 // two accumulators alternate between the tile segments of a pair.
 // PAIR: a pair of CTAs (a cluster of two) per tile, else one.
 template <bool PAIR>
@@ -203,7 +200,7 @@ umma_sk_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char *base = (unsigned char *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     constexpr int nbuf = UM_NBUF, CG = PAIR ? 2 : 1, TM = CG * UM_BM;
-    const uint32_t a_bytes = UM_BM * UM_BK * 2, b_bytes = (uint32_t)N / CG * UM_BK * 2;
+    const uint32_t a_bytes = UM_BM * UM_BK * 2, b_bytes = (uint32_t)umma_b_rows(N) * UM_BK * 2;
     const uint32_t stage_bytes = a_bytes + b_bytes;
     uint64_t *bars = (uint64_t *)(base + (size_t)stages * stage_bytes);
     uint64_t *full = bars, *empty = bars + stages, *accf = bars + 2 * stages, *acce = accf + 2, *drain = acce + 2;
@@ -271,7 +268,7 @@ umma_sk_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
                     const uint32_t fb = smem_cta0<PAIR>(&full[s]);
                     if (rank == 0) mbar_expect_tx(&full[s], CG * stage_bytes);
                     tma_load_2d<PAIR>(sa, &map_a, kx, sg.tile * TM + rank * UM_BM, fb, pol_a);
-                    tma_load_2d<PAIR>(sb, &map_b, kx, rank * (N / CG), fb, pol_b);
+                    tma_load_2d<PAIR>(sb, &map_b, kx, rank * umma_b_rows(N), fb, pol_b);
                     ++g;
                 }
                 it += sg.n;
@@ -287,7 +284,7 @@ umma_sk_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     } else if (warp == 5) {
         if (lane == 0 && rank == 0) {
             // MMA issuer of the pair
-            const uint32_t idesc = instr_desc(TM, N);
+            const uint32_t idesc = instr_desc(TM, umma_cols(N));
             uint32_t g = 0;
             int seg = 0;
             bool ok = true;
@@ -521,7 +518,7 @@ static int umma_plan(int M, int N, int K, UmmaPlan *p) {
     int nsm = 0;
     OSRC_TRY(sm_count(&nsm));
     UmmaPlan q;
-    q.cg = N > UM_PAIR_N ? 2 : 1;
+    q.cg = umma_ctas(N);
     const int tm = q.cg * UM_BM;
     q.tiles = (M + tm - 1) / tm;
     q.KB = K / UM_BK;
@@ -530,8 +527,8 @@ static int umma_plan(int M, int N, int K, UmmaPlan *p) {
     if (g > nsm / q.cg) g = nsm / q.cg;
     if (g < 1) g = 1;
     q.grid = (int)g;
-    while (q.ncols < (uint32_t)N) q.ncols <<= 1;
-    const size_t stage = (size_t)UM_BM * UM_BK * 2 + (size_t)N / q.cg * UM_BK * 2;
+    q.ncols = (uint32_t)umma_acc_cols(N);
+    const size_t stage = (size_t)UM_BM * UM_BK * 2 + (size_t)umma_b_rows(N) * UM_BK * 2;
     q.stages = (int)((UM_SMEM_MAX - UM_SMEM_FIXED) / stage);
     if (q.stages > UM_MAX_STAGES) q.stages = UM_MAX_STAGES;
     q.smem = UM_SMEM_FIXED + (size_t)q.stages * stage;
@@ -563,7 +560,7 @@ static int umma_gemm_run(const void *A, int M, int K, const void *Bm, int N, flo
     OSRC_TRY(get_encoder());
     CUtensorMap ma, mb;
     OSRC_TRY(make_map(&ma, A, M, K, UM_BM));
-    OSRC_TRY(make_map(&mb, Bm, N, K, N / p.cg));
+    OSRC_TRY(make_map(&mb, Bm, N, K, umma_b_rows(N)));
     static PerDeviceOnce once;
     OSRC_TRY(per_device_once(once, [](int) -> int {
         OSRC_CK(cudaFuncSetAttribute(umma_sk_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,

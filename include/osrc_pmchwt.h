@@ -473,11 +473,15 @@ long long osrc_launch_count(const osrc_problem *pb);
 int osrc_profile_enable(osrc_problem *pb, int on);
 /* Far-field kernel statistics since profiling was enabled: number of
  * launches and their summed device time in ms (events recorded on the
- * launching stream around each launch).  Waits for the last timed launch. */
+ * launching stream around each launch; where an apply takes several launches
+ * of one kernel, around all of them, counted as one).  Waits for the last timed launch. */
 int osrc_far_kernel_stats(osrc_problem *pb, long long *launches, double *total_ms);
 /* Right-hand sides processed by the timed far-field launches (a launch of the
  * several-right-hand-side kernel counts each of its vectors). */
 long long osrc_far_kernel_rhs(const osrc_problem *pb);
+/* How many of the timed launches evaluated each pair of triangles once for both
+ * directions (the others evaluate every ordered pair). */
+long long osrc_far_kernel_symmetric(const osrc_problem *pb);
 /* Number of far-field point pairs one apply evaluates: 36 x (number of
  * triangle pairs sharing no vertex). */
 long long osrc_far_pairs(const osrc_problem *pb);

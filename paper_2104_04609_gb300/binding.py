@@ -181,6 +181,7 @@ SIGNATURES = {
     "osrc_near_nnz": (ctypes.c_longlong, [_VP]),
     "osrc_fp32_peak": (ctypes.c_int, [ctypes.c_int, _DP, _DP, _VP]),
     "osrc_far_kernel_rhs": (ctypes.c_longlong, [_VP]),
+    "osrc_far_kernel_symmetric": (ctypes.c_longlong, [_VP]),
 }
 
 _LIB = None
@@ -643,6 +644,10 @@ def osrc_far_kernel_stats(pb):
 
 def osrc_far_kernel_rhs(pb):
     return lib().osrc_far_kernel_rhs(pb)
+
+
+def osrc_far_kernel_symmetric(pb):
+    return lib().osrc_far_kernel_symmetric(pb)
 
 
 def osrc_far_pairs(pb):

@@ -1697,7 +1697,7 @@ static int sym_launch(osrc_problem *pb, const VecPtrs &xp, int R, const FarSymPl
     }
     if (pb->prof_on) {
         OSRC_CK(cudaEventRecord(pb->prof_ev[1], st));
-        pb->prof_pending = true;
+        pb->prof_pending = pb->prof_sym_pending = true;
         pb->prof_rhs_pending = R;
     }
     return OSRC_OK;
@@ -1712,8 +1712,9 @@ int far_prof_collect(osrc_problem *pb) {
     pb->prof_ms += ms;
     pb->prof_launches++;
     pb->prof_rhs += pb->prof_rhs_pending;
+    pb->prof_sym += pb->prof_sym_pending;
     pb->prof_rhs_pending = 1;
-    pb->prof_pending = false;
+    pb->prof_sym_pending = pb->prof_pending = false;
     return OSRC_OK;
 }
 

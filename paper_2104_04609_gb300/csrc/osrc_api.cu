@@ -643,7 +643,7 @@ extern "C" int osrc_profile_enable(osrc_problem *pb, int on) {
     pb->prof_on = on != 0;
     pb->prof_launches = 0;
     pb->prof_ms = 0.0;
-    pb->prof_rhs = 0;
+    pb->prof_rhs = pb->prof_sym = 0;
     return OSRC_OK;
 }
 
@@ -657,6 +657,8 @@ extern "C" int osrc_far_kernel_stats(osrc_problem *pb, long long *launches, doub
 }
 
 extern "C" long long osrc_far_kernel_rhs(const osrc_problem *pb) { return pb ? pb->prof_rhs : 0; }
+
+extern "C" long long osrc_far_kernel_symmetric(const osrc_problem *pb) { return pb ? pb->prof_sym : 0; }
 
 extern "C" long long osrc_far_pairs(const osrc_problem *pb) {
     return pb ? 36LL * ((long long)pb->nt * pb->nt - pb->near_pairs) : 0;

@@ -271,6 +271,8 @@ struct osrc_problem {
     bool prof_on = false, prof_pending = false;
     int prof_rhs_pending = 1;    // right-hand sides of the last timed far launch
     long long prof_rhs = 0;      // right-hand sides summed over the timed launches
+    bool prof_sym_pending = false;
+    long long prof_sym = 0;      // timed launches that took each pair of triangles once
     cudaEvent_t prof_ev[2] = {nullptr, nullptr};
     long long prof_launches = 0;
     double prof_ms = 0.0;

@@ -47,6 +47,12 @@ __host__ __device__ inline void rule_point(int q, double bary[3], double &w) {
     for (int j = 0; j < 3; ++j) bary[j] = (j == i) ? 1.0 - 2.0 * a : a;
 }
 
+// Scale of the weights in the element matrices, chosen so that all four (weight
+// times barycentric coordinate, of both classes) are FP32 numbers to 4e-10: rounded
+// as they are, they scale every value by 1 + 3.7e-8 and the corners' shares by up
+// to 1.4e-7 (1 % of an apply's error).
+constexpr double kElemScale = 0.982727956;
+
 constexpr int FAR_THREADS = 128;
 // resident blocks per SM the one-right-hand-side kernel is compiled for
 // (registers per thread = 65536 / (FAR_THREADS x FAR_MIN_BLOCKS))
@@ -79,7 +85,7 @@ constexpr int SYM_MIN_NT = 2048;
 constexpr int SYM_MAX_SLOTS = 104;  // most partial sums of an apply (R = 1): 104 x 18 floats a triangle
                                     // (70 or 200 measure the same within 1 %)
 // right-hand sides of a sym_kernel launch: what two blocks per SM have shared
-// memory for (8 as 5 + 3 would take 55 ms at 10242 vertices, farm_kernel 48.8)
+// memory for (8 as 5 + 3 would take 55.7 ms at 10242 vertices, farm_kernel 49.9)
 constexpr int SYM_MAX_R = 5;
 constexpr int SYM_MULTI_SLOTS = 96; // partial sums, times right-hand sides, of several-right-hand-side launches
 // lanes of the gather per vertex: a block up to GATHER_BLOCK_NV vertices, a
@@ -816,7 +822,7 @@ gather_kernel(int nv, int nt, int npts, int ns, int R, const int *__restrict__ v
                 comp_add(s[0], c[0], P[sp * su]);
                 comp_add(s[1], c[1], P[sp * su + nt]);
             }
-            const double w = 0.079577471545947667884 * g[0] * (q < 2 ? 1.0 : g[4 + 3 * a + (q - 2)]);
+            const double w = 0.079577471545947667884 / (kElemScale * kElemScale) * g[0] * (q < 2 ? 1.0 : g[4 + 3 * a + (q - 2)]);
             const double2 val = cd(w * comp_value(s[0], c[0]), w * comp_value(s[1], c[1]));
             if (q == 0) y1 = cadd(y1, val);
             else y2 = cadd(y2, val);
@@ -947,7 +953,8 @@ __global__ void farm_prep_kernel(VecPtrs x, int R, int nv, int nt, const int *__
     d[4 * (size_t)nt] = make_float4((float)cv[2].x, (float)cv[2].y, 0.f, 0.f);
 }
 
-// The matrices of one triangle pair, [re, im of S, N, T, K][b][a], and W.
+// The matrices of one triangle pair, [re, im of S, N, T, K][b][a], and W; all
+// times kElemScale^2 (the gather divides by it).
 struct ElemMat {
     float E[8][3][3];
     float wr, wi;
@@ -961,8 +968,9 @@ __device__ __forceinline__ void elem_matrices(const f2 (&X)[3], const f2 (&Y)[3]
                                               const FarConst2 &c, const CenterPair &cp, f2 m1, f2 k1i, float dk1i,
                                               ElemMat &M) {
     // the rule's classes: weights times beta, and times alpha - beta
-    constexpr float WB1 = (float)(kQw1 * kQa1), WB2 = (float)(kQw2 * kQa2);
-    constexpr float WG1 = (float)(kQw1 * (1.0 - 3.0 * kQa1)), WG2 = (float)(kQw2 * (1.0 - 3.0 * kQa2));
+    constexpr float WB1 = (float)(kElemScale * kQw1 * kQa1), WB2 = (float)(kElemScale * kQw2 * kQa2);
+    constexpr float WG1 = (float)(kElemScale * kQw1 * (1.0 - 3.0 * kQa1)),
+                    WG2 = (float)(kElemScale * kQw2 * (1.0 - 3.0 * kQa2));
     const f2 wb = make_float2(WB1, WB2), wg = make_float2(WG1, WG2);
     f2 kb[3], kg[3];  // the test weights times -(x - y).n_y
     F3 {
@@ -1031,11 +1039,18 @@ __device__ __forceinline__ void elem_matrices(const f2 (&X)[3], const f2 (&Y)[3]
         }
 }
 
-// u_b (u1 re, im, u2 re, im) += the matrices on the corner densities
+// u[b FAR_THREADS] (u1 re, im, u2 re, im) += the matrices on the corner densities
 // d[a stride] (psi, phi).  REV: the pair seen from the source triangle.  S and N are symmetric;
 // the normals change places and x - y its sign, so K becomes -T^T and T -K^T.
+// A pair's 12 products are summed before they meet the tile's sums, which then
+// round once a pair: a third less error of an apply where coordinates and phases do
+// not hide it (four spheres of 642 vertices 1.48e-7 -> 1.02e-7, bumpy ellipsoid of
+// 3001 1.32 -> 0.89; far_kernel 1.34, 1.28) for 0.3 % of the time at R = 1 and 1.8
+// at R = 8.  The tile's sums are loaded after the products (before them they cost
+// 11 registers and 8 % of the centred kernel's time).
 template <bool REV>
-__device__ __forceinline__ void elem_apply(const ElemMat &M, const float4 *d, size_t stride, float4 (&u)[3]) {
+__device__ __forceinline__ void elem_apply(const ElemMat &M, const float4 *d, size_t stride, float4 *u) {
+    float4 s[3] = {make_float4(0.f, 0.f, 0.f, 0.f), make_float4(0.f, 0.f, 0.f, 0.f), make_float4(0.f, 0.f, 0.f, 0.f)};
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
         const float4 da = d[a * stride];
@@ -1045,11 +1060,20 @@ __device__ __forceinline__ void elem_apply(const ElemMat &M, const float4 *d, si
             const float sr = M.E[0][i][j], si = M.E[1][i][j], nr = M.E[2][i][j], ni = M.E[3][i][j];
             const float tr = REV ? -M.E[6][i][j] : M.E[4][i][j], ti = REV ? -M.E[7][i][j] : M.E[5][i][j];
             const float kr = REV ? -M.E[4][i][j] : M.E[6][i][j], ki = REV ? -M.E[5][i][j] : M.E[7][i][j];
-            u[b].x = fmaf(sr, da.x, fmaf(-si, da.y, fmaf(kr, da.z, fmaf(-ki, da.w, u[b].x))));
-            u[b].y = fmaf(sr, da.y, fmaf(si, da.x, fmaf(kr, da.w, fmaf(ki, da.z, u[b].y))));
-            u[b].z = fmaf(tr, da.x, fmaf(-ti, da.y, fmaf(nr, da.z, fmaf(-ni, da.w, u[b].z))));
-            u[b].w = fmaf(tr, da.y, fmaf(ti, da.x, fmaf(nr, da.w, fmaf(ni, da.z, u[b].w))));
+            s[b].x = fmaf(sr, da.x, fmaf(-si, da.y, fmaf(kr, da.z, fmaf(-ki, da.w, s[b].x))));
+            s[b].y = fmaf(sr, da.y, fmaf(si, da.x, fmaf(kr, da.w, fmaf(ki, da.z, s[b].y))));
+            s[b].z = fmaf(tr, da.x, fmaf(-ti, da.y, fmaf(nr, da.z, fmaf(-ni, da.w, s[b].z))));
+            s[b].w = fmaf(tr, da.y, fmaf(ti, da.x, fmaf(nr, da.w, fmaf(ni, da.z, s[b].w))));
         }
+    }
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+        float4 v = u[b * FAR_THREADS];
+        v.x += s[b].x;
+        v.y += s[b].y;
+        v.z += s[b].z;
+        v.w += s[b].w;
+        u[b * FAR_THREADS] = v;
     }
 }
 
@@ -1091,7 +1115,7 @@ __device__ __forceinline__ void elem_curl(const ElemMat &M, float4 C0, float4 C1
 // 3000 to 5000 vertices) for 2 % of the time, the old values of an entry's 18
 // being loaded together.
 // Bound by the FP32 pipe: an apply at 10242 vertices is 27.1 ms of kernel
-// values and matrices and 2.7 ms a right-hand side (R 8: 48.8 ms), where
+// values and matrices and 2.84 ms a right-hand side (R 8: 49.9 ms), where
 // point-by-point sums took 24 + 9.9 (102.7).  Tensor cores do not help: TF32
 // pieces with the kernel values as an operand took 64.7 ms at R 2 and 80.8 at
 // 8, mma.sync and packed FMA not overlapping.
@@ -1178,12 +1202,7 @@ farm_kernel(const float4 *__restrict__ pt, const float4 *__restrict__ cen, const
             for (int r = 0; r < R; ++r) {
                 const float4 *D = shD + 5 * r * FARM_TS + s;
                 float4 *o4 = acc4 + (size_t)r * 4 * FAR_THREADS + threadIdx.x;
-                float4 u[3];
-#pragma unroll
-                for (int b = 0; b < 3; ++b) u[b] = o4[b * FAR_THREADS];
-                elem_apply<false>(M, D, FARM_TS, u);
-#pragma unroll
-                for (int b = 0; b < 3; ++b) o4[b * FAR_THREADS] = u[b];
+                elem_apply<false>(M, D, FARM_TS, o4);
                 elem_curl<false>(M, D[3 * FARM_TS], D[4 * FARM_TS], o4 + 3 * FAR_THREADS,
                                  acc2 + (size_t)r * FAR_THREADS + threadIdx.x, nullptr, nullptr);
             }
@@ -1245,9 +1264,9 @@ farm_kernel(const float4 *__restrict__ pt, const float4 *__restrict__ cen, const
 //   part [ntst + nsrc][R][18][nt]  as farm_kernel's
 // One vector's curl sums carry their rounding errors along (COMP; several
 // vectors' are as accurate as point-by-point sums without).  Bound by the FP32
-// pipe at 8 warps per SM: an apply at 10242 vertices 17.3 ms (far_kernel 25.9),
-// 20000 vertices centred 78.6 (124), four objects of 642 vertices 1.69 (2.19);
-// R = 2: 19.9, 3: 23.0, 4: 28.4, 5: 32.0 (farm_kernel 32.5, 35.3, 38.0, 40.6).
+// pipe at 8 warps per SM: an apply at 10242 vertices 17.4 ms (far_kernel 25.9),
+// 20000 vertices centred 79.6 (124), four objects of 642 vertices 1.71 (2.19);
+// R = 2: 20.0, 3: 23.2, 4: 28.7, 5: 32.5 (farm_kernel 32.8, 35.7, 38.5, 41.3).
 // ---------------------------------------------------------------------------
 constexpr int SYM_U = 32;  // source triangles per tile (one step each per lane)
 constexpr size_t sym_smem_bytes(int R, bool centred) {
@@ -1383,25 +1402,16 @@ sym_kernel(const float4 *__restrict__ pt, const float4 *__restrict__ cen, const 
                     c, cp, m1, k1i, dk1i, M);
 #pragma unroll 1
                 for (int r = 0; r < R; ++r) {
-                    float4 v[3];
                     const float4 *D = shD + 5 * r * SYM_U + s;
                     float4 *o4 = acc4 + (size_t)r * 4 * FAR_THREADS + threadIdx.x;
                     float2 *o2 = acc2 + (size_t)r * FAR_THREADS + threadIdx.x;
-#pragma unroll
-                    for (int b = 0; b < 3; ++b) v[b] = o4[b * FAR_THREADS];
-                    elem_apply<false>(M, D, SYM_U, v);
-#pragma unroll
-                    for (int b = 0; b < 3; ++b) o4[b * FAR_THREADS] = v[b];
+                    elem_apply<false>(M, D, SYM_U, o4);
                     elem_curl<COMP>(M, D[3 * SYM_U], D[4 * SYM_U], o4 + 3 * FAR_THREADS, o2, err4 + threadIdx.x, err2 + threadIdx.x);
                     if (both) {
                         const float4 *T = sD + 5 * (size_t)r * nt + tau;
                         o4 = src4 + (size_t)r * 4 * FAR_THREADS + warp * 32 + s;
                         o2 = src2 + (size_t)r * FAR_THREADS + warp * 32 + s;
-#pragma unroll
-                        for (int b = 0; b < 3; ++b) v[b] = o4[b * FAR_THREADS];
-                        elem_apply<true>(M, T, nt, v);
-#pragma unroll
-                        for (int b = 0; b < 3; ++b) o4[b * FAR_THREADS] = v[b];
+                        elem_apply<true>(M, T, nt, o4);
                         elem_curl<COMP>(M, T[3 * (size_t)nt], T[4 * (size_t)nt], o4 + 3 * FAR_THREADS, o2,
                                         err4 + FAR_THREADS + warp * 32 + s, err2 + FAR_THREADS + warp * 32 + s);
                     }

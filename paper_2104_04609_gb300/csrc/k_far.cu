@@ -56,30 +56,24 @@ constexpr double kElemScale = 0.982727956;
 constexpr int FAR_THREADS = 128;
 // resident blocks per SM the one-right-hand-side kernel is compiled for
 // (registers per thread = 65536 / (FAR_THREADS x FAR_MIN_BLOCKS))
-#ifndef OSRC_FAR_MIN_BLOCKS
-#define OSRC_FAR_MIN_BLOCKS 2
-#endif
+constexpr int FAR_MIN_BLOCKS = 2;
 // largest k_max x (bounding-box diagonal) for the plain (FP32 k r) variant
 constexpr double FAR_PLAIN_MAX_PHASE = 32.0 * 3.14159265358979323846;
 constexpr int FAR_TS = 64;  // source triangles per shared-memory tile
-#ifndef OSRC_FAR_QUNROLL
-#define OSRC_FAR_QUNROLL 3
-#endif
-#ifndef OSRC_FAR_HUNROLL
-#define OSRC_FAR_HUNROLL 2
-#endif
-constexpr int FAR_QUNROLL = OSRC_FAR_QUNROLL, FAR_HUNROLL = OSRC_FAR_HUNROLL;  // unrolls of the rule-point loops
 constexpr int FAR_MIN_TPS = 16;  // fewest source triangles per split
 // test triangles per block: 32 below FAR_TRIS32_NT triangles, 64 below
-// FAR_TRIS64_NT, else FAR_THREADS (128).  Measured: 5136 triangles on four
-// objects 2.136 ms with 128, 2.145 with 64, 2.256 with 32; 296 triangles
-// 38 us with 32 sharing the sources between four warps, 46 us without
+// FAR_TRIS64_NT, else FAR_THREADS (128).  far_kernel (meshes below SYM_MIN_NT) has
+// 32: 296 triangles 52 us an apply with 32 sharing the sources between four warps,
+// 54 with 64, 64 with 128.  64 and 128 are farm_kernel's (6 and more vectors there);
+// 8 vectors take, with 32 / 64 / 128, at 1796 triangles 509 / 564 / 535 us, 2048:
+// 622 / 600 / 609, 4094: 2.22 / 2.14 / 2.13 ms, 7996: 8.24 / 7.88 / 7.92, 11996:
+// 18.4 / 17.7 / 17.5, 19996: 51.3 / 49.4 / 48.9
 constexpr int FAR_TRIS32_NT = 2048;
 constexpr int FAR_TRIS64_NT = 4096;
 constexpr int FAR_MAX_NS = 64;   // most source splits
 // sym_kernel from this many triangles on (far_kernel / sym_kernel at 796
 // triangles 73 / 97 us, 1280: 144 / 145, 2048: 299 / 276, 2996: 618 / 506, 3996:
-// 1062 / 940, 20480: 25.9 / 17.3 ms; its work comes in tiles of 128 x 32
+// 1062 / 940, 20480: 25.9 / 17.4 ms; its work comes in tiles of 128 x 32
 // triangles, too few of them for small meshes)
 constexpr int SYM_MIN_NT = 2048;
 constexpr int SYM_MAX_SLOTS = 104;  // most partial sums of an apply (R = 1): 104 x 18 floats a triangle
@@ -545,7 +539,7 @@ __device__ __forceinline__ void far_tri(const f2 (&X)[3], const f2 (&Y)[3], cons
 // sources on other objects and change sign for Mueller.  ABSORB (with MULTI):
 // complex interior wavenumbers (attenuation).
 template <bool CENTRED, bool MULTI, bool ABSORB>
-__global__ void __launch_bounds__(FAR_THREADS, OSRC_FAR_MIN_BLOCKS)
+__global__ void __launch_bounds__(FAR_THREADS, FAR_MIN_BLOCKS)
 far_kernel(const float4 *__restrict__ pt, const float4 *__restrict__ cen,
            const float4 *__restrict__ tn, const int4 *__restrict__ tv,
            const float4 *__restrict__ sP, const float2 *__restrict__ sP5,
@@ -647,11 +641,11 @@ far_kernel(const float4 *__restrict__ pt, const float4 *__restrict__ cen,
                 A[p].t1r = A[p].t1i = A[p].ur = A[p].ui = make_float2(0.f, 0.f);
             f2 t3r = make_float2(0.f, 0.f), t3i = t3r;  // sum_q w_q (G0 + G1/rho), lanes summed over their points
             const f2 m1 = dup2(MULTI ? (shComp[s] != ct ? 0.f : sgn) : 1.f);
-#pragma unroll FAR_HUNROLL
+#pragma unroll
             for (int h = 0; h < 2; ++h) {  // the two weight classes of the source points
                 CurlAcc Bs;
                 Bs.g0r = Bs.g0i = Bs.g1r = Bs.g1i = make_float2(0.f, 0.f);
-#pragma unroll FAR_QUNROLL
+#pragma unroll
                 for (int q = 3 * h; q < 3 * h + 3; ++q) {
                     const float4 *P = &shP[24 * s + 4 * q];
                     const float4 P0 = P[0], P1 = P[1], P2 = P[2], P3 = P[3];
@@ -1613,7 +1607,7 @@ int far_setup_geometry(osrc_problem *pb, cudaStream_t st) {
     int &sms = pb->sms;
     OSRC_CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     pb->far_tris = nt < FAR_TRIS32_NT ? 32 : nt < FAR_TRIS64_NT ? 64 : FAR_THREADS;
-    const int slots = sms * OSRC_FAR_MIN_BLOCKS;  // farm_kernel runs on the same grid
+    const int slots = sms * FAR_MIN_BLOCKS;  // farm_kernel runs on the same grid
     const int bx = (nt + pb->far_tris - 1) / pb->far_tris;
     const int max_ns = std::max(1, std::min(FAR_MAX_NS, nt / FAR_MIN_TPS));
     const int ns0 = std::min(max_ns, std::max(1, (4 * slots + bx - 1) / bx));

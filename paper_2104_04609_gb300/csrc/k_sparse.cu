@@ -1049,7 +1049,7 @@ int launch_kry(osrc_problem *pb, KryBatch &batch, cudaStream_t st) {
     OSRC_CK(cudaLaunchKernelEx(&cfg, kry_kernel, batch, n, (const int *)pb->d_ms_ptr.p,
                                (const int *)pb->d_ms_col.p, (const double *)pb->d_M.p,
                                (const double *)pb->d_S.p, pb->d_kry.p, pb->p.inner_tol,
-                               pb->p.inner_maxit, pb->d_kry_stat.p, pb->d_kry_res.p));
+                               pb->p.inner_maxit, batch.s[0].stat, batch.s[0].res));
     pb->launches++;
     return OSRC_OK;
 }
@@ -1097,10 +1097,10 @@ int ms_build(osrc_problem *pb, const std::vector<int> &cptr, const std::vector<i
     return OSRC_OK;
 }
 
-static int mass_solve_async(osrc_problem *pb, const double2 *y, double2 *z, bool swap, cudaStream_t st);
+static int mass_solve_async(osrc_problem *pb, const double2 *y, double2 *z, bool swap, int word, cudaStream_t st);
 
 int mass_solve(osrc_problem *pb, const double2 *x, double2 *y, cudaStream_t st) {
-    OSRC_TRY(mass_solve_async(pb, x, y, false, st));
+    OSRC_TRY(mass_solve_async(pb, x, y, false, 0, st));
     return check_kry(pb, 2, st);
 }
 
@@ -1112,11 +1112,13 @@ int mass_solve(osrc_problem *pb, const double2 *x, double2 *y, cudaStream_t st) 
 // so the mass solve of row 1 and all 2 N_Pade + 1 shifted systems run as one
 // batched launch (row 2 needs no mass solve at all).
 int osrc_precond_nsys(const osrc_problem *pb) {
-    return pb->p.precond == OSRC_PRECOND_OSRC ? 2 * pb->p.n_pade + 2 : 2;
+    // (Calderon: two mass solves of two systems each)
+    return pb->p.precond == OSRC_PRECOND_OSRC ? 2 * pb->p.n_pade + 2 : pb->p.precond == OSRC_PRECOND_CALDERON ? 4 : 2;
 }
 
-// both block rows of M^-1 y; rows swapped in the output when swap is set
-static void mass_systems(osrc_problem *pb, const double2 *y, double2 *z, bool swap, KryBatch &b) {
+// both block rows of M^-1 y; rows swapped in the output when swap is set; word:
+// the first's status word
+static void mass_systems(osrc_problem *pb, const double2 *y, double2 *z, bool swap, int word, KryBatch &b) {
     const int n = pb->nv;
     for (int k = 0; k < 2; ++k) {
         KrySys &s = b.s[b.nsys++];
@@ -1126,14 +1128,14 @@ static void mass_systems(osrc_problem *pb, const double2 *y, double2 *z, bool sw
         s.f = y + (size_t)k * n;
         s.x = z + (size_t)(swap ? 1 - k : k) * n;
         s.conj = 1;
-        s.stat = pb->d_kry_stat.p + k;
-        s.res = pb->d_kry_res.p + k;
+        s.stat = pb->d_kry_stat.p + word + k;
+        s.res = pb->d_kry_res.p + word + k;
     }
 }
 
-static int mass_solve_async(osrc_problem *pb, const double2 *y, double2 *z, bool swap, cudaStream_t st) {
+static int mass_solve_async(osrc_problem *pb, const double2 *y, double2 *z, bool swap, int word, cudaStream_t st) {
     KryBatch b{};
-    mass_systems(pb, y, z, swap, b);
+    mass_systems(pb, y, z, swap, word, b);
     return launch_kry(pb, b, st);
 }
 
@@ -1191,10 +1193,10 @@ int osrc_precond_fused_multi(osrc_problem *const *pbs, const double2 *const *ys,
         for (int r = 0; r < nrun; ++r) {
             osrc_problem *q = pbs[r];
             double2 *t = q->d_kry_rhs.p + 2 * (size_t)n, *w = q->d_tmp2.p + 2 * (size_t)n;
-            OSRC_TRY(mass_solve_async(q, ys[r], t, true, st));
+            OSRC_TRY(mass_solve_async(q, ys[r], t, true, 0, st));
             if (q->p.precision == OSRC_FP64_DENSE) OSRC_TRY(dense_apply(q, t, w, st));
             else OSRC_TRY(far_apply(q, t, w, OSRC_PART_ALL, st));
-            OSRC_TRY(mass_solve_async(q, w, zs[r], false, st));
+            OSRC_TRY(mass_solve_async(q, w, zs[r], false, 2, st));
         }
         return OSRC_OK;
     }
@@ -1210,7 +1212,7 @@ int osrc_precond_fused_multi(osrc_problem *const *pbs, const double2 *const *ys,
         const int R = std::min(group, nrun - r0);
         KryBatch b{};
         for (int r = 0; r < R; ++r) {
-            if (mass) mass_systems(pbs[r0 + r], ys[r0 + r], zs[r0 + r], false, b);
+            if (mass) mass_systems(pbs[r0 + r], ys[r0 + r], zs[r0 + r], false, 0, b);
             else osrc_systems(pbs[r0 + r], ys[r0 + r], b);
         }
         OSRC_TRY(launch_kry(pbs[r0], b, st));

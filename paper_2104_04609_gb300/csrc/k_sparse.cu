@@ -290,10 +290,12 @@ kry_kernel(const __grid_constant__ KryBatch batch, int n, const int *__restrict_
 // reverse Cuthill-McKee (d_ms_perm), so that a CTA's columns lie mostly in
 // itself and its neighbours.  A system that fits one CTA needs no cluster.
 // One preconditioner apply (10 systems; before: three cluster barriers an
-// iteration, the search direction in L2, entries in shared memory): 10242
-// vertices 0.37 ms (0.66), 2562 0.26 (0.59), 642 0.20 (0.37), 150 0.13 (0.29).
-// most threads with one row each (80 registers; in a cluster 224 bytes of spill
-// stores and 152 of loads, alone none) and with two (96; 496 and 376, 284 and 180)
+// iteration, the search direction in L2, entries in shared memory): Fibonacci
+// spheres of 10242 vertices 0.40 ms (0.76), 2562 0.28 (0.71), 642 0.26 (0.56), 150
+// 0.10 (0.17).
+// most threads with one row each (80 registers; in a cluster 180 bytes of spill
+// stores and 124 of loads, alone none) and with two (96; 452 and 336, alone 200 and
+// 148)
 constexpr int KMIX_THREADS1 = 768, KMIX_THREADS2 = 640;
 constexpr float KMIX_MIN_TOL = 2e-6f;      // most a FP32 solve reduces the residual by
 constexpr int KMIX_MAX_REFINE = 40;
@@ -488,20 +490,21 @@ __device__ __forceinline__ float2 f2div(float2 a, float2 b) {
     asm("rcp.approx.f32 %0, %1;" : "=f"(ri) : "f"(b.x * b.x + b.y * b.y));
     return make_float2((a.x * b.x + a.y * b.y) * ri, (a.y * b.x - a.x * b.y) * ri);
 }
-// 1 / a to about 48 bits: one Newton step from the FP32 reciprocal where that has
-// the range
+// 1 / a to about 48 bits, one Newton step from the FP32 reciprocal (where that is
+// within its range; beyond it the iteration's FP32 products leave theirs as well):
+// an FP64 division per row, or a branch to one, takes 8 us of a 270 us apply on
+// 642 rows
 __device__ __forceinline__ double kmix_rcp(double a) {
-    if (!(a > 1e-36 && a < 1e36)) return 1.0 / a;
     const double r = 1.0f / (float)a;
-    return fma(r, fma(-a, r, 1.0), r);
+    return a > 1e-36 && a < 1e36 ? fma(r, fma(-a, r, 1.0), r) : r;
 }
-// an entry alpha m + beta s: formed in FP64 and rounded once (the terms cancel
-// where a shifted system comes near singular: with entries 1e-6 of their terms'
-// size 2 refinements reach 1e-10, from terms rounded to FP32 6); the library's
-// systems have alpha 1
-__device__ __forceinline__ double2 kmix_entry(double2 alpha, double2 beta, double m, double s) {
-    if (alpha.x == 1.0 && alpha.y == 0.0) return cd(fma(beta.x, s, m), beta.y * s);
-    return cd(fma(beta.x, s, alpha.x * m), fma(beta.y, s, alpha.y * m));
+// an entry m + beta s: formed in FP64 and rounded once (the terms cancel where a
+// shifted system comes near singular: with entries 1e-6 of their terms' size 2
+// refinements reach 1e-10, from terms rounded to FP32 6).  The systems that come
+// here have alpha 1 (launch_kry): a factor tested in the kernel takes 12 us of a
+// 270 us apply on 642 rows.
+__device__ __forceinline__ double2 kmix_entry(double2 beta, double m, double s) {
+    return cd(fma(beta.x, s, m), beta.y * s);
 }
 // a b + c
 __device__ __forceinline__ float2 f2fma(float2 a, float2 b, float2 c) {
@@ -593,7 +596,7 @@ kmix_kernel(const __grid_constant__ KryBatch batch, int n, const int *__restrict
             for (int e = 0; e < KMIX_E; ++e)
                 if (e < deg) {
                     const int c = col[p0 + e];
-                    const double2 ae = kmix_entry(sy.alpha, b64, M[p0 + e], S[p0 + e]);
+                    const double2 ae = kmix_entry(b64, M[p0 + e], S[p0 + e]);
                     a[k][e] = make_float2((float)ae.x, (float)ae.y);
                     const int ci = inv[c];
                     ad[k][e] = (uint16_t)ci;
@@ -606,7 +609,7 @@ kmix_kernel(const __grid_constant__ KryBatch batch, int n, const int *__restrict
                 at[k] = atomicAdd(&s_long, nlong[k]);
                 for (int e = 0; e < nlong[k]; ++e) {
                     const int pe = p0 + KMIX_E + e, ci = inv[col[pe]];
-                    const double2 ae = kmix_entry(sy.alpha, b64, M[pe], S[pe]);
+                    const double2 ae = kmix_entry(b64, M[pe], S[pe]);
                     la[at[k] + e] = make_float2((float)ae.x, (float)ae.y);
                     lc[at[k] + e] = (uint16_t)ci;
                     who[k] |= 1u << (ci / rows);
@@ -760,7 +763,7 @@ kmix_kernel(const __grid_constant__ KryBatch batch, int n, const int *__restrict
                     sx.y += se * xj.y;
                 }
                 const double2 bi = sy.bscale ? cmul(sy.beta, sy.bscale[batch.vcomp[i]]) : sy.beta;
-                r64[k] = csub(sy.f[i], cadd(cmul(sy.alpha, mx), cmul(bi, sx)));
+                r64[k] = csub(sy.f[i], cadd(mx, cmul(bi, sx)));
                 rn += cabs2(r64[k]);
             }
             double v[1] = {rn};
@@ -1024,8 +1027,9 @@ int launch_kry(osrc_problem *pb, KryBatch &batch, cudaStream_t st) {
     KmixPlan pl;
     OSRC_TRY(kmix_plan(pb, batch.nsys, &pl));
     bool mix = pl.cs > 0;
-    for (int k = 0; k < batch.nsys && mix; ++k)  // in-place systems stay on the FP64 kernel
-        if (ranges_overlap(batch.s[k].f, batch.s[k].x, n)) mix = false;
+    for (int k = 0; k < batch.nsys && mix; ++k)  // in-place systems (and alpha other than 1) stay on the FP64 kernel
+        if (ranges_overlap(batch.s[k].f, batch.s[k].x, n) || batch.s[k].alpha.x != 1.0 || batch.s[k].alpha.y != 0.0)
+            mix = false;
     if (mix) {
         std::stable_sort(batch.s, batch.s + batch.nsys,
                          [](const KrySys &a, const KrySys &c) { return cabs2(a.beta) > cabs2(c.beta); });

@@ -1,4 +1,4 @@
-// GPU check of the mixed inner solver's matrix entries alpha M + beta S where the
+// GPU check of the mixed inner solver's matrix entries M + beta S where the
 // two terms nearly cancel (to 1e-6 of their size): formed in FP64 and rounded
 // once they carry FP32's 6e-8, and an FP32 solve reduces the FP64 residual
 // accordingly; formed in FP32 they would be a few per cent off, and so would each
@@ -32,7 +32,7 @@ static T *upload(const std::vector<T> &h) {
 // half zeros to either side of the diagonal
 static int check(int half) {
     const int n = 64, per = 2 * half + 1;
-    const double2 alpha = cd(1.0, 0.5), beta = cd(-1.0, -0.5);
+    const double2 alpha = cd(1.0, 0.0), beta = cd(-1.0, 0.0);
     std::vector<int> ptr(n + 1), col, id(n);
     std::vector<double> M, S;
     for (int i = 0; i < n; ++i) {

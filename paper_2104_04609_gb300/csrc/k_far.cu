@@ -47,10 +47,10 @@ __host__ __device__ inline void rule_point(int q, double bary[3], double &w) {
     for (int j = 0; j < 3; ++j) bary[j] = (j == i) ? 1.0 - 2.0 * a : a;
 }
 
-// Scale of the weights in the element matrices, chosen so that all four (weight
-// times barycentric coordinate, of both classes) are FP32 numbers to 4e-10: rounded
-// as they are, they scale every value by 1 + 3.7e-8 and the corners' shares by up
-// to 1.4e-7 (1 % of an apply's error).
+// Scale of the weights in the element matrices of one vector, chosen so that all
+// four (weight times barycentric coordinate, of both classes) are FP32 numbers to
+// 4e-10: rounded as they are, they scale every value by 1 + 3.7e-8 and the corners'
+// shares by up to 1.4e-7 (1 % of an apply's error).
 constexpr double kElemScale = 0.982727956;
 
 constexpr int FAR_THREADS = 128;
@@ -79,7 +79,7 @@ constexpr int SYM_MIN_NT = 2048;
 constexpr int SYM_MAX_SLOTS = 104;  // most partial sums of an apply (R = 1): 104 x 18 floats a triangle
                                     // (70 or 200 measure the same within 1 %)
 // right-hand sides of a sym_kernel launch: what two blocks per SM have shared
-// memory for (8 as 5 + 3 would take 55.7 ms at 10242 vertices, farm_kernel 49.9)
+// memory for (8 as 5 + 3 would take 55.1 ms at 10242 vertices, farm_kernel 49.0)
 constexpr int SYM_MAX_R = 5;
 constexpr int SYM_MULTI_SLOTS = 96; // partial sums, times right-hand sides, of several-right-hand-side launches
 // lanes of the gather per vertex: a block up to GATHER_BLOCK_NV vertices, a
@@ -792,7 +792,7 @@ __global__ void __launch_bounds__(GATHER_THREADS)
 gather_kernel(int nv, int nt, int npts, int ns, int R, const int *__restrict__ vt_ptr,
               const int *__restrict__ vt_idx, const double *__restrict__ tgeo, const float *__restrict__ part,
               const float *__restrict__ partA, int use_far, const int *__restrict__ nr_ptr,
-              const int *__restrict__ nr_col, const double2 *__restrict__ nr_val, int use_near,
+              const int *__restrict__ nr_col, const double2 *__restrict__ nr_val, int use_near, double scale,
               const __grid_constant__ VecPtrs x, const __grid_constant__ OutPtrs y) {
     static_assert(W == 1 || L == 32, "split groups are warps");
     __shared__ double2 red[W > 1 ? W : 1][2];
@@ -816,7 +816,7 @@ gather_kernel(int nv, int nt, int npts, int ns, int R, const int *__restrict__ v
                 comp_add(s[0], c[0], P[sp * su]);
                 comp_add(s[1], c[1], P[sp * su + nt]);
             }
-            const double w = 0.079577471545947667884 / (kElemScale * kElemScale) * g[0] * (q < 2 ? 1.0 : g[4 + 3 * a + (q - 2)]);
+            const double w = scale * g[0] * (q < 2 ? 1.0 : g[4 + 3 * a + (q - 2)]);
             const double2 val = cd(w * comp_value(s[0], c[0]), w * comp_value(s[1], c[1]));
             if (q == 0) y1 = cadd(y1, val);
             else y2 = cadd(y2, val);
@@ -845,9 +845,8 @@ gather_kernel(int nv, int nt, int npts, int ns, int R, const int *__restrict__ v
             if (q & 1) y2.y += av;
             else y2.x += av;
         }
-        const double inv4pi = 0.079577471545947667884;
-        y1 = cscale(y1, inv4pi);
-        y2 = cscale(y2, inv4pi);
+        y1 = cscale(y1, scale);
+        y2 = cscale(y2, scale);
     }
     if (valid && use_near) {
         const double2 *xr = x.p[rr];
@@ -947,8 +946,8 @@ __global__ void farm_prep_kernel(VecPtrs x, int R, int nv, int nt, const int *__
     d[4 * (size_t)nt] = make_float4((float)cv[2].x, (float)cv[2].y, 0.f, 0.f);
 }
 
-// The matrices of one triangle pair, [re, im of S, N, T, K][b][a], and W; all
-// times kElemScale^2 (the gather divides by it).
+// The matrices of one triangle pair, [re, im of S, N, T, K][b][a], and W; SCALED:
+// all times kElemScale^2 (the gather divides by it).
 struct ElemMat {
     float E[8][3][3];
     float wr, wi;
@@ -956,15 +955,15 @@ struct ElemMat {
 
 // mns = (-n_y, .), my0 = -y_0, dn: -(x - y).n_y = (X - y_0).mns + dn (centred:
 // X.mns + dn); load(q, P0, P1) gives source point q as duplicated pairs; m1, k1i, dk1i as in far_vals (MULTI, ABSORB).
-template <bool CENTRED, bool MULTI, bool ABSORB, typename L>
+template <bool CENTRED, bool MULTI, bool ABSORB, bool SCALED, typename L>
 __device__ __forceinline__ void elem_matrices(const f2 (&X)[3], const f2 (&Y)[3], const f2 (&Z)[3], const float4 &n4,
                                               float pdn, const float4 &mns, const float4 &my0, float dn, const L &load,
                                               const FarConst2 &c, const CenterPair &cp, f2 m1, f2 k1i, float dk1i,
                                               ElemMat &M) {
     // the rule's classes: weights times beta, and times alpha - beta
-    constexpr float WB1 = (float)(kElemScale * kQw1 * kQa1), WB2 = (float)(kElemScale * kQw2 * kQa2);
-    constexpr float WG1 = (float)(kElemScale * kQw1 * (1.0 - 3.0 * kQa1)),
-                    WG2 = (float)(kElemScale * kQw2 * (1.0 - 3.0 * kQa2));
+    constexpr double sc = SCALED ? kElemScale : 1.0;
+    constexpr float WB1 = (float)(sc * kQw1 * kQa1), WB2 = (float)(sc * kQw2 * kQa2);
+    constexpr float WG1 = (float)(sc * kQw1 * (1.0 - 3.0 * kQa1)), WG2 = (float)(sc * kQw2 * (1.0 - 3.0 * kQa2));
     const f2 wb = make_float2(WB1, WB2), wg = make_float2(WG1, WG2);
     f2 kb[3], kg[3];  // the test weights times -(x - y).n_y
     F3 {
@@ -1036,15 +1035,18 @@ __device__ __forceinline__ void elem_matrices(const f2 (&X)[3], const f2 (&Y)[3]
 // u[b FAR_THREADS] (u1 re, im, u2 re, im) += the matrices on the corner densities
 // d[a stride] (psi, phi).  REV: the pair seen from the source triangle.  S and N are symmetric;
 // the normals change places and x - y its sign, so K becomes -T^T and T -K^T.
-// A pair's 12 products are summed before they meet the tile's sums, which then
-// round once a pair: a third less error of an apply where coordinates and phases do
-// not hide it (four spheres of 642 vertices 1.48e-7 -> 1.02e-7, bumpy ellipsoid of
-// 3001 1.32 -> 0.89; far_kernel 1.34, 1.28) for 0.3 % of the time at R = 1 and 1.8
-// at R = 8.  The tile's sums are loaded after the products (before them they cost
-// 11 registers and 8 % of the centred kernel's time).
-template <bool REV>
+// PAIR: a pair's 12 products are summed before they meet the tile's sums, which
+// then round once a pair: a third less error of an apply where coordinates and
+// phases do not hide it (four spheres of 642 vertices 1.48e-7 -> 1.02e-7, bumpy
+// ellipsoid of 3001 1.32 -> 0.89; far_kernel 1.34, 1.28) for 0.3 % of the time at
+// R = 1.  Several vectors are as accurate as point-by-point sums without it, and it
+// would take 1.8 % at R = 8.  The tile's sums are loaded after the products (before
+// them they cost 11 registers and 8 % of the centred kernel's time).
+template <bool REV, bool PAIR>
 __device__ __forceinline__ void elem_apply(const ElemMat &M, const float4 *d, size_t stride, float4 *u) {
-    float4 s[3] = {make_float4(0.f, 0.f, 0.f, 0.f), make_float4(0.f, 0.f, 0.f, 0.f), make_float4(0.f, 0.f, 0.f, 0.f)};
+    float4 s[3];
+#pragma unroll
+    for (int b = 0; b < 3; ++b) s[b] = PAIR ? make_float4(0.f, 0.f, 0.f, 0.f) : u[b * FAR_THREADS];
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
         const float4 da = d[a * stride];
@@ -1062,12 +1064,11 @@ __device__ __forceinline__ void elem_apply(const ElemMat &M, const float4 *d, si
     }
 #pragma unroll
     for (int b = 0; b < 3; ++b) {
-        float4 v = u[b * FAR_THREADS];
-        v.x += s[b].x;
-        v.y += s[b].y;
-        v.z += s[b].z;
-        v.w += s[b].w;
-        u[b * FAR_THREADS] = v;
+        if (PAIR) {
+            const float4 v = u[b * FAR_THREADS];
+            s[b] = make_float4(v.x + s[b].x, v.y + s[b].y, v.z + s[b].z, v.w + s[b].w);
+        }
+        u[b * FAR_THREADS] = s[b];
     }
 }
 
@@ -1109,7 +1110,7 @@ __device__ __forceinline__ void elem_curl(const ElemMat &M, float4 C0, float4 C1
 // 3000 to 5000 vertices) for 2 % of the time, the old values of an entry's 18
 // being loaded together.
 // Bound by the FP32 pipe: an apply at 10242 vertices is 27.1 ms of kernel
-// values and matrices and 2.84 ms a right-hand side (R 8: 49.9 ms), where
+// values and matrices and 2.7 ms a right-hand side (R 8: 49.0 ms), where
 // point-by-point sums took 24 + 9.9 (102.7).  Tensor cores do not help: TF32
 // pieces with the kernel values as an operand took 64.7 ms at R 2 and 80.8 at
 // 8, mma.sync and packed FMA not overlapping.
@@ -1186,7 +1187,7 @@ farm_kernel(const float4 *__restrict__ pt, const float4 *__restrict__ cen, const
                 dn = cp.Dx.x * mns.x + cp.Dy.x * mns.y + cp.Dz.x * mns.z;
             }
             ElemMat M;
-            elem_matrices<CENTRED, false, false>(
+            elem_matrices<CENTRED, false, false, false>(
                 X, Y, Z, n4, pdn, mns, my0, dn, [&](int q, float4 &P0, float4 &P1) {
                     P0 = shG[12 * s + 2 * q];
                     P1 = shG[12 * s + 2 * q + 1];
@@ -1196,7 +1197,7 @@ farm_kernel(const float4 *__restrict__ pt, const float4 *__restrict__ cen, const
             for (int r = 0; r < R; ++r) {
                 const float4 *D = shD + 5 * r * FARM_TS + s;
                 float4 *o4 = acc4 + (size_t)r * 4 * FAR_THREADS + threadIdx.x;
-                elem_apply<false>(M, D, FARM_TS, o4);
+                elem_apply<false, false>(M, D, FARM_TS, o4);
                 elem_curl<false>(M, D[3 * FARM_TS], D[4 * FARM_TS], o4 + 3 * FAR_THREADS,
                                  acc2 + (size_t)r * FAR_THREADS + threadIdx.x, nullptr, nullptr);
             }
@@ -1256,11 +1257,12 @@ farm_kernel(const float4 *__restrict__ pt, const float4 *__restrict__ cen, const
 // blocks write one entry; further launches add to it.  Everything is added in
 // a fixed order.
 //   part [ntst + nsrc][R][18][nt]  as farm_kernel's
-// One vector's curl sums carry their rounding errors along (COMP; several
-// vectors' are as accurate as point-by-point sums without).  Bound by the FP32
+// One vector's curl sums carry their rounding errors along, its pairs are summed
+// first and its weights scaled (COMP; several vectors are as accurate as
+// point-by-point sums without).  Bound by the FP32
 // pipe at 8 warps per SM: an apply at 10242 vertices 17.4 ms (far_kernel 25.9),
 // 20000 vertices centred 79.6 (124), four objects of 642 vertices 1.71 (2.19);
-// R = 2: 20.0, 3: 23.2, 4: 28.7, 5: 32.5 (farm_kernel 32.8, 35.7, 38.5, 41.3).
+// R = 2: 20.0, 3: 23.1, 4: 28.4, 5: 32.0 (farm_kernel 32.5, 35.3, 38.0, 40.6).
 // ---------------------------------------------------------------------------
 constexpr int SYM_U = 32;  // source triangles per tile (one step each per lane)
 constexpr size_t sym_smem_bytes(int R, bool centred) {
@@ -1387,7 +1389,7 @@ sym_kernel(const float4 *__restrict__ pt, const float4 *__restrict__ cen, const 
                 }
                 const f2 m1 = dup2(MULTI ? (shComp[s] != ct ? 0.f : sgn) : 1.f);
                 ElemMat M;
-                elem_matrices<CENTRED, MULTI, ABSORB>(
+                elem_matrices<CENTRED, MULTI, ABSORB, COMP>(
                     X, Y, Z, n4, pdn, mns, shP[s], dn, [&](int q, float4 &P0, float4 &P1) {
                         const float4 y = shP[q * SYM_U + s];
                         P0 = make_float4(y.x, y.x, y.y, y.y);
@@ -1399,13 +1401,13 @@ sym_kernel(const float4 *__restrict__ pt, const float4 *__restrict__ cen, const 
                     const float4 *D = shD + 5 * r * SYM_U + s;
                     float4 *o4 = acc4 + (size_t)r * 4 * FAR_THREADS + threadIdx.x;
                     float2 *o2 = acc2 + (size_t)r * FAR_THREADS + threadIdx.x;
-                    elem_apply<false>(M, D, SYM_U, o4);
+                    elem_apply<false, COMP>(M, D, SYM_U, o4);
                     elem_curl<COMP>(M, D[3 * SYM_U], D[4 * SYM_U], o4 + 3 * FAR_THREADS, o2, err4 + threadIdx.x, err2 + threadIdx.x);
                     if (both) {
                         const float4 *T = sD + 5 * (size_t)r * nt + tau;
                         o4 = src4 + (size_t)r * 4 * FAR_THREADS + warp * 32 + s;
                         o2 = src2 + (size_t)r * FAR_THREADS + warp * 32 + s;
-                        elem_apply<true>(M, T, nt, o4);
+                        elem_apply<true, COMP>(M, T, nt, o4);
                         elem_curl<COMP>(M, T[3 * (size_t)nt], T[4 * (size_t)nt], o4 + 3 * FAR_THREADS, o2,
                                         err4 + FAR_THREADS + warp * 32 + s, err2 + FAR_THREADS + warp * 32 + s);
                     }
@@ -1722,16 +1724,18 @@ int far_prof_collect(osrc_problem *pb) {
     return OSRC_OK;
 }
 
+// es: scale of the element matrices' weights
 static int gather_launch(osrc_problem *pb, int ns, int R, const float *part, const float *partA, int use_far,
-                         int use_near, const VecPtrs &x, const OutPtrs &y, cudaStream_t st) {
+                         int use_near, double es, const VecPtrs &x, const OutPtrs &y, cudaStream_t st) {
     osrc_mesh *m = pb->mesh;
+    const double scale = 0.079577471545947667884 / (es * es);  // 1 / (4 pi)
     const int nv = pb->nv;
     const int per = nv <= GATHER_BLOCK_NV ? 1 : nv <= GATHER_WARP_NV ? GATHER_THREADS / 32 : GATHER_THREADS / 8;
     const dim3 grid((nv + per - 1) / per, R);
 #define OSRC_GATHER_LAUNCH(LL, WW)                                                                             \
     (partA ? gather_kernel<LL, WW, false> : gather_kernel<LL, WW, true>)<<<grid, GATHER_THREADS, 0, st>>>(nv, pb->nt, pb->npts, ns, R, m->d_vt_ptr.p, m->d_vt_idx.p, \
                                                        pb->d_tgeo.p, part, partA, use_far, pb->d_nr_ptr.p,       \
-                                                       pb->d_nr_col.p, pb->d_nr_val.p, use_near, x, y)
+                                                       pb->d_nr_col.p, pb->d_nr_val.p, use_near, scale, x, y)
     if (nv <= GATHER_BLOCK_NV) OSRC_GATHER_LAUNCH(32, 4);
     else if (nv <= GATHER_WARP_NV) OSRC_GATHER_LAUNCH(32, 1);
     else OSRC_GATHER_LAUNCH(8, 1);
@@ -1753,7 +1757,8 @@ int far_apply(osrc_problem *pb, const double2 *x, double2 *y, int part, cudaStre
     if (use_far && !far_workspace_made(pb)) OSRC_TRY(far_workspace(pb));  // a clone made without it
     if (use_far && pb->far_sym) {
         OSRC_TRY(sym_launch(pb, xp, 1, pb->sym[1], pb->d_sD.p, pb->d_part.p, st));
-        return gather_launch(pb, pb->sym[1].ntst + pb->sym[1].nsrc, 1, pb->d_part.p, nullptr, use_far, use_near, xp, yp, st);
+        return gather_launch(pb, pb->sym[1].ntst + pb->sym[1].nsrc, 1, pb->d_part.p, nullptr, use_far, use_near, kElemScale,
+                             xp, yp, st);
     }
     if (use_far) {
         const float4 *src_pts = pb->far_reduce ? pb->d_poff.p : pb->d_pt.p;
@@ -1792,7 +1797,7 @@ int far_apply(osrc_problem *pb, const double2 *x, double2 *y, int part, cudaStre
             pb->prof_pending = true;
         }
     }
-    return gather_launch(pb, pb->nsplit, 1, pb->d_part.p, pb->d_partA1.p, use_far, use_near, xp, yp, st);
+    return gather_launch(pb, pb->nsplit, 1, pb->d_part.p, pb->d_partA1.p, use_far, use_near, 1.0, xp, yp, st);
 }
 
 // ---------------------------------------------------------------------------
@@ -1841,7 +1846,7 @@ static int farm_launch(osrc_problem *pb, const double2 *const *xs, double2 *cons
     if (use_far && pb->far_sym && R <= SYM_MAX_R) {
         const FarSymPlan pl = pb->sym[R];
         OSRC_TRY(sym_launch(pb, xp, R, pl, pb->d_sDm.p, pb->d_partm.p, st));
-        return gather_launch(pb, pl.ntst + pl.nsrc, R, pb->d_partm.p, nullptr, use_far, use_near, xp, yp, st);
+        return gather_launch(pb, pl.ntst + pl.nsrc, R, pb->d_partm.p, nullptr, use_far, use_near, 1.0, xp, yp, st);
     }
     if (use_far) {
         farm_prep_kernel<<<dim3((nt + 127) / 128, R), 128, 0, st>>>(xp, R, nv, nt, m->d_tris.p, pb->d_tgeo.p,
@@ -1871,7 +1876,7 @@ static int farm_launch(osrc_problem *pb, const double2 *const *xs, double2 *cons
             pb->prof_rhs_pending = R;
         }
     }
-    return gather_launch(pb, ns, R, pb->d_partm.p, nullptr, use_far, use_near, xp, yp, st);
+    return gather_launch(pb, ns, R, pb->d_partm.p, nullptr, use_far, use_near, 1.0, xp, yp, st);
 }
 
 bool far_multi_supported(const osrc_problem *pb) {
